@@ -34,7 +34,8 @@
 // stops when the Newton step is below half the eps tolerance.  Lanes that
 // finish take the next stencil from a global counter, so a warp stays full
 // until the work runs out.  Groups of different stencil size are processed
-// largest first in the same persistent launch.
+// largest first in the same persistent launch.  Node sets that do not fill the
+// chip with a lane per stencil take the same steps on teams of lanes (team.cu).
 //
 // Weights (Eqs. grad_x_f_interp, surface_lap_P1): only the first row of
 // L_P = sum_d G^d G^d is needed, so with A symmetric
@@ -42,40 +43,16 @@
 //   w = (A^{-1} [v; 0])[:n] / r_s^2,
 // four solves and one pass over the pairs, equal in exact arithmetic to
 // forming the full G^d (which the oracle does).
-#include "common.cuh"
 #include "dd.cuh"
+#include "stencil.cuh"
 
 #include <algorithm>
 #include <cmath>
 #include <mutex>
+#include <cstring>
 
 namespace rbffd {
 namespace {
-
-constexpr int LANCZOS_KMAX = 24;
-constexpr double LANCZOS_RTOL = 1e-6;       // relative change that stops a Lanczos run
-// The A^{-1} run never stops before this many steps: when the second
-// smallest |eigenvalue| of A is within a factor 0.6-0.9 of the smallest, the
-// top Ritz value can sit on the second one for several steps (the component
-// of lambda_min's eigenvector grows by (1 + 2 sqrt(gap))^k per step), and
-// stopping on a stalled value misjudges kappa by 10-40 %.
-constexpr int LANCZOS_KMIN = 10;
-constexpr double ACCEPT_MARGIN = 1e-4;      // shrink the accept band by this
-// Early acceptance of a learned first guess.  Every Ritz value of the A^{-1}
-// run is a lower bound of 1 / min|lambda(A)| (and the A run's of
-// max|lambda(A)|), so the running estimate k_j = lambda_max theta_j never
-// exceeds kappa: k_j >= accept_lo kappa_T already proves the lower edge.
-// The upper edge needs the run's shortfall bounded: over 1.5M first
-// evaluations (1M-node sphere, n = 31 / 50 / 70 / 101, and the held-out
-// bumpy sphere, n = 50) the smallest ratio theta_j / theta_final was 0.44 at
-// step 6, 0.74 at step 7, 0.93 at step 8 and 0.998 at step 9.  A guess is
-// accepted at step j when k_j <= f_j accept_hi kappa_T with f_6..f_9 =
-// 0.25, 0.45, 0.7, 0.85 (1.1-1.8x below the worst ratios seen); otherwise
-// the same run continues to its full length and the usual test decides.
-__host__ __device__ inline double early_accept_factor(int steps) {
-    return steps == 6 ? 0.25 : steps == 7 ? 0.45 : steps == 8 ? 0.7 : steps == 9 ? 0.85 : 0.0;
-}
-constexpr double F_FAIL = 60.0;         // F value used when Phi is not numerically SPD
 
 // ---------------------------------------------------------------------------
 // lane-private scratch, interleaved across the warp
@@ -99,8 +76,6 @@ __device__ __forceinline__ LaneF float_view(const Lane& S, int region) {
     const int lane = threadIdx.x & 31;
     return LaneF{reinterpret_cast<float*>(S.p - lane + (int64_t)region * 32) + lane};
 }
-
-__host__ __device__ inline int pk(int i, int j) { return i * (i + 1) / 2 + j; }
 
 struct Layout {
     int m;       // padded stencil size (multiple of 4)
@@ -142,32 +117,8 @@ __host__ __device__ inline Layout make_layout(int m, bool full) {
 }
 
 // ---------------------------------------------------------------------------
-// kernels phi(eps r) and psi(r) = phi'(r)/r as functions of e2r2 = (eps r)^2
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ double phi_of(int kernel, double e2r2) {
-    return kernel == RBFFD_GAUSSIAN ? exp(-e2r2) : rsqrt(1.0 + e2r2);
-}
-// psi in scaled units: Gaussian -2 eps^2 phi, IMQ -eps^2 phi^3
-__device__ __forceinline__ double psi_from_phi(int kernel, double e2, double ph) {
-    return kernel == RBFFD_GAUSSIAN ? -2.0 * e2 * ph : -e2 * ph * ph * ph;
-}
-// psi = psi_scale * psi_shape(phi): the pair pass of the weights sums
-// psi_shape terms and applies the constant factor once per entry
-__device__ __forceinline__ double psi_shape(int kernel, double ph) {
-    return kernel == RBFFD_GAUSSIAN ? ph : ph * ph * ph;
-}
-__device__ __forceinline__ double psi_scale(int kernel, double e2) {
-    return kernel == RBFFD_GAUSSIAN ? -2.0 * e2 : -e2;
-}
-
-// ---------------------------------------------------------------------------
 // stencil geometry: centre-translated, r_s-scaled coordinates and normals
 // ---------------------------------------------------------------------------
-struct Geo {
-    double rs;        // stencil radius (max distance to the centre)
-    double mean_d;    // mean scaled distance of the n-1 neighbours
-};
-
 __device__ Geo load_geometry(const Lane& S, const Layout& ly, int n, const int32_t* __restrict__ idx,
                              int64_t off, int npad, int64_t lr, const double* __restrict__ X,
                              const double* __restrict__ NR, bool with_normals) {
@@ -225,7 +176,7 @@ __device__ void assemble_phi(const Lane& S, const Layout& ly, int n, int kernel,
         int base = pk(i, 0);
         if (i < n) {
             for (int j = 0; j < i; ++j) {
-                double v = phi_of(kernel, e2 * S[ly.R2 + base + j]);
+                double v = phi_of(kernel, e2, S[ly.R2 + base + j]);
                 S[dst + base + j] = v;
                 if (cpy >= 0) S[cpy + base + j] = v;
                 if (fcpy >= 0) F[base + j] = (float)v;
@@ -458,104 +409,6 @@ __device__ void chol_solve(const Lane& S, const Layout& ly, int V) {
     chol_solve_multi<1>(S, ly, R);
 }
 
-// ---------------------------------------------------------------------------
-// extreme eigenvalues of a symmetric tridiagonal (float32 Sturm bisection)
-// ---------------------------------------------------------------------------
-__device__ int sturm_below(const float* a, const float* b2, int k, float x) {
-    int c = 0;
-    float d = a[0] - x;
-    if (d < 0.f) ++c;
-    for (int i = 1; i < k; ++i) {
-        if (d == 0.f) d = -1e-30f;
-        d = (a[i] - x) - b2[i - 1] / d;
-        if (d < 0.f) ++c;
-    }
-    return c;
-}
-
-// extreme eigenvalues of T (alpha[0..k-1], beta[0..k-2], scaled into
-// [-1, 1]); returns the one of largest magnitude, signed, in double units
-__device__ double tri_extreme(const float* a, const float* b2, int k, double scale) {
-    float lo = -1.f, hi = 1.f;
-    // top eigenvalue: count(x) < k  <=>  x <= lambda_max
-    for (int it = 0; it < 26; ++it) {
-        float mid = 0.5f * (lo + hi);
-        if (sturm_below(a, b2, k, mid) < k) lo = mid; else hi = mid;
-    }
-    float top = 0.5f * (lo + hi);
-    lo = -1.f; hi = 1.f;
-    // bottom eigenvalue: count(x) >= 1  <=>  x > lambda_min
-    for (int it = 0; it < 26; ++it) {
-        float mid = 0.5f * (lo + hi);
-        if (sturm_below(a, b2, k, mid) >= 1) hi = mid; else lo = mid;
-    }
-    float bot = 0.5f * (lo + hi);
-    return scale * (double)(fabsf(top) >= fabsf(bot) ? top : bot);
-}
-
-__device__ double tri_max_abs(const float* a, const float* b2, int k, double scale) {
-    return fabs(tri_extreme(a, b2, k, scale));
-}
-
-// Eigenvector y (unit) of the symmetric tridiagonal T for its eigenvalue
-// theta: two steps of inverse iteration, each a solve with T - theta I by
-// Gaussian elimination with partial pivoting (the factor has two
-// superdiagonals after row exchanges).
-__device__ void tri_eigvec(const double* al, const double* be, int k, double theta, double* y) {
-    double d[LANCZOS_KMAX], du[LANCZOS_KMAX], du2[LANCZOS_KMAX], dl[LANCZOS_KMAX];
-    bool sw[LANCZOS_KMAX];
-    double tmax = 0.0;
-    for (int i = 0; i < k; ++i) tmax = fmax(tmax, fabs(al[i] - theta) + (i < k - 1 ? fabs(be[i]) : 0.0));
-    const double tiny = 1e-30 * (tmax > 0.0 ? tmax : 1.0);
-    for (int i = 0; i < k; ++i) {
-        d[i] = al[i] - theta;
-        du[i] = i < k - 1 ? be[i] : 0.0;
-        dl[i] = i < k - 1 ? be[i] : 0.0;
-        du2[i] = 0.0;
-        sw[i] = false;
-    }
-    for (int i = 0; i < k - 1; ++i) {
-        if (fabs(d[i]) >= fabs(dl[i])) {
-            if (d[i] == 0.0) d[i] = tiny;
-            double f = dl[i] / d[i];
-            dl[i] = f;
-            d[i + 1] -= f * du[i];
-        } else {   // exchange rows i and i + 1
-            double f = d[i] / dl[i];
-            d[i] = dl[i];
-            dl[i] = f;
-            double t = du[i];
-            du[i] = d[i + 1];
-            d[i + 1] = t - f * d[i + 1];
-            if (i < k - 2) {
-                du2[i] = du[i + 1];
-                du[i + 1] = -f * du[i + 1];
-            }
-            sw[i] = true;
-        }
-    }
-    if (d[k - 1] == 0.0) d[k - 1] = tiny;
-    for (int i = 0; i < k; ++i) y[i] = 1.0;
-    for (int pass = 0; pass < 2; ++pass) {
-        for (int i = 0; i < k - 1; ++i) {
-            if (sw[i]) {
-                double t = y[i];
-                y[i] = y[i + 1];
-                y[i + 1] = t - dl[i] * y[i + 1];
-            } else {
-                y[i + 1] -= dl[i] * y[i];
-            }
-        }
-        y[k - 1] /= d[k - 1];
-        if (k > 1) y[k - 2] = (y[k - 2] - du[k - 2] * y[k - 1]) / d[k - 2];
-        for (int i = k - 3; i >= 0; --i) y[i] = (y[i] - du[i] * y[i + 1] - du2[i] * y[i + 2]) / d[i];
-        double nrm = 0.0;
-        for (int i = 0; i < k; ++i) nrm = fmax(nrm, fabs(y[i]));
-        double inv = nrm > 0.0 ? 1.0 / nrm : 1.0;
-        for (int i = 0; i < k; ++i) y[i] *= inv;
-    }
-}
-
 // y = Phi x in float32 from the packed float32 copy F of Phi, x and y at
 // float offsets x, y of V.  Rows in blocks of four (four independent FMA
 // chains; each x_j loaded once per block): columns left of the block from
@@ -681,18 +534,6 @@ __device__ double lanczos_max_f32(const Lane& S, const Layout& ly, int n, double
     return ext;
 }
 
-// splitmix64 (Steele, Lea, Flood 2014) mapped to [-1, 1): the pseudo-random
-// start vector of the A^{-1} Lanczos run, seeded per stencil, so that no
-// stencil's symmetry can leave it (nearly) orthogonal to the eigenvector of
-// lambda_min, as a fixed smooth start vector can be.
-__device__ inline double unit_hash(uint64_t x) {
-    x += 0x9E3779B97F4A7C15ull;
-    x = (x ^ (x >> 30)) * 0xBF58476D1CE4E5B9ull;
-    x = (x ^ (x >> 27)) * 0x94D049BB133111EBull;
-    x ^= x >> 31;
-    return (double)(x >> 11) * (2.0 / 9007199254740992.0) - 1.0;
-}
-
 // Start vector of the A^{-1} Lanczos run, normalised, in region QB (m
 // entries) with its border entry returned: the previous evaluation's Ritz
 // vector (region RV, border *vb) when warm, else the stencil's
@@ -768,18 +609,24 @@ __device__ double lanczos_inv_ritz(const Lane& S, const Layout& ly, int n, doubl
         alpha_d[j] = a;
         beta_d[j] = bn;
         k = j + 1;
-        double G = 0.0;
-        for (int i = 0; i <= j; ++i) {
-            double r = fabs(alpha_d[i]) + (i < j ? beta_d[i] : 0.0) + (i > 0 ? beta_d[i - 1] : 0.0);
-            G = fmax(G, r);
+        // the extreme eigenvalue, at the steps whose tests use it: the stops
+        // from kmin on (which compare with the step before) and the early
+        // acceptance
+        const bool last = bn <= 1e-14 * fabs(a) || j + 1 == LANCZOS_KMAX;
+        if (j + 1 >= kmin - 1 || last || (early && early_accept_factor(j + 1) > 0.0)) {
+            double G = 0.0;
+            for (int i = 0; i <= j; ++i) {
+                double r = fabs(alpha_d[i]) + (i < j ? beta_d[i] : 0.0) + (i > 0 ? beta_d[i - 1] : 0.0);
+                G = fmax(G, r);
+            }
+            double ig = 1.0 / G;
+            for (int i = 0; i <= j; ++i) {
+                al[i] = (float)(alpha_d[i] * ig);
+                float bb = (float)(beta_d[i] * ig);
+                b2[i] = bb * bb;
+            }
+            ext = tri_extreme(al, b2, j + 1, G);
         }
-        double ig = 1.0 / G;
-        for (int i = 0; i <= j; ++i) {
-            al[i] = (float)(alpha_d[i] * ig);
-            float bb = (float)(beta_d[i] * ig);
-            b2[i] = bb * bb;
-        }
-        ext = tri_extreme(al, b2, j + 1, G);
         if (early && j + 1 < kmin) {
             // early acceptance of a learned guess (see early_accept_factor);
             // the caller needs no Ritz vector then
@@ -790,7 +637,7 @@ __device__ double lanczos_inv_ritz(const Lane& S, const Layout& ly, int n, doubl
             }
         }
         if (j + 1 >= kmin && fabs(fabs(ext) - prev) <= rtol * fabs(ext)) break;
-        if (bn <= 1e-14 * fabs(a) || j + 1 == LANCZOS_KMAX) break;
+        if (last) break;
         prev = fabs(ext);
         beta = bn;
         const double ib = 1.0 / bn;
@@ -892,136 +739,6 @@ __device__ double eval_kappa(const Lane& S, const Layout& ly, int n, int kernel,
 __device__ inline double kappa_slope(const Lane& S, const Layout& ly, int n, int kernel, double eps_s,
                                      double theta) {
     return -eps_s * theta * eig_derivative(S, ly, n, kernel, eps_s);
-}
-
-// ---------------------------------------------------------------------------
-// per-lane root finder: safeguarded Newton in x = ln eps_s
-// ---------------------------------------------------------------------------
-enum { PH_FIRST = 0, PH_NEWTON = 1, PH_DONE = 3 };
-
-struct Search {
-    double x_next;        // point to evaluate next
-    double lo, hi;        // bracket of the root: F(lo) > 0 > F(hi) (F decreases)
-    double x_ret, k_ret;  // result (eps_s = exp(x_ret)) and kappa reported for it
-    double dx_prev;
-    double f_prev;        // |F| at the previous iterate
-    double ulo, uhi;      // caller's search range of x (+-inf when none)
-    int phase, evals;
-    int status;
-};
-
-__device__ inline double clampd(double v, double lo, double hi) { return fmin(fmax(v, lo), hi); }
-
-// dF/dx near the root, about -(11 + n / 10) on quasi-uniform surface
-// stencils (measured); used when the computed derivative is unusable.
-__device__ inline double slope_model(int n) { return -(11.0 + 0.1 * n); }
-
-// A learned guess predicts the root (kappa = kappa_T).  The search starts a
-// slope model's step past it, at kappa ~0.85 kappa_T: early acceptance (see
-// early_accept_factor) needs the estimate well below the band's upper edge,
-// and the networks' errors leave more room below kappa_T than above it
-// inside [0.5, 2] kappa_T.  On the 1M-node sphere this aim moves more first
-// evaluations into the step-7 window than it pushes out of the band.
-constexpr double LEARNED_AIM = 0.85;
-__device__ inline double learned_start(float guess, int n) {
-    return (double)guess + log(LEARNED_AIM) / slope_model(n);
-}
-
-__device__ inline void finish(Search& s, double x, double k, int status) {
-    s.x_ret = x;
-    s.k_ret = k;
-    s.status = status;
-    s.phase = PH_DONE;
-}
-
-// Consume F(x_next) = f with derivative d and kappa k.
-//  * learned first guess: accepted when kappa is inside the band;
-//  * Newton step dx = -f/d (slope model if d is unusable), clamped to +-3,
-//    replaced by bisection of the bracket when it would leave it;
-//  * stop when the distance to the root is below xtol/2, when the bracket
-//    is narrower than xtol, or when the steps stop shrinking at the float64
-//    noise floor of kappa (distance below xtol, step at least 0.9 of the
-//    previous one); every stop returns the evaluated x, within xtol of the
-//    root (the oracle's Brent guarantee).
-__device__ void search_update(Search& s, double f, double d, double k, double tol_s, int max_evals,
-                              double acc_lo, double acc_hi, bool learned, int n) {
-    s.evals++;
-    const double x = s.x_next;
-    if (s.phase == PH_FIRST && learned && k >= acc_lo && k <= acc_hi) {
-        finish(s, x, k, RBFFD_STENCIL_ACCEPTED_PREDICTION);
-        return;
-    }
-    if (f == 0.0) {
-        finish(s, x, k, RBFFD_STENCIL_OK);
-        return;
-    }
-    if (f > 0.0) s.lo = fmax(s.lo, x); else s.hi = fmin(s.hi, x);
-    // the root lies outside the caller's range: kappa is still above kappa_T
-    // at its largest eps, or already below it at its smallest
-    if ((f > 0.0 && x >= s.uhi) || (f < 0.0 && x <= s.ulo)) {
-        finish(s, x, k, RBFFD_STENCIL_NO_BRACKET);
-        return;
-    }
-    const double xtol = tol_s / exp(x);
-    // the Hellmann-Feynman slope is trusted only within a factor 5 of the
-    // slope model (a Ritz vector from a clustered pair can be poor)
-    const double sm = slope_model(n);
-    const bool usable = isfinite(d) && isfinite(f) && f != F_FAIL && d <= 0.2 * sm && d >= 5.0 * sm;
-    const double sl = usable ? d : sm;
-    double dx = clampd(-f / sl, -3.0, 3.0);
-    double xn = x + dx;
-    const bool bracketed = isfinite(s.lo) && isfinite(s.hi);
-    // safeguard: bisect when the Newton point leaves the bracket, or when the
-    // last Newton step did not halve |F| (the bracket then still shrinks
-    // geometrically, whatever the quality of the slope)
-    const bool slow = s.phase == PH_NEWTON && fabs(f) > 0.5 * s.f_prev;
-    const bool bisect = bracketed && (!(xn > s.lo && xn < s.hi) || slow);
-    if (bisect) xn = 0.5 * (s.lo + s.hi);
-    xn = clampd(xn, s.ulo, s.uhi);
-    dx = xn - x;
-    // distance of x from the root: after a bisection x is an end of the
-    // bracket, so at most 2|dx|; after a Newton step |F| over the flatter of
-    // the computed slope and the model (a Ritz vector from a clustered pair
-    // can give a slope several times too steep, and with it a step that
-    // looks converged while x is still far from the root)
-    const double dist = bisect ? fabs(dx) : fabs(f) / fmin(fabs(sl), fabs(sm));
-    // every stop returns the evaluated x (its factorisation is still in
-    // scratch for the weights)
-    if (usable && dist < 0.5 * xtol) {
-        finish(s, x, k, RBFFD_STENCIL_OK);
-        return;
-    }
-    // without a usable slope: the same test with the flattest slope that
-    // would have been trusted (0.2 |model|); it stops an iteration sitting
-    // on the root (|F| at rounding level) whose Ritz vector gives no slope
-    if (!usable && f != F_FAIL && fabs(f) < 0.1 * xtol * fabs(sm)) {
-        finish(s, x, k, RBFFD_STENCIL_OK);
-        return;
-    }
-    if (bracketed && s.hi - s.lo < xtol) {
-        finish(s, x, k, RBFFD_STENCIL_OK);
-        return;
-    }
-    // float64 noise floor of kappa: tiny steps that no longer shrink (a
-    // linearly converging Newton, e.g. with a slope off by 2x, shrinks its
-    // steps by a constant factor and does not stop here; when it is slow the
-    // halving test above bisects instead)
-    if (s.phase == PH_NEWTON && usable && dist < xtol && fabs(dx) >= 0.9 * fabs(s.dx_prev)) {
-        finish(s, x, k, RBFFD_STENCIL_OK);
-        return;
-    }
-    if (s.evals >= max_evals) {
-        finish(s, x, k, bracketed ? RBFFD_STENCIL_NO_CONVERGENCE : RBFFD_STENCIL_NO_BRACKET);
-        return;
-    }
-    s.dx_prev = dx;
-    s.f_prev = fabs(f);
-    s.x_next = xn;
-    s.phase = PH_NEWTON;
-}
-
-__device__ inline double F_of(double k, double kT) {
-    return isfinite(k) ? log(k / kT) : F_FAIL;
 }
 
 // [c; d] = A^{-1} [f; 0] in place on region V (first n entries)
@@ -1151,28 +868,6 @@ __device__ void first_row_weights(const Lane& S, const Layout& ly, int n, int ke
     aug_solve0(S, ly, n, V, s);
 }
 
-struct SearchArgs {
-    const double* X;
-    const double* NR;
-    double* w64;
-    float* w32;
-    const int32_t* idx;
-    const int32_t* row_node;
-    GroupInfo gi;
-    double* scratch;
-    int lane_size;
-    int kernel;
-    double kT, tol, acc_lo, acc_hi;
-    double xlo, xhi;             // search range of ln(eps * r_s) (+-inf when none)
-    int max_evals;
-    const float* guess_rows;     // ln(eps_s) per internal row, or NULL
-    unsigned long long* counters;  // per group
-    double* eps;
-    double* kappa;
-    int32_t* evals;
-    int32_t* status;
-};
-
 __global__ void __launch_bounds__(128, 4) search_kernel(SearchArgs A) {
     const int lane_id = threadIdx.x & 31;
     const int64_t warp_global = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
@@ -1262,22 +957,6 @@ __global__ void __launch_bounds__(128, 4) search_kernel(SearchArgs A) {
 // ---------------------------------------------------------------------------
 // weights at a fixed eps per stencil
 // ---------------------------------------------------------------------------
-struct WeightArgs {
-    const double* X;
-    const double* NR;
-    const int32_t* idx;
-    const int32_t* row_node;
-    GroupInfo gi;
-    double* scratch;
-    int lane_size;
-    int kernel;
-    const double* eps_node;
-    double* w64;
-    float* w32;
-    int32_t* status;      // written only on failure
-    int* nfail;
-};
-
 __global__ void __launch_bounds__(128, 4) weights_kernel(WeightArgs A) {
     const int lane_id = threadIdx.x & 31;
     const int64_t warp_global = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
@@ -1343,15 +1022,9 @@ LaunchShape launch_shape(const rbffd_build_opts& o, int64_t rows) {
 rbffd_status build_search(rbffd_op* op, const double* nodes, const double* normals,
                           const rbffd_build_opts& o, const float* guess_rows, cudaStream_t st) {
     const GroupInfo& gi = op->gi;
-    int mmax = 0;
-    for (int g = 0; g < gi.ngroups; ++g) mmax = std::max(mmax, gi.npad[g]);
-    Layout ly = make_layout(mmax, false);
     LaunchShape ls = launch_shape(o, op->N);
     RBFFD_CHECK_ARG(ls.threads % 32 == 0 && ls.threads <= 128, "block_threads must be 32..128, x32");
-    int64_t lanes = (int64_t)ls.blocks * ls.threads;
-    double* scratch = nullptr;
     unsigned long long* ctr = nullptr;
-    RBFFD_CUDA_TRY(pool_alloc(&scratch, (size_t)lanes * ly.size * sizeof(double), st));
     RBFFD_CUDA_TRY(pool_alloc(&ctr, RBFFD_MAX_GROUPS * sizeof(unsigned long long), st));
     RBFFD_CUDA_TRY(cudaMemsetAsync(ctr, 0, RBFFD_MAX_GROUPS * sizeof(unsigned long long), st));
     SearchArgs A;
@@ -1362,8 +1035,6 @@ rbffd_status build_search(rbffd_op* op, const double* nodes, const double* norma
     A.idx = op->idx;
     A.row_node = op->row_node;
     A.gi = gi;
-    A.scratch = scratch;
-    A.lane_size = ly.size;
     A.kernel = o.kernel;
     A.kT = o.kappa_target;
     A.tol = o.eps_tol;
@@ -1378,10 +1049,27 @@ rbffd_status build_search(rbffd_op* op, const double* nodes, const double* norma
     A.kappa = op->kappa;
     A.evals = op->evals;
     A.status = op->status;
-    search_kernel<<<ls.blocks, ls.threads, 0, st>>>(A);
-    note_launch();
-    RBFFD_CUDA_TRY(cudaGetLastError());
-    RBFFD_CUDA_TRY(cudaFreeAsync(scratch, st));
+    // Operators that do not fill the chip with a lane per stencil go to the team
+    // kernel, unless the caller chose the lane kernel's launch shape.  One kernel
+    // takes all groups, largest stencils first: a launch per group was slower
+    // (1M nodes in four sizes, learned: 476 against 421 ms), because the last
+    // stencils of a large group then run alone.
+    int mmax = 0;
+    for (int g = 0; g < gi.ngroups; ++g) mmax = std::max(mmax, gi.npad[g]);
+    const bool shaped = o.block_threads > 0 || o.blocks_per_sm > 0;
+    if (!shaped && team_lanes(mmax, op->N) > 0) {
+        rbffd_status s = team_search(A, mmax, op->N, st);
+        if (s != RBFFD_OK) return s;
+    } else {
+        const Layout ly = make_layout(mmax, false);
+        const int64_t lanes = (int64_t)ls.blocks * ls.threads;
+        RBFFD_CUDA_TRY(pool_alloc(&A.scratch, (size_t)lanes * ly.size * sizeof(double), st));
+        A.lane_size = ly.size;
+        search_kernel<<<ls.blocks, ls.threads, 0, st>>>(A);
+        note_launch();
+        RBFFD_CUDA_TRY(cudaGetLastError());
+        RBFFD_CUDA_TRY(cudaFreeAsync(A.scratch, st));
+    }
     RBFFD_CUDA_TRY(cudaFreeAsync(ctr, st));
     return RBFFD_OK;
 }
@@ -1389,38 +1077,44 @@ rbffd_status build_search(rbffd_op* op, const double* nodes, const double* norma
 rbffd_status build_weights(rbffd_op* op, const double* nodes, const double* normals,
                            const rbffd_build_opts& o, const double* eps_node, cudaStream_t st) {
     const GroupInfo& gi = op->gi;
-    int mmax = 0;
-    for (int g = 0; g < gi.ngroups; ++g) mmax = std::max(mmax, gi.npad[g]);
-    Layout ly = make_layout(mmax, true);
     LaunchShape ls = launch_shape(o, op->N);
     RBFFD_CHECK_ARG(ls.threads % 32 == 0 && ls.threads <= 128, "block_threads must be 32..128, x32");
-    int64_t lanes = (int64_t)ls.blocks * ls.threads;
-    double* scratch = nullptr;
     int* nfail = nullptr;
-    RBFFD_CUDA_TRY(pool_alloc(&scratch, (size_t)lanes * ly.size * sizeof(double), st));
     RBFFD_CUDA_TRY(pool_alloc(&nfail, sizeof(int), st));
     RBFFD_CUDA_TRY(cudaMemsetAsync(nfail, 0, sizeof(int), st));
-    WeightArgs A;
+    TeamWeightArgs B;
+    memset(&B, 0, sizeof(B));
+    WeightArgs& A = B.w;
     A.X = nodes;
     A.NR = normals;
     A.idx = op->idx;
     A.row_node = op->row_node;
     A.gi = gi;
-    A.scratch = scratch;
-    A.lane_size = ly.size;
     A.kernel = o.kernel;
     A.eps_node = eps_node;
     A.w64 = op->w64;
     A.w32 = op->w32;
     A.status = op->status;
     A.nfail = nfail;
-    weights_kernel<<<ls.blocks, ls.threads, 0, st>>>(A);
-    note_launch();
-    RBFFD_CUDA_TRY(cudaGetLastError());
+    int mmax = 0;
+    for (int g = 0; g < gi.ngroups; ++g) mmax = std::max(mmax, gi.npad[g]);
+    const bool shaped = o.block_threads > 0 || o.blocks_per_sm > 0;
+    if (!shaped && team_weight_lanes(mmax, op->N) > 0) {
+        rbffd_status s = team_weights(B, 0, st);
+        if (s != RBFFD_OK) return s;
+    } else {
+        const Layout ly = make_layout(mmax, true);
+        const int64_t lanes = (int64_t)ls.blocks * ls.threads;
+        RBFFD_CUDA_TRY(pool_alloc(&A.scratch, (size_t)lanes * ly.size * sizeof(double), st));
+        A.lane_size = ly.size;
+        weights_kernel<<<ls.blocks, ls.threads, 0, st>>>(A);
+        note_launch();
+        RBFFD_CUDA_TRY(cudaGetLastError());
+        RBFFD_CUDA_TRY(cudaFreeAsync(A.scratch, st));
+    }
     int hf = 0;
     RBFFD_CUDA_TRY(cudaMemcpyAsync(&hf, nfail, sizeof(int), cudaMemcpyDeviceToHost, st));
     RBFFD_CUDA_TRY(cudaStreamSynchronize(st));
-    RBFFD_CUDA_TRY(cudaFreeAsync(scratch, st));
     RBFFD_CUDA_TRY(cudaFreeAsync(nfail, st));
     if (hf) {
         set_error("%d stencils have a local matrix that is not numerically positive definite", hf);
@@ -1443,90 +1137,6 @@ constexpr int64_t NOALLOC_SCRATCH_DOUBLES = (int64_t)4 << 20;   // 32 MiB of flo
 static __device__ __align__(256) double g_noalloc_scratch[NOALLOC_SCRATCH_DOUBLES];
 static __device__ int g_noalloc_fail;   // rows that failed in the current call
 
-// geometry of one stencil given as a row of node indices (centre first);
-// returns false when an index is outside [0, N)
-__device__ bool load_geometry_row(const Lane& S, const Layout& ly, int n, const int32_t* __restrict__ row,
-                                  const double* __restrict__ X, const double* __restrict__ NR, int64_t N,
-                                  Geo& g) {
-    for (int j = 0; j < n; ++j)
-        if (row[j] < 0 || (int64_t)row[j] >= N) return false;
-    int c = row[0];
-    double cx = X[3 * (int64_t)c], cy = X[3 * (int64_t)c + 1], cz = X[3 * (int64_t)c + 2];
-    double rs2 = 0.0;
-    for (int j = 0; j < n; ++j) {
-        int k = row[j];
-        double dx = X[3 * (int64_t)k] - cx, dy = X[3 * (int64_t)k + 1] - cy, dz = X[3 * (int64_t)k + 2] - cz;
-        S[ly.XS + j] = dx;
-        S[ly.XS + ly.m + j] = dy;
-        S[ly.XS + 2 * ly.m + j] = dz;
-        rs2 = fmax(rs2, dx * dx + dy * dy + dz * dz);
-        double nx = NR[3 * (int64_t)k], ny = NR[3 * (int64_t)k + 1], nz = NR[3 * (int64_t)k + 2];
-        double inv = rsqrt(nx * nx + ny * ny + nz * nz);
-        S[ly.NS + j] = nx * inv;
-        S[ly.NS + ly.m + j] = ny * inv;
-        S[ly.NS + 2 * ly.m + j] = nz * inv;
-    }
-    g.rs = sqrt(rs2);
-    double inv = 1.0 / g.rs;
-    for (int j = 0; j < n; ++j) {
-        S[ly.XS + j] *= inv;
-        S[ly.XS + ly.m + j] *= inv;
-        S[ly.XS + 2 * ly.m + j] *= inv;
-    }
-    g.mean_d = 0.0;
-    for (int i = 0; i < n; ++i) {
-        double xi = S[ly.XS + i], yi = S[ly.XS + ly.m + i], zi = S[ly.XS + 2 * ly.m + i];
-        int base = pk(i, 0);
-        for (int j = 0; j < i; ++j) {
-            double dx = xi - S[ly.XS + j], dy = yi - S[ly.XS + ly.m + j], dz = zi - S[ly.XS + 2 * ly.m + j];
-            S[ly.R2 + base + j] = dx * dx + dy * dy + dz * dz;
-        }
-        S[ly.R2 + base + i] = 0.0;
-    }
-    return true;
-}
-
-__global__ void __launch_bounds__(128)
-weights_rows_kernel(const double* __restrict__ X, const double* __restrict__ NR, int64_t N,
-                    const int32_t* __restrict__ stencils, int64_t rows, int n,
-                    const double* __restrict__ eps, int kernel, double* __restrict__ Wout,
-                    double* __restrict__ scratch, int lane_size) {
-    const int lane_id = threadIdx.x & 31;
-    const int64_t warp_global = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    Lane S{scratch + warp_global * 32 * (int64_t)lane_size + lane_id};
-    const int npad = (n + 3) / 4 * 4;
-    const Layout ly = make_layout(npad, true);
-    const int m = ly.m;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < rows; r += stride) {
-        double* w_row = Wout + r * (int64_t)n;
-        Geo geo;
-        bool ok = load_geometry_row(S, ly, n, stencils + r * (int64_t)n, X, NR, N, geo);
-        double eps_s = ok ? eps[r] * geo.rs : 0.0;
-        double s = 0.0;
-        if (ok) {
-            assemble_phi(S, ly, n, kernel, eps_s, ly.L, ly.PH);
-            ok = cholesky(S, ly, n) && isfinite(eps_s) && eps_s > 0.0;
-        }
-        if (ok) {
-            for (int i = 0; i < m; ++i) S[ly.U + i] = i < n ? 1.0 : 0.0;
-            chol_solve(S, ly, ly.U);
-            for (int i = 0; i < n; ++i) s += S[ly.U + i];
-            ok = s > 0.0 && isfinite(s);
-        }
-        if (!ok) {
-            atomicAdd(&g_noalloc_fail, 1);
-            for (int j = 0; j < n; ++j) w_row[j] = NAN;
-            continue;
-        }
-        // the build's own weight arithmetic (same steps, same order)
-        first_row_weights(S, ly, n, kernel, eps_s, s);
-        const int V = ly.Q0;
-        double inv_rs2 = 1.0 / (geo.rs * geo.rs);
-        for (int j = 0; j < n; ++j) w_row[j] = S[V + j] * inv_rs2;
-    }
-}
-
 // Device address of the scratch array, looked up once per device.
 constexpr int NOALLOC_MAX_DEVICES = 64;
 double* g_noalloc_ptr[NOALLOC_MAX_DEVICES] = {};
@@ -1546,13 +1156,6 @@ extern "C" rbffd_status rbffd_stencil_weights_noalloc(const double* nodes, const
     RBFFD_CHECK_ARG(N >= 2 && rows >= 0, "N must be >= 2 and rows >= 0");
     if (n < 2 || n > RBFFD_MAX_N || n > N) {
         set_error("rbffd_stencil_weights_noalloc: stencil size %d outside [2, min(N, %d)]", n, RBFFD_MAX_N);
-        return RBFFD_EINVAL;
-    }
-    const int npad = (n + 3) / 4 * 4;
-    const int lane_size = make_layout(npad, true).size;
-    int64_t lanes = NOALLOC_SCRATCH_DOUBLES / lane_size / 32 * 32;
-    if (lanes < 32) {   // cannot happen for n <= 128 with 32 MiB; kept as the size guard
-        set_error("rbffd_stencil_weights_noalloc: stencil size %d needs more than the fixed scratch", n);
         return RBFFD_EINVAL;
     }
     if (rows == 0) return RBFFD_OK;
@@ -1579,14 +1182,21 @@ extern "C" rbffd_status rbffd_stencil_weights_noalloc(const double* nodes, const
     // the failure counter must start at zero; the scratch itself is written
     // before it is read in every row, so it is not cleared
     RBFFD_CUDA_TRY(cudaMemsetAsync(fail, 0, sizeof(int), st));
-    int64_t need = (rows + 31) / 32 * 32;
-    lanes = std::min(lanes, need);
-    int threads = (int)std::min<int64_t>(128, lanes);
-    int blocks = (int)(lanes / threads);
-    weights_rows_kernel<<<blocks, threads, 0, st>>>(nodes, normals, N, stencils, rows, n, eps, kernel, weights,
-                                                    scratch, lane_size);
-    note_launch();
-    RBFFD_CUDA_TRY(cudaGetLastError());
+    TeamWeightArgs B;
+    memset(&B, 0, sizeof(B));
+    B.w.X = nodes;
+    B.w.NR = normals;
+    B.w.scratch = scratch;
+    B.w.kernel = kernel;
+    B.w.eps_node = eps;
+    B.w.w64 = weights;
+    B.w.nfail = fail;
+    B.stencils = stencils;
+    B.N = N;
+    B.rows = rows;
+    B.n = n;
+    const rbffd_status s = team_weights(B, NOALLOC_SCRATCH_DOUBLES, st);
+    if (s != RBFFD_OK) return s;
     int hfail = 0;
     RBFFD_CUDA_TRY(cudaMemcpyAsync(&hfail, fail, sizeof(int), cudaMemcpyDeviceToHost, st));
     RBFFD_CUDA_TRY(cudaStreamSynchronize(st));
