@@ -230,12 +230,13 @@ typedef struct {
  *                                    + 12 dt s(t^{n+1})
  * (s the optional source of params, zero without one),
  * each implicit system solved by BiCGSTAB from x0 = u^n (Section 4.2), or
- * by the banded LU factors (params->solver).  Operators with fewer than 1024
- * rows per SM: one cooperative persistent launch per step; larger ones:
- * BiCGSTAB as a sequence of kernels whose iteration loop runs on the device
- * (a WHILE node of the CUDA graph, or, with use_graph = 0, the same kernels
- * from a host loop).  Either path is replayed from a CUDA graph when
- * use_graph = 1 (captured at the first call, again whenever an argument
+ * by the banded LU factors (params->solver).  Operators that fit the chip's
+ * shared memory (up to about 30 MB of indices and weights) take all steps of
+ * the call in one launch; larger ones run BiCGSTAB as a sequence of kernels
+ * whose iteration loop runs on the device (a WHILE node of the CUDA graph, or,
+ * with use_graph = 0, the same kernels from a host loop), and they and the
+ * direct steps are replayed from a CUDA graph when use_graph = 1 (captured at
+ * the first call, again whenever an argument
  * changes).  Synchronises the stream at the end and fills report (may be
  * NULL).  Returns RBFFD_SOLVER_NOT_CONVERGED (with report->failed_step) or
  * RBFFD_TIMEOUT when a bounded wait gave up.

@@ -5,22 +5,14 @@
 //   SBDF2:  (3 I - 2 dt delta L) u^{n+1} = 4 u^n - u^{n-1} + 2 dt (2 f^n - f^{n-1})
 //   first step without history: (I - dt delta L) u^1 = u^0 + dt f^0
 //
-// GPU design: one cooperative persistent launch per time step.  Every
-// thread owns a fixed set of operator rows for the whole step; both species
-// are solved together so each pass over the ELL matrix (the bytes that
-// bound the step) serves two SpMVs.  Phases of BiCGSTAB are separated by a
-// grid barrier of our own with a bounded spin (a block that waits longer
-// than about a second sets an error flag and leaves, so nothing can hang);
-// dot products are reduced per block in float64, written to per-phase
-// slots, and every block sums the slots in the same fixed order, so all
-// blocks hold bit-identical scalars.  Vectors written inside the launch are
-// read with L1-bypassing loads.  The solution is updated in place in u
-// (after the right-hand side is formed, u is only read by its own row).
-// The launch can be captured once into a CUDA graph and replayed per step.
-//
-// Large operators take a second path with the same arithmetic per row:
-// BiCGSTAB as a sequence of full-occupancy phase kernels under a device-side
-// WHILE graph node (the phase-kernel section below says why and how).
+// GPU design: both species are solved together, so each pass over the ELL
+// matrix serves two products, and the solution is updated in place in u, v.
+// Operators that fit the shared memory of the chip (up to about 30 MB) run all
+// steps of a call in one launch with the matrix resident there
+// (step_resident.cuh).  Larger ones run BiCGSTAB as a sequence of
+// full-occupancy phase kernels under a device-side WHILE graph node (the
+// phase-kernel section below says why and how).  A direct step is three
+// launches: right-hand side, substitutions (lu.cu), report.
 #include "common.cuh"
 
 #include <algorithm>
@@ -55,7 +47,6 @@ struct rbffd_step_ws {
     int64_t N;
     size_t elem;
     void* vec;                     // 2 species x 7 vectors (b, r, rh, p, q, s, t), each padded to a multiple of 4
-    double* partial;               // phases x blocks x 8
     unsigned long long* bar;       // barrier counter
     int* flags;                    // [0] error (timeout), [1] not converged, [2] has_history,
                                    // [3] report slot of the next step, [4] order of the last step
@@ -63,18 +54,17 @@ struct rbffd_step_ws {
     double* rep_res;               // per step: relres_u, relres_v
     double* tstart;                // time of u at the start of the call (device copy)
     int64_t rep_cap;
-    int blocks, threads;
-    cudaGraphExec_t graph;            // captured step (memset + launch)
+    cudaGraphExec_t graph;            // captured step
     cudaStream_t cap;                 // library-owned stream used only for capture
     unsigned char graph_args[1024];   // kernel arguments the graph holds
     size_t graph_args_size;
-    int solver;                       // path the graph was captured with (0 cooperative, 1 LU, 2 phases)
+    int solver;                       // path the graph was captured with (1 LU, 2 phases)
     rbffd_lu* lu[4][2];               // banded LU factors by SBDF order and species
     rbffd_lu* graph_lu[4][2];         // the factors the captured graph's solve reads
     double* ywork;                    // the LU substitutions' work: per species 2 N + 16 float64
     PhaseCtl* ctl;                    // phase-kernel path: loop state
     double* pp;                       //   per-block partial sums
-    int phased;                       // 1: BiCGSTAB as phase kernels (large operators)
+    double* rpart;                    // resident kernel: per-block sums of two reductions
 };
 
 namespace rbffd {
@@ -82,7 +72,6 @@ namespace rbffd {
 void step_ws_free(rbffd_step_ws* ws) {
     if (!ws) return;
     cudaFree(ws->vec);
-    cudaFree(ws->partial);
     cudaFree(ws->bar);
     cudaFree(ws->flags);
     cudaFree(ws->rep);
@@ -95,13 +84,11 @@ void step_ws_free(rbffd_step_ws* ws) {
     cudaFree(ws->ywork);
     cudaFree(ws->ctl);
     cudaFree(ws->pp);
+    cudaFree(ws->rpart);
     delete ws;
 }
 
 namespace {
-
-constexpr int NPHASE = 6;
-constexpr int NSLOT = 8;
 
 template <typename T>
 struct Args {
@@ -127,12 +114,10 @@ struct Args {
     T delta[2];
     double tol;
     int maxit;
-    double* partial;
     unsigned long long* bar;
     int* flags;
     int* rep;
     double* rep_res;
-    int rhs_only;      // 1: form the right-hand side b only (a direct solve follows)
     PhaseCtl* ctl;                         // phase-kernel path: loop state and totals
     double* pp;                            //   per-block partial sums (blocks x 8)
     cudaGraphConditionalHandle cond;       //   WHILE handle of the step graph (0: host loop)
@@ -143,44 +128,6 @@ enum { VB = 0, VR = 1, VRH = 2, VP = 3, VQ = 4, VS = 5, VT = 6 };
 template <typename T>
 __host__ __device__ __forceinline__ T* V(const Args<T>& a, int sp, int k) {
     return a.vec + ((int64_t)sp * 7 + k) * a.ldv;
-}
-
-template <typename T>
-__device__ __forceinline__ T ldcg(const T* p) { return __ldcg(p); }
-
-// block-reduce K doubles into partial[phase][block][0..K-1]
-template <int K>
-__device__ void block_partial(double (&v)[K], double* partial, int phase) {
-    __shared__ double sh[K][32];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-        double x = v[k];
-        for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
-        if (lane == 0) sh[k][wid] = x;
-    }
-    __syncthreads();
-    if (threadIdx.x < K) {
-        double s = 0.0;
-        for (int w = 0; w < nw; ++w) s += sh[threadIdx.x][w];
-        partial[((int64_t)phase * gridDim.x + blockIdx.x) * NSLOT + threadIdx.x] = s;
-    }
-}
-
-// every block sums the per-block partials of a phase in block order
-template <int K>
-__device__ void grid_total(const double* partial, int phase, double (&out)[K]) {
-    __shared__ double tot[K];
-    if (threadIdx.x < K) {
-        double s = 0.0;
-        for (int b = 0; b < (int)gridDim.x; ++b)
-            s += __ldcg(partial + ((int64_t)phase * gridDim.x + b) * NSLOT + threadIdx.x);
-        tot[threadIdx.x] = s;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < K; ++k) out[k] = tot[k];
-    __syncthreads();
 }
 
 template <typename T>
@@ -206,13 +153,8 @@ __device__ __forceinline__ void react(const Args<T>& a, T u, T v, T& f, T& g) {
     }
 }
 
-// (L x0)_row and (L x1)_row in one pass over the row (x read L1-bypassing:
-// within one launch L1 is not coherent across SMs); software-pipelined so
-// that a chunk's index and weight loads overlap the previous chunk's gathers
 __device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
-template <typename T>
-__device__ __forceinline__ int4 ld_stream4(const int32_t* p) { return __ldcs(reinterpret_cast<const int4*>(p)); }
 __device__ __forceinline__ void load4s(const float* p, float (&w)[4]) {
     float4 v = __ldcs(reinterpret_cast<const float4*>(p));
     w[0] = v.x; w[1] = v.y; w[2] = v.z; w[3] = v.w;
@@ -221,71 +163,6 @@ __device__ __forceinline__ void load4s(const double* p, double (&w)[4]) {
     double2 a = __ldcs(reinterpret_cast<const double2*>(p));
     double2 b = __ldcs(reinterpret_cast<const double2*>(p + 2));
     w[0] = a.x; w[1] = a.y; w[2] = b.x; w[3] = b.y;
-}
-
-constexpr int PF_CHUNKS = 6;   // ELL chunks prefetched into L2 ahead of use
-
-// (L x0)_row and (L x1)_row in one pass over the row (x read L1-bypassing:
-// within one launch L1 is not coherent across SMs); software-pipelined so
-// that a chunk's index and weight loads overlap the previous chunk's
-// gathers, with an L2 prefetch PF_CHUNKS chunks ahead that runs on into the
-// thread's next row (rnext), and streaming (evict-first) loads of the
-// single-use ELL so that the Krylov vectors stay in L2
-template <typename T>
-__device__ __forceinline__ void row_L2(const Args<T>& a, int64_t r, int64_t rnext, const T* x0, const T* x1,
-                                       bool two, T& y0, T& y1) {
-    int g = group_of_row(a.gi, r);
-    const int npad = a.gi.npad[g], nch = npad >> 2;
-    const int64_t base = ell_elem(a.gi.ell_off[g], npad, r - a.gi.row_begin[g], 0);
-    int64_t nbase = -1;
-    int nnch = 0;
-    if (rnext < a.N) {
-        const int gn = group_of_row(a.gi, rnext);
-        nnch = a.gi.npad[gn] >> 2;
-        nbase = ell_elem(a.gi.ell_off[gn], a.gi.npad[gn], rnext - a.gi.row_begin[gn], 0);
-    }
-    T s0 = T(0), s1 = T(0);
-    int4 iv = __ldcs(reinterpret_cast<const int4*>(a.idx + base));
-    T wv[4];
-    load4s(a.w + base, wv);
-    for (int c = 0; c < nch; ++c) {
-        // L2 prefetch PF_CHUNKS ahead (into the next row past this one's end)
-        {
-            const int k = c + PF_CHUNKS;
-            int64_t e = -1;
-            if (k < nch) e = base + (int64_t)k * 128;
-            else if (k - nch < nnch && nbase >= 0) e = nbase + (int64_t)(k - nch) * 128;
-            if (e >= 0) {
-                prefetch_l2(a.idx + e);
-                prefetch_l2(a.w + e);
-            }
-        }
-        // the next chunk's index and weight loads go out before this chunk's gathers
-        int4 ivn = iv;
-        T wn[4] = {wv[0], wv[1], wv[2], wv[3]};
-        if (c + 1 < nch) {
-            const int64_t en = base + (int64_t)(c + 1) * 128;
-            ivn = __ldcs(reinterpret_cast<const int4*>(a.idx + en));
-            load4s(a.w + en, wn);
-        }
-        const int ii[4] = {iv.x, iv.y, iv.z, iv.w};
-        T g0[4], g1[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            g0[q] = ldcg(x0 + ii[q]);
-            g1[q] = two ? ldcg(x1 + ii[q]) : T(0);
-        }
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            s0 = fma(wv[q], g0[q], s0);
-            s1 = fma(wv[q], g1[q], s1);
-        }
-        iv = ivn;
-#pragma unroll
-        for (int q = 0; q < 4; ++q) wv[q] = wn[q];
-    }
-    y0 = s0;
-    y1 = two ? s1 : T(0);
 }
 
 // the SBDF order, report slot and coefficients of the current step (from
@@ -297,13 +174,13 @@ struct StepCoef {
 };
 
 template <typename T>
-__device__ __forceinline__ StepCoef<T> step_coef(const Args<T>& a) {
+__device__ __forceinline__ StepCoef<T> step_coef_at(const Args<T>& a, int nhist, int slot) {
     StepCoef<T> k;
     // past levels available -> the order of this step (SBDF1 .. SBDF4, the
     // first steps of a run without history climb one order per step)
-    k.nhist = *((volatile int*)(a.flags + 2));
-    k.ord = min(a.order, k.nhist + 1);
-    k.slot = *((volatile int*)(a.flags + 3));
+    k.nhist = nhist;
+    k.ord = min(a.order, nhist + 1);
+    k.slot = slot;
     // the SBDFk system scaled to integer coefficients:
     //   c0 u^{n+1} - cl delta L u^{n+1} = sum_j A_j u^{n-j} + cl sum_j B_j f^{n-j}
     // k = 1: c0 1, cl dt;  k = 2: 3, 2 dt;  k = 3: 11, 6 dt;  k = 4: 25, 12 dt
@@ -317,9 +194,12 @@ __device__ __forceinline__ StepCoef<T> step_coef(const Args<T>& a) {
     return k;
 }
 
-// Dot-product accumulators.  The cooperative kernel sums in float64 (the
-// float32 products are exact there).  The phase kernels sum float32 products
-// with the compensated dot product Dot2 (Ogita, Rump & Oishi, "Accurate sum
+template <typename T>
+__device__ __forceinline__ StepCoef<T> step_coef(const Args<T>& a) {
+    return step_coef_at(a, *((volatile int*)(a.flags + 2)), *((volatile int*)(a.flags + 3)));
+}
+
+// Dot-product accumulators.  The phase kernels sum float32 products with the compensated dot product Dot2 (Ogita, Rump & Oishi, "Accurate sum
 // and dot product", SIAM J. Sci. Comput. 26 (2005), Algorithm 5.3): each
 // product a b split exactly into p + e by an FMA (TwoProduct), the running
 // sum carried by Knuth's error-free TwoSum, the rounding errors of both
@@ -355,22 +235,17 @@ struct PhaseAcc<float> {
     using type = Dot2;
 };
 
-// phase R of one row (node i, with (L u)_i = Lu, (L v)_i = Lv): kinetics,
-// right-hand side b of the step's SBDF order, history rotation, r0 = b - A u,
-// r-hat = r0, p = q = 0; accumulates |b|^2, |r0|^2 per species into d[0..1],
-// d[3..4]
-template <typename T, typename A>
-__device__ __forceinline__ void rhs_row(const Args<T>& a, const StepCoef<T>& kc, int64_t i, T Lu, T Lv,
-                                        A (&d)[6]) {
+// kinetics and right-hand side b of the step's SBDF order at node i (values
+// ui, vi), and the rotation of its history
+template <typename T>
+__device__ __forceinline__ void rhs_values(const Args<T>& a, const StepCoef<T>& kc, int64_t i, T ui, T vi, T& bu,
+                                           T& bv) {
     const bool two = a.ns == 2;
     const int ord = kc.ord;
-    const T c0 = kc.c0, cl = kc.cl, k0 = kc.k0, k1 = kc.k1, samp = kc.samp;
-    T* u = a.u;
-    T* v = two ? a.v : nullptr;
-    T ui = u[i], vi = two ? v[i] : T(0);
+    const T cl = kc.cl, samp = kc.samp;
     T f, g;
     react(a, ui, vi, f, g);
-    T bu, bv = T(0);
+    bv = T(0);
     if (ord == 2) {
         bu = T(4) * ui - a.up[i] + T(2) * a.dt * (T(2) * f - a.fp[i]);
         if (two) bv = T(4) * vi - a.vp[i] + T(2) * a.dt * (T(2) * g - a.gp[i]);
@@ -403,14 +278,6 @@ __device__ __forceinline__ void rhs_row(const Args<T>& a, const StepCoef<T>& kc,
     }
     a.up[i] = ui;
     a.fp[i] = f;
-    T ru = bu - (c0 * ui - k0 * Lu);
-    V(a, 0, VB)[i] = bu;
-    V(a, 0, VR)[i] = ru;
-    V(a, 0, VRH)[i] = ru;
-    V(a, 0, VP)[i] = T(0);
-    V(a, 0, VQ)[i] = T(0);
-    acc_add(d[0], bu, bu);
-    acc_add(d[1], ru, ru);
     if (two) {
         if (a.order >= 4) {
             a.vp3[i] = a.vp2[i];
@@ -422,7 +289,29 @@ __device__ __forceinline__ void rhs_row(const Args<T>& a, const StepCoef<T>& kc,
         }
         a.vp[i] = vi;
         a.gp[i] = g;
-        T rv = bv - (c0 * vi - k1 * Lv);
+    }
+}
+
+// phase R of one row (node i, with (L u)_i = Lu, (L v)_i = Lv): the right-hand
+// side, r0 = b - A u, r-hat = r0, p = q = 0; accumulates |b|^2, |r0|^2 per
+// species into d[0..1], d[3..4]
+template <typename T, typename A>
+__device__ __forceinline__ void rhs_row(const Args<T>& a, const StepCoef<T>& kc, int64_t i, T Lu, T Lv,
+                                        A (&d)[6]) {
+    const bool two = a.ns == 2;
+    const T ui = a.u[i], vi = two ? a.v[i] : T(0);
+    T bu, bv;
+    rhs_values(a, kc, i, ui, vi, bu, bv);
+    const T ru = bu - (kc.c0 * ui - kc.k0 * Lu);
+    V(a, 0, VB)[i] = bu;
+    V(a, 0, VR)[i] = ru;
+    V(a, 0, VRH)[i] = ru;
+    V(a, 0, VP)[i] = T(0);
+    V(a, 0, VQ)[i] = T(0);
+    acc_add(d[0], bu, bu);
+    acc_add(d[1], ru, ru);
+    if (two) {
+        const T rv = bv - (kc.c0 * vi - kc.k1 * Lv);
         V(a, 1, VB)[i] = bv;
         V(a, 1, VR)[i] = rv;
         V(a, 1, VRH)[i] = rv;
@@ -433,250 +322,30 @@ __device__ __forceinline__ void rhs_row(const Args<T>& a, const StepCoef<T>& kc,
     }
 }
 
-// NT threads per block: 1024 (one block per SM, <= 64 registers) for large
-// operators (there only the LU step's right-hand side runs here), 256 for
-// small ones
-template <typename T, int NT>
-__global__ void __launch_bounds__(NT) step_kernel(Args<T> a) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    const int64_t t0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    const bool two = a.ns == 2;
+// right-hand side b of a step that a direct solve follows, and its SBDF order
+// for the solve (flags[4])
+template <typename T>
+__global__ void __launch_bounds__(256) lu_rhs_kernel(Args<T> a) {
     const StepCoef<T> kc = step_coef(a);
-    const int nhist = kc.nhist, ord = kc.ord, slot = kc.slot;
-    const T c0 = kc.c0, k0 = kc.k0, k1 = kc.k1;
-    unsigned long long target = 0;
-    T* u = a.u;
-    T* v = two ? a.v : nullptr;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < a.N; i += (int64_t)gridDim.x * blockDim.x) {
+        T bu, bv;
+        rhs_values(a, kc, i, a.u[i], a.ns == 2 ? a.v[i] : T(0), bu, bv);
+        V(a, 0, VB)[i] = bu;
+        if (a.ns == 2) V(a, 1, VB)[i] = bv;
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) a.flags[4] = kc.ord;
+}
 
-    // ---- phase R: reaction, right-hand side, r0 = b - A u, history rotation
-    {
-        double d[6] = {0, 0, 0, 0, 0, 0};   // |b|^2, |r|^2, (rh, r) per species
-        for (int64_t r = t0; r < a.N; r += stride) {
-            int i = a.row_node[r];
-            T Lu, Lv;
-            row_L2(a, r, r + stride, u, v, two, Lu, Lv);
-            rhs_row(a, kc, i, Lu, Lv, d);
-        }
-        block_partial<6>(d, a.partial, 0);
-    }
-    if (!grid_sync(a.bar, target += gridDim.x, a.flags)) return;
-    if (a.rhs_only) {
-        // the implicit systems are solved by the banded LU launch that
-        // follows (every block has read flags[2..3] before the barrier)
-        if (blockIdx.x == 0 && threadIdx.x == 0) {
-            int* rp = a.rep + (int64_t)slot * 3;
-            rp[0] = rp[1] = rp[2] = 0;
-            a.rep_res[(int64_t)slot * 2] = 0.0;
-            a.rep_res[(int64_t)slot * 2 + 1] = 0.0;
-            a.flags[2] = min(nhist + 1, max(a.order - 1, 1));
-            a.flags[3] = slot + 1;
-            a.flags[4] = ord;
-        }
-        return;
-    }
-    double tot[6];
-    grid_total<6>(a.partial, 0, tot);
-
-    double bnorm[2] = {sqrt(tot[0]), sqrt(tot[3])};
-    double rho[2] = {tot[1], tot[4]};    // (rh, r0) = |r0|^2
-    double rho_prev[2] = {1.0, 1.0}, alpha[2] = {1.0, 1.0}, omega[2] = {1.0, 1.0};
-    bool active[2], conv[2] = {false, false}, fail[2] = {false, false};
-    int iters[2] = {0, 0};
-    double relres[2];
-    for (int k = 0; k < 2; ++k) {
-        bool exists = k == 0 || two;
-        relres[k] = bnorm[k] > 0 ? sqrt(rho[k]) / bnorm[k] : 0.0;
-        conv[k] = !exists || bnorm[k] == 0.0 || relres[k] <= a.tol;
-        active[k] = !conv[k];
-    }
-    if (bnorm[0] == 0.0)   // b = 0: x = 0
-        for (int64_t r = t0; r < a.N; r += stride) u[a.row_node[r]] = T(0);
-    if (two && bnorm[1] == 0.0)
-        for (int64_t r = t0; r < a.N; r += stride) v[a.row_node[r]] = T(0);
-
-    int it = 0;
-    while ((active[0] || active[1]) && it < a.maxit) {
-        ++it;
-        // ---- A: p = r + beta (p - omega q)
-        double beta[2];
-        for (int k = 0; k < 2; ++k) {
-            beta[k] = (rho[k] / rho_prev[k]) * (alpha[k] / omega[k]);
-            if (active[k] && (rho[k] == 0.0 || !isfinite(beta[k]))) {
-                fail[k] = true;
-                active[k] = false;
-            }
-        }
-        for (int64_t r = t0; r < a.N; r += stride) {
-            int i = a.row_node[r];
-            for (int k = 0; k < 2; ++k) {
-                if (!active[k]) continue;
-                T* p = V(a, k, VP);
-                p[i] = V(a, k, VR)[i] + (T)beta[k] * (p[i] - (T)omega[k] * V(a, k, VQ)[i]);
-            }
-        }
-        if (!grid_sync(a.bar, target += gridDim.x, a.flags)) return;
-        // ---- B: q = A p ; (rh, q)
-        {
-            double d[2] = {0, 0};
-            for (int64_t r = t0; r < a.N; r += stride) {
-                int i = a.row_node[r];
-                T L0, L1;
-                row_L2(a, r, r + stride, V(a, 0, VP), two ? V(a, 1, VP) : nullptr, two && active[1], L0, L1);
-                if (active[0]) {
-                    T q = c0 * V(a, 0, VP)[i] - k0 * L0;
-                    V(a, 0, VQ)[i] = q;
-                    d[0] += (double)V(a, 0, VRH)[i] * q;
-                }
-                if (active[1]) {
-                    T q = c0 * V(a, 1, VP)[i] - k1 * L1;
-                    V(a, 1, VQ)[i] = q;
-                    d[1] += (double)V(a, 1, VRH)[i] * q;
-                }
-            }
-            block_partial<2>(d, a.partial, 1);
-        }
-        if (!grid_sync(a.bar, target += gridDim.x, a.flags)) return;
-        {
-            double s[2];
-            grid_total<2>(a.partial, 1, s);
-            for (int k = 0; k < 2; ++k) {
-                if (!active[k]) continue;
-                alpha[k] = rho[k] / s[k];
-                if (s[k] == 0.0 || !isfinite(alpha[k])) {
-                    fail[k] = true;
-                    active[k] = false;
-                }
-            }
-        }
-        // ---- C: s = r - alpha q ; |s|^2
-        {
-            double d[2] = {0, 0};
-            for (int64_t r = t0; r < a.N; r += stride) {
-                int i = a.row_node[r];
-                for (int k = 0; k < 2; ++k) {
-                    if (!active[k]) continue;
-                    T s = V(a, k, VR)[i] - (T)alpha[k] * V(a, k, VQ)[i];
-                    V(a, k, VS)[i] = s;
-                    d[k] += (double)s * s;
-                }
-            }
-            block_partial<2>(d, a.partial, 2);
-        }
-        if (!grid_sync(a.bar, target += gridDim.x, a.flags)) return;
-        bool early[2] = {false, false};
-        {
-            double s[2];
-            grid_total<2>(a.partial, 2, s);
-            for (int k = 0; k < 2; ++k) {
-                if (!active[k]) continue;
-                double rr = sqrt(s[k]) / bnorm[k];
-                if (rr <= a.tol) {
-                    early[k] = true;
-                    relres[k] = rr;
-                }
-            }
-        }
-        // ---- D: t = A s ; (t, s), (t, t)   (x += alpha p where s converged)
-        {
-            double d[4] = {0, 0, 0, 0};
-            bool need0 = active[0] && !early[0], need1 = active[1] && !early[1];
-            for (int64_t r = t0; r < a.N; r += stride) {
-                int i = a.row_node[r];
-                T L0 = T(0), L1 = T(0);
-                if (need0 || need1)
-                    row_L2(a, r, r + stride, V(a, 0, VS), two ? V(a, 1, VS) : nullptr, two && need1, L0, L1);
-                for (int k = 0; k < 2; ++k) {
-                    T* x = k == 0 ? u : v;
-                    if (early[k]) {
-                        x[i] += (T)alpha[k] * V(a, k, VP)[i];
-                    } else if (active[k]) {
-                        T s = V(a, k, VS)[i];
-                        T t = c0 * s - (k == 0 ? k0 * L0 : k1 * L1);
-                        V(a, k, VT)[i] = t;
-                        d[2 * k] += (double)t * s;
-                        d[2 * k + 1] += (double)t * t;
-                    }
-                }
-            }
-            block_partial<4>(d, a.partial, 3);
-        }
-        for (int k = 0; k < 2; ++k)
-            if (early[k]) {
-                active[k] = false;
-                conv[k] = true;
-                iters[k] = it;
-            }
-        if (!grid_sync(a.bar, target += gridDim.x, a.flags)) return;
-        {
-            double s[4];
-            grid_total<4>(a.partial, 3, s);
-            for (int k = 0; k < 2; ++k) {
-                if (!active[k]) continue;
-                omega[k] = s[2 * k] / s[2 * k + 1];
-                if (s[2 * k + 1] == 0.0 || !isfinite(omega[k])) {
-                    fail[k] = true;
-                    active[k] = false;
-                }
-            }
-        }
-        // ---- E: x += alpha p + omega s ; r = s - omega t ; (rh, r), |r|^2
-        {
-            double d[4] = {0, 0, 0, 0};
-            for (int64_t r = t0; r < a.N; r += stride) {
-                int i = a.row_node[r];
-                for (int k = 0; k < 2; ++k) {
-                    if (!active[k]) continue;
-                    T* x = k == 0 ? u : v;
-                    T s = V(a, k, VS)[i];
-                    x[i] += (T)alpha[k] * V(a, k, VP)[i] + (T)omega[k] * s;
-                    T rn = s - (T)omega[k] * V(a, k, VT)[i];
-                    V(a, k, VR)[i] = rn;
-                    d[2 * k] += (double)V(a, k, VRH)[i] * rn;
-                    d[2 * k + 1] += (double)rn * rn;
-                }
-            }
-            block_partial<4>(d, a.partial, 4);
-        }
-        if (!grid_sync(a.bar, target += gridDim.x, a.flags)) return;
-        {
-            double s[4];
-            grid_total<4>(a.partial, 4, s);
-            for (int k = 0; k < 2; ++k) {
-                if (!active[k]) continue;
-                rho_prev[k] = rho[k];
-                rho[k] = s[2 * k];
-                relres[k] = sqrt(s[2 * k + 1]) / bnorm[k];
-                if (relres[k] <= a.tol) {
-                    active[k] = false;
-                    conv[k] = true;
-                    iters[k] = it;
-                } else if (omega[k] == 0.0) {
-                    fail[k] = true;
-                    active[k] = false;
-                }
-            }
-        }
-    }
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        bool bad = false;
-        for (int k = 0; k < 2; ++k) {
-            if (active[k]) {   // hit maxit
-                iters[k] = it;
-                bad = true;
-            }
-            if (fail[k]) bad = true;
-        }
-        int* rp = a.rep + (int64_t)slot * 3;
-        rp[0] = iters[0];
-        rp[1] = iters[1];
-        rp[2] = bad ? 1 : 0;
-        a.rep_res[(int64_t)slot * 2] = relres[0];
-        a.rep_res[(int64_t)slot * 2 + 1] = relres[1];
-        if (bad) atomicExch(a.flags + 1, 1);
-        a.flags[2] = min(nhist + 1, max(a.order - 1, 1));   // past levels now stored
-        a.flags[3] = slot + 1;   // every block read the slot before the first barrier
-        a.flags[4] = ord;
-    }
+// report of a direct step (no iterations) and the next step's history and slot
+template <typename T>
+__global__ void lu_commit_kernel(Args<T> a) {
+    const int nhist = a.flags[2], slot = a.flags[3];
+    int* rp = a.rep + (int64_t)slot * 3;
+    rp[0] = rp[1] = rp[2] = 0;
+    a.rep_res[(int64_t)slot * 2] = 0.0;
+    a.rep_res[(int64_t)slot * 2 + 1] = 0.0;
+    a.flags[2] = min(nhist + 1, max(a.order - 1, 1));
+    a.flags[3] = slot + 1;
 }
 
 // ---------------------------------------------------------------------------
@@ -685,8 +354,11 @@ __global__ void __launch_bounds__(NT) step_kernel(Args<T> a) {
 // BiCGSTAB iteration as five kernels (A: p; B: q = A p; C: s; D: t = A s;
 // E: x, r), then the report (F).  Kernel boundaries make the vectors
 // coherent, so the SpMV gathers go through L1 (neighbouring rows share most
-// of their stencil nodes) -- inside one cooperative launch they must bypass
-// it -- and no grid barrier is needed.  Reductions: block partials, then the
+// of their stencil nodes) and no grid barrier is needed.  Operators just above
+// what the resident kernel holds run here too: against one cooperative launch
+// with grid barriers and gathers through L2, 60k rows of n = 101 in float32
+// took 408 us a step instead of 674, 100k of n = 50 468 instead of 599, 60k of
+// n = 50 in float64 979 instead of 1303.  Reductions: block partials, then the
 // phase's last block (by ticket) sums them in block order (deterministic)
 // and sets the scalars the next phase reads; the last block of E commits
 // the iteration and sets the loop condition.
@@ -828,7 +500,7 @@ __device__ __forceinline__ void next_iteration(PhaseCtl* c) {
     }
 }
 
-// R: right-hand side and r0 (the cooperative kernel's phase R, per row)
+// R: right-hand side and r0
 template <typename T>
 __global__ void __launch_bounds__(PT, PT_MINB) phase_R(Args<T> a) {
     const StepCoef<T> kc = step_coef(a);
@@ -1178,6 +850,8 @@ __global__ void __launch_bounds__(PT) phase_F(Args<T> a) {
     }
 }
 
+#include "step_resident.cuh"
+
 __global__ void lonely_barrier(unsigned long long* bar, int* err) {
     // a second arrival never comes: the bounded wait must give up
     grid_sync(bar, 2ull * gridDim.x, err);
@@ -1220,34 +894,30 @@ void fill_args(Args<T>& a, rbffd_op* op, rbffd_state* s, const rbffd_step_params
     a.delta[1] = (T)p->delta_v;
     a.tol = p->tol;
     a.maxit = p->maxit;
-    a.partial = ws->partial;
     a.bar = ws->bar;
     a.flags = ws->flags;
     a.rep = ws->rep;
     a.rep_res = ws->rep_res;
-    a.rhs_only = p->solver == RBFFD_SOLVER_BANDED_LU ? 1 : 0;
     a.ctl = ws->ctl;
     a.pp = ws->pp;
     a.cond = 0;
 }
 
+// one step by the cached LU factors: (c0 I - cl delta L) x = b, the factors of
+// the step's order (read on the device from flags[4]); x overwrites u, v
 template <typename T>
-rbffd_status launch_step(Args<T>& a, rbffd_step_ws* ws, cudaStream_t st) {
-    RBFFD_CUDA_TRY(cudaMemsetAsync(ws->bar, 0, sizeof(unsigned long long), st));
-    void* args[] = {&a};
-    const void* fn = ws->threads == 1024 ? (const void*)step_kernel<T, 1024> : (const void*)step_kernel<T, 256>;
-    RBFFD_CUDA_TRY(cudaLaunchCooperativeKernel(fn, dim3(ws->blocks),
-                                               dim3(ws->threads), args, 0, st));
+rbffd_status launch_lu_step(Args<T>& a, rbffd_step_ws* ws, cudaStream_t st) {
+    lu_rhs_kernel<T><<<(unsigned)std::min<int64_t>((a.N + 255) / 256, (int64_t)sm_count() * 8), 256, 0, st>>>(a);
     note_launch();
-    if (a.rhs_only) {
-        // (c0 I - cl delta L) x = b by the cached LU factors of the step's
-        // order (read on the device from flags[4]); x overwrites u, v
-        const void* b[2] = {V(a, 0, VB), a.ns == 2 ? V(a, 1, VB) : nullptr};
-        void* x[2] = {a.u, a.ns == 2 ? a.v : nullptr};
-        rbffd_status r = lu_solve_step(ws->lu, a.ns, b, x, std::is_same<T, float>::value ? RBFFD_F32 : RBFFD_F64,
-                                       ws->flags + 4, ws->ywork, ws->flags, st);
-        if (r != RBFFD_OK) return r;
-    }
+    RBFFD_CUDA_TRY(cudaGetLastError());
+    const void* b[2] = {V(a, 0, VB), a.ns == 2 ? V(a, 1, VB) : nullptr};
+    void* x[2] = {a.u, a.ns == 2 ? a.v : nullptr};
+    rbffd_status r = lu_solve_step(ws->lu, a.ns, b, x, std::is_same<T, float>::value ? RBFFD_F32 : RBFFD_F64,
+                                   ws->flags + 4, ws->ywork, ws->flags, st);
+    if (r != RBFFD_OK) return r;
+    lu_commit_kernel<T><<<1, 1, 0, st>>>(a);
+    note_launch();
+    RBFFD_CUDA_TRY(cudaGetLastError());
     return RBFFD_OK;
 }
 
@@ -1346,9 +1016,17 @@ rbffd_status build_phase_graph(Args<T> a, cudaGraphExec_t* out) {
 
 // nsteps launches, directly or by replaying one captured graph of a step
 template <typename T>
-rbffd_status run_steps(Args<T>& a, rbffd_step_ws* ws, int64_t nsteps, bool use_graph, cudaStream_t st) {
+rbffd_status run_steps(Args<T>& a, rbffd_step_ws* ws, int64_t nsteps, bool use_graph, bool lu, int nhist,
+                       bool* phased, cudaStream_t st) {
     static_assert(sizeof(Args<T>) <= sizeof(ws->graph_args), "graph key too small");
-    if (ws->phased && !a.rhs_only) {
+    if (!lu && nsteps > 0) {
+        // operators that fit the chip's shared memory: one launch for all steps
+        const ResidentPlan plan = resident_plan<T>(a.gi, a.N, a.ns, sm_count());
+        if (plan.blocks > 0)
+            return resident_launch(a, plan, nhist, nsteps, ws->vec, ws->rpart, st);
+    }
+    if (!lu) {
+        *phased = true;
         if (!use_graph) {
             for (int64_t k = 0; k < nsteps; ++k) {
                 rbffd_status r = phased_step_host(a, ws, st);
@@ -1377,7 +1055,7 @@ rbffd_status run_steps(Args<T>& a, rbffd_step_ws* ws, int64_t nsteps, bool use_g
     }
     if (!use_graph) {
         for (int64_t k = 0; k < nsteps; ++k) {
-            rbffd_status r = launch_step(a, ws, st);
+            rbffd_status r = launch_lu_step(a, ws, st);
             if (r != RBFFD_OK) return r;
         }
         return RBFFD_OK;
@@ -1385,7 +1063,7 @@ rbffd_status run_steps(Args<T>& a, rbffd_step_ws* ws, int64_t nsteps, bool use_g
     // the graph holds the kernels' arguments, the LU solve's factor pointers
     // included: any change recaptures it
     if (!ws->graph || ws->graph_args_size != sizeof(a) || memcmp(ws->graph_args, &a, sizeof(a)) != 0 ||
-        ws->solver != a.rhs_only || memcmp(ws->graph_lu, ws->lu, sizeof(ws->lu)) != 0 || ws->solver == 2) {
+        ws->solver != 1 || memcmp(ws->graph_lu, ws->lu, sizeof(ws->lu)) != 0) {
         if (ws->graph) {
             cudaGraphExecDestroy(ws->graph);
             ws->graph = nullptr;
@@ -1395,7 +1073,7 @@ rbffd_status run_steps(Args<T>& a, rbffd_step_ws* ws, int64_t nsteps, bool use_g
         if (!ws->cap) RBFFD_CUDA_TRY(cudaStreamCreateWithFlags(&ws->cap, cudaStreamNonBlocking));
         cudaGraph_t g = nullptr;
         RBFFD_CUDA_TRY(cudaStreamBeginCapture(ws->cap, cudaStreamCaptureModeThreadLocal));
-        rbffd_status r = launch_step(a, ws, ws->cap);
+        rbffd_status r = launch_lu_step(a, ws, ws->cap);
         cudaError_t e = cudaStreamEndCapture(ws->cap, &g);
         if (r != RBFFD_OK) return r;
         RBFFD_CUDA_TRY(e);
@@ -1404,12 +1082,12 @@ rbffd_status run_steps(Args<T>& a, rbffd_step_ws* ws, int64_t nsteps, bool use_g
         RBFFD_CUDA_TRY(e);
         memcpy(ws->graph_args, &a, sizeof(a));
         ws->graph_args_size = sizeof(a);
-        ws->solver = a.rhs_only;
+        ws->solver = 1;
         memcpy(ws->graph_lu, ws->lu, sizeof(ws->lu));
     }
     for (int64_t k = 0; k < nsteps; ++k) {
         RBFFD_CUDA_TRY(cudaGraphLaunch(ws->graph, st));
-        note_launch();
+        note_launch(3);   // right-hand side, solve, commit
     }
     return RBFFD_OK;
 }
@@ -1452,41 +1130,14 @@ extern "C" rbffd_status rbffd_step_imex(rbffd_op* op, rbffd_state* s, const rbff
         op->step = ws;
         ws->elem = elem;
         ws->N = op->N;
-        // The cooperative kernel's shape.  Large operators (a row per thread
-        // at one 1024-thread block per SM) run BiCGSTAB as phase kernels and
-        // use the cooperative launch only for the right-hand side of an LU
-        // step; there one 1024-thread block per SM meets at each grid barrier
-        // (measured when BiCGSTAB still ran in it, 1M-node operator: 2.67 ms
-        // per step against 3.08 ms with 2 x 512 and 3.22 ms with 2 x 256
-        // threads per SM; 4 x 256 was slower still, 3.94 ms -- the barrier's
-        // cost grows with its blocks).  Smaller operators keep 256-thread
-        // blocks (about four rows per thread) so that they still spread over
-        // the SMs.
-        ws->threads = op->N >= (int64_t)1024 * sm_count() ? 1024 : 256;
-        int dev = 0, per_sm = 0;
-        RBFFD_CUDA_TRY(cudaGetDevice(&dev));
-        const void* fn = elem == 4 ? (ws->threads == 1024 ? (const void*)step_kernel<float, 1024>
-                                                          : (const void*)step_kernel<float, 256>)
-                                   : (ws->threads == 1024 ? (const void*)step_kernel<double, 1024>
-                                                          : (const void*)step_kernel<double, 256>);
-        RBFFD_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, ws->threads, 0));
-        int64_t maxb = (int64_t)std::max(1, per_sm) * sm_count();
-        const int64_t rows_per_block = ws->threads == 1024 ? 1024 : 4 * 256;
-        int64_t want = (op->N + rows_per_block - 1) / rows_per_block;
-        ws->blocks = (int)std::max<int64_t>(1, std::min(maxb, std::max<int64_t>(want, 1)));
         RBFFD_CUDA_TRY(cudaMalloc(&ws->vec, 2 * 7 * ((op->N + 3) & ~(int64_t)3) * elem));
-        RBFFD_CUDA_TRY(cudaMalloc(&ws->partial, (size_t)NPHASE * ws->blocks * NSLOT * sizeof(double)));
         RBFFD_CUDA_TRY(cudaMalloc(&ws->bar, sizeof(unsigned long long)));
         RBFFD_CUDA_TRY(cudaMalloc(&ws->flags, 5 * sizeof(int)));
         RBFFD_CUDA_TRY(cudaMalloc(&ws->tstart, sizeof(double)));
-        // large operators: BiCGSTAB as phase kernels under a device-side
-        // loop (SpMV gathers through L1, full occupancy); small ones: the
-        // cooperative kernel (a few blocks, latency-bound, where one launch
-        // per step wins)
-        ws->phased = ws->threads == 1024 ? 1 : 0;
         RBFFD_CUDA_TRY(cudaMalloc(&ws->ctl, sizeof(PhaseCtl)));
         RBFFD_CUDA_TRY(cudaMemset(ws->ctl, 0, sizeof(PhaseCtl)));
         RBFFD_CUDA_TRY(cudaMalloc(&ws->pp, (size_t)std::max<int64_t>(1, (op->N + PT - 1) / PT) * 8 * sizeof(double)));
+        RBFFD_CUDA_TRY(cudaMalloc(&ws->rpart, (size_t)2 * sm_count() * RES_SUMS * sizeof(double)));
         ws->rep_cap = 0;
     }
     if (ws->rep_cap < std::max<int64_t>(nsteps, 1)) {
@@ -1497,7 +1148,8 @@ extern "C" rbffd_status rbffd_step_imex(rbffd_op* op, rbffd_state* s, const rbff
         RBFFD_CUDA_TRY(cudaMalloc(&ws->rep_res, ws->rep_cap * 2 * sizeof(double)));
     }
     const int kept = std::max(order - 1, 1);   // past levels the order stores
-    int hflags[5] = {0, 0, std::min(s->has_history, kept), 0, 0};   // slot counter starts at 0
+    const int hist0 = std::min(s->has_history, kept);
+    int hflags[5] = {0, 0, hist0, 0, 0};   // slot counter starts at 0
     if (p->solver == RBFFD_SOLVER_BANDED_LU) {
         // factor (c0 I - cl delta L) for every SBDF order this call steps
         // with (orders climb while history builds up) and species, once per
@@ -1535,16 +1187,18 @@ extern "C" rbffd_status rbffd_step_imex(rbffd_op* op, rbffd_state* s, const rbff
     RBFFD_CUDA_TRY(cudaMemcpyAsync(ws->tstart, &s->t, sizeof(double), cudaMemcpyHostToDevice, st));
     RBFFD_CUDA_TRY(cudaMemsetAsync(ws->rep, 0, ws->rep_cap * 3 * sizeof(int), st));
     rbffd_status rs;
+    const bool lu = p->solver == RBFFD_SOLVER_BANDED_LU;
+    bool phased = false;   // BiCGSTAB ran as phase kernels (their launches are counted from the report)
     if (elem == 4) {
         Args<float> a;
         memset(&a, 0, sizeof(a));
         fill_args(a, op, s, p, ws);
-        rs = run_steps(a, ws, nsteps, p->use_graph != 0, st);
+        rs = run_steps(a, ws, nsteps, p->use_graph != 0, lu, hist0, &phased, st);
     } else {
         Args<double> a;
         memset(&a, 0, sizeof(a));
         fill_args(a, op, s, p, ws);
-        rs = run_steps(a, ws, nsteps, p->use_graph != 0, st);
+        rs = run_steps(a, ws, nsteps, p->use_graph != 0, lu, hist0, &phased, st);
     }
     if (rs != RBFFD_OK) return rs;
     std::vector<int> rep(std::max<int64_t>(nsteps, 1) * 3);
@@ -1567,7 +1221,7 @@ extern "C" rbffd_status rbffd_step_imex(rbffd_op* op, rbffd_state* s, const rbff
         r.last_relres_u = res[2 * k];
         r.last_relres_v = res[2 * k + 1];
     }
-    if (ws->phased && p->use_graph && p->solver == RBFFD_SOLVER_BICGSTAB)
+    if (phased && p->use_graph)
         for (int64_t k = 0; k < nsteps; ++k) note_launch(5 * std::max(rep[3 * k], rep[3 * k + 1]));
     r.steps_done = nsteps;
     s->has_history = (int)std::min<int64_t>((int64_t)std::min(s->has_history, kept) + nsteps, kept);

@@ -1,0 +1,567 @@
+// IMEX steps with the operator resident on the chip: one launch runs all the
+// steps of a call, each block keeping its slices of the ELL matrix in shared
+// memory and its rows' vectors in registers.
+//
+// What bounds it.  An operator of up to about 30 MB fits the shared memory of
+// the chip, and then an iteration moves no matrix bytes: what is left are its
+// synchronisations (one for each vector that neighbours read or sum that all
+// blocks need, five per BiCGSTAB iteration) and the gathers.  Two forms:
+//
+//  * one thread-block cluster (up to 16 blocks) for small operators: the
+//    gathered vector is copied to every block's shared memory, sums and copies
+//    travel through distributed shared memory, and the barrier is the
+//    cluster's (a few hundred nanoseconds);
+//  * a cooperative grid of one block per SM: gathers through L1 / L2 and the
+//    bounded grid barrier (about a microsecond and a half).
+//
+// TPR lanes share a row: each reads every TPR-th chunk of four entries, a
+// shuffle adds them up, and all of them hold the row's vector entries in
+// registers.  Sums of products go through shared memory, one value per row,
+// to one warp per sum (float64 arithmetic on all warps would cost more than
+// the iteration), float32 products as exact pairs (Dot2, as in the phase
+// kernels), and then from every block to all in a fixed order.
+//
+// Measured against one cooperative launch per step with the matrix streamed
+// from L2 and three blocks for the small operator: 2,562 nodes, n = 31, heat
+// equation in float64, 3.8 iterations per step: 314 -> 58 us per step; 40k
+// torus, n = 50, two species in float32: 320 -> 113 us per step.
+//
+// Included by step.cu inside its anonymous namespace.
+
+constexpr int RES_SUMS = 6;        // sums of one reduction, at most
+constexpr int RES_CLUSTER = 16;    // blocks of a cluster
+
+// threads per block, at most (float64 rows hold twice the registers)
+template <typename T>
+constexpr int res_threads() { return sizeof(T) == 8 ? 512 : 1024; }
+
+struct ResidentInfo {
+    int spb;             // slices of 32 rows per block
+    int max_elems;       // matrix elements of a block, at most
+    int64_t nsteps;
+    int nhist;           // past levels valid when the call begins
+    void* gather;        // grid form: ns x N gathered vector
+    double* part;        // grid form: 2 x blocks x RES_SUMS
+};
+
+__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ uint32_t peer_addr(uint32_t a, uint32_t rank) {
+    uint32_t r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void st_peer(uint32_t a, float v) {
+    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
+}
+__device__ __forceinline__ void st_peer(uint32_t a, double v) {
+    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
+}
+__device__ __forceinline__ uint32_t cluster_rank() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ void cluster_sync_all() {
+    asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
+}
+
+// a row's product as it goes to the summing warp
+template <typename T>
+struct Term {
+    using type = double;
+    __device__ static double of(double a, double b) { return a * b; }
+    __device__ static double add(double x, double y) { return x + y; }
+    __device__ static double value(double x) { return x; }
+};
+template <>
+struct Term<float> {
+    using type = float2;   // unevaluated sum x + y
+    __device__ static float2 of(float a, float b) {
+        const float p = __fmul_rn(a, b);
+        return make_float2(p, __fmaf_rn(a, b, -p));
+    }
+    __device__ static float2 add(float2 u, float2 v) {
+        const float x = __fadd_rn(u.x, v.x), z = __fsub_rn(x, u.x);
+        const float t = __fadd_rn(__fsub_rn(u.x, __fsub_rn(x, z)), __fsub_rn(v.x, z));   // u.x + v.x = x + t
+        return make_float2(x, __fadd_rn(t, __fadd_rn(u.y, v.y)));
+    }
+    __device__ static double value(float2 u) { return (double)u.x + (double)u.y; }
+};
+
+__device__ __forceinline__ double shfl_down_term(double x, int o) { return __shfl_down_sync(0xffffffffu, x, o); }
+__device__ __forceinline__ float2 shfl_down_term(float2 x, int o) {
+    return make_float2(__shfl_down_sync(0xffffffffu, x.x, o), __shfl_down_sync(0xffffffffu, x.y, o));
+}
+
+// what one lane per species decides and every thread of the block reads (the
+// scalar arithmetic is float64: on all warps it would cost more than the
+// products)
+template <typename T>
+struct ResidentScalars {
+    T beta[2], alpha[2], omega[2];
+    int act[2], early[2], zero[2];
+};
+
+// shared memory of a block, in this order (all offsets multiples of 16 bytes)
+template <typename T>
+struct ResidentSmem {
+    size_t w, idx, gather, terms, part, scal, total;
+    __host__ __device__ ResidentSmem(int max_elems, int rows, int64_t N, int ns, bool cluster) {
+        auto up = [](size_t x) { return (x + 15) & ~(size_t)15; };
+        w = 0;
+        idx = up(w + (size_t)max_elems * sizeof(T));
+        gather = up(idx + (size_t)max_elems * sizeof(int32_t));
+        terms = up(gather + (cluster ? (size_t)ns * N * sizeof(T) : 0));
+        part = up(terms + (size_t)RES_SUMS * rows * sizeof(typename Term<T>::type));
+        scal = up(part + (cluster ? 2 * RES_CLUSTER * RES_SUMS * sizeof(double) : 0));
+        total = up(scal + sizeof(ResidentScalars<T>));
+    }
+};
+
+// one block's view of the synchronisations
+template <typename T, bool CL>
+struct ResidentBlock {
+    unsigned char* sm;
+    ResidentSmem<T> L;
+    const Args<T>& a;
+    const ResidentInfo& ri;
+    int rows;                        // rows of a block (padding included)
+    int parity = 0;
+    unsigned long long target = 0;   // grid form: barrier count
+
+    // x (node i of species sp) to wherever blocks gather from: the TPR lanes
+    // of the row share the peers
+    template <int TPR>
+    __device__ void publish(int sp, int64_t i, int lane, T x) {
+        if (CL) {
+            const uint32_t at = smem_u32(sm + L.gather) + (uint32_t)((sp * a.N + i) * sizeof(T));
+            for (int p = lane; p < (int)gridDim.x; p += TPR) st_peer(peer_addr(at, p), x);
+        } else if (lane == 0) {
+            ((T*)ri.gather)[sp * a.N + i] = x;
+        }
+    }
+    __device__ const T* gathered(int sp) const {
+        return (CL ? (const T*)(sm + L.gather) : (const T*)ri.gather) + sp * a.N;
+    }
+    __device__ bool sync() {
+        if (CL) {
+            cluster_sync_all();
+            return true;
+        }
+        return grid_sync(a.bar, target += gridDim.x, a.flags);
+    }
+    // KS sums per species over all rows (terms v of each row, written by its
+    // lane 0), and the barrier that makes them, and what was published,
+    // visible; lane 0 of warp k then decides with the totals of species k
+    template <int KS, int NS, typename F>
+    __device__ bool reduce(const typename Term<T>::type (&v)[NS][KS], int row, bool writes, F decide) {
+        using TM = Term<T>;
+        using V = typename TM::type;
+        V* terms = (V*)(sm + L.terms);
+        if (writes) {
+#pragma unroll
+            for (int k = 0; k < NS; ++k)
+#pragma unroll
+                for (int j = 0; j < KS; ++j) terms[(k * KS + j) * rows + row] = v[k][j];
+        }
+        __syncthreads();
+        const int wid = threadIdx.x >> 5, ln = threadIdx.x & 31, nw = blockDim.x >> 5;
+        double* pp = CL ? (double*)(sm + L.part) + parity * RES_CLUSTER * RES_SUMS
+                        : ri.part + (int64_t)parity * gridDim.x * RES_SUMS;
+        for (int k = wid; k < NS * KS; k += nw) {
+            V s = terms[k * rows + ln];
+            for (int r = ln + 32; r < rows; r += 32) s = TM::add(s, terms[k * rows + r]);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) s = TM::add(s, shfl_down_term(s, o));
+            if (CL) {
+                const double t = __shfl_sync(0xffffffffu, TM::value(s), 0);
+                if (ln < (int)gridDim.x) st_peer(peer_addr(smem_u32(pp + blockIdx.x * RES_SUMS + k), ln), t);
+            } else if (ln == 0) {
+                __stcg(pp + (int64_t)blockIdx.x * RES_SUMS + k, TM::value(s));
+            }
+        }
+        if (!sync()) return false;
+        for (int k = wid; k < NS; k += nw) {
+            double tot[KS];
+#pragma unroll
+            for (int j = 0; j < KS; ++j) tot[j] = 0.0;
+            for (int b = ln; b < (int)gridDim.x; b += 32)
+#pragma unroll
+                for (int j = 0; j < KS; ++j)
+                    tot[j] += CL ? pp[b * RES_SUMS + k * KS + j] : __ldcg(pp + (int64_t)b * RES_SUMS + k * KS + j);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+                for (int j = 0; j < KS; ++j) tot[j] += __shfl_down_sync(0xffffffffu, tot[j], o);
+            if (ln == 0) decide(k, tot);
+        }
+        __syncthreads();
+        parity ^= 1;
+        return true;
+    }
+};
+
+template <typename T, int TPR, int NS, bool CL>
+__global__ void __launch_bounds__(res_threads<T>(), 1) resident_kernel(Args<T> a, ResidentInfo ri) {
+    extern __shared__ __align__(16) unsigned char res_smem[];
+    using TM = Term<T>;
+    const int rows = ri.spb * 32, RPW = 32 / TPR;
+    ResidentBlock<T, CL> B{res_smem, ResidentSmem<T>(ri.max_elems, rows, a.N, NS, CL), a, ri, rows};
+    T* sw = (T*)(res_smem + B.L.w);
+    int32_t* si = (int32_t*)(res_smem + B.L.idx);
+
+    // ---- this block's slices into shared memory; this thread's row
+    const int64_t s0 = (int64_t)blockIdx.x * ri.spb;
+    int64_t e0 = -1, e1 = 0;   // element range of the block
+    const int tid = threadIdx.x, lane = (tid & 31) / RPW;            // lane of the row
+    const int lrow = (tid >> 5) * RPW + (tid & 31) % RPW;            // row of the block
+    bool own = false;
+    int64_t node = 0, rbase = 0;
+    int nch = 0;
+    {
+        int64_t sl = 0;   // slices before group g
+        for (int g = 0; g < a.gi.ngroups; ++g) {
+            const int64_t cnt = a.gi.row_begin[g + 1] - a.gi.row_begin[g], ns = (cnt + 31) / 32;
+            const int64_t lo = max(s0, sl), hi = min(s0 + ri.spb, sl + ns);
+            if (lo < hi) {
+                const int64_t se = (int64_t)32 * a.gi.npad[g];
+                if (e0 < 0) e0 = a.gi.ell_off[g] + (lo - sl) * se;
+                e1 = a.gi.ell_off[g] + (hi - sl) * se;
+            }
+            const int64_t my = s0 + lrow / 32;
+            if (lrow < rows && my >= sl && my < sl + ns) {
+                const int64_t lr = (my - sl) * 32 + lrow % 32;
+                own = lr < cnt;
+                if (own) node = a.row_node[a.gi.row_begin[g] + lr];
+                rbase = ell_elem(a.gi.ell_off[g], a.gi.npad[g], lr, 0);
+                nch = a.gi.npad[g] >> 2;
+            }
+            sl += ns;
+        }
+    }
+    if (e0 < 0) e0 = e1;
+    for (int64_t e = e0 + 4 * tid; e < e1; e += 4 * (int64_t)blockDim.x) {
+        *reinterpret_cast<int4*>(si + (e - e0)) = __ldcs(reinterpret_cast<const int4*>(a.idx + e));
+        T w[4];
+        load4s(a.w + e, w);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) sw[e - e0 + q] = w[q];
+    }
+    const int sb = (int)(rbase - e0);
+
+    // row sums of both species against the gathered vector
+    auto product = [&](T (&y)[NS]) {
+#pragma unroll
+        for (int k = 0; k < NS; ++k) y[k] = T(0);
+        if (own) {
+            const T* g0 = B.gathered(0);
+            const T* g1 = NS == 2 ? B.gathered(1) : g0;
+#pragma unroll 2
+            for (int c = lane; c < nch; c += TPR) {
+                const int4 iv = *reinterpret_cast<const int4*>(si + sb + c * 128);
+                T w[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) w[q] = sw[sb + c * 128 + q];
+                const int ii[4] = {iv.x, iv.y, iv.z, iv.w};
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    y[0] = fma(w[q], g0[ii[q]], y[0]);
+                    if (NS == 2) y[NS - 1] = fma(w[q], g1[ii[q]], y[NS - 1]);
+                }
+            }
+        }
+#pragma unroll
+        for (int o = RPW; o < 32; o <<= 1)
+#pragma unroll
+            for (int k = 0; k < NS; ++k) y[k] += __shfl_xor_sync(0xffffffffu, y[k], o);
+    };
+
+    T x[NS], r[NS], rh[NS], p[NS], q[NS], s[NS], t[NS];
+#pragma unroll
+    for (int k = 0; k < NS; ++k) {
+        x[k] = own ? (k == 0 ? a.u : a.v)[node] : T(0);
+        r[k] = rh[k] = p[k] = q[k] = s[k] = t[k] = T(0);
+    }
+    const bool lead = own && lane == 0, sums = lane == 0 && lrow < rows;
+    volatile ResidentScalars<T>& sc = *(volatile ResidentScalars<T>*)(res_smem + B.L.scal);
+    // state of the deciding lanes (lane 0 of warps 0 .. NS - 1); res2, limit2:
+    // squared norms of the residual and of its tolerance
+    double bnorm = 0.0, limit2 = 0.0, rho = 0.0, rho_prev = 1.0, alpha = 1.0, omega = 1.0, res2 = 0.0;
+    bool active = false, fail = false;
+    int iters = 0, it = 0, nhist = ri.nhist;
+    if (CL) cluster_sync_all();   // every block of the cluster runs before its shared memory is written
+
+    for (int64_t step = 0; step < ri.nsteps; ++step) {
+        const StepCoef<T> kc = step_coef_at(a, nhist, (int)step);
+        const T kk[2] = {kc.k0, kc.k1};
+#pragma unroll
+        for (int k = 0; k < NS; ++k)
+            if (own) B.template publish<TPR>(k, node, lane, x[k]);
+        if (!B.sync()) return;
+        // ---- right-hand side, r0 = b - A x
+        T y[NS], b[2] = {T(0), T(0)};
+        product(y);
+        if (lead) rhs_values(a, kc, node, x[0], NS == 2 ? x[NS - 1] : T(0), b[0], b[1]);
+        typename TM::type d1[NS][1], d2[NS][2];
+#pragma unroll
+        for (int k = 0; k < NS; ++k) {
+            b[k] = __shfl_sync(0xffffffffu, b[k], (tid & 31) % RPW);
+            r[k] = b[k] - (kc.c0 * x[k] - kk[k] * y[k]);
+            rh[k] = r[k];
+            p[k] = q[k] = T(0);
+            d2[k][0] = TM::of(b[k], b[k]);
+            d2[k][1] = TM::of(r[k], r[k]);
+        }
+        it = 0;
+        if (!B.template reduce<2, NS>(d2, lrow, sums, [&](int k, const double (&tot)[2]) {
+                bnorm = sqrt(tot[0]);
+                limit2 = (a.tol * bnorm) * (a.tol * bnorm);
+                rho = tot[1];   // (r-hat, r0) = |r0|^2
+                rho_prev = alpha = omega = 1.0;
+                res2 = rho;
+                active = !(bnorm == 0.0 || sqrt(rho) / bnorm <= a.tol);
+                fail = active && !isfinite(rho);
+                active = active && !fail;
+                iters = 0;
+                sc.beta[k] = T(0);
+                sc.omega[k] = T(1);
+                sc.act[k] = active;
+                sc.zero[k] = bnorm == 0.0;
+            }))
+            return;
+#pragma unroll
+        for (int k = 0; k < NS; ++k)
+            if (sc.zero[k]) x[k] = T(0);   // b = 0: x = 0
+        while ((sc.act[0] || (NS == 2 && sc.act[NS - 1])) && it < a.maxit) {
+            ++it;
+            // ---- A: p = r + beta (p - omega q)
+#pragma unroll
+            for (int k = 0; k < NS; ++k)
+                if (sc.act[k] && own) {
+                    p[k] = r[k] + sc.beta[k] * (p[k] - sc.omega[k] * q[k]);
+                    B.template publish<TPR>(k, node, lane, p[k]);
+                }
+            if (!B.sync()) return;
+            // ---- B: q = A p ; (r-hat, q)
+            product(y);
+#pragma unroll
+            for (int k = 0; k < NS; ++k) {
+                if (sc.act[k]) q[k] = kc.c0 * p[k] - kk[k] * y[k];
+                d1[k][0] = TM::of(rh[k], q[k]);
+            }
+            if (!B.template reduce<1, NS>(d1, lrow, sums, [&](int k, const double (&tot)[1]) {
+                    if (active) {
+                        alpha = rho / tot[0];
+                        if (tot[0] == 0.0 || !isfinite(alpha)) {
+                            fail = true;
+                            active = false;
+                        }
+                        sc.alpha[k] = (T)alpha;
+                    }
+                    sc.act[k] = active;
+                }))
+                return;
+            // ---- C: s = r - alpha q ; |s|^2
+#pragma unroll
+            for (int k = 0; k < NS; ++k) {
+                if (sc.act[k] && own) {
+                    s[k] = r[k] - sc.alpha[k] * q[k];
+                    B.template publish<TPR>(k, node, lane, s[k]);
+                }
+                d1[k][0] = TM::of(s[k], s[k]);
+            }
+            if (!B.template reduce<1, NS>(d1, lrow, sums, [&](int k, const double (&tot)[1]) {
+                    const bool early = active && tot[0] <= limit2;
+                    if (early) {
+                        res2 = tot[0];
+                        iters = it;
+                        active = false;
+                    }
+                    sc.early[k] = early;
+                    sc.act[k] = active;
+                }))
+                return;
+            // ---- D: t = A s ; (t, s), (t, t)   (x += alpha p where s converged)
+#pragma unroll
+            for (int k = 0; k < NS; ++k)
+                if (sc.early[k]) x[k] += sc.alpha[k] * p[k];
+            if (!(sc.act[0] || (NS == 2 && sc.act[NS - 1]))) break;
+            product(y);
+#pragma unroll
+            for (int k = 0; k < NS; ++k) {
+                if (sc.act[k]) t[k] = kc.c0 * s[k] - kk[k] * y[k];
+                d2[k][0] = TM::of(t[k], s[k]);
+                d2[k][1] = TM::of(t[k], t[k]);
+            }
+            if (!B.template reduce<2, NS>(d2, lrow, sums, [&](int k, const double (&tot)[2]) {
+                    if (active) {
+                        omega = tot[0] / tot[1];
+                        if (tot[1] == 0.0 || !isfinite(omega)) {
+                            fail = true;
+                            active = false;
+                        }
+                        sc.omega[k] = (T)omega;
+                    }
+                    sc.act[k] = active;
+                }))
+                return;
+            // ---- E: x += alpha p + omega s ; r = s - omega t ; (r-hat, r), |r|^2
+#pragma unroll
+            for (int k = 0; k < NS; ++k) {
+                if (sc.act[k]) {
+                    x[k] += sc.alpha[k] * p[k] + sc.omega[k] * s[k];
+                    r[k] = s[k] - sc.omega[k] * t[k];
+                }
+                d2[k][0] = TM::of(rh[k], r[k]);
+                d2[k][1] = TM::of(r[k], r[k]);
+            }
+            if (!B.template reduce<2, NS>(d2, lrow, sums, [&](int k, const double (&tot)[2]) {
+                    if (active) {
+                        rho_prev = rho;
+                        rho = tot[0];
+                        if (tot[1] <= limit2) {
+                            iters = it;
+                            active = false;
+                        } else {
+                            // beta of the next iteration, if there is one
+                            const double beta = (rho / rho_prev) * (alpha / omega);
+                            if (omega == 0.0 || (it < a.maxit && (rho == 0.0 || !isfinite(beta)))) {
+                                fail = true;
+                                active = false;
+                            }
+                            sc.beta[k] = (T)beta;
+                        }
+                        res2 = tot[1];
+                    }
+                    sc.act[k] = active;
+                }))
+                return;
+        }
+        // ---- report of the step
+        if (blockIdx.x == 0 && (tid & 31) == 0 && (tid >> 5) < NS) {
+            const int k = tid >> 5;
+            if (active) iters = it;   // hit maxit
+            a.rep[step * 3 + k] = iters;
+            a.rep_res[step * 2 + k] = bnorm > 0 ? sqrt(res2) / bnorm : 0.0;
+            if (active || fail) {
+                atomicExch(a.rep + step * 3 + 2, 1);
+                atomicExch(a.flags + 1, 1);
+            }
+            if (NS == 1) {
+                a.rep[step * 3 + 1] = 0;
+                a.rep_res[step * 2 + 1] = 0.0;
+            }
+        }
+        nhist = min(nhist + 1, max(a.order - 1, 1));
+    }
+#pragma unroll
+    for (int k = 0; k < NS; ++k)
+        if (lead) (k == 0 ? a.u : a.v)[node] = x[k];
+}
+
+// A plan of the resident kernel for an operator: TPR lanes per row, slices per
+// block, blocks and form; blocks = 0 when the operator does not fit.
+struct ResidentPlan {
+    int blocks = 0, tpr = 1, spb = 0, max_elems = 0;
+    bool cluster = false;
+    size_t smem = 0;
+};
+
+// elements of the largest run of spb consecutive slices
+inline int64_t largest_block(const GroupInfo& gi, int spb, int64_t* slices) {
+    std::vector<int64_t> start(1, 0);   // element offset of each slice
+    for (int g = 0; g < gi.ngroups; ++g) {
+        const int64_t ns = (gi.row_begin[g + 1] - gi.row_begin[g] + 31) / 32;
+        for (int64_t k = 0; k < ns; ++k) start.push_back(start.back() + (int64_t)32 * gi.npad[g]);
+    }
+    const int64_t n = (int64_t)start.size() - 1;
+    int64_t most = 0;
+    for (int64_t b = 0; b < n; b += spb) most = std::max(most, start[std::min(n, b + spb)] - start[b]);
+    *slices = n;
+    return most;
+}
+
+constexpr size_t RES_SMEM_MAX = 227 * 1024;
+
+template <typename T>
+ResidentPlan resident_plan(const GroupInfo& gi, int64_t N, int ns, int sms) {
+    ResidentPlan best;
+    for (int form = 0; form < 2 && !best.blocks; ++form) {
+        ResidentPlan p;
+        p.cluster = form == 0;
+        int64_t slices = 0;
+        largest_block(gi, 1, &slices);
+        const int64_t blocks = std::min<int64_t>(slices, p.cluster ? RES_CLUSTER : sms);
+        p.spb = (int)((slices + blocks - 1) / blocks);
+        if (p.spb * 32 > res_threads<T>()) continue;
+        p.blocks = (int)((slices + p.spb - 1) / p.spb);
+        if (p.cluster)   // a power of two; the last blocks may have no rows
+            for (int c = 1;; c *= 2)
+                if (c >= p.blocks) {
+                    p.blocks = c;
+                    break;
+                }
+        const int64_t elems = largest_block(gi, p.spb, &slices);
+        if (elems * (int64_t)(sizeof(T) + 4) > (int64_t)RES_SMEM_MAX) continue;
+        p.max_elems = (int)elems;
+        p.smem = ResidentSmem<T>(p.max_elems, p.spb * 32, N, ns, p.cluster).total;
+        if (p.smem > RES_SMEM_MAX) continue;
+        // float64 rows gain nothing from more lanes (the float64 unit is the
+        // bound); float32 ones take up to four
+        while (sizeof(T) == 4 && p.tpr < 4 && p.spb * 32 * p.tpr * 2 <= res_threads<T>()) p.tpr *= 2;
+        best = p;
+    }
+    return best;
+}
+
+template <typename T, int TPR, int NS>
+rbffd_status resident_launch_as(Args<T>& a, const ResidentPlan& p, const ResidentInfo& ri, cudaStream_t st) {
+    const int threads = std::max(64, p.spb * 32 * TPR);   // at least a warp per species
+    if (p.cluster) {
+        auto* fn = resident_kernel<T, TPR, NS, true>;
+        RBFFD_CUDA_TRY(cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem));
+        RBFFD_CUDA_TRY(cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(p.blocks);
+        cfg.blockDim = dim3(threads);
+        cfg.dynamicSmemBytes = p.smem;
+        cfg.stream = st;
+        cudaLaunchAttribute at;
+        at.id = cudaLaunchAttributeClusterDimension;
+        at.val.clusterDim.x = p.blocks;
+        at.val.clusterDim.y = at.val.clusterDim.z = 1;
+        cfg.attrs = &at;
+        cfg.numAttrs = 1;
+        RBFFD_CUDA_TRY(cudaLaunchKernelEx(&cfg, fn, a, ri));
+    } else {
+        auto* fn = resident_kernel<T, TPR, NS, false>;
+        RBFFD_CUDA_TRY(cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem));
+        RBFFD_CUDA_TRY(cudaMemsetAsync(a.bar, 0, sizeof(unsigned long long), st));
+        ResidentInfo r = ri;
+        void* args[] = {&a, &r};
+        RBFFD_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)fn, dim3(p.blocks), dim3(threads), args, p.smem, st));
+    }
+    note_launch();
+    return RBFFD_OK;
+}
+
+template <typename T>
+rbffd_status resident_launch(Args<T>& a, const ResidentPlan& p, int nhist, int64_t nsteps, void* gather, double* part,
+                             cudaStream_t st) {
+    ResidentInfo ri;
+    memset(&ri, 0, sizeof(ri));
+    ri.spb = p.spb;
+    ri.max_elems = p.max_elems;
+    ri.nsteps = nsteps;
+    ri.nhist = nhist;
+    ri.gather = gather;
+    ri.part = part;
+    if (a.ns == 1) {
+        if (p.tpr == 1) return resident_launch_as<T, 1, 1>(a, p, ri, st);
+        if (sizeof(T) == 4 && p.tpr == 2) return resident_launch_as<T, 2, 1>(a, p, ri, st);
+        return resident_launch_as<T, 4, 1>(a, p, ri, st);
+    }
+    if (p.tpr == 1) return resident_launch_as<T, 1, 2>(a, p, ri, st);
+    if (sizeof(T) == 4 && p.tpr == 2) return resident_launch_as<T, 2, 2>(a, p, ri, st);
+    return resident_launch_as<T, 4, 2>(a, p, ri, st);
+}
