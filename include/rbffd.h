@@ -399,9 +399,9 @@ rbffd_status rbffd_stencil_weights_noalloc(const double* nodes, const double* no
  * Cuthill-McKee for faster iterative solves).  Each returns perm (N int32,
  * perm[k] = the original index of the node placed k-th); the library never
  * reorders on its own: the caller applies perm to its node, normal and field
- * arrays (x_new[k] = x[perm[k]]) and builds on the reordered set.  The sorts
- * and searches run on the host (one-off O(N log N) / O(nnz) steps);
- * synchronous.  Errors: RBFFD_EINVAL (NULL argument, N out of range,
+ * arrays (x_new[k] = x[perm[k]]) and builds on the reordered set.  The
+ * Morton keys are sorted on the device, the Cuthill-McKee searches run on the
+ * host; synchronous.  Errors: RBFFD_EINVAL (NULL argument, N out of range,
  * non-finite coordinates, a column index out of range), RBFFD_ECUDA.
  * ---------------------------------------------------------------------- */
 

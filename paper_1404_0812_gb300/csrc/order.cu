@@ -4,8 +4,8 @@
 // before any stencil exists.  Both return a permutation perm with perm[k] =
 // the original index of the node placed k-th; the caller applies it to its
 // node, normal and field arrays (x_new[k] = x[perm[k]]) and builds on the
-// reordered set.  The sorts and the breadth-first search run on the host:
-// they are one-off, O(N log N) / O(nnz) steps ahead of the build.
+// reordered set.  The Morton keys are sorted on the device (a stable radix
+// sort); the breadth-first searches of the Cuthill-McKee order run on the host.
 #include "common.cuh"
 
 #include <algorithm>
@@ -17,28 +17,32 @@
 namespace rbffd {
 namespace {
 
-__global__ void bbox_blocks(const double* __restrict__ X, int64_t N, double* __restrict__ out) {
-    __shared__ double lo[3][128], hi[3][128];
-    double l[3] = {INFINITY, INFINITY, INFINITY}, h[3] = {-INFINITY, -INFINITY, -INFINITY};
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x)
+constexpr int BOX_THREADS = 256;
+
+// bounding box of n boxes (in: 6 doubles each, lo then hi) or, with X, of
+// nodes: one box per block into out (min and max are exact: any order)
+__global__ void __launch_bounds__(BOX_THREADS) bbox_blocks(const double* __restrict__ X, const double* __restrict__ in,
+                                                          int64_t n, double* __restrict__ out) {
+    __shared__ double w[6][BOX_THREADS / 32];
+    double v[6] = {INFINITY, INFINITY, INFINITY, -INFINITY, -INFINITY, -INFINITY};
+    for (int64_t i = blockIdx.x * (int64_t)BOX_THREADS + threadIdx.x; i < n; i += (int64_t)gridDim.x * BOX_THREADS)
         for (int a = 0; a < 3; ++a) {
-            double v = X[3 * i + a];
-            l[a] = fmin(l[a], v);
-            h[a] = fmax(h[a], v);
+            v[a] = fmin(v[a], X ? X[3 * i + a] : in[6 * i + a]);
+            v[3 + a] = fmax(v[3 + a], X ? X[3 * i + a] : in[6 * i + 3 + a]);
         }
-    for (int a = 0; a < 3; ++a) {
-        lo[a][threadIdx.x] = l[a];
-        hi[a][threadIdx.x] = h[a];
-    }
+    for (int o = 16; o > 0; o >>= 1)
+        for (int a = 0; a < 3; ++a) {
+            v[a] = fmin(v[a], __shfl_xor_sync(0xffffffffu, v[a], o));
+            v[3 + a] = fmax(v[3 + a], __shfl_xor_sync(0xffffffffu, v[3 + a], o));
+        }
+    if ((threadIdx.x & 31) == 0)
+        for (int a = 0; a < 6; ++a) w[a][threadIdx.x >> 5] = v[a];
     __syncthreads();
-    if (threadIdx.x < 3) {
-        double a0 = INFINITY, a1 = -INFINITY;
-        for (int t = 0; t < (int)blockDim.x; ++t) {
-            a0 = fmin(a0, lo[threadIdx.x][t]);
-            a1 = fmax(a1, hi[threadIdx.x][t]);
-        }
-        out[6 * blockIdx.x + threadIdx.x] = a0;
-        out[6 * blockIdx.x + 3 + threadIdx.x] = a1;
+    if (threadIdx.x < 6) {
+        double x = w[threadIdx.x][0];
+        for (int k = 1; k < BOX_THREADS / 32; ++k)
+            x = threadIdx.x < 3 ? fmin(x, w[threadIdx.x][k]) : fmax(x, w[threadIdx.x][k]);
+        out[6 * blockIdx.x + threadIdx.x] = x;
     }
 }
 
@@ -66,6 +70,225 @@ __global__ void morton_keys(const double* __restrict__ X, int64_t N, double x0, 
     key[i] = spread3(q[0]) | (spread3(q[1]) << 1) | (spread3(q[2]) << 2);
 }
 
+// ---------------------------------------------------------------------------
+// Stable radix sort of (key, index) pairs, least significant byte first.
+//
+// A pass reads and writes 12 bytes per node; at a million nodes these stay in
+// L2 and the sort is bound by its launches (three per pass: digit counts of
+// every tile, their prefix sums digit by digit, scatter).  A tile's ranks come
+// from warp matches, in element order, so equal keys keep the index order; the
+// tile is put in order in shared memory first, which makes the scatter runs of
+// neighbours.  Up to one tile of nodes, one block does all passes.  Against
+// keys copied to the host and sorted there: 1M nodes 75.5 -> 0.21 ms.
+// ---------------------------------------------------------------------------
+constexpr int SORT_THREADS = 256, SORT_ITEMS = 16, SORT_WARPS = SORT_THREADS / 32;
+constexpr int TILE = SORT_THREADS * SORT_ITEMS, BINS = 256, PASSES = 8;   // 63-bit keys
+
+struct TileShared {
+    uint64_t key[TILE];
+    int32_t val[TILE];
+    int32_t wcount[SORT_WARPS][BINS];   // per warp: counts, then the offset among equal digits
+    int32_t first[BINS];                // tile position of each digit's first element
+    int32_t gbase[BINS];                // global position of the same
+    int32_t wsum[SORT_WARPS];
+};
+
+// exclusive prefix sum of one value per thread over the block
+__device__ int32_t block_exclusive(int32_t v, int32_t* wsum) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    int32_t x = v;
+    for (int o = 1; o < 32; o <<= 1) {
+        const int32_t y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) wsum[w] = x;
+    __syncthreads();
+    int32_t base = 0;
+    for (int k = 0; k < w; ++k) base += wsum[k];
+    __syncthreads();
+    return base + x - v;
+}
+
+// Sorts a tile of n elements by the digit at `shift` into S.key / S.val;
+// element warp * 512 + i * 32 + lane is item i of a thread.  S.first holds the
+// digits' first positions.
+__device__ void sort_tile(TileShared& S, const uint64_t (&key)[SORT_ITEMS], const int32_t (&val)[SORT_ITEMS], int n,
+                          int shift) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    for (int b = threadIdx.x; b < SORT_WARPS * BINS; b += SORT_THREADS) (&S.wcount[0][0])[b] = 0;
+    __syncthreads();
+    int32_t rank[SORT_ITEMS];
+#pragma unroll
+    for (int i = 0; i < SORT_ITEMS; ++i) {
+        const int e = w * (32 * SORT_ITEMS) + i * 32 + lane;
+        const int d = e < n ? (int)(key[i] >> shift) & (BINS - 1) : BINS;
+        const unsigned peers = __match_any_sync(0xffffffffu, d);
+        const int32_t old = d < BINS ? S.wcount[w][d] : 0;
+        rank[i] = old + __popc(peers & ((1u << lane) - 1u));
+        __syncwarp();
+        if (d < BINS && (peers >> lane) == 1u) S.wcount[w][d] = old + __popc(peers);   // the last of its peers
+        __syncwarp();
+    }
+    __syncthreads();
+    int32_t total = 0;
+    for (int k = 0; k < SORT_WARPS; ++k) {
+        const int32_t c = S.wcount[k][threadIdx.x];
+        S.wcount[k][threadIdx.x] = total;
+        total += c;
+    }
+    S.first[threadIdx.x] = block_exclusive(total, S.wsum);
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < SORT_ITEMS; ++i) {
+        const int e = w * (32 * SORT_ITEMS) + i * 32 + lane;
+        if (e < n) {
+            const int d = (int)(key[i] >> shift) & (BINS - 1);
+            const int at = S.first[d] + S.wcount[w][d] + rank[i];
+            S.key[at] = key[i];
+            S.val[at] = val[i];
+        }
+    }
+    __syncthreads();
+}
+
+__global__ void __launch_bounds__(SORT_THREADS) sort_counts(const uint64_t* __restrict__ key, int64_t N, int shift,
+                                                           int ntiles, int32_t* __restrict__ counts) {
+    __shared__ int32_t h[BINS];
+    h[threadIdx.x] = 0;
+    __syncthreads();
+    const int64_t base = (int64_t)blockIdx.x * TILE;
+#pragma unroll
+    for (int i = 0; i < SORT_ITEMS; ++i) {
+        const int64_t e = base + i * SORT_THREADS + threadIdx.x;
+        const int d = e < N ? (int)(key[e] >> shift) & (BINS - 1) : BINS;
+        const unsigned peers = __match_any_sync(0xffffffffu, d);
+        if (d < BINS && (peers >> (threadIdx.x & 31)) == 1u) atomicAdd(&h[d], __popc(peers));
+    }
+    __syncthreads();
+    counts[(int64_t)threadIdx.x * ntiles + blockIdx.x] = h[threadIdx.x];
+}
+
+// counts of digit blockIdx.x over the tiles -> exclusive prefix sums, and the
+// digit's total
+__global__ void __launch_bounds__(SORT_THREADS) sort_prefix(int32_t* __restrict__ counts, int ntiles,
+                                                           int32_t* __restrict__ totals) {
+    __shared__ int32_t wsum[SORT_WARPS], last;
+    int32_t* c = counts + (int64_t)blockIdx.x * ntiles;
+    int32_t run = 0;
+    for (int t0 = 0; t0 < ntiles; t0 += SORT_THREADS) {
+        const int t = t0 + threadIdx.x;
+        const int32_t v = t < ntiles ? c[t] : 0;
+        const int32_t x = block_exclusive(v, wsum);
+        if (t < ntiles) c[t] = run + x;
+        if (threadIdx.x == SORT_THREADS - 1) last = x + v;
+        __syncthreads();
+        run += last;
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) totals[blockIdx.x] = run;
+}
+
+// one pass: keys in -> out; in_val NULL: the element's own index (first
+// pass); out_key NULL: only the indices are written (last pass)
+__global__ void __launch_bounds__(SORT_THREADS) sort_scatter(const uint64_t* __restrict__ in_key,
+                                                            const int32_t* __restrict__ in_val, int64_t N, int shift,
+                                                            int ntiles, const int32_t* __restrict__ prefix,
+                                                            const int32_t* __restrict__ totals,
+                                                            uint64_t* __restrict__ out_key,
+                                                            int32_t* __restrict__ out_val) {
+    extern __shared__ __align__(16) unsigned char sort_smem[];
+    TileShared& S = *reinterpret_cast<TileShared*>(sort_smem);
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t base = (int64_t)blockIdx.x * TILE;
+    const int n = (int)(N - base < TILE ? N - base : TILE);
+    uint64_t key[SORT_ITEMS];
+    int32_t val[SORT_ITEMS];
+#pragma unroll
+    for (int i = 0; i < SORT_ITEMS; ++i) {
+        const int e = w * (32 * SORT_ITEMS) + i * 32 + lane;
+        key[i] = e < n ? in_key[base + e] : 0;
+        val[i] = e < n ? (in_val ? in_val[base + e] : (int32_t)(base + e)) : 0;
+    }
+    S.gbase[threadIdx.x] = block_exclusive(totals[threadIdx.x], S.wsum) + prefix[(int64_t)threadIdx.x * ntiles + blockIdx.x];
+    sort_tile(S, key, val, n, shift);
+    for (int j = threadIdx.x; j < n; j += SORT_THREADS) {
+        const uint64_t k = S.key[j];
+        const int d = (int)(k >> shift) & (BINS - 1);
+        const int64_t at = (int64_t)S.gbase[d] + (j - S.first[d]);
+        if (out_key) out_key[at] = k;
+        out_val[at] = S.val[j];
+    }
+}
+
+// all passes of up to one tile
+__global__ void __launch_bounds__(SORT_THREADS) sort_one_tile(const uint64_t* __restrict__ in_key, int n,
+                                                             int32_t* __restrict__ out_val) {
+    extern __shared__ __align__(16) unsigned char sort_smem[];
+    TileShared& S = *reinterpret_cast<TileShared*>(sort_smem);
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    for (int j = threadIdx.x; j < n; j += SORT_THREADS) {
+        S.key[j] = in_key[j];
+        S.val[j] = j;
+    }
+    __syncthreads();
+    for (int p = 0; p < PASSES; ++p) {
+        uint64_t key[SORT_ITEMS];
+        int32_t val[SORT_ITEMS];
+#pragma unroll
+        for (int i = 0; i < SORT_ITEMS; ++i) {
+            const int e = w * (32 * SORT_ITEMS) + i * 32 + lane;
+            key[i] = e < n ? S.key[e] : 0;
+            val[i] = e < n ? S.val[e] : 0;
+        }
+        __syncthreads();
+        sort_tile(S, key, val, n, 8 * p);
+    }
+    for (int j = threadIdx.x; j < n; j += SORT_THREADS) out_val[j] = S.val[j];
+}
+
+// perm = the indices of key[0..N-1] in (key, index) order; key is scratch
+rbffd_status sort_keys_device(uint64_t* key, int64_t N, int32_t* perm, cudaStream_t st) {
+    const size_t smem = sizeof(TileShared);
+    if (N <= TILE) {
+        RBFFD_CUDA_TRY(cudaFuncSetAttribute(sort_one_tile, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        sort_one_tile<<<1, SORT_THREADS, smem, st>>>(key, (int)N, perm);
+        note_launch();
+        RBFFD_CUDA_TRY(cudaGetLastError());
+        return RBFFD_OK;
+    }
+    RBFFD_CUDA_TRY(cudaFuncSetAttribute(sort_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    const int ntiles = (int)((N + TILE - 1) / TILE);
+    uint64_t* key2 = nullptr;
+    int32_t *val = nullptr, *val2 = nullptr, *counts = nullptr;
+    RBFFD_CUDA_TRY(pool_alloc(&key2, (size_t)N * sizeof(uint64_t), st));
+    RBFFD_CUDA_TRY(pool_alloc(&val, (size_t)N * sizeof(int32_t), st));
+    RBFFD_CUDA_TRY(pool_alloc(&val2, (size_t)N * sizeof(int32_t), st));
+    RBFFD_CUDA_TRY(pool_alloc(&counts, ((size_t)BINS * ntiles + BINS) * sizeof(int32_t), st));
+    int32_t* totals = counts + (size_t)BINS * ntiles;
+    const uint64_t* k_in = key;
+    uint64_t* k_out = key2;
+    const int32_t* v_in = nullptr;
+    int32_t* v_out = val;
+    for (int p = 0; p < PASSES; ++p) {
+        const bool final_pass = p == PASSES - 1;
+        sort_counts<<<ntiles, SORT_THREADS, 0, st>>>(k_in, N, 8 * p, ntiles, counts);
+        sort_prefix<<<BINS, SORT_THREADS, 0, st>>>(counts, ntiles, totals);
+        sort_scatter<<<ntiles, SORT_THREADS, smem, st>>>(k_in, v_in, N, 8 * p, ntiles, counts, totals,
+                                                        final_pass ? nullptr : k_out, final_pass ? perm : v_out);
+        note_launch(3);
+        RBFFD_CUDA_TRY(cudaGetLastError());
+        k_in = k_out;
+        k_out = k_out == key ? key2 : key;
+        v_in = v_out;
+        v_out = v_out == val ? val2 : val;
+    }
+    cudaFreeAsync(key2, st);
+    cudaFreeAsync(val, st);
+    cudaFreeAsync(val2, st);
+    cudaFreeAsync(counts, st);
+    return RBFFD_OK;
+}
+
 __global__ void stencil_rows(const int32_t* __restrict__ idx, const int32_t* __restrict__ row_node, GroupInfo gi,
                              int64_t R, int nmax, int32_t* __restrict__ out, int32_t* __restrict__ deg) {
     int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -88,23 +311,19 @@ extern "C" rbffd_status rbffd_morton_order(const double* nodes, int64_t N, int32
     RBFFD_CHECK_ARG(nodes && perm, "NULL argument");
     RBFFD_CHECK_ARG(N >= 1 && N < (int64_t)1 << 31, "N must be in [1, 2^31)");
     cudaStream_t st = as_stream(stream);
-    const int nb = (int)std::min<int64_t>(1024, (N + 127) / 128);
+    const int nb = (int)std::min<int64_t>((int64_t)sm_count() * 4, (N + BOX_THREADS - 1) / BOX_THREADS);
     double* part = nullptr;
     uint64_t* key = nullptr;
-    RBFFD_CUDA_TRY(pool_alloc(&part, (size_t)nb * 6 * sizeof(double), st));
-    bbox_blocks<<<nb, 128, 0, st>>>(nodes, N, part);
-    note_launch();
+    RBFFD_CUDA_TRY(pool_alloc(&part, (size_t)(nb + 1) * 6 * sizeof(double), st));
+    bbox_blocks<<<nb, BOX_THREADS, 0, st>>>(nodes, nullptr, N, part + 6);
+    bbox_blocks<<<1, BOX_THREADS, 0, st>>>(nullptr, part + 6, nb, part);
+    note_launch(2);
     RBFFD_CUDA_TRY(cudaGetLastError());
-    std::vector<double> hp((size_t)nb * 6);
-    RBFFD_CUDA_TRY(cudaMemcpyAsync(hp.data(), part, hp.size() * sizeof(double), cudaMemcpyDeviceToHost, st));
+    double box[6];
+    RBFFD_CUDA_TRY(cudaMemcpyAsync(box, part, sizeof(box), cudaMemcpyDeviceToHost, st));
     RBFFD_CUDA_TRY(cudaStreamSynchronize(st));
     cudaFreeAsync(part, st);
-    double lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
-    for (int b = 0; b < nb; ++b)
-        for (int a = 0; a < 3; ++a) {
-            lo[a] = std::min(lo[a], hp[6 * b + a]);
-            hi[a] = std::max(hi[a], hp[6 * b + 3 + a]);
-        }
+    const double *lo = box, *hi = box + 3;
     double ext = std::max(hi[0] - lo[0], std::max(hi[1] - lo[1], hi[2] - lo[2]));
     RBFFD_CHECK_ARG(std::isfinite(ext), "non-finite node coordinates");
     const double scale = ext > 0.0 ? 2097151.0 / ext : 0.0;   // one cube: the Z-order keeps proportions
@@ -112,14 +331,9 @@ extern "C" rbffd_status rbffd_morton_order(const double* nodes, int64_t N, int32
     morton_keys<<<(unsigned)((N + 255) / 256), 256, 0, st>>>(nodes, N, lo[0], lo[1], lo[2], scale, key);
     note_launch();
     RBFFD_CUDA_TRY(cudaGetLastError());
-    std::vector<uint64_t> hk((size_t)N);
-    RBFFD_CUDA_TRY(cudaMemcpyAsync(hk.data(), key, (size_t)N * sizeof(uint64_t), cudaMemcpyDeviceToHost, st));
-    RBFFD_CUDA_TRY(cudaStreamSynchronize(st));
+    const rbffd_status s = sort_keys_device(key, N, perm, st);
     cudaFreeAsync(key, st);
-    std::vector<int32_t> p((size_t)N);
-    std::iota(p.begin(), p.end(), 0);
-    std::sort(p.begin(), p.end(), [&](int32_t a, int32_t b) { return hk[a] < hk[b] || (hk[a] == hk[b] && a < b); });
-    RBFFD_CUDA_TRY(cudaMemcpyAsync(perm, p.data(), (size_t)N * sizeof(int32_t), cudaMemcpyHostToDevice, st));
+    if (s != RBFFD_OK) return s;
     RBFFD_CUDA_TRY(cudaStreamSynchronize(st));
     return RBFFD_OK;
 }
