@@ -147,6 +147,7 @@ struct rbffd_lu {
     int32_t* piv;               // N
     void* work;                 // 2 N + 16 values: b and y of rbffd_lu_solve
     int* err;                   // device flag: a bounded wait of the solve gave up
+    int interchanges;           // some step of the factorisation interchanged rows
 };
 
 struct rbffd_mlp {
