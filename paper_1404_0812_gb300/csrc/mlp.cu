@@ -10,7 +10,9 @@
 // whole forward and backward pass in shared memory (4x4 register tiles for
 // the three dense products); each CTA writes its gradient contribution to
 // its own row of a partial buffer, and a second kernel sums the rows in a
-// fixed order (deterministic) and applies Adam.  The products are far too
+// fixed order (deterministic) and applies Adam.  A mini-batch is too few tiles
+// for the chip (1,024 samples: 16); mlp_tile_cluster then spreads each tile
+// over a cluster of CTAs, with the same sums in the same order.  The products are far too
 // small (64 x 64 x <=303 per tile) for tensor-core tiles to pay, and the
 // network is specified in float32, so they run on the FP32 pipes.
 #include "common.cuh"
@@ -283,16 +285,255 @@ mlp_tile(const float* __restrict__ params, int D, const float* __restrict__ feat
     }
 }
 
+// ---------------------------------------------------------------------------
+// forward + backward of one tile on a cluster of C CTAs (mode 1 of mlp_tile
+// for mini-batches).  A step is bound by latency: 16 tiles of 1,024 samples
+// keep 16 of 152 SMs busy for 85 us.  Here a CTA runs TS / C samples forward
+// and back to dZ1, copies its samples' H1, H2, dZ2 and dZ1 to its peers through
+// distributed shared memory, and after one cluster barrier forms 1 / C of the
+// gradient's rows over all samples of the tile.  Every element keeps its sum in
+// sample order, so the gradient has the bits of mlp_tile's.  n = 50, batches of
+// 1,024: 93 -> 14 us per training step.
+// ---------------------------------------------------------------------------
+constexpr int W2S = H + 1;   // row stride of W2 in shared memory (rows and columns are read)
+
+struct ClusterTile {         // float offsets in shared memory
+    int X, XC, W1, W2, W3, Z1, Z2, H1, H2, D2, D1, dy, sq, total;
+    __host__ __device__ ClusterTile(int D, int C) {
+        const int own = TS / C, slice = (D + C - 1) / C;
+        int o = 0;
+        W1 = o; o += D * H;
+        W3 = o; o += H;
+        X = o; o += own * D;          // own samples' features
+        XC = o; o += TS * slice;      // all samples' features of this CTA's gradient rows
+        W2 = o; o += H * W2S;
+        Z1 = o; o += own * H;
+        Z2 = o; o += own * H;
+        o = (o + 3) / 4 * 4;
+        // all samples, filled by the cluster (H1: the columns of this CTA's rows
+        // of dW2 beside its own samples; H2: complete on the last CTA)
+        H1 = o; o += TS * H;
+        H2 = o; o += TS * H;
+        D2 = o; o += TS * H;
+        D1 = o; o += TS * H;
+        dy = o; o += TS;
+        sq = o; o += TS;
+        total = o;
+    }
+};
+
+__device__ __forceinline__ void st_peer4(uint32_t a, float4 v) {
+    asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(a), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w)
+                 : "memory");
+}
+
+__device__ __forceinline__ void cp4(float* dst, const float* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void cp16(float* dst, const float* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+
+template <int C>
+__global__ void __launch_bounds__(NT)
+mlp_tile_cluster(const float* __restrict__ params, int D, const float* __restrict__ feats,
+                 const float* __restrict__ target, const int32_t* __restrict__ sel, int64_t count, float inv_B,
+                 float* __restrict__ partial, float* __restrict__ loss_part) {
+    extern __shared__ __align__(16) float smc[];
+    constexpr int OWN = TS / C, PER = OWN / 4;   // samples of this CTA; outputs per thread of a layer
+    const ClusterTile L(D, C);
+    const View P = view(params, D);
+    const int t = threadIdx.x, rank = blockIdx.x % C;
+    const int64_t tile = blockIdx.x / C, s0 = tile * TS;
+    const int ns = (int)((count - s0) < TS ? (count - s0) : TS);
+    const int first = rank * OWN;                // tile sample of this CTA's sample 0
+    const int slice = (D + C - 1) / C, d0 = rank * slice, d1 = min(D, d0 + slice);
+    asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory");   // peers have started (waited for below)
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    // weights and features by asynchronous copies, all in flight together
+    // (loads in the products' loops cost 15 us of L2 latency)
+    __shared__ int64_t row[TS];
+    if (t < TS) row[t] = t < ns ? (sel ? (int64_t)sel[s0 + t] : s0 + t) : -1;
+    __syncthreads();
+    for (int s = t >> 5; s < TS; s += NT / 32) {        // a warp per sample
+        const float* f = feats + row[s] * D;
+        const bool real = row[s] >= 0;
+        for (int d = d0 + (t & 31); d < d0 + slice; d += 32) {
+            float* to = smc + L.XC + s * slice + d - d0;
+            if (real && d < D) cp4(to, f + d); else *to = 0.f;
+        }
+        if (s >= first && s < first + OWN)
+            for (int d = t & 31; d < D; d += 32) {
+                float* to = smc + L.X + (s - first) * D + d;
+                if (real) cp4(to, f + d); else *to = 0.f;
+            }
+    }
+    // the weights after the step before this one has updated them
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    for (int e = 4 * t; e < D * H; e += 4 * NT) cp16(smc + L.W1 + e, P.W1 + e);
+    for (int e = t; e < H; e += NT) cp4(smc + L.W3 + e, P.W3 + e);
+    for (int e = t; e < H * H; e += NT) cp4(smc + L.W2 + (e / H) * W2S + e % H, P.W2 + e);
+    asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
+    __syncthreads();
+    const float tgt = t < OWN && first + t < ns ? target[row[first + t]] : 0.f;
+    const int h = t & 63, sb = t >> 6;           // this thread's unit; samples sb + 4 i
+    float* const H1 = smc + L.H1 + first * H;    // own samples' rows of the shared arrays
+    float* const H2 = smc + L.H2 + first * H;
+    float* const D2 = smc + L.D2 + first * H;
+    float* const D1 = smc + L.D1 + first * H;
+    float acc[PER];
+#pragma unroll
+    for (int i = 0; i < PER; ++i) acc[i] = P.b1[h];
+#pragma unroll 8
+    for (int d = 0; d < D; ++d) {
+        const float w = smc[L.W1 + d * H + h];
+#pragma unroll
+        for (int i = 0; i < PER; ++i) acc[i] = fmaf(smc[L.X + (sb + 4 * i) * D + d], w, acc[i]);
+    }
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+        smc[L.Z1 + (sb + 4 * i) * H + h] = acc[i];
+        H1[(sb + 4 * i) * H + h] = gelu(acc[i]);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < PER; ++i) acc[i] = P.b2[h];
+#pragma unroll 8
+    for (int k = 0; k < H; ++k) {
+        const float w = smc[L.W2 + k * W2S + h];
+#pragma unroll
+        for (int i = 0; i < PER; ++i) acc[i] = fmaf(H1[(sb + 4 * i) * H + k], w, acc[i]);
+    }
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+        smc[L.Z2 + (sb + 4 * i) * H + h] = acc[i];
+        H2[(sb + 4 * i) * H + h] = gelu(acc[i]);
+    }
+    __syncthreads();
+    if (t < OWN) {
+        float y = P.b3[0];
+#pragma unroll 16
+        for (int k = 0; k < H; ++k) y = fmaf(H2[t * H + k], smc[L.W3 + k], y);
+        float r = 0.f;
+        if (first + t < ns) r = y - tgt;
+        smc[L.dy + first + t] = 2.f * r * inv_B;
+        smc[L.sq + first + t] = r * r;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+        const int s = sb + 4 * i;
+        D2[s * H + h] = smc[L.dy + first + s] * smc[L.W3 + h] * gelu_grad(smc[L.Z2 + s * H + h]);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < PER; ++i) acc[i] = 0.f;
+#pragma unroll 8
+    for (int k = 0; k < H; ++k) {
+        const float w = smc[L.W2 + h * W2S + k];   // unit h of layer 1
+#pragma unroll
+        for (int i = 0; i < PER; ++i) acc[i] = fmaf(D2[(sb + 4 * i) * H + k], w, acc[i]);
+    }
+#pragma unroll
+    for (int i = 0; i < PER; ++i) D1[(sb + 4 * i) * H + h] = acc[i] * gelu_grad(smc[L.Z1 + (sb + 4 * i) * H + h]);
+    __syncthreads();
+    // ---- own samples to the peers
+    asm volatile("barrier.cluster.wait;" ::: "memory");
+    const uint32_t base = (uint32_t)__cvta_generic_to_shared(smc);
+    for (int e = t; e < C * OWN * (H / 4); e += NT) {
+        const int p = e / (OWN * (H / 4)), q = e - p * (OWN * (H / 4));
+        if (p == rank) continue;
+        uint32_t pb;
+        asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(pb) : "r"(base), "r"(p));
+        const int off = first * H + 4 * q;
+        const int col = (4 * q) % H;
+        if (col >= p * (H / C) && col < (p + 1) * (H / C))
+            st_peer4(pb + 4 * (L.H1 + off), *reinterpret_cast<const float4*>(smc + L.H1 + off));
+        if (p == C - 1) st_peer4(pb + 4 * (L.H2 + off), *reinterpret_cast<const float4*>(smc + L.H2 + off));
+        st_peer4(pb + 4 * (L.D2 + off), *reinterpret_cast<const float4*>(smc + L.D2 + off));
+        st_peer4(pb + 4 * (L.D1 + off), *reinterpret_cast<const float4*>(smc + L.D1 + off));
+        if (q < 2 * OWN / 4) {   // dy and sq of the own samples
+            const int o1 = (q < OWN / 4 ? L.dy : L.sq) + first + 4 * (q % (OWN / 4));
+            st_peer4(pb + 4 * o1, *reinterpret_cast<const float4*>(smc + o1));
+        }
+    }
+    asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
+    // ---- this CTA's rows of the tile's gradient
+    const int64_t Pc = param_count(D);
+    float* G = partial + tile * Pc;
+    float* gW1 = G;
+    float* gb1 = gW1 + (int64_t)D * H;
+    float* gW2 = gb1 + H;
+    float* gb2 = gW2 + H * H;
+    float* gW3 = gb2 + H;
+    float* gb3 = gW3 + H;
+    const int ha = (t & 15) * 4, rg = t >> 4;
+    for (int d = d0 + rg; d < d1; d += NT / 16) {
+        float a[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 8
+        for (int s = 0; s < TS; ++s) {
+            const float x = smc[L.XC + s * slice + (d - d0)];
+            const float4 dz = *reinterpret_cast<const float4*>(smc + L.D1 + s * H + ha);
+            a[0] = fmaf(x, dz.x, a[0]);
+            a[1] = fmaf(x, dz.y, a[1]);
+            a[2] = fmaf(x, dz.z, a[2]);
+            a[3] = fmaf(x, dz.w, a[3]);
+        }
+        for (int b = 0; b < 4; ++b) gW1[(int64_t)d * H + ha + b] = a[b];   // a tile's partial starts at any float
+    }
+    for (int k = rank * (H / C) + rg; k < (rank + 1) * (H / C); k += NT / 16) {
+        float a[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 8
+        for (int s = 0; s < TS; ++s) {
+            const float x = smc[L.H1 + s * H + k];
+            const float4 dz = *reinterpret_cast<const float4*>(smc + L.D2 + s * H + ha);
+            a[0] = fmaf(x, dz.x, a[0]);
+            a[1] = fmaf(x, dz.y, a[1]);
+            a[2] = fmaf(x, dz.z, a[2]);
+            a[3] = fmaf(x, dz.w, a[3]);
+        }
+        for (int b = 0; b < 4; ++b) gW2[k * H + ha + b] = a[b];
+    }
+    if (rank == 0 && t < H) {
+        float g2 = 0.f, g1 = 0.f;
+#pragma unroll 8
+        for (int s = 0; s < TS; ++s) {
+            g2 += smc[L.D2 + s * H + t];
+            g1 += smc[L.D1 + s * H + t];
+        }
+        gb2[t] = g2;
+        gb1[t] = g1;
+    } else if (rank == C - 1 && t < H) {
+        float g = 0.f;
+#pragma unroll 8
+        for (int s = 0; s < TS; ++s) g = fmaf(smc[L.H2 + s * H + t], smc[L.dy + s], g);
+        gW3[t] = g;
+    } else if (rank == C - 1 && t == H) {
+        float g = 0.f, l = 0.f;
+        for (int s = 0; s < TS; ++s) {
+            g += smc[L.dy + s];
+            l += smc[L.sq + s];
+        }
+        gb3[0] = g;
+        loss_part[tile] = l;
+    }
+}
+
 // grad[p] = sum over tiles of partial[c][p] (fixed order); optionally Adam.
 __global__ void reduce_grad(const float* __restrict__ partial, int ntiles, int64_t P,
                             const float* __restrict__ loss_part, float* __restrict__ grad,
                             float* __restrict__ loss_out, float* __restrict__ params,
                             float* __restrict__ m, float* __restrict__ v, int adam_t, float lr,
                             int loss_slot) {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < P;
          p += (int64_t)gridDim.x * blockDim.x) {
         float g = 0.f;
-        for (int c = 0; c < ntiles; ++c) g += partial[(int64_t)c * P + p];
+#pragma unroll 16
+        for (int c = 0; c < ntiles; ++c) g += __ldcs(partial + (int64_t)c * P + p);
         if (grad) grad[p] = g;
         if (params) {
             const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
@@ -314,9 +555,82 @@ __global__ void reduce_grad(const float* __restrict__ partial, int ntiles, int64
 
 size_t tile_smem(int D) { return (size_t)(TS * D + 4 * TS * H + 2 * TS) * sizeof(float); }
 
+template <int C>
+rbffd_status launch_cluster_tiles(const rbffd_mlp* m, const float* feats, const float* target, const int32_t* sel,
+                                  int64_t count, int tiles, float* loss_part, cudaStream_t st) {
+    const size_t smem = (size_t)ClusterTile(m->D, C).total * sizeof(float);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(tiles * C));
+    cfg.blockDim = dim3(NT);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = C;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // see launch_reduce
+    at[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 2;
+    RBFFD_CUDA_TRY(cudaLaunchKernelEx(&cfg, mlp_tile_cluster<C>, (const float*)m->params, m->D, feats, target, sel,
+                                      count, 1.f / (float)count, m->partial, loss_part));
+    note_launch();
+    return RBFFD_OK;
+}
+
+// Gradient partials of `count` samples (sel: their rows, or NULL): clusters of
+// eight or four CTAs per tile while those stay within one wave of the chip, a
+// CTA per tile beyond (its register tiles move fewer shared-memory bytes per
+// FMA, and there are tiles enough), or where the weights of a large network
+// leave no room for a cluster's arrays.
+constexpr size_t CLUSTER_SMEM_MAX = 227 * 1024;
+template <int C>
+bool cluster_fits(int D) { return ClusterTile(D, C).total * sizeof(float) + 1024 <= CLUSTER_SMEM_MAX; }
+
+rbffd_status gradient_tiles(const rbffd_mlp* m, const float* feats, const float* target, const int32_t* sel,
+                            int64_t count, float* loss_part, cudaStream_t st) {
+    const int64_t tiles = (count + TS - 1) / TS;
+    if (tiles * 8 <= sm_count() && cluster_fits<8>(m->D))
+        return launch_cluster_tiles<8>(m, feats, target, sel, count, (int)tiles, loss_part, st);
+    if (tiles * 4 <= sm_count() && cluster_fits<4>(m->D))
+        return launch_cluster_tiles<4>(m, feats, target, sel, count, (int)tiles, loss_part, st);
+    mlp_tile<<<(unsigned)tiles, NT, tile_smem(m->D), st>>>(m->params, m->D, feats, target, sel, count,
+                                                           1.f / (float)count, 1, nullptr, m->partial, loss_part);
+    note_launch();
+    RBFFD_CUDA_TRY(cudaGetLastError());
+    return RBFFD_OK;
+}
+
+// The sum over tiles (and Adam).  Launched, like the cluster tiles, as a
+// programmatic dependent: the kernel starts while the one before it drains, and
+// waits for its results (griddepcontrol.wait) only before it reads them, which
+// takes the launch latencies of a step's two kernels off its path.
+rbffd_status launch_reduce(const rbffd_mlp* m, int tiles, float* grad, float* params, float* am, float* av, int adam_t,
+                           float lr, int slot, cudaStream_t st) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)((m->P + 127) / 128));
+    cfg.blockDim = dim3(128);
+    cfg.stream = st;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    RBFFD_CUDA_TRY(cudaLaunchKernelEx(&cfg, reduce_grad, (const float*)m->partial, tiles, m->P,
+                                      (const float*)(m->loss + 4096), grad, m->loss, params, am, av, adam_t, lr, slot));
+    note_launch();
+    return RBFFD_OK;
+}
+
 rbffd_status ensure_smem(int D) {
     RBFFD_CUDA_TRY(cudaFuncSetAttribute(mlp_tile, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         (int)tile_smem(D)));
+    if (cluster_fits<8>(D))
+        RBFFD_CUDA_TRY(cudaFuncSetAttribute(mlp_tile_cluster<8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        (int)(ClusterTile(D, 8).total * sizeof(float))));
+    if (cluster_fits<4>(D))
+        RBFFD_CUDA_TRY(cudaFuncSetAttribute(mlp_tile_cluster<4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        (int)(ClusterTile(D, 4).total * sizeof(float))));
     return RBFFD_OK;
 }
 
@@ -479,16 +793,10 @@ rbffd_status rbffd_mlp_loss_grad(const rbffd_mlp* mc, const float* feats, const 
     if (s != RBFFD_OK) return s;
     s = ensure_smem(m->D);
     if (s != RBFFD_OK) return s;
-    mlp_tile<<<(unsigned)tiles, NT, tile_smem(m->D), st>>>(m->params, m->D, feats, target, nullptr, count,
-                                                           1.f / (float)count, 1, nullptr, m->partial,
-                                                           m->loss + 4096);
-    note_launch();
-    RBFFD_CUDA_TRY(cudaGetLastError());
-    reduce_grad<<<(unsigned)((m->P + 255) / 256), 256, 0, st>>>(m->partial, (int)tiles, m->P, m->loss + 4096,
-                                                                grad, m->loss, nullptr, nullptr, nullptr, 0,
-                                                                0.f, 0);
-    note_launch();
-    RBFFD_CUDA_TRY(cudaGetLastError());
+    s = gradient_tiles(m, feats, target, nullptr, count, m->loss + 4096, st);
+    if (s != RBFFD_OK) return s;
+    s = launch_reduce(m, (int)tiles, grad, nullptr, nullptr, nullptr, 0, 0.f, 0, st);
+    if (s != RBFFD_OK) return s;
     if (loss) {
         // mean squared error = sum of squares / count
         float hl = 0.f;
@@ -514,36 +822,40 @@ rbffd_status rbffd_mlp_train(rbffd_mlp* m, const float* feats, const float* targ
     if (s != RBFFD_OK) return s;
     int32_t* perm_d = nullptr;
     RBFFD_CUDA_TRY(pool_alloc(&perm_d, count * sizeof(int32_t), st));
-    std::vector<int32_t> perm(count);
+    std::vector<int32_t> perm(count), next;
     for (int64_t i = 0; i < count; ++i) perm[i] = (int32_t)i;
     std::mt19937_64 rng(seed);
     int64_t steps_per_epoch = (count + batch - 1) / batch;
     RBFFD_CHECK_ARG(steps_per_epoch <= 4096, "count / batch must be <= 4096");
     std::vector<float> lossv(steps_per_epoch);
-    for (int ep = 0; ep < epochs; ++ep) {
+    auto shuffle = [&](std::vector<int32_t>& p) {
         for (int64_t i = count - 1; i > 0; --i) {
             int64_t j = (int64_t)(rng() % (uint64_t)(i + 1));
-            std::swap(perm[i], perm[j]);
+            std::swap(p[i], p[j]);
         }
+    };
+    shuffle(perm);
+    for (int ep = 0; ep < epochs; ++ep) {
         RBFFD_CUDA_TRY(cudaMemcpyAsync(perm_d, perm.data(), count * sizeof(int32_t), cudaMemcpyHostToDevice, st));
         for (int64_t b = 0; b < steps_per_epoch; ++b) {
             int64_t b0 = b * batch;
             int64_t nb = std::min<int64_t>(batch, count - b0);
             unsigned tiles = (unsigned)((nb + TS - 1) / TS);
             ++m->adam_t;   // the step counter lives with the network's moments
-            mlp_tile<<<tiles, NT, tile_smem(m->D), st>>>(m->params, m->D, feats, target, perm_d + b0, nb,
-                                                         1.f / (float)nb, 1, nullptr, m->partial,
-                                                         m->loss + 4096);
-            note_launch();
-            reduce_grad<<<(unsigned)((m->P + 255) / 256), 256, 0, st>>>(
-                m->partial, (int)tiles, m->P, m->loss + 4096, nullptr, m->loss, m->params, m->adam_m,
-                m->adam_v, m->adam_t, lr, (int)b);
-            note_launch();
+            s = gradient_tiles(m, feats, target, perm_d + b0, nb, m->loss + 4096, st);
+            if (s != RBFFD_OK) return s;
+            s = launch_reduce(m, (int)tiles, nullptr, m->params, m->adam_m, m->adam_v, m->adam_t, lr, (int)b, st);
+            if (s != RBFFD_OK) return s;
         }
         RBFFD_CUDA_TRY(cudaGetLastError());
+        if (ep + 1 < epochs) {   // the next epoch's order while the device works on this one
+            next = perm;
+            shuffle(next);
+        }
         RBFFD_CUDA_TRY(cudaMemcpyAsync(lossv.data(), m->loss, steps_per_epoch * sizeof(float),
                                        cudaMemcpyDeviceToHost, st));
         RBFFD_CUDA_TRY(cudaStreamSynchronize(st));
+        perm.swap(next);
         if (loss_host) {
             double tot = 0.0;
             for (float l : lossv) tot += l;
