@@ -1057,7 +1057,7 @@ rbffd_status build_search(rbffd_op* op, const double* nodes, const double* norma
     int mmax = 0;
     for (int g = 0; g < gi.ngroups; ++g) mmax = std::max(mmax, gi.npad[g]);
     const bool shaped = o.block_threads > 0 || o.blocks_per_sm > 0;
-    if (!shaped && team_lanes(mmax, op->N) > 0) {
+    if (!shaped && team_lanes(mmax, op->N, guess_rows != nullptr) > 0) {
         rbffd_status s = team_search(A, mmax, op->N, st);
         if (s != RBFFD_OK) return s;
     } else {

@@ -353,9 +353,9 @@ struct TeamWeightArgs {
 };
 
 // team.cu: lanes per stencil for a search over (weights of) rows stencils of
-// padded size m (0: the lane-per-stencil kernel is the faster one); the search
+// padded size m, with learned guesses or without (0: the lane-per-stencil kernel is the faster one); the search
 // and the weights on teams
-int team_lanes(int m, int64_t rows);
+int team_lanes(int m, int64_t rows, bool guesses);
 int team_weight_lanes(int m, int64_t rows);
 rbffd_status team_search(SearchArgs A, int m, int64_t rows, cudaStream_t st);
 rbffd_status team_weights(TeamWeightArgs B, int64_t scratch_doubles, cudaStream_t st);

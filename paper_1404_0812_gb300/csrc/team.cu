@@ -1137,23 +1137,31 @@ rbffd_status weights_with(TeamWeightArgs B, int mmax, int64_t rows, int64_t scra
 // Measured on one GB300 (sphere, IMQ, kappa_T 1e12, plain search; ms for a
 // lane / 4 / 8 / 16 lanes per stencil, the chosen one marked):
 //   n = 31:   1.3k 17.3/-/3.6/2.9*   5k 23.7/8.0/6.2*/8.2   10k 23.5/8.9*/10.0/16.9
-//             20k 30.8/17.0*/22.2/35.4   80k 80.7/60.2*/88.1/-   320k 296/249*/391/-
+//             20k 30.8/17.0*/22.2/35.4   80k 80.7*/60.2/88.1/-   320k 296*/249/391/-
 //   n = 50:   5k 60.7/20.1/13.0*/15.8   10k 90.1/29.1/23.4*/31.7   20k 83.3/32.3*/35.8/63.3
-//             160k 264/241*/352/-   320k 468/446*/691/-
+//             50k 103/78.0*/93.6/-   160k 264*/241/352/-   320k 468*/446/691/-
+//   n = 58:   10k 86.2/29.5/24.1*/34.0   25k 95.2/56.3/55.9*/-   50k 109*/101/113/-   80k 157*/161/184/-
+//   n = 78:   5k 122/34.4/25.7*/25.5   25k 154/129/89.6*/-   50k 187*/261/184/-
 //   n = 101:  5k 180/80/46.6/39.3*   20k 205/215/127*/129   80k 399*/758/447/-
 // Few stencils want many lanes each (all schedulers busy), many want few
-// (fewer float64 instructions per stencil).  From n = 61 the vectors of
-// eight teams of 4 lanes leave too few warps per SM.
-int team_lanes(int m, int64_t rows) {
+// (fewer float64 instructions per stencil).  From n = 57 the vectors of eight
+// teams of 4 lanes leave too few warps per SM.  With fewer evaluations per
+// stencil the lane kernel catches up earlier (torus, kappa_T 1e8, lane / team:
+// n = 15 20k 4.7/6.1, 51k 9.6/12.4; n = 31 51k 23.2/31.1; n = 50 51k 63.7/63.0,
+// 120k sphere 132/152), so it takes over there.  From learned guesses (about
+// one evaluation each) it is the other way round, since few rounds leave its
+// long instruction stream exposed (n = 31: 80k 24.9/14.2, 250k 40.7/34.6; n = 50:
+// 160k 98.9/57.0, 250k 71.0/67.5; n = 101: 50k 144/65.2, 80k 127/96, 160k 264/271).
+int team_lanes(int m, int64_t rows, bool guesses) {
     if (rows < 900) return 32;
     if (rows < (m > 80 ? 12000 : 3500)) return 16;
-    if (m > 60) return rows < 60000 ? 8 : 0;
-    if (rows < (m > 32 ? 15000 : 8000)) return 8;
-    return rows < (m > 24 ? 500000 : 250000) ? 4 : 0;
+    if (m > 56) return rows < (guesses ? 100000 : 40000) ? 8 : 0;
+    if (rows < (m > 32 ? 18000 : 8000)) return 8;
+    return rows < (guesses ? 250000 : m > 36 ? 80000 : m > 24 ? 40000 : 25000) ? 4 : 0;
 }
 
 rbffd_status team_search(SearchArgs A, int mmax, int64_t rows, cudaStream_t st) {
-    switch (team_lanes(mmax, rows)) {
+    switch (team_lanes(mmax, rows, A.guess_rows != nullptr)) {
         case 4: return search_with<4>(A, mmax, rows, st);
         case 16: return search_with<16>(A, mmax, rows, st);
         case 32: return search_with<32>(A, mmax, rows, st);
