@@ -23,20 +23,17 @@
 // Loop state of the phase-kernel BiCGSTAB (device memory).  Each phase
 // kernel reads it as its previous kernel left it; only the last block of a
 // phase (by ticket) writes it, after every other block of that phase has
-// finished reading.
+// finished reading, a lane per species (the phase kernels' threads do no
+// float64 scalar arithmetic).
+struct SpeciesState {
+    double bnorm, limit2;              // |b|; squared norm at which the residual has converged
+    double rho, rho_prev, alpha, omega, res2;   // committed: (r-hat, r), ..., |r|^2
+    double beta, alpha_n, omega_n;     // the current iteration's scalars
+    int active, fail, iters, zero;
+    int actA, actB, early, actE;       //   and its decisions
+};
 struct PhaseCtl {
-    double totR[6];              // phase R: |b|^2, |r0|^2 (u: 0, 1; v: 3, 4)
-    double totB[2];              // (r-hat, q)
-    double totC[2];              // |s|^2
-    double totD[4];              // (t, s), (t, t) per species
-    double totE[4];              // (r-hat, r), |r|^2 per species
-    double bnorm[2], rho[2], rho_prev[2], alpha[2], omega[2], relres[2];
-    int active[2], conv[2], fail[2], iters[2], zero[2];
-    // the current iteration's scalars and decisions, each set once by the
-    // last block of the phase that makes it (the phase kernels' threads only
-    // read them: no per-thread float64 scalar arithmetic)
-    double beta[2], alpha_n[2], omega_n[2];
-    int actA[2], actB[2], early[2], actE[2];
+    SpeciesState s[2];
     int it;                      // iterations done in this step
     int more;                    // the loop continues (host-loop mode reads it)
     unsigned int ticket;
@@ -224,6 +221,16 @@ __device__ __forceinline__ void acc_add(double& s, float a, float b) { s += (dou
 __device__ __forceinline__ void acc_add(double& s, double a, double b) { s += a * b; }
 __device__ __forceinline__ double acc_value(const Dot2& s) { return (double)s.hi + (double)s.lo; }
 __device__ __forceinline__ double acc_value(double s) { return s; }
+__device__ __forceinline__ Dot2 acc_merge(const Dot2& u, const Dot2& v) {
+    const float x = __fadd_rn(u.hi, v.hi), z = __fsub_rn(x, u.hi);
+    const float t = __fadd_rn(__fsub_rn(u.hi, __fsub_rn(x, z)), __fsub_rn(v.hi, z));   // u.hi + v.hi = x + t exactly
+    return Dot2{x, __fadd_rn(t, __fadd_rn(u.lo, v.lo))};
+}
+__device__ __forceinline__ double acc_merge(double u, double v) { return u + v; }
+__device__ __forceinline__ Dot2 acc_shfl_down(const Dot2& s, int o) {
+    return Dot2{__shfl_down_sync(0xffffffffu, s.hi, o), __shfl_down_sync(0xffffffffu, s.lo, o)};
+}
+__device__ __forceinline__ double acc_shfl_down(double s, int o) { return __shfl_down_sync(0xffffffffu, s, o); }
 
 // the phase kernels' accumulator for state type T
 template <typename T>
@@ -294,10 +301,10 @@ __device__ __forceinline__ void rhs_values(const Args<T>& a, const StepCoef<T>& 
 
 // phase R of one row (node i, with (L u)_i = Lu, (L v)_i = Lv): the right-hand
 // side, r0 = b - A u, r-hat = r0, p = q = 0; accumulates |b|^2, |r0|^2 per
-// species into d[0..1], d[3..4]
+// species into d[0..1], d[2..3]
 template <typename T, typename A>
 __device__ __forceinline__ void rhs_row(const Args<T>& a, const StepCoef<T>& kc, int64_t i, T Lu, T Lv,
-                                        A (&d)[6]) {
+                                        A (&d)[4]) {
     const bool two = a.ns == 2;
     const T ui = a.u[i], vi = two ? a.v[i] : T(0);
     T bu, bv;
@@ -317,8 +324,8 @@ __device__ __forceinline__ void rhs_row(const Args<T>& a, const StepCoef<T>& kc,
         V(a, 1, VRH)[i] = rv;
         V(a, 1, VP)[i] = T(0);
         V(a, 1, VQ)[i] = T(0);
-        acc_add(d[3], bv, bv);
-        acc_add(d[4], rv, rv);
+        acc_add(d[2], bv, bv);
+        acc_add(d[3], rv, rv);
     }
 }
 
@@ -376,9 +383,9 @@ constexpr int VG = 2;       // four-element groups a thread of phases A and C lo
 // next row (rnext)
 constexpr int ROW_PF = 2;
 
-template <typename T>
+template <typename T, bool two>
 __device__ __forceinline__ void row_L1(const Args<T>& a, int64_t r, int64_t rnext, const T* __restrict__ x0,
-                                       const T* __restrict__ x1, bool two, T& y0, T& y1) {
+                                       const T* __restrict__ x1, T& y0, T& y1) {
     const int g = group_of_row(a.gi, r);
     const int npad = a.gi.npad[g], nch = npad >> 2;
     const int64_t base = ell_elem(a.gi.ell_off[g], npad, r - a.gi.row_begin[g], 0);
@@ -425,79 +432,105 @@ __device__ __forceinline__ void row_L1(const Args<T>& a, int64_t r, int64_t rnex
     y1 = two ? s1 : T(0);
 }
 
-constexpr int RED_ROUNDS = 4;   // rounds of partials the last block loads at once
+// the product of the species that still run (L0, L1; the other stays unset): a
+// second species' gathers, and the branch around them, only where both run
+// (one species in float64, 300k rows, n = 50: 946 -> 692 us a step)
+template <typename T>
+__device__ __forceinline__ void row_species(const Args<T>& a, int64_t r, int64_t rnext, const T* x0, const T* x1, bool on0,
+                                            bool on1, T& L0, T& L1) {
+    if (on0 && on1) {
+        row_L1<T, true>(a, r, rnext, x0, x1, L0, L1);
+    } else {
+        T y, none;
+        const T* x = on0 ? x0 : x1;
+        row_L1<T, false>(a, r, rnext, x, x, y, none);
+        L0 = L1 = y;
+    }
+}
 
-// K sums per block (each thread's accumulators, in float64 from here on)
-// into pp[block][0..K-1]; the last block of the grid sums them in block
-// order into tot[0..K-1] and returns true.  Blocks of NTB <= 1024 threads.
+// K sums per block into pp[block][0..K-1]; the last block of the grid sums
+// them in a fixed order and returns the totals (in shared memory; NULL in the
+// other blocks).  Only one warp per sum does float64 arithmetic: one float64
+// warp instruction takes the SM 16 clocks, and a float64 shuffle tree in every
+// warp cost the vector phases more than their memory traffic (two species,
+// float32, 1M rows: 5.63 -> 5.07 ms a step).
 template <int K, int NTB, typename A>
-__device__ bool phase_reduce(const A (&v)[K], double* pp, double* tot, unsigned int* ticket) {
-    __shared__ double sh[K][NTB / 32];
+__device__ const double* phase_reduce(const A (&v)[K], double* pp, unsigned int* ticket) {
+    constexpr bool PAIRS = sizeof(A) == sizeof(Dot2) && !std::is_same<A, double>::value;
+    __shared__ A sh[K][PAIRS ? NTB / 32 : NTB];
+    __shared__ double tot[K];
     __shared__ int last;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    static_assert(K <= NTB / 32, "a warp per sum");
+    if (PAIRS) {   // float32 pairs: a shuffle tree per warp, then one thread per sum over the warps
 #pragma unroll
-    for (int k = 0; k < K; ++k) {
-        double x = acc_value(v[k]);
-        for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
-        if (lane == 0) sh[k][wid] = x;
-    }
-    __syncthreads();
-    if (threadIdx.x < K) {
-        double t = 0.0;
-        for (int w = 0; w < NTB / 32; ++w) t += sh[threadIdx.x][w];
-        pp[(int64_t)blockIdx.x * 8 + threadIdx.x] = t;
-        __threadfence();
+        for (int k = 0; k < K; ++k) {
+            A x = v[k];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) x = acc_merge(x, acc_shfl_down(x, o));
+            if (lane == 0) sh[k][wid] = x;
+        }
+        __syncthreads();
+        if (threadIdx.x < K) {
+            A t = sh[threadIdx.x][0];
+#pragma unroll
+            for (int w = 1; w < NTB / 32; ++w) t = acc_merge(t, sh[threadIdx.x][w]);
+            pp[(int64_t)blockIdx.x * 8 + threadIdx.x] = acc_value(t);
+            __threadfence();
+        }
+    } else {       // float64: one warp per sum over the threads' values
+#pragma unroll
+        for (int k = 0; k < K; ++k) sh[k][threadIdx.x] = v[k];
+        __syncthreads();
+        if (wid < K) {
+            A t = sh[wid][lane];
+#pragma unroll
+            for (int w = 1; w < NTB / 32; ++w) t = acc_merge(t, sh[wid][w * 32 + lane]);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) t = acc_merge(t, acc_shfl_down(t, o));
+            if (lane == 0) {
+                pp[(int64_t)blockIdx.x * 8 + wid] = acc_value(t);
+                __threadfence();
+            }
+        }
     }
     __syncthreads();
     if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == gridDim.x - 1;
     __syncthreads();
-    if (!last) return false;
+    if (!last) return nullptr;
     __threadfence();
-    // fixed order: thread t sums blocks t, t + NTB, ...; then a fixed tree
-    // over the threads' sums.  The loads of the first RED_ROUNDS rounds go
-    // out together (one L2 round trip instead of one per round and sum)
-    __shared__ double acc[K][NTB];
-    double part[K][RED_ROUNDS];
+    // lane t of warp k sums blocks t, t + 32, ..., four loads in flight; then a fixed tree
+    if (wid < K) {
+        double s = 0.0;
+        for (int64_t b0 = lane; b0 < gridDim.x; b0 += 128) {
+            double x[4];
 #pragma unroll
-    for (int u = 0; u < RED_ROUNDS; ++u) {
-        const int64_t b = threadIdx.x + (int64_t)u * NTB;
+            for (int u = 0; u < 4; ++u) x[u] = b0 + 32 * u < gridDim.x ? __ldcg(pp + (b0 + 32 * u) * 8 + wid) : 0.0;
 #pragma unroll
-        for (int k = 0; k < K; ++k) part[k][u] = b < gridDim.x ? __ldcg(pp + b * 8 + k) : 0.0;
+            for (int u = 0; u < 4; ++u) s += x[u];
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+        if (lane == 0) tot[wid] = s;
     }
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-        double t = 0.0;
-#pragma unroll
-        for (int u = 0; u < RED_ROUNDS; ++u)
-            if (threadIdx.x + (int64_t)u * NTB < gridDim.x) t += part[k][u];
-        for (int64_t b = threadIdx.x + (int64_t)RED_ROUNDS * NTB; b < gridDim.x; b += NTB) t += __ldcg(pp + b * 8 + k);
-        acc[k][threadIdx.x] = t;
-    }
-    __syncthreads();
-    for (int h = NTB / 2; h > 0; h >>= 1) {
-        if (threadIdx.x < h)
-#pragma unroll
-            for (int k = 0; k < K; ++k) acc[k][threadIdx.x] += acc[k][threadIdx.x + h];
-        __syncthreads();
-    }
-    if (threadIdx.x < K) tot[threadIdx.x] = acc[threadIdx.x][0];
     if (threadIdx.x == 0) *ticket = 0u;
     __syncthreads();
-    return true;
+    return tot;
 }
 
+// the loop continues while a species runs (m: ballot of the deciding lanes)
 __device__ __forceinline__ void set_more(PhaseCtl* c, cudaGraphConditionalHandle h, int more) {
-    c->more = more;
-    if (h) cudaGraphSetConditional(h, (unsigned)more);
+    if (threadIdx.x == 0) {
+        c->more = more;
+        if (h) cudaGraphSetConditional(h, (unsigned)more);
+    }
 }
 
 // beta and the A-decision of the next iteration, from the committed state
-__device__ __forceinline__ void next_iteration(PhaseCtl* c) {
-    for (int k = 0; k < 2; ++k) {
-        c->beta[k] = (c->rho[k] / c->rho_prev[k]) * (c->alpha[k] / c->omega[k]);
-        c->actA[k] = c->active[k] && !(c->rho[k] == 0.0 || !isfinite(c->beta[k]));
-        c->actB[k] = c->early[k] = c->actE[k] = 0;
-    }
+__device__ __forceinline__ void next_iteration(SpeciesState& z) {
+    z.beta = (z.rho / z.rho_prev) * (z.alpha / z.omega);
+    z.actA = z.active && !(z.rho == 0.0 || !isfinite(z.beta));
+    z.actB = z.early = z.actE = 0;
 }
 
 // R: right-hand side and r0
@@ -505,34 +538,33 @@ template <typename T>
 __global__ void __launch_bounds__(PT, PT_MINB) phase_R(Args<T> a) {
     const StepCoef<T> kc = step_coef(a);
     const bool two = a.ns == 2;
-    typename PhaseAcc<T>::type d[6];
+    typename PhaseAcc<T>::type d[4];
     for (auto& x : d) acc_zero(x);
     for (int64_t r = blockIdx.x * (int64_t)PT + threadIdx.x; r < a.N; r += (int64_t)gridDim.x * PT) {
         const int64_t i = a.row_node[r];
         T Lu, Lv;
-        row_L1(a, r, r + (int64_t)gridDim.x * PT, a.u, two ? a.v : a.u, two, Lu, Lv);
+        row_species(a, r, r + (int64_t)gridDim.x * PT, (const T*)a.u, (const T*)a.v, true, two, Lu, Lv);
         rhs_row(a, kc, i, Lu, Lv, d);
     }
     PhaseCtl* c = a.ctl;
-    if (phase_reduce<6, PT>(d, a.pp, c->totR, &c->ticket) && threadIdx.x == 0) {
-        int more = 0;
-        for (int k = 0; k < 2; ++k) {
-            const bool exists = k == 0 || two;
-            const double bn = sqrt(c->totR[3 * k]), rr = c->totR[3 * k + 1];
-            c->bnorm[k] = bn;
-            c->rho[k] = rr;   // (r-hat, r0) = |r0|^2
-            c->rho_prev[k] = c->alpha[k] = c->omega[k] = 1.0;
-            c->relres[k] = bn > 0 ? sqrt(rr) / bn : 0.0;
-            c->conv[k] = !exists || bn == 0.0 || c->relres[k] <= a.tol;
-            c->active[k] = !c->conv[k];
-            c->fail[k] = 0;
-            c->iters[k] = 0;
-            c->zero[k] = exists && bn == 0.0;   // b = 0: x = 0
-            more |= c->active[k];
-        }
+    const double* tot = phase_reduce<4, PT>(d, a.pp, &c->ticket);
+    if (tot && threadIdx.x < 2) {
+        const int k = threadIdx.x;
+        const bool exists = k == 0 || two;
+        SpeciesState z;
+        z.bnorm = sqrt(tot[2 * k]);
+        z.limit2 = (a.tol * z.bnorm) * (a.tol * z.bnorm);
+        z.rho = z.res2 = tot[2 * k + 1];   // (r-hat, r0) = |r0|^2
+        z.rho_prev = z.alpha = z.omega = 1.0;
+        z.alpha_n = z.omega_n = 0.0;
+        z.active = exists && z.bnorm != 0.0 && !(sqrt(z.res2) / z.bnorm <= a.tol);
+        z.fail = z.iters = 0;
+        z.zero = exists && z.bnorm == 0.0;   // b = 0: x = 0
+        next_iteration(z);
+        c->s[k] = z;
         c->it = 0;
-        next_iteration(c);
-        set_more(c, a.cond, more && a.maxit > 0);
+        const unsigned m = __ballot_sync(3u, z.active);
+        set_more(c, a.cond, m != 0 && a.maxit > 0);
     }
 }
 
@@ -568,8 +600,8 @@ __global__ void __launch_bounds__(PV, PV_BPS) phase_A(Args<T> a) {
     const PhaseCtl* c = a.ctl;
     const int64_t S = (int64_t)gridDim.x * PV, t0 = blockIdx.x * (int64_t)PV + threadIdx.x;
     for (int k = 0; k < a.ns; ++k) {
-        if (!c->actA[k]) continue;
-        const T beta = (T)c->beta[k], omega = (T)c->omega[k];
+        if (!c->s[k].actA) continue;
+        const T beta = (T)c->s[k].beta, omega = (T)c->s[k].omega;
         T* __restrict__ p = V(a, k, VP);
         const T* __restrict__ r = V(a, k, VR);
         const T* __restrict__ q = V(a, k, VQ);
@@ -611,7 +643,7 @@ __device__ __forceinline__ int64_t back_row(int64_t k, int64_t Np) { return Np -
 template <typename T>
 __global__ void __launch_bounds__(PT, PT_MINB) phase_B(Args<T> a) {
     PhaseCtl* c = a.ctl;
-    const bool a0 = c->actA[0], a1 = a.ns == 2 && c->actA[1];
+    const bool a0 = c->s[0].actA, a1 = a.ns == 2 && c->s[1].actA;
     const StepCoef<T> kc = step_coef(a);
     typename PhaseAcc<T>::type d[2];
     for (auto& x : d) acc_zero(x);
@@ -622,7 +654,7 @@ __global__ void __launch_bounds__(PT, PT_MINB) phase_B(Args<T> a) {
         const int64_t rn = k + S >= Np ? a.N : (B_BACK ? back_row(k + S, Np) : k + S);
         const int64_t i = a.row_node[r];
         T L0, L1;
-        row_L1(a, r, rn, V(a, 0, VP), a.ns == 2 ? V(a, 1, VP) : V(a, 0, VP), a1, L0, L1);
+        row_species(a, r, rn, (const T*)V(a, 0, VP), (const T*)V(a, 1, VP), a0, a1, L0, L1);
         if (a0) {
             const T q = kc.c0 * V(a, 0, VP)[i] - kc.k0 * L0;
             V(a, 0, VQ)[i] = q;
@@ -634,11 +666,15 @@ __global__ void __launch_bounds__(PT, PT_MINB) phase_B(Args<T> a) {
             acc_add(d[1], V(a, 1, VRH)[i], q);
         }
     }
-    if (phase_reduce<2, PT>(d, a.pp, c->totB, &c->ticket) && threadIdx.x == 0)
-        for (int k = 0; k < 2; ++k) {
-            c->alpha_n[k] = c->actA[k] ? c->rho[k] / c->totB[k] : 0.0;
-            c->actB[k] = c->actA[k] && !(c->totB[k] == 0.0 || !isfinite(c->alpha_n[k]));
-        }
+    const double* tot = phase_reduce<2, PT>(d, a.pp, &c->ticket);
+    if (tot && threadIdx.x < 2) {
+        const int k = threadIdx.x;
+        SpeciesState& z = c->s[k];
+        const int act = z.actA;
+        const double alpha = act ? z.rho / tot[k] : 0.0;
+        z.alpha_n = alpha;
+        z.actB = act && !(tot[k] == 0.0 || !isfinite(alpha));
+    }
 }
 
 // C: s = r - alpha q ; |s|^2
@@ -649,8 +685,8 @@ __global__ void __launch_bounds__(PV, PV_BPS) phase_C(Args<T> a) {
     for (auto& x : d) acc_zero(x);
     const int64_t S = (int64_t)gridDim.x * PV, t0 = blockIdx.x * (int64_t)PV + threadIdx.x;
     for (int k = 0; k < a.ns; ++k) {
-        if (!c->actB[k]) continue;
-        const T alpha = (T)c->alpha_n[k];
+        if (!c->s[k].actB) continue;
+        const T alpha = (T)c->s[k].alpha_n;
         const T* __restrict__ r = V(a, k, VR);
         const T* __restrict__ q = V(a, k, VQ);
         T* __restrict__ sv = V(a, k, VS);
@@ -685,8 +721,13 @@ __global__ void __launch_bounds__(PV, PV_BPS) phase_C(Args<T> a) {
             acc_add(d[k], x, x);
         }
     }
-    if (phase_reduce<2, PV>(d, a.pp, c->totC, &c->ticket) && threadIdx.x == 0)
-        for (int k = 0; k < 2; ++k) c->early[k] = c->actB[k] && sqrt(c->totC[k]) / c->bnorm[k] <= a.tol;
+    const double* tot = phase_reduce<2, PV>(d, a.pp, &c->ticket);
+    if (tot && threadIdx.x < 2) {
+        SpeciesState& z = c->s[threadIdx.x];
+        const int early = z.actB && tot[threadIdx.x] <= z.limit2;
+        z.early = early;
+        if (early) z.res2 = tot[threadIdx.x];
+    }
 }
 
 // D: t = A s ; (t, s), (t, t)   (x += alpha p where s already converged)
@@ -695,19 +736,21 @@ __global__ void __launch_bounds__(PT, PT_MINB) phase_D(Args<T> a) {
     PhaseCtl* c = a.ctl;
     const StepCoef<T> kc = step_coef(a);
     const bool two = a.ns == 2;
-    const bool e0 = c->early[0], e1 = two && c->early[1];
-    const bool b0 = c->actB[0], b1 = two && c->actB[1];
+    const bool e0 = c->s[0].early, e1 = two && c->s[1].early;
+    const bool b0 = c->s[0].actB, b1 = two && c->s[1].actB;
     const bool need0 = b0 && !e0, need1 = b1 && !e1;
     typename PhaseAcc<T>::type d[4];
     for (auto& x : d) acc_zero(x);
     for (int64_t r = blockIdx.x * (int64_t)PT + threadIdx.x; (b0 || b1) && r < a.N; r += (int64_t)gridDim.x * PT) {
         const int64_t i = a.row_node[r];
         T L0 = T(0), L1 = T(0);
-        if (need0 || need1) row_L1(a, r, r + (int64_t)gridDim.x * PT, V(a, 0, VS), two ? V(a, 1, VS) : V(a, 0, VS), need1, L0, L1);
+        if (need0 || need1)
+            row_species(a, r, r + (int64_t)gridDim.x * PT, (const T*)V(a, 0, VS), (const T*)V(a, 1, VS), need0, need1, L0,
+                        L1);
         for (int k = 0; k < a.ns; ++k) {
             T* x = k == 0 ? a.u : a.v;
             if (k == 0 ? e0 : e1) {
-                x[i] += (T)c->alpha_n[k] * V(a, k, VP)[i];
+                x[i] += (T)c->s[k].alpha_n * V(a, k, VP)[i];
             } else if (k == 0 ? b0 : b1) {
                 const T sv = V(a, k, VS)[i];
                 const T t = kc.c0 * sv - (k == 0 ? kc.k0 * L0 : kc.k1 * L1);
@@ -717,11 +760,15 @@ __global__ void __launch_bounds__(PT, PT_MINB) phase_D(Args<T> a) {
             }
         }
     }
-    if (phase_reduce<4, PT>(d, a.pp, c->totD, &c->ticket) && threadIdx.x == 0)
-        for (int k = 0; k < 2; ++k) {
-            c->omega_n[k] = c->totD[2 * k] / c->totD[2 * k + 1];
-            c->actE[k] = c->actB[k] && !c->early[k] && !(c->totD[2 * k + 1] == 0.0 || !isfinite(c->omega_n[k]));
-        }
+    const double* tot = phase_reduce<4, PT>(d, a.pp, &c->ticket);
+    if (tot && threadIdx.x < 2) {
+        const int k = threadIdx.x;
+        SpeciesState& z = c->s[k];
+        const int act = z.actB && !z.early;
+        const double omega = tot[2 * k] / tot[2 * k + 1];
+        z.omega_n = omega;
+        z.actE = act && !(tot[2 * k + 1] == 0.0 || !isfinite(omega));
+    }
 }
 
 // E: x += alpha p + omega s ; r = s - omega t ; (r-hat, r), |r|^2; the last
@@ -739,8 +786,8 @@ __global__ void __launch_bounds__(PV, PV_BPS) phase_E(Args<T> a) {
     for (auto& x : d) acc_zero(x);
     const int64_t S = (int64_t)gridDim.x * PV, t0 = blockIdx.x * (int64_t)PV + threadIdx.x;
     for (int k = 0; k < a.ns; ++k) {
-        if (!c->actE[k]) continue;
-        const T alpha = (T)c->alpha_n[k], omega = (T)c->omega_n[k];
+        if (!c->s[k].actE) continue;
+        const T alpha = (T)c->s[k].alpha_n, omega = (T)c->s[k].omega_n;
         T* __restrict__ x = k == 0 ? a.u : a.v;
         const T* __restrict__ p = V(a, k, VP);
         const T* __restrict__ sv = V(a, k, VS);
@@ -778,42 +825,37 @@ __global__ void __launch_bounds__(PV, PV_BPS) phase_E(Args<T> a) {
             acc_add(d[2 * k + 1], rn, rn);
         }
     }
-    if (phase_reduce<4, PV>(d, a.pp, c->totE, &c->ticket) && threadIdx.x == 0) {
-        const int it = c->it + 1;
-        int more = 0;
-        for (int k = 0; k < 2; ++k) {
-            if (!c->active[k]) continue;
-            if (!c->actA[k] || !c->actB[k]) {
-                c->fail[k] = 1;
-                c->active[k] = 0;
-            } else if (c->early[k]) {
-                c->relres[k] = sqrt(c->totC[k]) / c->bnorm[k];
-                c->conv[k] = 1;
-                c->active[k] = 0;
-                c->iters[k] = it;
-            } else if (!c->actE[k]) {
-                c->fail[k] = 1;
-                c->active[k] = 0;
+    const double* tot = phase_reduce<4, PV>(d, a.pp, &c->ticket);
+    if (tot && threadIdx.x < 2) {
+        const int k = threadIdx.x, it = c->it + 1;
+        SpeciesState z = c->s[k];
+        if (z.active) {
+            if (!z.actA || !z.actB || (!z.early && !z.actE)) {
+                z.fail = 1;
+                z.active = 0;
+            } else if (z.early) {
+                z.active = 0;
+                z.iters = it;
             } else {
-                c->rho_prev[k] = c->rho[k];
-                c->rho[k] = c->totE[2 * k];
-                c->alpha[k] = c->alpha_n[k];
-                c->omega[k] = c->omega_n[k];
-                c->relres[k] = sqrt(c->totE[2 * k + 1]) / c->bnorm[k];
-                if (c->relres[k] <= a.tol) {
-                    c->conv[k] = 1;
-                    c->active[k] = 0;
-                    c->iters[k] = it;
-                } else if (c->omega_n[k] == 0.0) {
-                    c->fail[k] = 1;
-                    c->active[k] = 0;
+                z.rho_prev = z.rho;
+                z.rho = tot[2 * k];
+                z.alpha = z.alpha_n;
+                z.omega = z.omega_n;
+                z.res2 = tot[2 * k + 1];
+                if (z.res2 <= z.limit2) {
+                    z.active = 0;
+                    z.iters = it;
+                } else if (z.omega_n == 0.0) {
+                    z.fail = 1;
+                    z.active = 0;
                 }
             }
-            more |= c->active[k];
         }
+        next_iteration(z);
+        const unsigned m = __ballot_sync(3u, z.active);   // both lanes have read c->it
+        c->s[k] = z;
         c->it = it;
-        next_iteration(c);
-        set_more(c, a.cond, more && it < a.maxit);
+        set_more(c, a.cond, m != 0 && it < a.maxit);
     }
 }
 
@@ -822,27 +864,21 @@ template <typename T>
 __global__ void __launch_bounds__(PT) phase_F(Args<T> a) {
     const PhaseCtl* c = a.ctl;
     for (int k = 0; k < a.ns; ++k) {
-        if (!c->zero[k]) continue;
+        if (!c->s[k].zero) continue;
         T* x = k == 0 ? a.u : a.v;
         for (int64_t i = blockIdx.x * (int64_t)PT + threadIdx.x; i < a.N; i += (int64_t)gridDim.x * PT) x[i] = T(0);
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         const StepCoef<T> kc = step_coef(a);
-        int iters[2] = {c->iters[0], c->iters[1]};
+        int* rp = a.rep + (int64_t)kc.slot * 3;
         bool bad = false;
         for (int k = 0; k < 2; ++k) {
-            if (c->active[k]) {   // hit maxit
-                iters[k] = c->it;
-                bad = true;
-            }
-            if (c->fail[k]) bad = true;
+            const SpeciesState& z = c->s[k];
+            bad = bad || z.active || z.fail;   // still active: hit maxit
+            rp[k] = z.active ? c->it : z.iters;
+            a.rep_res[(int64_t)kc.slot * 2 + k] = z.bnorm > 0 ? sqrt(z.res2) / z.bnorm : 0.0;
         }
-        int* rp = a.rep + (int64_t)kc.slot * 3;
-        rp[0] = iters[0];
-        rp[1] = iters[1];
         rp[2] = bad ? 1 : 0;
-        a.rep_res[(int64_t)kc.slot * 2] = c->relres[0];
-        a.rep_res[(int64_t)kc.slot * 2 + 1] = c->relres[1];
         if (bad) atomicExch(a.flags + 1, 1);
         a.flags[2] = min(kc.nhist + 1, max(a.order - 1, 1));
         a.flags[3] = kc.slot + 1;

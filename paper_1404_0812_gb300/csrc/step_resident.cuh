@@ -65,33 +65,18 @@ __device__ __forceinline__ void cluster_sync_all() {
     asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
 }
 
-// a row's product as it goes to the summing warp
+// a row's product as it goes to the summing warp: float64, or an exact pair of
+// float32 values
 template <typename T>
 struct Term {
-    using type = double;
-    __device__ static double of(double a, double b) { return a * b; }
-    __device__ static double add(double x, double y) { return x + y; }
-    __device__ static double value(double x) { return x; }
-};
-template <>
-struct Term<float> {
-    using type = float2;   // unevaluated sum x + y
-    __device__ static float2 of(float a, float b) {
-        const float p = __fmul_rn(a, b);
-        return make_float2(p, __fmaf_rn(a, b, -p));
+    using type = typename PhaseAcc<T>::type;
+    __device__ static type of(T a, T b) {
+        type t;
+        acc_zero(t);
+        acc_add(t, a, b);
+        return t;
     }
-    __device__ static float2 add(float2 u, float2 v) {
-        const float x = __fadd_rn(u.x, v.x), z = __fsub_rn(x, u.x);
-        const float t = __fadd_rn(__fsub_rn(u.x, __fsub_rn(x, z)), __fsub_rn(v.x, z));   // u.x + v.x = x + t
-        return make_float2(x, __fadd_rn(t, __fadd_rn(u.y, v.y)));
-    }
-    __device__ static double value(float2 u) { return (double)u.x + (double)u.y; }
 };
-
-__device__ __forceinline__ double shfl_down_term(double x, int o) { return __shfl_down_sync(0xffffffffu, x, o); }
-__device__ __forceinline__ float2 shfl_down_term(float2 x, int o) {
-    return make_float2(__shfl_down_sync(0xffffffffu, x.x, o), __shfl_down_sync(0xffffffffu, x.y, o));
-}
 
 // what one lane per species decides and every thread of the block reads (the
 // scalar arithmetic is float64: on all warps it would cost more than the
@@ -155,8 +140,7 @@ struct ResidentBlock {
     // visible; lane 0 of warp k then decides with the totals of species k
     template <int KS, int NS, typename F>
     __device__ bool reduce(const typename Term<T>::type (&v)[NS][KS], int row, bool writes, F decide) {
-        using TM = Term<T>;
-        using V = typename TM::type;
+        using V = typename Term<T>::type;
         V* terms = (V*)(sm + L.terms);
         if (writes) {
 #pragma unroll
@@ -170,14 +154,14 @@ struct ResidentBlock {
                         : ri.part + (int64_t)parity * gridDim.x * RES_SUMS;
         for (int k = wid; k < NS * KS; k += nw) {
             V s = terms[k * rows + ln];
-            for (int r = ln + 32; r < rows; r += 32) s = TM::add(s, terms[k * rows + r]);
+            for (int r = ln + 32; r < rows; r += 32) s = acc_merge(s, terms[k * rows + r]);
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) s = TM::add(s, shfl_down_term(s, o));
+            for (int o = 16; o > 0; o >>= 1) s = acc_merge(s, acc_shfl_down(s, o));
             if (CL) {
-                const double t = __shfl_sync(0xffffffffu, TM::value(s), 0);
+                const double t = __shfl_sync(0xffffffffu, acc_value(s), 0);
                 if (ln < (int)gridDim.x) st_peer(peer_addr(smem_u32(pp + blockIdx.x * RES_SUMS + k), ln), t);
             } else if (ln == 0) {
-                __stcg(pp + (int64_t)blockIdx.x * RES_SUMS + k, TM::value(s));
+                __stcg(pp + (int64_t)blockIdx.x * RES_SUMS + k, acc_value(s));
             }
         }
         if (!sync()) return false;
