@@ -22,13 +22,23 @@ MODELS = {"none": MODEL_NONE, "linear": MODEL_LINEAR, "schnakenberg": MODEL_SCHN
           "gray_scott": MODEL_GRAY_SCOTT, "barrio": MODEL_BARRIO}
 
 
+# Addresses and streams go to ctypes as plain integers (the signatures convert
+# them), and the current stream's handle is asked for directly: building a
+# c_void_p and a torch Stream object for each call took longer than a small
+# apply's kernel (2,562 rows: 13.9 -> 8.1 us a call, 4.4 of them the kernel).
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _ptr(t):
-    return None if t is None else C.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _stream(stream=None):
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return C.c_void_p(s.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_stream is None:
+        return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(torch.cuda.current_device())
 
 
 def _dev(t, dtype):

@@ -124,6 +124,8 @@ def library_path() -> str:
 def load(build: bool = True):
     """Load (building first if needed) the C-ABI library.  Raises if absent."""
     global _handle
+    if _handle is not None:
+        return _handle
     with _lock:
         if _handle is not None:
             return _handle
