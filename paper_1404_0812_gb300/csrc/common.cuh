@@ -79,25 +79,28 @@ struct GroupInfo {
 // every block adds 1 to *bar and waits until it reaches target (which grows
 // by gridDim.x per barrier).  A block that has polled for about a second, or
 // that sees *err set, gives up, sets *err and returns false, so that no wait
-// can hang; the caller then leaves the kernel.
-constexpr long long GRID_SYNC_MAX_POLLS = 20000000;   // ~1-2 s with 32 ns sleeps
+// can hang; the caller then leaves the kernel.  Release / acquire accesses of
+// one thread order the block's (a full fence and sleeps between the polls cost
+// the resident step a fifth of its time: 40k torus, two species, 111 -> 90 us).
+constexpr long long GRID_SYNC_MAX_POLLS = 20000000;   // bound of waits with a sleep per poll (lu.cu)
+constexpr long long GRID_SYNC_POLLS = 3000000;        // ~1 s of L2 round trips
 __device__ __forceinline__ bool grid_sync(unsigned long long* bar, unsigned long long target, int* err) {
     __shared__ int ok;
     __syncthreads();
     if (threadIdx.x == 0) {
         ok = 1;
-        __threadfence();
-        atomicAdd(bar, 1ull);
+        asm volatile("red.release.gpu.add.u64 [%0], 1;" ::"l"(bar) : "memory");
         long long polls = 0;
-        while (*((volatile unsigned long long*)bar) < target) {
-            if (++polls > GRID_SYNC_MAX_POLLS || *((volatile int*)err)) {
+        for (;;) {
+            unsigned long long seen;
+            asm volatile("ld.acquire.gpu.u64 %0, [%1];" : "=l"(seen) : "l"(bar) : "memory");
+            if (seen >= target) break;
+            if (++polls > GRID_SYNC_POLLS || ((polls & 63) == 0 && *((volatile int*)err))) {
                 ok = 0;
                 atomicExch(err, 1);
                 break;
             }
-            __nanosleep(32);
         }
-        __threadfence();
     }
     __syncthreads();
     return ok != 0;

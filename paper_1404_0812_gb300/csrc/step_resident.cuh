@@ -12,7 +12,7 @@
 //    travel through distributed shared memory, and the barrier is the
 //    cluster's (a few hundred nanoseconds);
 //  * a cooperative grid of one block per SM: gathers through L1 / L2 and the
-//    bounded grid barrier (about a microsecond and a half).
+//    bounded grid barrier (about a microsecond).
 //
 // TPR lanes share a row: each reads every TPR-th chunk of four entries, a
 // shuffle adds them up, and all of them hold the row's vector entries in
@@ -23,8 +23,8 @@
 //
 // Measured against one cooperative launch per step with the matrix streamed
 // from L2 and three blocks for the small operator: 2,562 nodes, n = 31, heat
-// equation in float64, 3.8 iterations per step: 314 -> 58 us per step; 40k
-// torus, n = 50, two species in float32: 320 -> 113 us per step.
+// equation in float64, 3.8 iterations per step: 314 -> 52 us per step; 40k
+// torus, n = 50, two species in float32: 320 -> 90 us per step.
 //
 // Included by step.cu inside its anonymous namespace.
 
@@ -154,6 +154,7 @@ struct ResidentBlock {
                         : ri.part + (int64_t)parity * gridDim.x * RES_SUMS;
         for (int k = wid; k < NS * KS; k += nw) {
             V s = terms[k * rows + ln];
+#pragma unroll 4
             for (int r = ln + 32; r < rows; r += 32) s = acc_merge(s, terms[k * rows + r]);
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) s = acc_merge(s, acc_shfl_down(s, o));
@@ -169,12 +170,26 @@ struct ResidentBlock {
             double tot[KS];
 #pragma unroll
             for (int j = 0; j < KS; ++j) tot[j] = 0.0;
-            for (int b = ln; b < (int)gridDim.x; b += 32)
+            if (CL) {   // at most 16 blocks
 #pragma unroll
-                for (int j = 0; j < KS; ++j)
-                    tot[j] += CL ? pp[b * RES_SUMS + k * KS + j] : __ldcg(pp + (int64_t)b * RES_SUMS + k * KS + j);
+                for (int j = 0; j < KS; ++j) tot[j] = ln < (int)gridDim.x ? pp[ln * RES_SUMS + k * KS + j] : 0.0;
+            } else {
+                for (int b0 = ln; b0 < (int)gridDim.x; b0 += 160) {   // five loads per lane in flight
+                    double x[5][KS];
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1)
+                    for (int u = 0; u < 5; ++u)
+#pragma unroll
+                        for (int j = 0; j < KS; ++j)
+                            x[u][j] = b0 + 32 * u < (int)gridDim.x
+                                          ? __ldcg(pp + (int64_t)(b0 + 32 * u) * RES_SUMS + k * KS + j) : 0.0;
+#pragma unroll
+                    for (int u = 0; u < 5; ++u)
+#pragma unroll
+                        for (int j = 0; j < KS; ++j) tot[j] += x[u][j];
+                }
+            }
+#pragma unroll
+            for (int o = CL ? RES_CLUSTER / 2 : 16; o > 0; o >>= 1)
 #pragma unroll
                 for (int j = 0; j < KS; ++j) tot[j] += __shfl_down_sync(0xffffffffu, tot[j], o);
             if (ln == 0) decide(k, tot);
