@@ -106,6 +106,10 @@ __device__ __forceinline__ bool grid_sync(unsigned long long* bar, unsigned long
     return ok != 0;
 }
 
+__device__ __forceinline__ void cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
+}
+
 // exclusive prefix sum of n int32 values on the device (knn.cu)
 rbffd_status exclusive_scan(const int32_t* in, int32_t* out, int64_t n, cudaStream_t st);
 

@@ -517,9 +517,6 @@ __device__ __forceinline__ void st_cluster(uint32_t a, double v) {
 __device__ __forceinline__ void st_cluster(uint32_t a, float v) {
     asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
 }
-__device__ __forceinline__ void cluster_barrier() {
-    asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
-}
 
 // One triangular sweep: forward with L, or (BACK) with U on mirrored rows
 // r' = N - 1 - r.  in / out: the right-hand side and the result by row.

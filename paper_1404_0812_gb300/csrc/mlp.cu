@@ -293,18 +293,19 @@ mlp_tile(const float* __restrict__ params, int D, const float* __restrict__ feat
 // distributed shared memory, and after one cluster barrier forms 1 / C of the
 // gradient's rows over all samples of the tile.  Every element keeps its sum in
 // sample order, so the gradient has the bits of mlp_tile's.  n = 50, batches of
-// 1,024: 93 -> 14 us per training step.
+// 1,024: 85 -> 13 us for the gradient of a step.
 // ---------------------------------------------------------------------------
 constexpr int W2S = H + 1;   // row stride of W2 in shared memory (rows and columns are read)
 
 struct ClusterTile {         // float offsets in shared memory
-    int X, XC, W1, W2, W3, Z1, Z2, H1, H2, D2, D1, dy, sq, total;
+    int X, XS, XC, W1, W2, W3, Z1, Z2, H1, H2, D2, D1, dy, sq, total;
     __host__ __device__ ClusterTile(int D, int C) {
         const int own = TS / C, slice = (D + C - 1) / C;
+        XS = (D + 3) / 4 * 4;         // row stride of X (read four features at a time)
         int o = 0;
         W1 = o; o += D * H;
         W3 = o; o += H;
-        X = o; o += own * D;          // own samples' features
+        X = o; o += own * XS;         // own samples' features
         XC = o; o += TS * slice;      // all samples' features of this CTA's gradient rows
         W2 = o; o += H * W2S;
         Z1 = o; o += own * H;
@@ -322,6 +323,12 @@ struct ClusterTile {         // float offsets in shared memory
     }
 };
 
+// acc + a[0] w[0] + ... + a[3] w[3], in this order (a: 16-byte aligned, shared memory)
+__device__ __forceinline__ float dot4(const float* a, const float (&w)[4], float acc) {
+    const float4 x = *reinterpret_cast<const float4*>(a);
+    return fmaf(x.w, w[3], fmaf(x.z, w[2], fmaf(x.y, w[1], fmaf(x.x, w[0], acc))));
+}
+
 __device__ __forceinline__ void st_peer4(uint32_t a, float4 v) {
     asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(a), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w)
                  : "memory");
@@ -336,25 +343,14 @@ __device__ __forceinline__ void cp16(float* dst, const float* src) {
                  : "memory");
 }
 
+// rows and features of the tile's samples, by asynchronous copies (loads in the
+// products' loops cost 15 us of L2 latency); they need no weights, so a step's
+// are on their way while the step before it still updates those
 template <int C>
-__global__ void __launch_bounds__(NT)
-mlp_tile_cluster(const float* __restrict__ params, int D, const float* __restrict__ feats,
-                 const float* __restrict__ target, const int32_t* __restrict__ sel, int64_t count, float inv_B,
-                 float* __restrict__ partial, float* __restrict__ loss_part) {
-    extern __shared__ __align__(16) float smc[];
-    constexpr int OWN = TS / C, PER = OWN / 4;   // samples of this CTA; outputs per thread of a layer
-    const ClusterTile L(D, C);
-    const View P = view(params, D);
-    const int t = threadIdx.x, rank = blockIdx.x % C;
-    const int64_t tile = blockIdx.x / C, s0 = tile * TS;
-    const int ns = (int)((count - s0) < TS ? (count - s0) : TS);
-    const int first = rank * OWN;                // tile sample of this CTA's sample 0
-    const int slice = (D + C - 1) / C, d0 = rank * slice, d1 = min(D, d0 + slice);
-    asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory");   // peers have started (waited for below)
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    // weights and features by asynchronous copies, all in flight together
-    // (loads in the products' loops cost 15 us of L2 latency)
-    __shared__ int64_t row[TS];
+__device__ __forceinline__ void load_samples(float* smc, const ClusterTile& L, int64_t* row, int D,
+                                             const float* feats, const int32_t* sel, int64_t s0, int ns, int rank) {
+    constexpr int OWN = TS / C;
+    const int t = threadIdx.x, first = rank * OWN, slice = (D + C - 1) / C, d0 = rank * slice;
     if (t < TS) row[t] = t < ns ? (sel ? (int64_t)sel[s0 + t] : s0 + t) : -1;
     __syncthreads();
     for (int s = t >> 5; s < TS; s += NT / 32) {        // a warp per sample
@@ -366,31 +362,52 @@ mlp_tile_cluster(const float* __restrict__ params, int D, const float* __restric
         }
         if (s >= first && s < first + OWN)
             for (int d = t & 31; d < D; d += 32) {
-                float* to = smc + L.X + (s - first) * D + d;
+                float* to = smc + L.X + (s - first) * L.XS + d;
                 if (real) cp4(to, f + d); else *to = 0.f;
             }
     }
-    // the weights after the step before this one has updated them
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+// weights, forward and backward pass, and the tile's gradient partial; start:
+// the peers' first barrier phase is still to be waited for
+template <int C>
+__device__ __forceinline__ void cluster_gradient(float* smc, const ClusterTile& L, const int64_t* row, const View& P,
+                                                 int D, const float* target, int ns, float inv_B, int rank,
+                                                 bool start, float* G, float* loss_part) {
+    constexpr int OWN = TS / C, PER = OWN / 4;   // samples of this CTA; outputs per thread of a layer
+    const int t = threadIdx.x;
+    const int first = rank * OWN;                // tile sample of this CTA's sample 0
+    const int slice = (D + C - 1) / C, d0 = rank * slice, d1 = min(D, d0 + slice);
     for (int e = 4 * t; e < D * H; e += 4 * NT) cp16(smc + L.W1 + e, P.W1 + e);
     for (int e = t; e < H; e += NT) cp4(smc + L.W3 + e, P.W3 + e);
     for (int e = t; e < H * H; e += NT) cp4(smc + L.W2 + (e / H) * W2S + e % H, P.W2 + e);
+    const int h = t & 63, sb = t >> 6;           // this thread's unit; samples sb + 4 i
+    const float bias1 = __ldcg(P.b1 + h), bias2 = __ldcg(P.b2 + h), bias3 = __ldcg(P.b3);
     asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
     __syncthreads();
     const float tgt = t < OWN && first + t < ns ? target[row[first + t]] : 0.f;
-    const int h = t & 63, sb = t >> 6;           // this thread's unit; samples sb + 4 i
     float* const H1 = smc + L.H1 + first * H;    // own samples' rows of the shared arrays
     float* const H2 = smc + L.H2 + first * H;
     float* const D2 = smc + L.D2 + first * H;
     float* const D1 = smc + L.D1 + first * H;
     float acc[PER];
 #pragma unroll
-    for (int i = 0; i < PER; ++i) acc[i] = P.b1[h];
-#pragma unroll 8
-    for (int d = 0; d < D; ++d) {
+    for (int i = 0; i < PER; ++i) acc[i] = bias1;
+    // four features of a sample per load: one word of shared memory per FMA
+    // and load cost the layers twice the reads
+    int d = 0;
+#pragma unroll 4
+    for (; d + 4 <= D; d += 4) {
+        float w[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) w[q] = smc[L.W1 + (d + q) * H + h];
+#pragma unroll
+        for (int i = 0; i < PER; ++i) acc[i] = dot4(smc + L.X + (sb + 4 * i) * L.XS + d, w, acc[i]);
+    }
+    for (; d < D; ++d) {
         const float w = smc[L.W1 + d * H + h];
 #pragma unroll
-        for (int i = 0; i < PER; ++i) acc[i] = fmaf(smc[L.X + (sb + 4 * i) * D + d], w, acc[i]);
+        for (int i = 0; i < PER; ++i) acc[i] = fmaf(smc[L.X + (sb + 4 * i) * L.XS + d], w, acc[i]);
     }
 #pragma unroll
     for (int i = 0; i < PER; ++i) {
@@ -399,12 +416,14 @@ mlp_tile_cluster(const float* __restrict__ params, int D, const float* __restric
     }
     __syncthreads();
 #pragma unroll
-    for (int i = 0; i < PER; ++i) acc[i] = P.b2[h];
-#pragma unroll 8
-    for (int k = 0; k < H; ++k) {
-        const float w = smc[L.W2 + k * W2S + h];
+    for (int i = 0; i < PER; ++i) acc[i] = bias2;
+#pragma unroll 4
+    for (int k = 0; k < H; k += 4) {
+        float w[4];
 #pragma unroll
-        for (int i = 0; i < PER; ++i) acc[i] = fmaf(H1[(sb + 4 * i) * H + k], w, acc[i]);
+        for (int q = 0; q < 4; ++q) w[q] = smc[L.W2 + (k + q) * W2S + h];
+#pragma unroll
+        for (int i = 0; i < PER; ++i) acc[i] = dot4(H1 + (sb + 4 * i) * H + k, w, acc[i]);
     }
 #pragma unroll
     for (int i = 0; i < PER; ++i) {
@@ -413,7 +432,7 @@ mlp_tile_cluster(const float* __restrict__ params, int D, const float* __restric
     }
     __syncthreads();
     if (t < OWN) {
-        float y = P.b3[0];
+        float y = bias3;
 #pragma unroll 16
         for (int k = 0; k < H; ++k) y = fmaf(H2[t * H + k], smc[L.W3 + k], y);
         float r = 0.f;
@@ -430,17 +449,19 @@ mlp_tile_cluster(const float* __restrict__ params, int D, const float* __restric
     __syncthreads();
 #pragma unroll
     for (int i = 0; i < PER; ++i) acc[i] = 0.f;
-#pragma unroll 8
-    for (int k = 0; k < H; ++k) {
-        const float w = smc[L.W2 + h * W2S + k];   // unit h of layer 1
+#pragma unroll 4
+    for (int k = 0; k < H; k += 4) {
+        float w[4];
 #pragma unroll
-        for (int i = 0; i < PER; ++i) acc[i] = fmaf(D2[(sb + 4 * i) * H + k], w, acc[i]);
+        for (int q = 0; q < 4; ++q) w[q] = smc[L.W2 + h * W2S + k + q];   // unit h of layer 1
+#pragma unroll
+        for (int i = 0; i < PER; ++i) acc[i] = dot4(D2 + (sb + 4 * i) * H + k, w, acc[i]);
     }
 #pragma unroll
     for (int i = 0; i < PER; ++i) D1[(sb + 4 * i) * H + h] = acc[i] * gelu_grad(smc[L.Z1 + (sb + 4 * i) * H + h]);
     __syncthreads();
     // ---- own samples to the peers
-    asm volatile("barrier.cluster.wait;" ::: "memory");
+    if (start) asm volatile("barrier.cluster.wait;" ::: "memory");
     const uint32_t base = (uint32_t)__cvta_generic_to_shared(smc);
     for (int e = t; e < C * OWN * (H / 4); e += NT) {
         const int p = e / (OWN * (H / 4)), q = e - p * (OWN * (H / 4));
@@ -461,8 +482,6 @@ mlp_tile_cluster(const float* __restrict__ params, int D, const float* __restric
     }
     asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
     // ---- this CTA's rows of the tile's gradient
-    const int64_t Pc = param_count(D);
-    float* G = partial + tile * Pc;
     float* gW1 = G;
     float* gb1 = gW1 + (int64_t)D * H;
     float* gW2 = gb1 + H;
@@ -517,8 +536,47 @@ mlp_tile_cluster(const float* __restrict__ params, int D, const float* __restric
             l += smc[L.sq + s];
         }
         gb3[0] = g;
-        loss_part[tile] = l;
+        *loss_part = l;
     }
+}
+
+template <int C>
+__global__ void __launch_bounds__(NT)
+mlp_tile_cluster(const float* __restrict__ params, int D, const float* __restrict__ feats,
+                 const float* __restrict__ target, const int32_t* __restrict__ sel, int64_t count, float inv_B,
+                 float* __restrict__ partial, float* __restrict__ loss_part) {
+    extern __shared__ __align__(16) float smc[];
+    __shared__ int64_t row[TS];
+    const ClusterTile L(D, C);
+    const int rank = blockIdx.x % C;
+    const int64_t tile = blockIdx.x / C, s0 = tile * TS;
+    const int ns = (int)((count - s0) < TS ? (count - s0) : TS);
+    asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory");   // peers have started (waited for below)
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    load_samples<C>(smc, L, row, D, feats, sel, s0, ns, rank);
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    cluster_gradient<C>(smc, L, row, view(params, D), D, target, ns, inv_B, rank, true,
+                        partial + tile * param_count(D), loss_part + tile);
+}
+
+// p's gradient: the sum over tiles in a fixed order
+__device__ __forceinline__ float sum_tiles(const float* partial, int ntiles, int64_t P, int64_t p) {
+    float g = 0.f;
+#pragma unroll 16
+    for (int c = 0; c < ntiles; ++c) g += __ldcg(partial + (int64_t)c * P + p);
+    return g;
+}
+
+__device__ __forceinline__ void adam_update(float* params, float* m, float* v, int64_t p, float g, int adam_t,
+                                            float lr) {
+    const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
+    float mm = b1 * m[p] + (1.f - b1) * g;
+    float vv = b2 * v[p] + (1.f - b2) * g * g;
+    m[p] = mm;
+    v[p] = vv;
+    float mh = mm / (1.f - powf(b1, (float)adam_t));
+    float vh = vv / (1.f - powf(b2, (float)adam_t));
+    params[p] -= lr * mh / (sqrtf(vh) + eps);
 }
 
 // grad[p] = sum over tiles of partial[c][p] (fixed order); optionally Adam.
@@ -531,26 +589,73 @@ __global__ void reduce_grad(const float* __restrict__ partial, int ntiles, int64
     asm volatile("griddepcontrol.wait;" ::: "memory");
     for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < P;
          p += (int64_t)gridDim.x * blockDim.x) {
-        float g = 0.f;
-#pragma unroll 16
-        for (int c = 0; c < ntiles; ++c) g += __ldcs(partial + (int64_t)c * P + p);
+        const float g = sum_tiles(partial, ntiles, P, p);
         if (grad) grad[p] = g;
-        if (params) {
-            const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
-            float mm = b1 * m[p] + (1.f - b1) * g;
-            float vv = b2 * v[p] + (1.f - b2) * g * g;
-            m[p] = mm;
-            v[p] = vv;
-            float mh = mm / (1.f - powf(b1, (float)adam_t));
-            float vh = vv / (1.f - powf(b2, (float)adam_t));
-            params[p] -= lr * mh / (sqrtf(vh) + eps);
-        }
+        if (params) adam_update(params, m, v, p, g, adam_t, lr);
     }
     if (blockIdx.x == 0 && threadIdx.x == 0 && loss_out) {
         float l = 0.f;
         for (int c = 0; c < ntiles; ++c) l += loss_part[c];
         loss_out[loss_slot] = l;
     }
+}
+
+// ---------------------------------------------------------------------------
+// a whole epoch of mini-batch steps in one cooperative launch of clusters: the
+// CTAs stay on their SMs, a step's two kernels become two halves between grid
+// barriers (each parameter's sum and Adam update by one thread of the grid),
+// and the next step's features are fetched under the barrier.  With a pair of
+// launches per step the host's launch calls were the bound (n = 50, batches of
+// 1,024: 29 us a step, 18 of them the kernels; 20 us in this kernel).
+// The barriers are bounded: a CTA that gives up leaves its loop, and a last
+// cluster barrier keeps its shared memory in place until a peer that passed the
+// same grid barrier has stored to it.
+// ---------------------------------------------------------------------------
+struct EpochArgs {
+    float *params, *adam_m, *adam_v, *partial, *loss_part, *loss_out;
+    const float *feats, *target;
+    const int32_t* sel;
+    int64_t count, P;
+    int D, batch, adam_t;   // adam_t: steps taken before this epoch
+    float lr;
+    unsigned long long* bar;
+    int* err;
+};
+
+template <int C>
+__global__ void __launch_bounds__(NT) mlp_epoch_cluster(EpochArgs a) {
+    extern __shared__ __align__(16) float smc[];
+    __shared__ int64_t row[TS];
+    const ClusterTile L(a.D, C);
+    const int rank = blockIdx.x % C, tile = blockIdx.x / C;
+    const View P = view(a.params, a.D);
+    const int64_t s0 = (int64_t)tile * TS;
+    unsigned long long target = 0;
+    asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory");
+    int step = 0;
+    for (int64_t b0 = 0; b0 < a.count; b0 += a.batch, ++step) {
+        const int64_t nb = min((int64_t)a.batch, a.count - b0);
+        const int tiles = (int)((nb + TS - 1) / TS);
+        const bool mine = tile < tiles;             // (a last, smaller batch leaves clusters idle)
+        const int ns = (int)min((int64_t)TS, nb - s0);
+        if (mine) load_samples<C>(smc, L, row, a.D, a.feats, a.sel + b0, s0, ns, rank);
+        if (step > 0 && !grid_sync(a.bar, target += gridDim.x, a.err)) break;   // the weights are updated
+        if (mine)
+            cluster_gradient<C>(smc, L, row, P, a.D, a.target, ns, __fdiv_rn(1.f, (float)nb), rank, step == 0,
+                                a.partial + tile * a.P, a.loss_part + tile);
+        if (!grid_sync(a.bar, target += gridDim.x, a.err)) break;               // the partials are complete
+        for (int64_t p = blockIdx.x * (int64_t)NT + threadIdx.x; p < a.P; p += (int64_t)gridDim.x * NT)
+            adam_update(a.params, a.adam_m, a.adam_v, p, sum_tiles(a.partial, tiles, a.P, p), a.adam_t + step + 1,
+                        a.lr);
+        if (blockIdx.x == gridDim.x - 1 && threadIdx.x == NT - 1) {
+            float l = 0.f;
+#pragma unroll 16
+            for (int c = 0; c < tiles; ++c) l += __ldcg(a.loss_part + c);
+            a.loss_out[step] = l;
+        }
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    cluster_barrier();
 }
 
 size_t tile_smem(int D) { return (size_t)(TS * D + 4 * TS * H + 2 * TS) * sizeof(float); }
@@ -622,6 +727,70 @@ rbffd_status launch_reduce(const rbffd_mlp* m, int tiles, float* grad, float* pa
     return RBFFD_OK;
 }
 
+// The grid barrier's words, behind the losses.
+unsigned long long* barrier_words(const rbffd_mlp* m) {
+    return reinterpret_cast<unsigned long long*>(m->loss + 4096 + (m->partial_rows + 1) / 2 * 2);
+}
+
+template <int C>
+rbffd_status launch_epoch(const rbffd_mlp* m, EpochArgs a, int tiles, cudaStream_t st, bool* done) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(tiles * C));
+    cfg.blockDim = dim3(NT);
+    cfg.dynamicSmemBytes = (size_t)ClusterTile(m->D, C).total * sizeof(float);
+    cfg.stream = st;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = C;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeCooperative;
+    at[1].val.cooperative = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 2;
+    RBFFD_CUDA_TRY(cudaFuncSetAttribute(mlp_epoch_cluster<C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        (int)cfg.dynamicSmemBytes));
+    int resident = 0;
+    RBFFD_CUDA_TRY(cudaOccupancyMaxActiveClusters(&resident, mlp_epoch_cluster<C>, &cfg));
+    if (resident < tiles) return RBFFD_OK;
+    a.bar = barrier_words(m);
+    a.err = reinterpret_cast<int*>(a.bar + 1);
+    RBFFD_CUDA_TRY(cudaMemsetAsync(a.bar, 0, 2 * sizeof(unsigned long long), st));
+    RBFFD_CUDA_TRY(cudaLaunchKernelEx(&cfg, mlp_epoch_cluster<C>, a));
+    note_launch();
+    *done = true;
+    return RBFFD_OK;
+}
+
+// One epoch (the samples in the order sel) in one launch where its clusters are
+// all resident at once: of eight CTAs per tile, else of four (batches of more
+// tiles than 1,024 samples have).  Otherwise *done stays false.
+rbffd_status epoch_launch(const rbffd_mlp* m, const float* feats, const float* target, const int32_t* sel,
+                          int64_t count, int batch, float lr, cudaStream_t st, bool* done) {
+    EpochArgs a = {};
+    a.params = m->params;
+    a.adam_m = m->adam_m;
+    a.adam_v = m->adam_v;
+    a.partial = m->partial;
+    a.loss_part = m->loss + 4096;
+    a.loss_out = m->loss;
+    a.feats = feats;
+    a.target = target;
+    a.sel = sel;
+    a.count = count;
+    a.P = m->P;
+    a.D = m->D;
+    a.batch = batch;
+    a.adam_t = m->adam_t;
+    a.lr = lr;
+    const int64_t tiles = (std::min<int64_t>(batch, count) + TS - 1) / TS;
+    *done = false;
+    rbffd_status s = RBFFD_OK;
+    if (tiles * 8 <= sm_count() && cluster_fits<8>(m->D)) s = launch_epoch<8>(m, a, (int)tiles, st, done);
+    if (s == RBFFD_OK && !*done && tiles * 4 <= sm_count() && cluster_fits<4>(m->D))
+        s = launch_epoch<4>(m, a, (int)tiles, st, done);
+    return s;
+}
+
 rbffd_status ensure_smem(int D) {
     RBFFD_CUDA_TRY(cudaFuncSetAttribute(mlp_tile, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         (int)tile_smem(D)));
@@ -646,7 +815,7 @@ rbffd_status ensure_train_ws(rbffd_mlp* m, int64_t tiles) {
         cudaFree(m->loss);
         m->partial = nullptr;
         RBFFD_CUDA_TRY(cudaMalloc(&m->partial, tiles * m->P * sizeof(float)));
-        RBFFD_CUDA_TRY(cudaMalloc(&m->loss, (tiles + 4096) * sizeof(float)));
+        RBFFD_CUDA_TRY(cudaMalloc(&m->loss, (tiles + 4096 + 6) * sizeof(float))   /* and barrier words */);
         m->partial_rows = tiles;
     }
     return RBFFD_OK;
@@ -837,7 +1006,11 @@ rbffd_status rbffd_mlp_train(rbffd_mlp* m, const float* feats, const float* targ
     shuffle(perm);
     for (int ep = 0; ep < epochs; ++ep) {
         RBFFD_CUDA_TRY(cudaMemcpyAsync(perm_d, perm.data(), count * sizeof(int32_t), cudaMemcpyHostToDevice, st));
-        for (int64_t b = 0; b < steps_per_epoch; ++b) {
+        bool whole;
+        s = epoch_launch(m, feats, target, perm_d, count, batch, lr, st, &whole);
+        if (s != RBFFD_OK) return s;
+        if (whole) m->adam_t += (int)steps_per_epoch;
+        for (int64_t b = 0; !whole && b < steps_per_epoch; ++b) {
             int64_t b0 = b * batch;
             int64_t nb = std::min<int64_t>(batch, count - b0);
             unsigned tiles = (unsigned)((nb + TS - 1) / TS);
@@ -852,9 +1025,17 @@ rbffd_status rbffd_mlp_train(rbffd_mlp* m, const float* feats, const float* targ
             next = perm;
             shuffle(next);
         }
+        int gave_up = 0;
         RBFFD_CUDA_TRY(cudaMemcpyAsync(lossv.data(), m->loss, steps_per_epoch * sizeof(float),
                                        cudaMemcpyDeviceToHost, st));
+        if (whole)
+            RBFFD_CUDA_TRY(cudaMemcpyAsync(&gave_up, barrier_words(m) + 1, sizeof(int), cudaMemcpyDeviceToHost, st));
         RBFFD_CUDA_TRY(cudaStreamSynchronize(st));
+        if (gave_up) {
+            cudaFreeAsync(perm_d, st);
+            set_error("rbffd_mlp_train: a grid barrier of the training kernel gave up");
+            return RBFFD_ECUDA;
+        }
         perm.swap(next);
         if (loss_host) {
             double tot = 0.0;
