@@ -498,8 +498,9 @@ __global__ void __launch_bounds__(SOLVE_THREADS) solve_kernel(SolveArgs<T, TV> a
 // to all CTAs while they update the rest, so a block costs one triangle, one
 // 32-column update of 32 rows and a cluster barrier.  The back substitution is
 // the same on mirrored rows, its rows scaled by 1 / U_ii so that the triangle's
-// chain has no division.  2,400 rows, bands of about 300: 4.2 -> 0.7 ms per
-// solve of two species.
+// chain has no division.  2,400 rows, bands of about 300: 4.2 -> 0.6 ms per
+// solve of two species (0.88 with the next block's coefficients loaded in the
+// step that uses them).
 // ---------------------------------------------------------------------------
 constexpr int NB = 32;                 // rows of a block
 constexpr int BLK_CTAS = 8;            // CTAs of the cluster
@@ -522,7 +523,7 @@ __device__ __forceinline__ void st_cluster(uint32_t a, float v) {
 // r' = N - 1 - r.  in / out: the right-hand side and the result by row.
 template <typename T, bool BACK, typename TI, typename TO>
 __device__ void block_sweep(const SolveSys<T>& f, int64_t N, int64_t kl, int64_t ku, const TI* in, TO* out, T* ring,
-                            int slots, T (*ybuf)[NB], T (*part)[NB], int rank) {
+                            int slots, T (*ybuf)[NB], T (*part)[NB], T (*tri)[NB], int rank) {
     const int64_t bw = BACK ? kl + ku : kl, ldab = 2 * kl + ku + 1;
     const int64_t nblk = (N + NB - 1) / NB, reach = (bw + NB - 1) / NB;   // blocks a block reaches below itself
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -538,21 +539,36 @@ __device__ void block_sweep(const SolveSys<T>& f, int64_t N, int64_t kl, int64_t
         const int64_t r = b * NB + lane;
         slot(b)[lane] = r < N ? (T)in[BACK ? N - 1 - r : r] : T(0);
     };
+    // A block's coefficients are fetched in the step before their use, at its
+    // start (the barrier at its end waits for loads still in flight), by the
+    // UPD warps that update the next block: eight columns of the update each,
+    // kept in registers, and eight of the triangle, put in shared memory
+    // scaled by U's diagonal (back sweep).
+    constexpr int CW = NB / UPD;
+    T tcol[CW], upd[CW], diag = T(1);
+    auto fetch = [&](int64_t b) {
+        const int64_t r0 = b * NB, r = r0 + lane;
+#pragma unroll
+        for (int c = 0; c < CW; ++c) {
+            const int q = warp * CW + c;
+            tcol[c] = q < lane ? coef(r, r0 + q) : T(0);
+            upd[c] = b > 0 ? coef(r, r0 - NB + q) : T(0);
+        }
+        if (BACK) diag = r < N ? f.udiag[N - 1 - r] : T(1);
+    };
+    auto store_triangle = [&]() {
+        const T d = BACK ? T(1) / diag : T(1);
+#pragma unroll
+        for (int c = 0; c < CW; ++c) tri[warp * CW + c][lane] = BACK ? tcol[c] * d : tcol[c];
+        if (warp == 0) tri[NB][lane] = d;
+    };
     // solve the triangle of block b (its rows updated) by one warp, copy the
     // result to all CTAs and to `out`
     auto solve = [&](int64_t b, T y) {
-        const int64_t r0 = b * NB, r = r0 + lane;
-        T l[NB];
+        const int64_t r = b * NB + lane;
+        if (BACK) y *= tri[NB][lane];
 #pragma unroll
-        for (int c = 0; c < NB; ++c) l[c] = c < lane ? coef(r, r0 + c) : T(0);
-        if (BACK) {
-            const T d = r < N ? T(1) / f.udiag[N - 1 - r] : T(1);
-            y *= d;
-#pragma unroll
-            for (int c = 0; c < NB; ++c) l[c] *= d;
-        }
-#pragma unroll
-        for (int c = 0; c < NB; ++c) y = fma(-l[c], __shfl_sync(0xffffffffu, y, c), y);
+        for (int c = 0; c < NB; ++c) y = fma(-tri[c][lane], __shfl_sync(0xffffffffu, y, c), y);
 #pragma unroll
         for (int p = 0; p < BLK_CTAS; ++p) st_cluster(peer_smem(&ybuf[b & 1][lane], p), y);
         if (r < N) out[BACK ? N - 1 - r : r] = (TO)y;
@@ -561,20 +577,25 @@ __device__ void block_sweep(const SolveSys<T>& f, int64_t N, int64_t kl, int64_t
     for (int64_t b = rank + (int64_t)warp * BLK_CTAS; b <= min(reach + 1, nblk - 1); b += (int64_t)BLK_WARPS * BLK_CTAS)
         load(b);
     __syncthreads();
+    if (rank < 2 && warp < UPD) {
+        fetch(rank);
+        store_triangle();
+    }
+    __syncthreads();
     if (rank == 0 && warp == 0) solve(0, slot(0)[lane]);
     cluster_barrier();
     for (int64_t k = 0; k + 1 < nblk; ++k) {
         const T* y = ybuf[k & 1];
         const int64_t nx = k + 1;
-        const bool owner = nx % BLK_CTAS == rank;
-        // the owner's first warps bring the next block up to date and solve it
-        if (owner && warp < UPD) {
-            constexpr int CW = NB / UPD;
-            T a[CW], s = T(0);
+        const bool owner = nx % BLK_CTAS == rank, ahead = (nx + 1) % BLK_CTAS == rank;
+        if (ahead && warp < UPD) {
+            fetch(nx + 1);
+            store_triangle();
+        } else if (owner && warp < UPD) {
+            // the owner's first warps bring the next block up to date and solve it
+            T s = T(0);
 #pragma unroll
-            for (int c = 0; c < CW; ++c) a[c] = coef(nx * NB + lane, k * NB + warp * CW + c);
-#pragma unroll
-            for (int c = 0; c < CW; ++c) s = fma(a[c], y[warp * CW + c], s);
+            for (int c = 0; c < CW; ++c) s = fma(upd[c], y[warp * CW + c], s);
             part[warp][lane] = s;
             asm volatile("bar.sync 1, %0;" ::"n"(UPD * 32) : "memory");
             if (warp == 0) {
@@ -583,20 +604,23 @@ __device__ void block_sweep(const SolveSys<T>& f, int64_t N, int64_t kl, int64_t
                 for (int w = 0; w < UPD; ++w) v -= part[w][lane];
                 solve(nx, v);
             }
-        }
-        // the other warps update the rows below it, a warp per block, and load
-        // the block that enters the window
-        const int w0 = owner ? UPD : 0, nw = BLK_WARPS - w0;
-        if (warp >= w0) {
+        } else {
+            // the other warps update the rows below it, a warp per block, and
+            // load the block that enters the window
+            const int w0 = owner || ahead ? UPD : 0, nw = BLK_WARPS - w0;
             const int64_t first = nx + 1 + ((rank - (nx + 1)) % BLK_CTAS + BLK_CTAS) % BLK_CTAS;
             for (int64_t b = first + (int64_t)(warp - w0) * BLK_CTAS; b <= min(k + reach, nblk - 1);
                  b += (int64_t)nw * BLK_CTAS) {
                 const int64_t r = b * NB + lane;
-                T v = slot(b)[lane], a[NB];
+                T v = slot(b)[lane];
+#pragma unroll 1
+                for (int h = 0; h < NB; h += 16) {   // 16 loads in flight (32 spill)
+                    T a[16];
 #pragma unroll
-                for (int c = 0; c < NB; ++c) a[c] = coef(r, k * NB + c);
+                    for (int c = 0; c < 16; ++c) a[c] = coef(r, k * NB + h + c);
 #pragma unroll
-                for (int c = 0; c < NB; ++c) v = fma(-a[c], y[c], v);
+                    for (int c = 0; c < 16; ++c) v = fma(-a[c], y[h + c], v);
+                }
                 slot(b)[lane] = v;
             }
             const int64_t enter = k + reach + 2;
@@ -612,7 +636,7 @@ __host__ __device__ inline int block_slots(int64_t bw) { return (int)(((bw + NB 
 template <typename T, typename TV>
 __global__ void __cluster_dims__(BLK_CTAS, 1, 1) __launch_bounds__(BLK_THREADS) solve_blocks_kernel(SolveArgs<T, TV> a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ T ybuf[2][NB], part[UPD][NB];
+    __shared__ T ybuf[2][NB], part[UPD][NB], tri[NB + 1][NB];
     T* ring = reinterpret_cast<T*>(smem_raw);
     const int sp = blockIdx.x / BLK_CTAS, rank = blockIdx.x % BLK_CTAS;
     const int ord = a.ord_flag ? *((volatile const int*)a.ord_flag) : 1;
@@ -620,11 +644,11 @@ __global__ void __cluster_dims__(BLK_CTAS, 1, 1) __launch_bounds__(BLK_THREADS) 
     T* wy = a.work + sp * (2 * a.N + 16);
     const int slots = block_slots(a.kl + a.ku);
     cluster_barrier();   // all CTAs run before their shared memory is written
-    block_sweep<T, false>(f, a.N, a.kl, a.ku, a.b[sp], wy, ring, slots, ybuf, part, rank);
+    block_sweep<T, false>(f, a.N, a.kl, a.ku, a.b[sp], wy, ring, slots, ybuf, part, tri, rank);
     // the forward results, written by every CTA, are read by all
     __threadfence();
     cluster_barrier();
-    block_sweep<T, true>(f, a.N, a.kl, a.ku, wy, a.x[sp], ring, slots, ybuf, part, rank);
+    block_sweep<T, true>(f, a.N, a.kl, a.ku, wy, a.x[sp], ring, slots, ybuf, part, tri, rank);
 }
 
 template <typename T>
