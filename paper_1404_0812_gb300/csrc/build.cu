@@ -175,7 +175,21 @@ __device__ void assemble_phi(const Lane& S, const Layout& ly, int n, int kernel,
     for (int i = 0; i < ly.m; ++i) {
         int base = pk(i, 0);
         if (i < n) {
-            for (int j = 0; j < i; ++j) {
+            int j = 0;
+            for (; j + 4 <= i; j += 4) {   // four loads ahead of the stores
+                double v[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) v[q] = S[ly.R2 + base + j + q];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) v[q] = phi_of(kernel, e2, v[q]);
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    S[dst + base + j + q] = v[q];
+                    if (cpy >= 0) S[cpy + base + j + q] = v[q];
+                    if (fcpy >= 0) F[base + j + q] = (float)v[q];
+                }
+            }
+            for (; j < i; ++j) {
                 double v = phi_of(kernel, e2, S[ly.R2 + base + j]);
                 S[dst + base + j] = v;
                 if (cpy >= 0) S[cpy + base + j] = v;
@@ -220,6 +234,27 @@ __device__ __forceinline__ void chol_tile_accumulate(const Lane& S, int L, int i
         for (int a = 0; a < R; ++a) xa[a] = xn[a];
 #pragma unroll
         for (int b = 0; b < 4; ++b) yb[b] = yn[b];
+    }
+}
+
+// The diagonal tile (ib = jb): its lower half only, ten of sixteen FMAs and
+// half the loads of a step.
+__device__ __forceinline__ void chol_diag_accumulate(const Lane& S, int L, int jb, double (&acc)[4][4]) {
+    const int r = L + pk(jb, 0);
+    double x[4];
+#pragma unroll
+    for (int a = 0; a < 4; ++a) x[a] = S[r + a * jb + a * (a + 1) / 2];
+    for (int k = 0; k < jb; ++k) {
+        double xn[4];
+        const int kn = k + 1 < jb ? k + 1 : k;
+#pragma unroll
+        for (int a = 0; a < 4; ++a) xn[a] = S[r + a * jb + a * (a + 1) / 2 + kn];
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+#pragma unroll
+            for (int b = 0; b <= a; ++b) acc[a][b] = fma(-x[a], x[b], acc[a][b]);
+#pragma unroll
+        for (int a = 0; a < 4; ++a) x[a] = xn[a];
     }
 }
 
@@ -268,7 +303,7 @@ __device__ bool cholesky(const Lane& S, const Layout& ly, int n) {
             for (int a = 0; a < 4; ++a)
 #pragma unroll
                 for (int b = 0; b < 4; ++b) acc[a][b] = (a >= b) ? S[L + pk(ib + a, jb + b)] : 0.0;
-            if (jb > 0) chol_tile_accumulate<4>(S, L, ib, jb, acc);
+            if (jb > 0) chol_diag_accumulate(S, L, jb, acc);
 #pragma unroll
             for (int b = 0; b < 4; ++b) {
                 double d = acc[b][b];
@@ -475,28 +510,38 @@ __device__ double lanczos_max_f32(const Lane& S, const Layout& ly, int n, double
         // [Phi q + qb 1; 1^T q]
         phi_mul_f32(F, V, q_, w, m);
         float sum = 0.f;
-        for (int i = 0; i < n; ++i) {
-            sum += V[q_ + i];
-            V[w + i] += qb;
-        }
+        for (int i = 0; i < n; ++i) sum += V[q_ + i];
         float wb = fmaf(-beta, qpb, sum);
         float ap[4] = {0.f, 0.f, 0.f, 0.f};
         for (int i = 0; i < m; i += 4) {
+            float v[4], x[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) v[q] = V[w + i + q];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) x[q] = V[qp + i + q];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) v[q] = fmaf(-beta, x[q], i + q < n ? v[q] + qb : v[q]);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) x[q] = V[q_ + i + q];
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                const float v = fmaf(-beta, V[qp + i + q], V[w + i + q]);
-                V[w + i + q] = v;
-                ap[q] = fmaf(V[q_ + i + q], v, ap[q]);
+                V[w + i + q] = v[q];
+                ap[q] = fmaf(x[q], v[q], ap[q]);
             }
         }
         const float a = fmaf(qb, wb, (ap[0] + ap[1]) + (ap[2] + ap[3]));
         float bp[4] = {0.f, 0.f, 0.f, 0.f};
         for (int i = 0; i < m; i += 4) {
+            float v[4], x[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) v[q] = V[w + i + q];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) x[q] = V[q_ + i + q];
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                const float v = fmaf(-a, V[q_ + i + q], V[w + i + q]);
-                V[w + i + q] = v;
-                bp[q] = fmaf(v, v, bp[q]);
+                v[q] = fmaf(-a, x[q], v[q]);
+                V[w + i + q] = v[q];
+                bp[q] = fmaf(v[q], v[q], bp[q]);
             }
         }
         wb = fmaf(-a, qb, wb);
@@ -573,7 +618,13 @@ __device__ double lanczos_inv_ritz(const Lane& S, const Layout& ly, int n, doubl
         const int qj = ly.QB + j * m, qp = ly.QB + (j - 1) * m;
         // [c; d] = A^{-1} [f; g]: c0 = Phi^{-1} f, d = (1^T c0 - g) / s, c = c0 - d u
         if (j > 0 || !w0_ready) {
-            for (int i = 0; i < m; ++i) S[w + i] = S[qj + i];
+            for (int i = 0; i < m; i += 4) {
+                double v[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) v[q] = S[qj + i + q];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) S[w + i + q] = v[q];
+            }
             chol_solve(S, ly, w);
         }
         double sp[4] = {0.0, 0.0, 0.0, 0.0};
@@ -581,27 +632,45 @@ __device__ double lanczos_inv_ritz(const Lane& S, const Layout& ly, int n, doubl
 #pragma unroll
             for (int q = 0; q < 4; ++q) sp[q] += S[w + i + q];
         double dd = ((sp[0] + sp[1]) + (sp[2] + sp[3]) - qbord[j]) / s;
-        for (int i = 0; i < n; ++i) S[w + i] = fma(-dd, S[ly.U + i], S[w + i]);
         double wb = dd;
         double ap[4] = {0.0, 0.0, 0.0, 0.0};
-        for (int i = 0; i < m; i += 4) {
+        for (int i = 0; i < m; i += 4) {   // the loads of four elements ahead of the stores
+            double v[4], x[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) v[q] = S[w + i + q];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) x[q] = S[ly.U + i + q];
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (i + q < n) v[q] = fma(-dd, x[q], v[q]);
+            if (j > 0) {
+#pragma unroll
+                for (int q = 0; q < 4; ++q) x[q] = S[qp + i + q];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) v[q] = fma(-beta, x[q], v[q]);
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) x[q] = S[qj + i + q];
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                double v = S[w + i + q];
-                if (j > 0) v = fma(-beta, S[qp + i + q], v);
-                S[w + i + q] = v;
-                ap[q] = fma(S[qj + i + q], v, ap[q]);
+                S[w + i + q] = v[q];
+                ap[q] = fma(x[q], v[q], ap[q]);
             }
         }
         if (j > 0) wb = fma(-beta, qbord[j - 1], wb);
         double a = fma(qbord[j], wb, (ap[0] + ap[1]) + (ap[2] + ap[3]));
         double bp[4] = {0.0, 0.0, 0.0, 0.0};
         for (int i = 0; i < m; i += 4) {
+            double v[4], x[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) v[q] = S[w + i + q];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) x[q] = S[qj + i + q];
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                double v = fma(-a, S[qj + i + q], S[w + i + q]);
-                S[w + i + q] = v;
-                bp[q] = fma(v, v, bp[q]);
+                v[q] = fma(-a, x[q], v[q]);
+                S[w + i + q] = v[q];
+                bp[q] = fma(v[q], v[q], bp[q]);
             }
         }
         wb = fma(-a, qbord[j], wb);
@@ -642,7 +711,13 @@ __device__ double lanczos_inv_ritz(const Lane& S, const Layout& ly, int n, doubl
         beta = bn;
         const double ib = 1.0 / bn;
         const int qn = ly.QB + (j + 1) * m;
-        for (int i = 0; i < m; ++i) S[qn + i] = S[w + i] * ib;
+        for (int i = 0; i < m; i += 4) {
+            double v[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) v[q] = S[w + i + q];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) S[qn + i + q] = v[q] * ib;
+        }
         qbord[j + 1] = wb * ib;
     }
     // Ritz vector  v = sum_j y_j q_j
