@@ -56,6 +56,19 @@ namespace {
 
 // ---------------------------------------------------------------------------
 // lane-private scratch, interleaved across the warp
+//
+// Size of the code.  The warps of an SM are in different phases of their
+// stencils, and with the loops unrolled as the compiler likes the search was
+// 483 KB of instructions: warps waited longer for instructions than for
+// anything else (38 % of their time, 1M nodes in four sizes 421 ms).  So the
+// lane functions' loops are not unrolled (unroll 1) where their bodies already
+// keep loads in flight, the triangular solves are functions called from several
+// places, views and layouts go by value (a reference is read again after every
+// store), and the kernel function is a template argument: 192 KB, 385 ms.  Only
+// the solves' chunk loops keep the compiler's unrolling (404 ms without, 397
+// with, before the other changes).  For the same reason variants with more code
+// were slower: the solves' next chunk fetched ahead 461 ms, 168 registers for
+// it on three blocks per SM 449 ms.
 // ---------------------------------------------------------------------------
 struct Lane {
     double* p;   // points at element 0 of this lane
@@ -119,12 +132,13 @@ __host__ __device__ inline Layout make_layout(int m, bool full) {
 // ---------------------------------------------------------------------------
 // stencil geometry: centre-translated, r_s-scaled coordinates and normals
 // ---------------------------------------------------------------------------
-__device__ Geo load_geometry(const Lane& S, const Layout& ly, int n, const int32_t* __restrict__ idx,
+__device__ Geo load_geometry(const Lane S, const Layout ly, int n, const int32_t* __restrict__ idx,
                              int64_t off, int npad, int64_t lr, const double* __restrict__ X,
                              const double* __restrict__ NR, bool with_normals) {
     int c = idx[ell_elem(off, npad, lr, 0)];
     double cx = X[3 * (int64_t)c], cy = X[3 * (int64_t)c + 1], cz = X[3 * (int64_t)c + 2];
     double rs2 = 0.0;
+#pragma unroll 1
     for (int j = 0; j < n; ++j) {
         int k = idx[ell_elem(off, npad, lr, j)];
         double dx = X[3 * (int64_t)k] - cx, dy = X[3 * (int64_t)k + 1] - cy,
@@ -145,6 +159,7 @@ __device__ Geo load_geometry(const Lane& S, const Layout& ly, int n, const int32
     g.rs = sqrt(rs2);
     double inv = 1.0 / g.rs;
     double sum = 0.0;
+#pragma unroll 1
     for (int j = 0; j < n; ++j) {
         double x = S[ly.XS + j] * inv, y = S[ly.XS + ly.m + j] * inv, z = S[ly.XS + 2 * ly.m + j] * inv;
         S[ly.XS + j] = x;
@@ -154,9 +169,11 @@ __device__ Geo load_geometry(const Lane& S, const Layout& ly, int n, const int32
     }
     g.mean_d = sum / (double)(n - 1);
     // pairwise squared distances (lower triangle, diagonal 0)
+#pragma unroll 1
     for (int i = 0; i < n; ++i) {
         double xi = S[ly.XS + i], yi = S[ly.XS + ly.m + i], zi = S[ly.XS + 2 * ly.m + i];
         int base = pk(i, 0);
+#pragma unroll 1
         for (int j = 0; j < i; ++j) {
             double dx = xi - S[ly.XS + j], dy = yi - S[ly.XS + ly.m + j], dz = zi - S[ly.XS + 2 * ly.m + j];
             S[ly.R2 + base + j] = dx * dx + dy * dy + dz * dz;
@@ -168,14 +185,16 @@ __device__ Geo load_geometry(const Lane& S, const Layout& ly, int n, const int32
 
 // Phi(eps) into region dst (lower packed, m x m, identity on the padding);
 // optionally a copy into region cpy and a float32 copy into region fcpy.
-__device__ void assemble_phi(const Lane& S, const Layout& ly, int n, int kernel, double eps_s,
+__device__ void assemble_phi(const Lane S, const Layout ly, int n, int kernel, double eps_s,
                              int dst, int cpy, int fcpy = -1) {
     double e2 = eps_s * eps_s;
     const LaneF F = float_view(S, fcpy >= 0 ? fcpy : 0);
+#pragma unroll 1
     for (int i = 0; i < ly.m; ++i) {
         int base = pk(i, 0);
         if (i < n) {
             int j = 0;
+#pragma unroll 1
             for (; j + 4 <= i; j += 4) {   // four loads ahead of the stores
                 double v[4];
 #pragma unroll
@@ -189,6 +208,7 @@ __device__ void assemble_phi(const Lane& S, const Layout& ly, int n, int kernel,
                     if (fcpy >= 0) F[base + j + q] = (float)v[q];
                 }
             }
+#pragma unroll 1
             for (; j < i; ++j) {
                 double v = phi_of(kernel, e2, S[ly.R2 + base + j]);
                 S[dst + base + j] = v;
@@ -196,6 +216,7 @@ __device__ void assemble_phi(const Lane& S, const Layout& ly, int n, int kernel,
                 if (fcpy >= 0) F[base + j] = (float)v;
             }
         } else {
+#pragma unroll 1
             for (int j = 0; j < i; ++j) {
                 S[dst + base + j] = 0.0;
                 if (cpy >= 0) S[cpy + base + j] = 0.0;
@@ -219,6 +240,7 @@ __device__ __forceinline__ void chol_tile_accumulate(const Lane& S, int L, int i
     for (int a = 0; a < R; ++a) xa[a] = S[ra + a * ib + a * (a + 1) / 2];
 #pragma unroll
     for (int b = 0; b < 4; ++b) yb[b] = S[rb + b * jb + b * (b + 1) / 2];
+#pragma unroll 1
     for (int k = 0; k < jb; ++k) {
         double xn[R], yn[4];
         const int kn = k + 1 < jb ? k + 1 : k;
@@ -244,6 +266,7 @@ __device__ __forceinline__ void chol_diag_accumulate(const Lane& S, int L, int j
     double x[4];
 #pragma unroll
     for (int a = 0; a < 4; ++a) x[a] = S[r + a * jb + a * (a + 1) / 2];
+#pragma unroll 1
     for (int k = 0; k < jb; ++k) {
         double xn[4];
         const int kn = k + 1 < jb ? k + 1 : k;
@@ -263,7 +286,7 @@ __device__ __forceinline__ void chol_diag_accumulate(const Lane& S, int L, int j
 // row block, whose other rows are padding (identity rows of Phi: their L
 // entries stay the zeros the assembly wrote, and no real row reads them).
 template <int R>
-__device__ __forceinline__ void chol_tile_offdiag(const Lane& S, const Layout& ly, int ib, int jb,
+__device__ __forceinline__ void chol_tile_offdiag(const Lane S, const Layout ly, int ib, int jb,
                                                   const double (&Ld)[4][4]) {
     const int L = ly.L;
     double acc[R][4];
@@ -290,9 +313,10 @@ __device__ __forceinline__ void chol_tile_offdiag(const Lane& S, const Layout& l
 // ID receives 1 / L_ii.  Returns false when a pivot is not positive.  Rows
 // n .. m-1 are padding (identity in Phi and in L): the off-diagonal tiles of
 // the last row block leave them out.
-__device__ bool cholesky(const Lane& S, const Layout& ly, int n) {
+__device__ bool cholesky(const Lane S, const Layout ly, int n) {
     const int m = ly.m, L = ly.L;
     bool ok = true;
+#pragma unroll 1
     for (int jb = 0; jb < m; jb += 4) {
         double Ld[4][4];
         {
@@ -330,6 +354,7 @@ __device__ bool cholesky(const Lane& S, const Layout& ly, int n) {
                     S[L + pk(jb + a, jb + b)] = acc[a][b];
                 }
         }
+#pragma unroll 1
         for (int ib = jb + 4; ib < m; ib += 4) {
             const int rows = n - ib;   // >= 1: padding is less than one block
             if (rows >= 4) chol_tile_offdiag<4>(S, ly, ib, jb, Ld);
@@ -342,7 +367,7 @@ __device__ bool cholesky(const Lane& S, const Layout& ly, int n) {
     return true;
 }
 
-// x_d <- Phi^{-1} x_d for NR right-hand sides (regions V[d], length m) using
+// x_d <- Phi^{-1} x_d for NR right-hand sides (regions V0 + d VS, length m) using
 // L and ID: forward L y = x, then backward L^T x = y, in blocks of four rows.
 // A chunk of C = 4 / NR columns (forward) or rows (backward) is loaded before
 // its FMAs issue, so each step keeps 4 C + NR C loads in flight for 4 C NR
@@ -350,7 +375,7 @@ __device__ bool cholesky(const Lane& S, const Layout& ly, int n) {
 // receives the blocks' updates from the last block down (backward), whatever
 // NR is, so a right-hand side gets the same bits alone or with others.
 template <int NR>
-__device__ void chol_solve_multi(const Lane& S, const Layout& ly, const int (&V)[NR]) {
+__device__ __noinline__ void chol_solve_multi(const Lane S, const Layout ly, int V0, int VS) {
     constexpr int C = NR == 1 ? 4 : NR == 2 ? 2 : 1;
     const int m = ly.m, L = ly.L;
     for (int ib = 0; ib < m; ib += 4) {   // forward
@@ -358,14 +383,14 @@ __device__ void chol_solve_multi(const Lane& S, const Layout& ly, const int (&V)
 #pragma unroll
         for (int a = 0; a < 4; ++a)
 #pragma unroll
-            for (int d = 0; d < NR; ++d) t[a][d] = S[V[d] + ib + a];
+            for (int d = 0; d < NR; ++d) t[a][d] = S[V0 + d * VS + ib + a];
         const int r = pk(ib, 0);   // row ib + a starts at r + a ib + a (a + 1) / 2
         for (int k = 0; k < ib; k += C) {   // ib is a multiple of 4, hence of C
             double y[C][NR], l[4][C];
 #pragma unroll
             for (int q = 0; q < C; ++q)
 #pragma unroll
-                for (int d = 0; d < NR; ++d) y[q][d] = S[V[d] + k + q];
+                for (int d = 0; d < NR; ++d) y[q][d] = S[V0 + d * VS + k + q];
 #pragma unroll
             for (int a = 0; a < 4; ++a)
 #pragma unroll
@@ -389,7 +414,7 @@ __device__ void chol_solve_multi(const Lane& S, const Layout& ly, const int (&V)
 #pragma unroll
             for (int d = 0; d < NR; ++d) {
                 t[a][d] *= id;
-                S[V[d] + ib + a] = t[a][d];
+                S[V0 + d * VS + ib + a] = t[a][d];
             }
         }
     }
@@ -398,7 +423,7 @@ __device__ void chol_solve_multi(const Lane& S, const Layout& ly, const int (&V)
 #pragma unroll
         for (int b = 3; b >= 0; --b) {
 #pragma unroll
-            for (int d = 0; d < NR; ++d) t[b][d] = S[V[d] + kb + b];
+            for (int d = 0; d < NR; ++d) t[b][d] = S[V0 + d * VS + kb + b];
 #pragma unroll
             for (int c = b + 1; c < 4; ++c) {
                 const double l = S[L + pk(kb + c, kb + b)];
@@ -409,7 +434,7 @@ __device__ void chol_solve_multi(const Lane& S, const Layout& ly, const int (&V)
 #pragma unroll
             for (int d = 0; d < NR; ++d) {
                 t[b][d] *= id;
-                S[V[d] + kb + b] = t[b][d];
+                S[V0 + d * VS + kb + b] = t[b][d];
             }
         }
         const int r0 = pk(kb, 0), r1 = pk(kb + 1, 0), r2 = pk(kb + 2, 0), r3 = pk(kb + 3, 0);
@@ -422,7 +447,7 @@ __device__ void chol_solve_multi(const Lane& S, const Layout& ly, const int (&V)
                 l[2][q] = S[L + r2 + i + q];
                 l[3][q] = S[L + r3 + i + q];
 #pragma unroll
-                for (int d = 0; d < NR; ++d) v[q][d] = S[V[d] + i + q];
+                for (int d = 0; d < NR; ++d) v[q][d] = S[V0 + d * VS + i + q];
             }
 #pragma unroll
             for (int b = 0; b < 4; ++b)
@@ -433,15 +458,14 @@ __device__ void chol_solve_multi(const Lane& S, const Layout& ly, const int (&V)
 #pragma unroll
             for (int q = 0; q < C; ++q)
 #pragma unroll
-                for (int d = 0; d < NR; ++d) S[V[d] + i + q] = v[q][d];
+                for (int d = 0; d < NR; ++d) S[V0 + d * VS + i + q] = v[q][d];
         }
     }
 }
 
 // x <- Phi^{-1} x (x in region V of length m)
-__device__ void chol_solve(const Lane& S, const Layout& ly, int V) {
-    const int R[1] = {V};
-    chol_solve_multi<1>(S, ly, R);
+__device__ void chol_solve(const Lane S, const Layout ly, int V) {
+    chol_solve_multi<1>(S, ly, V, 0);
 }
 
 // y = Phi x in float32 from the packed float32 copy F of Phi, x and y at
@@ -450,7 +474,7 @@ __device__ void chol_solve(const Lane& S, const Layout& ly, int V) {
 // the block's rows, the 4 x 4 diagonal block, and columns right of it from
 // the rows below (symmetry).  The padding rows of Phi are the identity and
 // entries n..m-1 of x are zero, so the loops run to m.
-__device__ void phi_mul_f32(const LaneF& F, const LaneF& V, int x, int y, int m) {
+__device__ void phi_mul_f32(const LaneF F, const LaneF V, int x, int y, int m) {
     for (int ib = 0; ib < m; ib += 4) {
         float acc[4] = {0.f, 0.f, 0.f, 0.f};
         const int r = pk(ib, 0);   // row ib + a starts at r + a ib + a (a + 1) / 2
@@ -486,13 +510,14 @@ __device__ void phi_mul_f32(const LaneF& F, const LaneF& V, int x, int y, int m)
 // conditioned (Weyl: float32 rounding of Phi and of the products moves it
 // by ~sqrt(m) 6e-8 relative), so float32 costs kappa no accuracy that the
 // root finder would notice and takes the run off the float64 pipe.
-__device__ double lanczos_max_f32(const Lane& S, const Layout& ly, int n, double rtol) {
+__device__ double lanczos_max_f32(const Lane S, const Layout ly, int n, double rtol) {
     const int m = ly.m;
     const LaneF F = float_view(S, ly.PF), V = float_view(S, ly.FV);
     float al[LANCZOS_KMAX], b2[LANCZOS_KMAX];
     double alpha_d[LANCZOS_KMAX], beta_d[LANCZOS_KMAX];
     int qp = 0, q_ = m, w = 2 * m;
     float nrm2 = 0.f;
+#pragma unroll 1
     for (int i = 0; i < m; ++i) {
         const float v = i < n ? 1.0f + 0.01f * (__cosf(1.7f * (float)i + 0.3f) + 0.1f) : 0.f;
         V[q_ + i] = v;
@@ -502,17 +527,21 @@ __device__ double lanczos_max_f32(const Lane& S, const Layout& ly, int n, double
     float qb = 0.1f, qpb = 0.f;
     nrm2 = fmaf(qb, qb, nrm2);
     const float inrm = rsqrtf(nrm2);
+#pragma unroll 1
     for (int i = 0; i < n; ++i) V[q_ + i] *= inrm;
     qb *= inrm;
     float beta = 0.f;
     double prev = -1.0, ext = 0.0;
+#pragma unroll 1
     for (int j = 0; j < LANCZOS_KMAX; ++j) {
         // [Phi q + qb 1; 1^T q]
         phi_mul_f32(F, V, q_, w, m);
         float sum = 0.f;
+#pragma unroll 1
         for (int i = 0; i < n; ++i) sum += V[q_ + i];
         float wb = fmaf(-beta, qpb, sum);
         float ap[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 1
         for (int i = 0; i < m; i += 4) {
             float v[4], x[4];
 #pragma unroll
@@ -531,6 +560,7 @@ __device__ double lanczos_max_f32(const Lane& S, const Layout& ly, int n, double
         }
         const float a = fmaf(qb, wb, (ap[0] + ap[1]) + (ap[2] + ap[3]));
         float bp[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 1
         for (int i = 0; i < m; i += 4) {
             float v[4], x[4];
 #pragma unroll
@@ -550,11 +580,13 @@ __device__ double lanczos_max_f32(const Lane& S, const Layout& ly, int n, double
         beta_d[j] = bn;
         // scaled tridiagonal (Gershgorin bound as the scale)
         double G = 0.0;
+#pragma unroll 1
         for (int i = 0; i <= j; ++i) {
             double r = fabs(alpha_d[i]) + (i < j ? beta_d[i] : 0.0) + (i > 0 ? beta_d[i - 1] : 0.0);
             G = fmax(G, r);
         }
         const double ig = 1.0 / G;
+#pragma unroll 1
         for (int i = 0; i <= j; ++i) {
             al[i] = (float)(alpha_d[i] * ig);
             const float bb = (float)(beta_d[i] * ig);
@@ -573,6 +605,7 @@ __device__ double lanczos_max_f32(const Lane& S, const Layout& ly, int n, double
         q_ = w;
         w = t;
         qpb = qb;
+#pragma unroll 1
         for (int i = 0; i < n; ++i) V[q_ + i] *= ib;
         qb = wb * ib;
     }
@@ -583,10 +616,11 @@ __device__ double lanczos_max_f32(const Lane& S, const Layout& ly, int n, double
 // entries) with its border entry returned: the previous evaluation's Ritz
 // vector (region RV, border *vb) when warm, else the stencil's
 // pseudo-random vector.
-__device__ double lanczos_inv_start(const Lane& S, const Layout& ly, int n, bool warm, const double* vb,
+__device__ double lanczos_inv_start(const Lane S, const Layout ly, int n, bool warm, const double* vb,
                                     uint64_t seed) {
     const int m = ly.m;
     double nrm2 = 0.0;
+#pragma unroll 1
     for (int i = 0; i < m; ++i) {
         double v = i < n ? (warm ? S[ly.RV + i] : unit_hash(seed * 131u + i)) : 0.0;
         S[ly.QB + i] = v;
@@ -595,6 +629,7 @@ __device__ double lanczos_inv_start(const Lane& S, const Layout& ly, int n, bool
     double qb = warm ? *vb : unit_hash(seed * 131u + n);
     nrm2 += qb * qb;
     double inrm = rsqrt(nrm2);
+#pragma unroll 1
     for (int i = 0; i < n; ++i) S[ly.QB + i] *= inrm;
     return qb * inrm;
 }
@@ -604,7 +639,7 @@ __device__ double lanczos_inv_start(const Lane& S, const Layout& ly, int n, bool
 // Phi^{-1} product is already in region Q2): returns the signed Ritz value
 // theta of largest magnitude and writes the unit Ritz vector (m entries,
 // border in *vb) to region RV.
-__device__ double lanczos_inv_ritz(const Lane& S, const Layout& ly, int n, double s, double rtol, bool warm,
+__device__ double lanczos_inv_ritz(const Lane S, const Layout ly, int n, double s, double rtol, bool warm,
                                    double qb0, bool w0_ready, double* vb, double lmax = 0.0,
                                    double acc_lo = 0.0, double acc_hi = 0.0, bool* early = nullptr) {
     const int m = ly.m, w = ly.Q2;
@@ -614,10 +649,12 @@ __device__ double lanczos_inv_ritz(const Lane& S, const Layout& ly, int n, doubl
     const int kmin = warm ? 2 : LANCZOS_KMIN;
     double beta = 0.0, prev = -1.0, ext = 0.0;
     int k = 0;
+#pragma unroll 1
     for (int j = 0; j < LANCZOS_KMAX; ++j) {
         const int qj = ly.QB + j * m, qp = ly.QB + (j - 1) * m;
         // [c; d] = A^{-1} [f; g]: c0 = Phi^{-1} f, d = (1^T c0 - g) / s, c = c0 - d u
         if (j > 0 || !w0_ready) {
+#pragma unroll 1
             for (int i = 0; i < m; i += 4) {
                 double v[4];
 #pragma unroll
@@ -628,12 +665,14 @@ __device__ double lanczos_inv_ritz(const Lane& S, const Layout& ly, int n, doubl
             chol_solve(S, ly, w);
         }
         double sp[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 1
         for (int i = 0; i < m; i += 4)
 #pragma unroll
             for (int q = 0; q < 4; ++q) sp[q] += S[w + i + q];
         double dd = ((sp[0] + sp[1]) + (sp[2] + sp[3]) - qbord[j]) / s;
         double wb = dd;
         double ap[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 1
         for (int i = 0; i < m; i += 4) {   // the loads of four elements ahead of the stores
             double v[4], x[4];
 #pragma unroll
@@ -660,6 +699,7 @@ __device__ double lanczos_inv_ritz(const Lane& S, const Layout& ly, int n, doubl
         if (j > 0) wb = fma(-beta, qbord[j - 1], wb);
         double a = fma(qbord[j], wb, (ap[0] + ap[1]) + (ap[2] + ap[3]));
         double bp[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 1
         for (int i = 0; i < m; i += 4) {
             double v[4], x[4];
 #pragma unroll
@@ -684,11 +724,13 @@ __device__ double lanczos_inv_ritz(const Lane& S, const Layout& ly, int n, doubl
         const bool last = bn <= 1e-14 * fabs(a) || j + 1 == LANCZOS_KMAX;
         if (j + 1 >= kmin - 1 || last || (early && early_accept_factor(j + 1) > 0.0)) {
             double G = 0.0;
+#pragma unroll 1
             for (int i = 0; i <= j; ++i) {
                 double r = fabs(alpha_d[i]) + (i < j ? beta_d[i] : 0.0) + (i > 0 ? beta_d[i - 1] : 0.0);
                 G = fmax(G, r);
             }
             double ig = 1.0 / G;
+#pragma unroll 1
             for (int i = 0; i <= j; ++i) {
                 al[i] = (float)(alpha_d[i] * ig);
                 float bb = (float)(beta_d[i] * ig);
@@ -711,6 +753,7 @@ __device__ double lanczos_inv_ritz(const Lane& S, const Layout& ly, int n, doubl
         beta = bn;
         const double ib = 1.0 / bn;
         const int qn = ly.QB + (j + 1) * m;
+#pragma unroll 1
         for (int i = 0; i < m; i += 4) {
             double v[4];
 #pragma unroll
@@ -724,15 +767,19 @@ __device__ double lanczos_inv_ritz(const Lane& S, const Layout& ly, int n, doubl
     double y[LANCZOS_KMAX];
     tri_eigvec(alpha_d, beta_d, k, ext, y);
     double vbr = 0.0, nv = 0.0;
+#pragma unroll 1
     for (int j = 0; j < k; ++j) vbr = fma(y[j], qbord[j], vbr);
+#pragma unroll 1
     for (int i = 0; i < m; ++i) {
         double v = 0.0;
+#pragma unroll 1
         for (int j = 0; j < k; ++j) v = fma(y[j], S[ly.QB + j * m + i], v);
         S[ly.RV + i] = v;
         nv = fma(v, v, nv);
     }
     nv = fma(vbr, vbr, nv);
     double inv = nv > 0.0 ? rsqrt(nv) : 0.0;
+#pragma unroll 1
     for (int i = 0; i < m; ++i) S[ly.RV + i] *= inv;
     *vb = vbr * inv;
     return ext;
@@ -740,13 +787,15 @@ __device__ double lanczos_inv_ritz(const Lane& S, const Layout& ly, int n, doubl
 
 // d lambda / d eps_s = v^T (dA/d eps_s) v for the unit eigenvector v in RV
 // (Hellmann-Feynman; the border of A does not depend on eps).
-__device__ double eig_derivative(const Lane& S, const Layout& ly, int n, int kernel, double eps_s) {
+__device__ double eig_derivative(const Lane S, const Layout ly, int n, int kernel, double eps_s) {
     double acc[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 1
     for (int i = 1; i < n; ++i) {
         const int base = pk(i, 0);
         const double vi = S[ly.RV + i];
         double row[4] = {0.0, 0.0, 0.0, 0.0};
         int j = 0;
+#pragma unroll 1
         for (; j + 4 <= i; j += 4) {
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
@@ -755,6 +804,7 @@ __device__ double eig_derivative(const Lane& S, const Layout& ly, int n, int ker
                 row[q] = fma(g * S[ly.R2 + base + j + q], S[ly.RV + j + q], row[q]);
             }
         }
+#pragma unroll 1
         for (; j < i; ++j) {
             double ph = S[ly.PH + base + j];
             double g = kernel == RBFFD_GAUSSIAN ? 2.0 * ph : ph * ph * ph;
@@ -776,7 +826,7 @@ __device__ double eig_derivative(const Lane& S, const Layout& ly, int n, int ker
 // With acc_hi > 0 (a learned first guess) the A^{-1} run may stop early and
 // set *early when the guess is proven acceptable (see early_accept_factor);
 // kappa is then the run's lower estimate and no Ritz vector is formed.
-__device__ double eval_kappa(const Lane& S, const Layout& ly, int n, int kernel, double eps_s, bool warm,
+__device__ double eval_kappa(const Lane S, const Layout ly, int n, int kernel, double eps_s, bool warm,
                              double* vb, double* theta_out, double* schur, uint64_t seed,
                              double acc_lo = 0.0, double acc_hi = 0.0, bool* early = nullptr) {
     double* dF = theta_out;
@@ -787,15 +837,14 @@ __device__ double eval_kappa(const Lane& S, const Layout& ly, int n, int kernel,
     // u = Phi^{-1} 1 and the A^{-1} run's first product Phi^{-1} q_0 in one
     // pass over L
     const double qb0 = lanczos_inv_start(S, ly, n, warm, vb, seed);
+#pragma unroll 1
     for (int i = 0; i < ly.m; ++i) {
         S[ly.U + i] = i < n ? 1.0 : 0.0;
         S[ly.Q2 + i] = S[ly.QB + i];
     }
-    {
-        const int R[2] = {ly.U, ly.Q2};
-        chol_solve_multi<2>(S, ly, R);
-    }
+    chol_solve_multi<2>(S, ly, ly.U, ly.Q2 - ly.U);
     double s = 0.0;
+#pragma unroll 1
     for (int i = 0; i < n; ++i) s += S[ly.U + i];
     if (!(s > 0.0)) return INFINITY;
     *schur = s;
@@ -811,34 +860,38 @@ __device__ double eval_kappa(const Lane& S, const Layout& ly, int n, int kernel,
 }
 
 // dF/dx from the Ritz vector left in RV by eval_kappa (theta = its Ritz value)
-__device__ inline double kappa_slope(const Lane& S, const Layout& ly, int n, int kernel, double eps_s,
+__device__ inline double kappa_slope(const Lane S, const Layout ly, int n, int kernel, double eps_s,
                                      double theta) {
     return -eps_s * theta * eig_derivative(S, ly, n, kernel, eps_s);
 }
 
 // [c; d] = A^{-1} [f; 0] in place on region V (first n entries)
-__device__ void aug_solve0(const Lane& S, const Layout& ly, int n, int V, double s) {
+__device__ void aug_solve0(const Lane S, const Layout ly, int n, int V, double s) {
     chol_solve(S, ly, V);
     double sum = 0.0;
+#pragma unroll 1
     for (int i = 0; i < n; ++i) sum += S[V + i];
     double d = sum / s;
+#pragma unroll 1
     for (int i = 0; i < n; ++i) S[V + i] = fma(-d, S[ly.U + i], S[V + i]);
 }
 
 // Three right-hand sides (regions V, V + m, V + 2m) solved together: every
 // element of L is loaded once for three FMAs.
-__device__ void chol_solve_x3(const Lane& S, const Layout& ly, int V) {
-    const int R[3] = {V, V + ly.m, V + 2 * ly.m};
-    chol_solve_multi<3>(S, ly, R);
+__device__ void chol_solve_x3(const Lane S, const Layout ly, int V) {
+    chol_solve_multi<3>(S, ly, V, ly.m);
 }
 
-__device__ void aug_solve0_x3(const Lane& S, const Layout& ly, int n, int V, double s) {
+__device__ void aug_solve0_x3(const Lane S, const Layout ly, int n, int V, double s) {
     const int m = ly.m;
     chol_solve_x3(S, ly, V);
+#pragma unroll 1
     for (int d = 0; d < 3; ++d) {
         double sum = 0.0;
+#pragma unroll 1
         for (int i = 0; i < n; ++i) sum += S[V + d * m + i];
         double dd = sum / s;
+#pragma unroll 1
         for (int i = 0; i < n; ++i) S[V + d * m + i] = fma(-dd, S[ly.U + i], S[V + d * m + i]);
     }
 }
@@ -848,13 +901,16 @@ __device__ void aug_solve0_x3(const Lane& S, const Layout& ly, int n, int V, dou
 //   g_d = (A^{-1} [B^d row 0; 0])[:n],  h_i = P_i g_i,
 //   v_j = sum_i psi_ij (x_i - x_j) . h_i,  w = (A^{-1} [v; 0])[:n].
 // Leaves the scaled weights (times r_s^2) in region Q0.
-__device__ void first_row_weights(const Lane& S, const Layout& ly, int n, int kernel, double eps_s, double s) {
+__device__ void first_row_weights(const Lane S, const Layout ly, int n, int kernel, double eps_s, double s) {
     const int XS = ly.XS, m = ly.m;
     const double e2 = eps_s * eps_s;
     // centre projector P_0 = I - n_0 n_0^T; rhs_d,j = psi(r_0j) [P_0 (x_0 - x_j)]_d
     double n0x = S[ly.NS], n0y = S[ly.NS + m], n0z = S[ly.NS + 2 * m];
+#pragma unroll 1
     for (int d = 0; d < 3; ++d)
+#pragma unroll 1
         for (int i = 0; i < m; ++i) S[ly.GV + d * m + i] = 0.0;
+#pragma unroll 1
     for (int j = 1; j < n; ++j) {
         double ph = S[ly.PH + pk(j, 0)];
         double ps = psi_from_phi(kernel, e2, ph);
@@ -866,6 +922,7 @@ __device__ void first_row_weights(const Lane& S, const Layout& ly, int n, int ke
     }
     aug_solve0_x3(S, ly, n, ly.GV, s);
     // h_i = P_i g_i
+#pragma unroll 1
     for (int i = 0; i < n; ++i) {
         double gx = S[ly.GV + i], gy = S[ly.GV + m + i], gz = S[ly.GV + 2 * m + i];
         double nx = S[ly.NS + i], ny = S[ly.NS + m + i], nz = S[ly.NS + 2 * m + i];
@@ -875,6 +932,7 @@ __device__ void first_row_weights(const Lane& S, const Layout& ly, int n, int ke
         S[ly.HV + 2 * m + i] = gz - nz * nd;
     }
     const int V = ly.Q0;
+#pragma unroll 1
     for (int i = 0; i < m; ++i) S[V + i] = 0.0;
     // pair (i, j), j < i: v_j += psi (x_i - x_j) . h_i ; v_i += psi (x_j - x_i) . h_j,
     // summed with psi_shape and scaled by psi_scale at the end.
@@ -883,6 +941,7 @@ __device__ void first_row_weights(const Lane& S, const Layout& ly, int n, int ke
     // Every v_j still receives the rows' contributions in row order and every
     // row sums its own in column order, so the result is the same bit for bit.
     int i = 0;
+#pragma unroll 1
     for (; i + 4 <= n; i += 4) {
         double xi[4], yi[4], zi[4], hx[4], hy[4], hz[4], vi[4];
 #pragma unroll
@@ -896,6 +955,7 @@ __device__ void first_row_weights(const Lane& S, const Layout& ly, int n, int ke
             vi[a] = 0.0;
         }
         const int r0 = pk(i, 0);   // row i + a starts at r0 + a i + a (a + 1) / 2
+#pragma unroll 1
         for (int j = 0; j < i; ++j) {
             const double xj = S[XS + j], yj = S[XS + m + j], zj = S[XS + 2 * m + j];
             const double hjx = S[ly.HV + j], hjy = S[ly.HV + m + j], hjz = S[ly.HV + 2 * m + j];
@@ -924,11 +984,13 @@ __device__ void first_row_weights(const Lane& S, const Layout& ly, int n, int ke
             S[V + i + a] += vi[a];
         }
     }
+#pragma unroll 1
     for (; i < n; ++i) {
         double xi = S[XS + i], yi = S[XS + m + i], zi = S[XS + 2 * m + i];
         double hx = S[ly.HV + i], hy = S[ly.HV + m + i], hz = S[ly.HV + 2 * m + i];
         double vi = 0.0;
         int base = pk(i, 0);
+#pragma unroll 1
         for (int j = 0; j < i; ++j) {
             double ps = psi_shape(kernel, S[ly.PH + base + j]);
             double dx = xi - S[XS + j], dy = yi - S[XS + m + j], dz = zi - S[XS + 2 * m + j];
@@ -939,10 +1001,12 @@ __device__ void first_row_weights(const Lane& S, const Layout& ly, int n, int ke
         S[V + i] += vi;
     }
     const double cs = psi_scale(kernel, e2);
+#pragma unroll 1
     for (int j = 0; j < n; ++j) S[V + j] *= cs;
     aug_solve0(S, ly, n, V, s);
 }
 
+template <int KERNEL>
 __global__ void __launch_bounds__(128, 4) search_kernel(SearchArgs A) {
     const int lane_id = threadIdx.x & 31;
     const int64_t warp_global = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
@@ -999,11 +1063,11 @@ __global__ void __launch_bounds__(128, 4) search_kernel(SearchArgs A) {
             double theta;
             const bool first_guess = learned && st.phase == PH_FIRST;
             bool early = false;
-            double k = eval_kappa(S, ly, n, A.kernel, eps_s, false, &vborder, &theta, &schur,
+            double k = eval_kappa(S, ly, n, KERNEL, eps_s, false, &vborder, &theta, &schur,
                                   (uint64_t)A.row_node[r], acc_lo, first_guess ? acc_hi : 0.0, &early);
             // the slope is needed unless a learned guess is accepted now
             const bool accept_now = first_guess && (early || (k >= acc_lo && k <= acc_hi));
-            dF = (isfinite(k) && !accept_now) ? kappa_slope(S, ly, n, A.kernel, eps_s, theta) : NAN;
+            dF = (isfinite(k) && !accept_now) ? kappa_slope(S, ly, n, KERNEL, eps_s, theta) : NAN;
             search_update(st, F_of(k, A.kT), dF, k, tol_s, A.max_evals, acc_lo, acc_hi, learned, n);
             if (st.phase == PH_DONE) {
                 // the search stopped at its last evaluated point, whose
@@ -1012,8 +1076,9 @@ __global__ void __launch_bounds__(128, 4) search_kernel(SearchArgs A) {
                 const int npad = A.gi.npad[g];
                 const int64_t off = A.gi.ell_off[g];
                 const bool valid = isfinite(st.k_ret) && schur > 0.0;
-                if (valid) first_row_weights(S, ly, n, A.kernel, exp(st.x_ret), schur);
+                if (valid) first_row_weights(S, ly, n, KERNEL, exp(st.x_ret), schur);
                 const double inv_rs2 = 1.0 / (geo.rs * geo.rs);
+#pragma unroll 1
                 for (int j = 0; j < npad; ++j) {
                     double w = (valid && j < n) ? S[ly.Q0 + j] * inv_rs2 : 0.0;
                     A.w64[ell_elem(off, npad, lr, j)] = w;
@@ -1140,7 +1205,8 @@ rbffd_status build_search(rbffd_op* op, const double* nodes, const double* norma
         const int64_t lanes = (int64_t)ls.blocks * ls.threads;
         RBFFD_CUDA_TRY(pool_alloc(&A.scratch, (size_t)lanes * ly.size * sizeof(double), st));
         A.lane_size = ly.size;
-        search_kernel<<<ls.blocks, ls.threads, 0, st>>>(A);
+        if (A.kernel == RBFFD_GAUSSIAN) search_kernel<RBFFD_GAUSSIAN><<<ls.blocks, ls.threads, 0, st>>>(A);
+        else search_kernel<RBFFD_IMQ><<<ls.blocks, ls.threads, 0, st>>>(A);
         note_launch();
         RBFFD_CUDA_TRY(cudaGetLastError());
         RBFFD_CUDA_TRY(cudaFreeAsync(A.scratch, st));

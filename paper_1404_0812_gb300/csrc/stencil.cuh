@@ -69,6 +69,7 @@ __device__ int sturm_below(const float* a, const float* b2, int k, float x) {
     int c = 0;
     float d = a[0] - x;
     if (d < 0.f) ++c;
+#pragma unroll 1
     for (int i = 1; i < k; ++i) {
         if (d == 0.f) d = -1e-30f;
         d = (a[i] - x) - b2[i - 1] / d;
@@ -79,9 +80,10 @@ __device__ int sturm_below(const float* a, const float* b2, int k, float x) {
 
 // extreme eigenvalues of T (alpha[0..k-1], beta[0..k-2], scaled into
 // [-1, 1]); returns the one of largest magnitude, signed, in double units
-__device__ double tri_extreme(const float* a, const float* b2, int k, double scale) {
+__device__ __noinline__ double tri_extreme(const float* a, const float* b2, int k, double scale) {
     float lo = -1.f, hi = 1.f;
     // top eigenvalue: count(x) < k  <=>  x <= lambda_max
+#pragma unroll 1
     for (int it = 0; it < 26; ++it) {
         float mid = 0.5f * (lo + hi);
         if (sturm_below(a, b2, k, mid) < k) lo = mid; else hi = mid;
@@ -89,6 +91,7 @@ __device__ double tri_extreme(const float* a, const float* b2, int k, double sca
     float top = 0.5f * (lo + hi);
     lo = -1.f; hi = 1.f;
     // bottom eigenvalue: count(x) >= 1  <=>  x > lambda_min
+#pragma unroll 1
     for (int it = 0; it < 26; ++it) {
         float mid = 0.5f * (lo + hi);
         if (sturm_below(a, b2, k, mid) >= 1) hi = mid; else lo = mid;
@@ -105,12 +108,14 @@ __device__ double tri_max_abs(const float* a, const float* b2, int k, double sca
 // theta: two steps of inverse iteration, each a solve with T - theta I by
 // Gaussian elimination with partial pivoting (the factor has two
 // superdiagonals after row exchanges).
-__device__ void tri_eigvec(const double* al, const double* be, int k, double theta, double* y) {
+__device__ __noinline__ void tri_eigvec(const double* al, const double* be, int k, double theta, double* y) {
     double d[LANCZOS_KMAX], du[LANCZOS_KMAX], du2[LANCZOS_KMAX], dl[LANCZOS_KMAX];
     bool sw[LANCZOS_KMAX];
     double tmax = 0.0;
+#pragma unroll 1
     for (int i = 0; i < k; ++i) tmax = fmax(tmax, fabs(al[i] - theta) + (i < k - 1 ? fabs(be[i]) : 0.0));
     const double tiny = 1e-30 * (tmax > 0.0 ? tmax : 1.0);
+#pragma unroll 1
     for (int i = 0; i < k; ++i) {
         d[i] = al[i] - theta;
         du[i] = i < k - 1 ? be[i] : 0.0;
@@ -118,6 +123,7 @@ __device__ void tri_eigvec(const double* al, const double* be, int k, double the
         du2[i] = 0.0;
         sw[i] = false;
     }
+#pragma unroll 1
     for (int i = 0; i < k - 1; ++i) {
         if (fabs(d[i]) >= fabs(dl[i])) {
             if (d[i] == 0.0) d[i] = tiny;
@@ -139,8 +145,11 @@ __device__ void tri_eigvec(const double* al, const double* be, int k, double the
         }
     }
     if (d[k - 1] == 0.0) d[k - 1] = tiny;
+#pragma unroll 1
     for (int i = 0; i < k; ++i) y[i] = 1.0;
+#pragma unroll 1
     for (int pass = 0; pass < 2; ++pass) {
+#pragma unroll 1
         for (int i = 0; i < k - 1; ++i) {
             if (sw[i]) {
                 double t = y[i];
@@ -152,10 +161,13 @@ __device__ void tri_eigvec(const double* al, const double* be, int k, double the
         }
         y[k - 1] /= d[k - 1];
         if (k > 1) y[k - 2] = (y[k - 2] - du[k - 2] * y[k - 1]) / d[k - 2];
+#pragma unroll 1
         for (int i = k - 3; i >= 0; --i) y[i] = (y[i] - du[i] * y[i + 1] - du2[i] * y[i + 2]) / d[i];
         double nrm = 0.0;
+#pragma unroll 1
         for (int i = 0; i < k; ++i) nrm = fmax(nrm, fabs(y[i]));
         double inv = nrm > 0.0 ? 1.0 / nrm : 1.0;
+#pragma unroll 1
         for (int i = 0; i < k; ++i) y[i] *= inv;
     }
 }
@@ -221,7 +233,7 @@ __device__ inline void finish(Search& s, double x, double k, int status) {
 //    noise floor of kappa (distance below xtol, step at least 0.9 of the
 //    previous one); every stop returns the evaluated x, within xtol of the
 //    root (the oracle's Brent guarantee).
-__device__ void search_update(Search& s, double f, double d, double k, double tol_s, int max_evals,
+__device__ __noinline__ void search_update(Search& s, double f, double d, double k, double tol_s, int max_evals,
                               double acc_lo, double acc_hi, bool learned, int n) {
     s.evals++;
     const double x = s.x_next;

@@ -121,6 +121,7 @@ __device__ Geo team_geometry(const Tm& C, const TeamLayout& ly, int n, bool on, 
     if (on) {
         const int c = node(0);
         const double cx = X[3 * (int64_t)c], cy = X[3 * (int64_t)c + 1], cz = X[3 * (int64_t)c + 2];
+#pragma unroll 1
         for (int j = C.l; j < n; j += T) {
             const int k = node(j);
             const double dx = X[3 * (int64_t)k] - cx, dy = X[3 * (int64_t)k + 1] - cy,
@@ -142,6 +143,7 @@ __device__ Geo team_geometry(const Tm& C, const TeamLayout& ly, int n, bool on, 
     g.mean_d = 0.0;
     const double inv = 1.0 / g.rs;
     if (on)
+#pragma unroll 1
         for (int j = C.l; j < n; j += T) {
             const double x = C.V(XV + j) * inv, y = C.V(XV + m + j) * inv, z = C.V(XV + 2 * m + j) * inv;
             C.V(XV + j) = x;
@@ -155,12 +157,15 @@ __device__ Geo team_geometry(const Tm& C, const TeamLayout& ly, int n, bool on, 
     __syncwarp();
     if (want_mean) {
         double sum = 0.0;
+#pragma unroll 1
         for (int j = 1; j < n; ++j) sum += C.V(ly.W + j);
         g.mean_d = sum / (double)(n - 1);
     }
+#pragma unroll 1
     for (int i = 0; i < n; ++i) {
         const double xi = C.V(XV + i), yi = C.V(XV + m + i), zi = C.V(XV + 2 * m + i);
         const int base = ly.R2 + pk(i, 0);
+#pragma unroll 1
         for (int j = C.l; j <= i; j += T) {
             const double dx = xi - C.V(XV + j), dy = yi - C.V(XV + m + j), dz = zi - C.V(XV + 2 * m + j);
             if (on) C.G(base + j) = dx * dx + dy * dy + dz * dz;   // 0 on the diagonal
@@ -185,12 +190,14 @@ __device__ void team_assemble(const Tm& C, const TeamLayout& ly, int n, int kern
         C.G(ly.PH + e) = v;
         if (f32) C.GF(ly.PF, e) = (float)v;
     }
+#pragma unroll 1
     for (int e = real + C.l; e < ly.P; e += T) {
         C.G(ly.L + e) = 0.0;
         C.G(ly.PH + e) = 0.0;
         if (f32) C.GF(ly.PF, e) = 0.f;
     }
     __syncwarp();
+#pragma unroll 1
     for (int i = C.l; i < ly.m; i += T) {
         const int e = pk(i, i);
         C.G(ly.L + e) = 1.0;
@@ -443,12 +450,14 @@ __device__ __noinline__ double team_tri_extreme(const Tm C, int AL, int BE, int 
     constexpr int LV = T >= 32 ? 4 : T >= 16 ? 3 : T >= 8 ? 2 : 1, HALF = T / 2, LEVELS = 26;
     // scale (Gershgorin bound)
     double G = 0.0;
+#pragma unroll 1
     for (int i = C.l; i < k; i += T) {
         const double r = fabs(C.V(AL + i)) + (i < k - 1 ? C.V(BE + i) : 0.0) + (i > 0 ? C.V(BE + i - 1) : 0.0);
         G = fmax(G, r);
     }
     G = C.team_max(G);
     const double ig = 1.0 / G;
+#pragma unroll 1
     for (int i = C.l; i < k; i += T) {
         C.VF(A32, i) = (float)(C.V(AL + i) * ig);
         const float bb = (float)(C.V(BE + i) * ig);
@@ -459,6 +468,7 @@ __device__ __noinline__ double team_tri_extreme(const Tm C, int AL, int BE, int 
     const int node = (top ? C.l : C.l - HALF) + 1;   // heap index of this lane's midpoint, 1 = the next
     const int depth = 31 - __clz(node);
     float lo = -1.f, hi = 1.f;
+#pragma unroll 1
     for (int done = 0; done < LEVELS; done += LV) {
         const int lv = min(LV, LEVELS - done);
         // this lane's midpoint: the path of its heap index from the root
@@ -471,6 +481,7 @@ __device__ __noinline__ double team_tri_extreme(const Tm C, int AL, int BE, int 
             }
         float dd = C.VF(A32, 0) - x;
         int cnt = dd < 0.f ? 1 : 0;
+#pragma unroll 1
         for (int i = 1; i < k; ++i) {
             if (dd == 0.f) dd = -1e-30f;
             dd = (C.VF(A32, i) - x) - C.VF(A32, LANCZOS_KMAX + i - 1) / dd;
@@ -479,6 +490,7 @@ __device__ __noinline__ double team_tri_extreme(const Tm C, int AL, int BE, int 
         // up: the eigenvalue lies above this midpoint (top: fewer than k below; bottom: none below)
         const unsigned votes = __ballot_sync(FULL, top ? cnt < k : cnt < 1);
         int h = 1;
+#pragma unroll 1
         for (int d = 0; d < lv; ++d) {
             const bool up = (votes >> (((top ? 0 : HALF) + h - 1) * S + C.t)) & 1u;
             const float c = 0.5f * (lo + hi);
@@ -600,9 +612,11 @@ template <typename Tm>
 __device__ double team_lanczos_start(const Tm& C, const TeamLayout& ly, int n, int q, uint64_t seed) {
     constexpr int T = Tm::T;
     const int m = ly.m;
+#pragma unroll 1
     for (int i = C.l; i < m; i += T) C.V(q + i) = i < n ? unit_hash(seed * 131u + i) : 0.0;
     __syncwarp();
     double nrm2 = 0.0;
+#pragma unroll 1
     for (int i = 0; i < m; ++i) {
         const double v = C.V(q + i);
         nrm2 += v * v;
@@ -611,6 +625,7 @@ __device__ double team_lanczos_start(const Tm& C, const TeamLayout& ly, int n, i
     nrm2 += qb * qb;
     const double inrm = rsqrt(nrm2);
     __syncwarp();
+#pragma unroll 1
     for (int i = C.l; i < n; i += T) C.V(q + i) *= inrm;
     __syncwarp();
     return qb * inrm;
@@ -624,6 +639,7 @@ __device__ __noinline__ void team_ritz_vector(const Tm C, int m, int k, double e
     const int RV = ly.G + 2 * m;
     {
         double al[LANCZOS_KMAX], be[LANCZOS_KMAX], y[LANCZOS_KMAX];
+#pragma unroll 1
         for (int i = 0; i < k; ++i) {
             al[i] = C.V(ly.AL + i);
             be[i] = C.V(ly.BE + i);
@@ -631,18 +647,23 @@ __device__ __noinline__ void team_ritz_vector(const Tm C, int m, int k, double e
         tri_eigvec(al, be, k, ext, y);
         __syncwarp();
         if (C.l == 0)
+#pragma unroll 1
             for (int i = 0; i < k; ++i) C.V(ly.Y + i) = y[i];
     }
     __syncwarp();
     double vbr = 0.0;
+#pragma unroll 1
     for (int j = 0; j < k; ++j) vbr = fma(C.V(ly.Y + j), C.V(ly.QBD + j), vbr);
+#pragma unroll 1
     for (int i = C.l; i < m; i += T) {
         double v = 0.0;
+#pragma unroll 1
         for (int j = 0; j < k; ++j) v = fma(C.V(ly.Y + j), C.G(ly.QB + j * m + i), v);
         C.V(RV + i) = v;
     }
     __syncwarp();
     double nv = 0.0;
+#pragma unroll 1
     for (int i = 0; i < m; ++i) {
         const double v = C.V(RV + i);
         nv = fma(v, v, nv);
@@ -650,6 +671,7 @@ __device__ __noinline__ void team_ritz_vector(const Tm C, int m, int k, double e
     nv = fma(vbr, vbr, nv);
     const double inv = nv > 0.0 ? rsqrt(nv) : 0.0;
     __syncwarp();
+#pragma unroll 1
     for (int i = C.l; i < m; i += T) C.V(RV + i) *= inv;
     __syncwarp();
 }
@@ -913,6 +935,7 @@ __global__ void __launch_bounds__(32) team_search_kernel(SearchArgs A, int refil
     const Tm C = make_team<Tm>(A.scratch, blockIdx.x, A.lane_size, team_smem);
     const double acc_lo = A.acc_lo * A.kT * (1.0 + ACCEPT_MARGIN);
     const double acc_hi = A.acc_hi * A.kT * (1.0 - ACCEPT_MARGIN);
+#pragma unroll 1
     for (int g = 0; g < A.gi.ngroups; ++g) {
         const int n = A.gi.n[g], m = A.gi.npad[g];
         const TeamLayout ly = team_layout(m, true);
@@ -973,6 +996,7 @@ __global__ void __launch_bounds__(32) team_search_kernel(SearchArgs A, int refil
             const bool spd = team_cholesky(C, m, true);
             const double lmax = team_lanczos_max(C, m, n, LANCZOS_RTOL);
             const double qb0 = team_lanczos_start(C, ly, n, ly.G, (uint64_t)node);
+#pragma unroll 1
             for (int i = C.l; i < m; i += T) C.V(ly.W + i) = C.V(ly.G + i);
             const double s = team_schur<true>(C, ly, true, n);
             const bool sound = spd && s > 0.0;
@@ -999,6 +1023,7 @@ __global__ void __launch_bounds__(32) team_search_kernel(SearchArgs A, int refil
                 if (finished) {
                     const bool valid = isfinite(st.k_ret) && schur > 0.0;
                     const double inv_rs2 = 1.0 / (geo.rs * geo.rs);
+#pragma unroll 1
                     for (int j = C.l; j < m; j += T) {
                         const double w = (valid && j < n) ? C.V(ly.W + j) * inv_rs2 : 0.0;
                         const int64_t e = ell_elem(off, m, lr, j);
@@ -1031,11 +1056,13 @@ __global__ void __launch_bounds__(32) team_weights_kernel(TeamWeightArgs B) {
     const Tm C = make_team<Tm>(A.scratch, blockIdx.x, A.lane_size, team_smem);
     const bool dense = B.stencils != nullptr;
     const int groups = dense ? 1 : A.gi.ngroups;
+#pragma unroll 1
     for (int g = 0; g < groups; ++g) {
         const int n = dense ? B.n : A.gi.n[g], m = (n + 3) / 4 * 4;
         const TeamLayout ly = team_layout(m, false);
         const int64_t off = dense ? 0 : A.gi.ell_off[g], row0 = dense ? 0 : A.gi.row_begin[g];
         const int64_t cnt = dense ? B.rows : A.gi.row_begin[g + 1] - row0;
+#pragma unroll 1
         for (int64_t first = (int64_t)blockIdx.x * S; first < cnt; first += (int64_t)gridDim.x * S) {
             const int64_t lr = first + C.t;
             const bool have = lr < cnt;
@@ -1043,6 +1070,7 @@ __global__ void __launch_bounds__(32) team_weights_kernel(TeamWeightArgs B) {
             const int32_t* row = dense ? B.stencils + (have ? lr : 0) * n : nullptr;
             if (dense) {
                 if (have)
+#pragma unroll 1
                     for (int j = C.l; j < n; j += T) ok = ok && row[j] >= 0 && (int64_t)row[j] < B.N;
                 // every lane of the team has to agree
                 const unsigned bad = __ballot_sync(FULL, have && !ok);
@@ -1066,8 +1094,10 @@ __global__ void __launch_bounds__(32) team_weights_kernel(TeamWeightArgs B) {
                 if (!dense) A.status[node] = RBFFD_STENCIL_SINGULAR;
             }
             if (have && dense) {
+#pragma unroll 1
                 for (int j = C.l; j < n; j += T) A.w64[lr * n + j] = ok ? C.V(ly.W + j) * inv_rs2 : NAN;
             } else if (have) {
+#pragma unroll 1
                 for (int j = C.l; j < m; j += T) {
                     const double w = ok && j < n ? C.V(ly.W + j) * inv_rs2 : 0.0;
                     const int64_t e = ell_elem(off, m, lr, j);
@@ -1190,6 +1220,7 @@ rbffd_status team_weights(TeamWeightArgs B, int64_t scratch_doubles, cudaStream_
         mmax = (B.n + 3) / 4 * 4;
     } else {
         rows = B.w.gi.row_begin[B.w.gi.ngroups];
+#pragma unroll 1
         for (int g = 0; g < B.w.gi.ngroups; ++g) mmax = std::max(mmax, B.w.gi.npad[g]);
     }
     int T = std::max(8, team_weight_lanes(mmax, rows));
