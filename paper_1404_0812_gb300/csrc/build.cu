@@ -67,8 +67,8 @@ namespace {
 // store), and the kernel function is a template argument: 192 KB, 385 ms.  Only
 // the solves' chunk loops keep the compiler's unrolling (404 ms without, 397
 // with, before the other changes).  For the same reason variants with more code
-// were slower: the solves' next chunk fetched ahead 461 ms, 168 registers for
-// it on three blocks per SM 449 ms.
+// were slower: the solves' next chunk fetched ahead 461 ms (392 on the smaller
+// code, its registers spill), 168 registers for it on three blocks per SM 449 ms.
 // ---------------------------------------------------------------------------
 struct Lane {
     double* p;   // points at element 0 of this lane
