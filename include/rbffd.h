@@ -160,9 +160,9 @@ typedef struct {
     int model;          /* reaction kinetics, see coef below */
     int nspecies;       /* 1 (u only, heat/forced diffusion) or 2 (u, v) */
     int dtype;          /* RBFFD_F32 or RBFFD_F64 state and arithmetic
-                           (float32 dot products accumulate in float64, or,
-                           for large operators, in compensated float32 --
-                           Ogita-Rump-Oishi Dot2 -- of the same accuracy) */
+                           (float32 dot products are summed at least as
+                           accurately as in float64, with Ogita-Rump-Oishi
+                           DotK in scaled float32, whatever the fields' scale) */
     double dt;          /* time step */
     double delta_u, delta_v;   /* diffusion coefficients */
     double coef[8];     /* LINEAR: lu, lv.  SCHNAKENBERG: a, b, gamma.

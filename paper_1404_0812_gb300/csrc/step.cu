@@ -16,6 +16,7 @@
 #include "common.cuh"
 
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <type_traits>
 #include <vector>
@@ -29,6 +30,7 @@ struct SpeciesState {
     double bnorm, limit2;              // |b|; squared norm at which the residual has converged
     double rho, rho_prev, alpha, omega, res2;   // committed: (r-hat, r), ..., |r|^2
     double beta, alpha_n, omega_n;     // the current iteration's scalars
+    int e0, e;                         // exponents of r-hat and of the iteration's vectors in the sums
     int active, fail, iters, zero;
     int actA, actB, early, actE;       //   and its decisions
 };
@@ -196,50 +198,153 @@ __device__ __forceinline__ StepCoef<T> step_coef(const Args<T>& a) {
     return step_coef_at(a, *((volatile int*)(a.flags + 2)), *((volatile int*)(a.flags + 3)));
 }
 
-// Dot-product accumulators.  The phase kernels sum float32 products with the compensated dot product Dot2 (Ogita, Rump & Oishi, "Accurate sum
-// and dot product", SIAM J. Sci. Comput. 26 (2005), Algorithm 5.3): each
-// product a b split exactly into p + e by an FMA (TwoProduct), the running
-// sum carried by Knuth's error-free TwoSum, the rounding errors of both
-// summed apart and added at the end.  The result is as accurate as the sum
-// computed in twice the working precision, with float32 instructions only
-// (the float64 pipe of this GPU is a small fraction of the float32 one).
-struct Dot2 {
-    float hi, lo;
+// Dot-product accumulators.  Float64 sums and those of a right-hand side are
+// float64.  The float32 sums of an iteration are carried in three float32 values
+// by the dot product DotK with K = 3 (Ogita, Rump & Oishi, "Accurate sum and dot
+// product", SIAM J. Sci. Comput. 26 (2005), Algorithm 5.10, the last level a plain
+// sum): each product a b split exactly into p + e by an FMA (TwoProduct), sums by
+// Knuth's error-free TwoSum, the errors of the second level added at the end.  The
+// rounding error is about 2^-72 of the sum of |a b|, below that of a float64 sum,
+// with float32 instructions only: the float64 unit takes a warp 64 clocks for an
+// FMA (two species, 1M rows: 5.28 ms a step with float64 sums, 5.06 with these;
+// 500k rows of n = 17: 986 and 902 us; pairs of float32 values, about 2^-48 and not
+// scaled, took 5.06 ms and 892 us).
+// TwoProduct is exact, and the sum finite, while the terms stay within float32's
+// range, so the factors are scaled to about one by powers of two (exactly).
+struct Dot3 {
+    float h, m, l;
 };
-__device__ __forceinline__ void acc_zero(Dot2& s) { s.hi = s.lo = 0.f; }
+__device__ __forceinline__ float two_sum(float a, float b, float& err) {
+    const float x = __fadd_rn(a, b), z = __fsub_rn(x, a);
+    err = __fadd_rn(__fsub_rn(a, __fsub_rn(x, z)), __fsub_rn(b, z));
+    return x;
+}
+__device__ __forceinline__ void acc_zero(Dot3& s) { s.h = s.m = s.l = 0.f; }
 __device__ __forceinline__ void acc_zero(double& s) { s = 0.0; }
-__device__ __forceinline__ void acc_add(Dot2& s, float a, float b) {
+__device__ __forceinline__ void acc_pair(Dot3& s, float p, float e) {
+    float t, u, w;
+    s.h = two_sum(s.h, p, t);
+    s.m = two_sum(s.m, e, u);
+    s.m = two_sum(s.m, t, w);
+    s.l = __fadd_rn(s.l, __fadd_rn(u, w));
+}
+__device__ __forceinline__ void acc_add(Dot3& s, float a, float b) {
     const float p = __fmul_rn(a, b);
-    const float e = __fmaf_rn(a, b, -p);                    // a b = p + e exactly
-    const float x = __fadd_rn(s.hi, p);
-    const float z = __fsub_rn(x, s.hi);
-    const float t = __fadd_rn(__fsub_rn(s.hi, __fsub_rn(x, z)), __fsub_rn(p, z));   // s.hi + p = x + t exactly
-    s.hi = x;
-    s.lo = __fadd_rn(s.lo, __fadd_rn(t, e));
+    acc_pair(s, p, __fmaf_rn(a, b, -p));   // a b = p + e exactly
 }
-__device__ __forceinline__ void acc_add(double& s, float a, float b) { s += (double)a * b; }
 __device__ __forceinline__ void acc_add(double& s, double a, double b) { s += a * b; }
-__device__ __forceinline__ double acc_value(const Dot2& s) { return (double)s.hi + (double)s.lo; }
-__device__ __forceinline__ double acc_value(double s) { return s; }
-__device__ __forceinline__ Dot2 acc_merge(const Dot2& u, const Dot2& v) {
-    const float x = __fadd_rn(u.hi, v.hi), z = __fsub_rn(x, u.hi);
-    const float t = __fadd_rn(__fsub_rn(u.hi, __fsub_rn(x, z)), __fsub_rn(v.hi, z));   // u.hi + v.hi = x + t exactly
-    return Dot2{x, __fadd_rn(t, __fadd_rn(u.lo, v.lo))};
-}
-__device__ __forceinline__ double acc_merge(double u, double v) { return u + v; }
-__device__ __forceinline__ Dot2 acc_shfl_down(const Dot2& s, int o) {
-    return Dot2{__shfl_down_sync(0xffffffffu, s.hi, o), __shfl_down_sync(0xffffffffu, s.lo, o)};
-}
-__device__ __forceinline__ double acc_shfl_down(double s, int o) { return __shfl_down_sync(0xffffffffu, s, o); }
 
-// the phase kernels' accumulator for state type T
+// the exponent by which values of about 2^e are scaled: 2^-e and its inverse are
+// normal float32 numbers
+__device__ __forceinline__ int unit_exp(int e) { return min(max(e, -126), 126); }
+__device__ __forceinline__ float unit_scale(int e) { return __int_as_float((127 - e) << 23); }   // 2^-e
+
+// The sum of a warp's values, in fixed point: each value is cut into three integers
+// of 20 bits (by adding and subtracting 1.5 2^23), relative to the largest of them
+// all, and integers are summed exactly by warp reductions.  What is cut off is below
+// 2^-55 of the largest value, a float64 rounding's share.  (With a shuffle tree of
+// Dot3 values, 40k torus, two species: 84.5 us a step, with this 80.)
+struct Fixed {
+    long long n;   // value n 2^e
+    int e;
+};
+__device__ __forceinline__ Fixed warp_sum(const Dot3& s, int e) {
+    const float x[3] = {s.h, s.m, s.l};
+    unsigned m = 0;   // largest magnitude (the bits order like integers)
+#pragma unroll
+    for (int i = 0; i < 3; ++i) m = max(m, __float_as_uint(x[i]) & 0x7fffffffu);
+    m = __reduce_max_sync(0xffffffffu, m);
+    const int E = max((int)(m >> 23) - 127, -110);
+    const float S = __int_as_float((127 + 15 - E) << 23), R = 12582912.f;   // to below 2^16; 1.5 2^23
+    int n[3] = {0, 0, 0};
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        float y = x[i], f = S;
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            const float t = __fmaf_rn(y, f, R);
+            n[q] += __float_as_int(t) - __float_as_int(R);
+            y = __fmaf_rn(y, f, -__fsub_rn(t, R));   // exactly what is left
+            f = 1048576.f;
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < 3; ++q) n[q] = __reduce_add_sync(0xffffffffu, n[q]);
+    Fixed r;
+    r.n = ((long long)n[0] << 40) + ((long long)n[1] << 20) + n[2];
+    r.e = m < 0x7f800000u ? e + E - 55 : INT_MAX;   // infinite or NaN
+    return r;
+}
+__device__ __forceinline__ double fixed_value(const Fixed& f) {
+    if (f.e == INT_MAX) return NAN;
+    // n as a float64 (its halves placed in the mantissas of 2^84 and 2^52)
+    const double x = (__hiloint2double(0x45300000, (int)(f.n >> 32) ^ (int)0x80000000) - 19342822341709703277445120.0) +
+                     __hiloint2double(0x43300000, (int)f.n);
+    return f.n == 0 ? 0.0 : __hiloint2double(__double2hiint(x) + (f.e << 20), __double2loint(x));
+}
+
+// Squared norms of two vectors whose scale is not known yet: float32 threads scale
+// by their largest element so far, and a warp agrees on one exponent at the end.
+struct Norms64 {
+    double b = 0.0, r = 0.0;
+    __device__ void add(double x, double y) {
+        acc_add(b, x, x);
+        acc_add(r, y, y);
+    }
+    __device__ int finish(double& sb, double& sr) const {
+        sb = b;
+        sr = r;
+        return 0;
+    }
+};
+struct Norms32 {
+    Dot3 b{0.f, 0.f, 0.f}, r{0.f, 0.f, 0.f};
+    int e = -126;
+    // |g| <= 1: the sums at another exponent (what underflows is far below them)
+    __device__ static void rescale(Dot3& s, float g) {
+        s.h *= g;
+        s.m *= g;
+        s.l *= g;
+    }
+    __device__ void to(int en) {
+        const float g = en - e < 63 ? unit_scale(2 * (en - e)) : 0.f;
+        rescale(b, g);
+        rescale(r, g);
+        e = en;
+    }
+    __device__ void add(float x, float y) {
+        const unsigned m = max(__float_as_uint(x) & 0x7fffffffu, __float_as_uint(y) & 0x7fffffffu);
+        const int en = unit_exp((int)(m >> 23) - 127);
+        if (en > e + 8) to(en);
+        const float f = unit_scale(e), xs = x * f, ys = y * f;
+        acc_add(b, xs, xs);
+        acc_add(r, ys, ys);
+    }
+    __device__ int finish(Dot3& sb, Dot3& sr) {
+        to(__reduce_max_sync(0xffffffffu, e));
+        sb = b;
+        sr = r;
+        return e;
+    }
+};
+
+// the steps' accumulators for state type T, and their factors' scaling
 template <typename T>
 struct PhaseAcc {
     using type = double;
+    using norms = Norms64;
+    __device__ static double scaled(double x, float) { return x; }
+    __device__ static int exp_of(double) { return 0; }
 };
 template <>
 struct PhaseAcc<float> {
-    using type = Dot2;
+    using type = Dot3;
+    using norms = Norms32;
+    __device__ static float scaled(float x, float f) { return x * f; }
+    // the exponent of a vector by its squared norm
+    __device__ static int exp_of(double norm2) {
+        return unit_exp((((__double2hiint(norm2) >> 20) & 0x7ff) - 1023) >> 1);
+    }
 };
 
 // kinetics and right-hand side b of the step's SBDF order at node i (values
@@ -302,9 +407,9 @@ __device__ __forceinline__ void rhs_values(const Args<T>& a, const StepCoef<T>& 
 // phase R of one row (node i, with (L u)_i = Lu, (L v)_i = Lv): the right-hand
 // side, r0 = b - A u, r-hat = r0, p = q = 0; accumulates |b|^2, |r0|^2 per
 // species into d[0..1], d[2..3]
-template <typename T, typename A>
+template <typename T>
 __device__ __forceinline__ void rhs_row(const Args<T>& a, const StepCoef<T>& kc, int64_t i, T Lu, T Lv,
-                                        A (&d)[4]) {
+                                        typename PhaseAcc<T>::norms (&d)[2]) {
     const bool two = a.ns == 2;
     const T ui = a.u[i], vi = two ? a.v[i] : T(0);
     T bu, bv;
@@ -315,8 +420,7 @@ __device__ __forceinline__ void rhs_row(const Args<T>& a, const StepCoef<T>& kc,
     V(a, 0, VRH)[i] = ru;
     V(a, 0, VP)[i] = T(0);
     V(a, 0, VQ)[i] = T(0);
-    acc_add(d[0], bu, bu);
-    acc_add(d[1], ru, ru);
+    d[0].add(bu, ru);
     if (two) {
         const T rv = bv - (kc.c0 * vi - kc.k1 * Lv);
         V(a, 1, VB)[i] = bv;
@@ -324,8 +428,7 @@ __device__ __forceinline__ void rhs_row(const Args<T>& a, const StepCoef<T>& kc,
         V(a, 1, VRH)[i] = rv;
         V(a, 1, VP)[i] = T(0);
         V(a, 1, VQ)[i] = T(0);
-        acc_add(d[2], bv, bv);
-        acc_add(d[3], rv, rv);
+        d[1].add(bv, rv);
     }
 }
 
@@ -453,46 +556,46 @@ __device__ __forceinline__ void row_species(const Args<T>& a, int64_t r, int64_t
 // other blocks).  Only one warp per sum does float64 arithmetic: one float64
 // warp instruction takes the SM 16 clocks, and a float64 shuffle tree in every
 // warp cost the vector phases more than their memory traffic (two species,
-// float32, 1M rows: 5.63 -> 5.07 ms a step).
-template <int K, int NTB, typename A>
-__device__ const double* phase_reduce(const A (&v)[K], double* pp, unsigned int* ticket) {
-    constexpr bool PAIRS = sizeof(A) == sizeof(Dot2) && !std::is_same<A, double>::value;
-    __shared__ A sh[K][PAIRS ? NTB / 32 : NTB];
+// float32, 1M rows: 5.63 -> 5.06 ms a step).  exp_of(k): the exponent of float32
+// sum k (warp_sum).
+template <int K, int NTB, typename A, typename F>
+__device__ const double* phase_reduce(const A (&v)[K], double* pp, unsigned int* ticket, F exp_of) {
+    using F32 = std::is_same<A, Dot3>;
+    constexpr int NW = NTB / 32;
+    using Shared = typename std::conditional<F32::value, Fixed, double>::type;
+    __shared__ Shared sh[K][F32::value ? NW : NTB];
     __shared__ double tot[K];
     __shared__ int last;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    static_assert(K <= NTB / 32, "a warp per sum");
-    if (PAIRS) {   // float32 pairs: a shuffle tree per warp, then one thread per sum over the warps
+    static_assert(K <= NW && NW <= 32, "a warp per sum");
+    double t = 0.0;
+    if constexpr (F32::value) {   // a warp's sum in fixed point, then one warp per sum over the warps
 #pragma unroll
         for (int k = 0; k < K; ++k) {
-            A x = v[k];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) x = acc_merge(x, acc_shfl_down(x, o));
+            const Fixed x = warp_sum(v[k], exp_of(k));
             if (lane == 0) sh[k][wid] = x;
         }
         __syncthreads();
-        if (threadIdx.x < K) {
-            A t = sh[threadIdx.x][0];
+        if (wid < K) {
+            if (lane < NW) t = fixed_value(sh[wid][lane]);
 #pragma unroll
-            for (int w = 1; w < NTB / 32; ++w) t = acc_merge(t, sh[threadIdx.x][w]);
-            pp[(int64_t)blockIdx.x * 8 + threadIdx.x] = acc_value(t);
-            __threadfence();
+            for (int o = NW / 2; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
         }
-    } else {       // float64: one warp per sum over the threads' values
+    } else {                      // float64: one warp per sum over the threads' values
 #pragma unroll
         for (int k = 0; k < K; ++k) sh[k][threadIdx.x] = v[k];
         __syncthreads();
         if (wid < K) {
-            A t = sh[wid][lane];
+            t = sh[wid][lane];
 #pragma unroll
-            for (int w = 1; w < NTB / 32; ++w) t = acc_merge(t, sh[wid][w * 32 + lane]);
+            for (int w = 1; w < NW; ++w) t += sh[wid][w * 32 + lane];
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) t = acc_merge(t, acc_shfl_down(t, o));
-            if (lane == 0) {
-                pp[(int64_t)blockIdx.x * 8 + wid] = acc_value(t);
-                __threadfence();
-            }
+            for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
         }
+    }
+    if (wid < K && lane == 0) {
+        pp[(int64_t)blockIdx.x * 8 + wid] = t;
+        __threadfence();
     }
     __syncthreads();
     if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == gridDim.x - 1;
@@ -538,8 +641,7 @@ template <typename T>
 __global__ void __launch_bounds__(PT, PT_MINB) phase_R(Args<T> a) {
     const StepCoef<T> kc = step_coef(a);
     const bool two = a.ns == 2;
-    typename PhaseAcc<T>::type d[4];
-    for (auto& x : d) acc_zero(x);
+    typename PhaseAcc<T>::norms d[2];
     for (int64_t r = blockIdx.x * (int64_t)PT + threadIdx.x; r < a.N; r += (int64_t)gridDim.x * PT) {
         const int64_t i = a.row_node[r];
         T Lu, Lv;
@@ -547,7 +649,10 @@ __global__ void __launch_bounds__(PT, PT_MINB) phase_R(Args<T> a) {
         rhs_row(a, kc, i, Lu, Lv, d);
     }
     PhaseCtl* c = a.ctl;
-    const double* tot = phase_reduce<4, PT>(d, a.pp, &c->ticket);
+    typename PhaseAcc<T>::type v[4];
+    int e[2];
+    for (int k = 0; k < 2; ++k) e[k] = d[k].finish(v[2 * k], v[2 * k + 1]);
+    const double* tot = phase_reduce<4, PT>(v, a.pp, &c->ticket, [&](int j) { return 2 * e[j >> 1]; });
     if (tot && threadIdx.x < 2) {
         const int k = threadIdx.x;
         const bool exists = k == 0 || two;
@@ -555,8 +660,10 @@ __global__ void __launch_bounds__(PT, PT_MINB) phase_R(Args<T> a) {
         z.bnorm = sqrt(tot[2 * k]);
         z.limit2 = (a.tol * z.bnorm) * (a.tol * z.bnorm);
         z.rho = z.res2 = tot[2 * k + 1];   // (r-hat, r0) = |r0|^2
-        z.rho_prev = z.alpha = z.omega = 1.0;
+        z.rho_prev = z.rho;   // beta = 1 (p = q = 0: any finite value)
+        z.alpha = z.omega = 1.0;
         z.alpha_n = z.omega_n = 0.0;
+        z.e0 = z.e = PhaseAcc<T>::exp_of(z.rho);
         z.active = exists && z.bnorm != 0.0 && !(sqrt(z.res2) / z.bnorm <= a.tol);
         z.fail = z.iters = 0;
         z.zero = exists && z.bnorm == 0.0;   // b = 0: x = 0
@@ -645,8 +752,11 @@ __global__ void __launch_bounds__(PT, PT_MINB) phase_B(Args<T> a) {
     PhaseCtl* c = a.ctl;
     const bool a0 = c->s[0].actA, a1 = a.ns == 2 && c->s[1].actA;
     const StepCoef<T> kc = step_coef(a);
-    typename PhaseAcc<T>::type d[2];
+    using PA = PhaseAcc<T>;
+    typename PA::type d[2];
     for (auto& x : d) acc_zero(x);
+    const int e0[2] = {c->s[0].e0, c->s[1].e0}, e[2] = {c->s[0].e, c->s[1].e};
+    const float f0[2] = {unit_scale(e0[0]), unit_scale(e0[1])}, f[2] = {unit_scale(e[0]), unit_scale(e[1])};
     const int64_t S = (int64_t)gridDim.x * PT, Np = (a.N + 31) & ~(int64_t)31;
     for (int64_t k = blockIdx.x * (int64_t)PT + threadIdx.x; (a0 || a1) && k < Np; k += S) {
         const int64_t r = B_BACK ? back_row(k, Np) : k;
@@ -658,15 +768,15 @@ __global__ void __launch_bounds__(PT, PT_MINB) phase_B(Args<T> a) {
         if (a0) {
             const T q = kc.c0 * V(a, 0, VP)[i] - kc.k0 * L0;
             V(a, 0, VQ)[i] = q;
-            acc_add(d[0], V(a, 0, VRH)[i], q);
+            acc_add(d[0], PA::scaled(V(a, 0, VRH)[i], f0[0]), PA::scaled(q, f[0]));
         }
         if (a1) {
             const T q = kc.c0 * V(a, 1, VP)[i] - kc.k1 * L1;
             V(a, 1, VQ)[i] = q;
-            acc_add(d[1], V(a, 1, VRH)[i], q);
+            acc_add(d[1], PA::scaled(V(a, 1, VRH)[i], f0[1]), PA::scaled(q, f[1]));
         }
     }
-    const double* tot = phase_reduce<2, PT>(d, a.pp, &c->ticket);
+    const double* tot = phase_reduce<2, PT>(d, a.pp, &c->ticket, [&](int k) { return e0[k] + e[k]; });
     if (tot && threadIdx.x < 2) {
         const int k = threadIdx.x;
         SpeciesState& z = c->s[k];
@@ -681,12 +791,16 @@ __global__ void __launch_bounds__(PT, PT_MINB) phase_B(Args<T> a) {
 template <typename T>
 __global__ void __launch_bounds__(PV, PV_BPS) phase_C(Args<T> a) {
     PhaseCtl* c = a.ctl;
-    typename PhaseAcc<T>::type d[2];
+    using PA = PhaseAcc<T>;
+    typename PA::type d[2];
     for (auto& x : d) acc_zero(x);
     const int64_t S = (int64_t)gridDim.x * PV, t0 = blockIdx.x * (int64_t)PV + threadIdx.x;
-    for (int k = 0; k < a.ns; ++k) {
-        if (!c->s[k].actB) continue;
+    const int e[2] = {c->s[0].e, c->s[1].e};
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        if (k >= a.ns || !c->s[k].actB) continue;
         const T alpha = (T)c->s[k].alpha_n;
+        const float f = unit_scale(e[k]);
         const T* __restrict__ r = V(a, k, VR);
         const T* __restrict__ q = V(a, k, VQ);
         T* __restrict__ sv = V(a, k, VS);
@@ -698,9 +812,9 @@ __global__ void __launch_bounds__(PV, PV_BPS) phase_C(Args<T> a) {
 #pragma unroll
                 for (int u = 0; u < VG; ++u)
                     if (g0 + u * S < G) {
-                        const int64_t e = 4 * (g0 + u * S);
-                        ld4v(r + e, rv[u]);
-                        ld4v(q + e, qv[u]);
+                        const int64_t i4 = 4 * (g0 + u * S);
+                        ld4v(r + i4, rv[u]);
+                        ld4v(q + i4, qv[u]);
                     }
 #pragma unroll
                 for (int u = 0; u < VG; ++u)
@@ -708,7 +822,8 @@ __global__ void __launch_bounds__(PV, PV_BPS) phase_C(Args<T> a) {
 #pragma unroll
                         for (int j = 0; j < 4; ++j) {
                             rv[u][j] = rv[u][j] - alpha * qv[u][j];
-                            acc_add(d[k], rv[u][j], rv[u][j]);
+                            const T y = PA::scaled(rv[u][j], f);
+                            acc_add(d[k], y, y);
                         }
                         st4v(sv + 4 * (g0 + u * S), rv[u]);
                     }
@@ -718,10 +833,10 @@ __global__ void __launch_bounds__(PV, PV_BPS) phase_C(Args<T> a) {
         for (; i < a.N; i += S) {
             const T x = r[i] - alpha * q[i];
             sv[i] = x;
-            acc_add(d[k], x, x);
+            acc_add(d[k], PA::scaled(x, f), PA::scaled(x, f));
         }
     }
-    const double* tot = phase_reduce<2, PV>(d, a.pp, &c->ticket);
+    const double* tot = phase_reduce<2, PV>(d, a.pp, &c->ticket, [&](int k) { return 2 * e[k]; });
     if (tot && threadIdx.x < 2) {
         SpeciesState& z = c->s[threadIdx.x];
         const int early = z.actB && tot[threadIdx.x] <= z.limit2;
@@ -739,15 +854,19 @@ __global__ void __launch_bounds__(PT, PT_MINB) phase_D(Args<T> a) {
     const bool e0 = c->s[0].early, e1 = two && c->s[1].early;
     const bool b0 = c->s[0].actB, b1 = two && c->s[1].actB;
     const bool need0 = b0 && !e0, need1 = b1 && !e1;
-    typename PhaseAcc<T>::type d[4];
+    using PA = PhaseAcc<T>;
+    typename PA::type d[4];
     for (auto& x : d) acc_zero(x);
+    const int e[2] = {c->s[0].e, c->s[1].e};
+    const float f[2] = {unit_scale(e[0]), unit_scale(e[1])};
     for (int64_t r = blockIdx.x * (int64_t)PT + threadIdx.x; (b0 || b1) && r < a.N; r += (int64_t)gridDim.x * PT) {
         const int64_t i = a.row_node[r];
         T L0 = T(0), L1 = T(0);
         if (need0 || need1)
             row_species(a, r, r + (int64_t)gridDim.x * PT, (const T*)V(a, 0, VS), (const T*)V(a, 1, VS), need0, need1, L0,
                         L1);
-        for (int k = 0; k < a.ns; ++k) {
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {   // (e1 and b1 only with two species)
             T* x = k == 0 ? a.u : a.v;
             if (k == 0 ? e0 : e1) {
                 x[i] += (T)c->s[k].alpha_n * V(a, k, VP)[i];
@@ -755,12 +874,13 @@ __global__ void __launch_bounds__(PT, PT_MINB) phase_D(Args<T> a) {
                 const T sv = V(a, k, VS)[i];
                 const T t = kc.c0 * sv - (k == 0 ? kc.k0 * L0 : kc.k1 * L1);
                 V(a, k, VT)[i] = t;
-                acc_add(d[2 * k], t, sv);
-                acc_add(d[2 * k + 1], t, t);
+                const T ts = PA::scaled(t, f[k]);
+                acc_add(d[2 * k], ts, PA::scaled(sv, f[k]));
+                acc_add(d[2 * k + 1], ts, ts);
             }
         }
     }
-    const double* tot = phase_reduce<4, PT>(d, a.pp, &c->ticket);
+    const double* tot = phase_reduce<4, PT>(d, a.pp, &c->ticket, [&](int j) { return 2 * e[j >> 1]; });
     if (tot && threadIdx.x < 2) {
         const int k = threadIdx.x;
         SpeciesState& z = c->s[k];
@@ -782,12 +902,16 @@ __device__ __forceinline__ void e_update(T alpha, T omega, T& x, T p, T s, T t, 
 template <typename T>
 __global__ void __launch_bounds__(PV, PV_BPS) phase_E(Args<T> a) {
     PhaseCtl* c = a.ctl;
-    typename PhaseAcc<T>::type d[4];
+    using PA = PhaseAcc<T>;
+    typename PA::type d[4];
     for (auto& x : d) acc_zero(x);
     const int64_t S = (int64_t)gridDim.x * PV, t0 = blockIdx.x * (int64_t)PV + threadIdx.x;
-    for (int k = 0; k < a.ns; ++k) {
-        if (!c->s[k].actE) continue;
+    const int e0[2] = {c->s[0].e0, c->s[1].e0}, e[2] = {c->s[0].e, c->s[1].e};
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        if (k >= a.ns || !c->s[k].actE) continue;
         const T alpha = (T)c->s[k].alpha_n, omega = (T)c->s[k].omega_n;
+        const float f0 = unit_scale(e0[k]), f = unit_scale(e[k]);
         T* __restrict__ x = k == 0 ? a.u : a.v;
         const T* __restrict__ p = V(a, k, VP);
         const T* __restrict__ sv = V(a, k, VS);
@@ -798,21 +922,22 @@ __global__ void __launch_bounds__(PV, PV_BPS) phase_E(Args<T> a) {
         if (a.vec4) {
             const int64_t G = a.N >> 2;
             for (int64_t g = t0; g < G; g += S) {
-                const int64_t e = 4 * g;
+                const int64_t i4 = 4 * g;
                 T xv[4], pv[4], s_[4], tv[4], hv[4], rn[4];
-                ld4v(x + e, xv);
-                ld4v(p + e, pv);
-                ld4v(sv + e, s_);
-                ld4v(t + e, tv);
-                ld4v(rh + e, hv);
+                ld4v(x + i4, xv);
+                ld4v(p + i4, pv);
+                ld4v(sv + i4, s_);
+                ld4v(t + i4, tv);
+                ld4v(rh + i4, hv);
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     e_update(alpha, omega, xv[j], pv[j], s_[j], tv[j], rn[j]);
-                    acc_add(d[2 * k], hv[j], rn[j]);
-                    acc_add(d[2 * k + 1], rn[j], rn[j]);
+                    const T y = PA::scaled(rn[j], f);
+                    acc_add(d[2 * k], PA::scaled(hv[j], f0), y);
+                    acc_add(d[2 * k + 1], y, y);
                 }
-                st4v(x + e, xv);
-                st4v(r + e, rn);
+                st4v(x + i4, xv);
+                st4v(r + i4, rn);
             }
             i = 4 * G + t0;
         }
@@ -821,11 +946,13 @@ __global__ void __launch_bounds__(PV, PV_BPS) phase_E(Args<T> a) {
             e_update(alpha, omega, xi, p[i], sv[i], t[i], rn);
             x[i] = xi;
             r[i] = rn;
-            acc_add(d[2 * k], rh[i], rn);
-            acc_add(d[2 * k + 1], rn, rn);
+            const T y = PA::scaled(rn, f);
+            acc_add(d[2 * k], PA::scaled(rh[i], f0), y);
+            acc_add(d[2 * k + 1], y, y);
         }
     }
-    const double* tot = phase_reduce<4, PV>(d, a.pp, &c->ticket);
+    const double* tot =
+        phase_reduce<4, PV>(d, a.pp, &c->ticket, [&](int j) { return (j & 1 ? e[j >> 1] : e0[j >> 1]) + e[j >> 1]; });
     if (tot && threadIdx.x < 2) {
         const int k = threadIdx.x, it = c->it + 1;
         SpeciesState z = c->s[k];
@@ -842,6 +969,7 @@ __global__ void __launch_bounds__(PV, PV_BPS) phase_E(Args<T> a) {
                 z.alpha = z.alpha_n;
                 z.omega = z.omega_n;
                 z.res2 = tot[2 * k + 1];
+                z.e = PA::exp_of(z.res2);
                 if (z.res2 <= z.limit2) {
                     z.active = 0;
                     z.iters = it;

@@ -18,13 +18,15 @@
 // shuffle adds them up, and all of them hold the row's vector entries in
 // registers.  Sums of products go through shared memory, one value per row,
 // to one warp per sum (float64 arithmetic on all warps would cost more than
-// the iteration), float32 products as exact pairs (Dot2, as in the phase
-// kernels), and then from every block to all in a fixed order.
+// the iteration; float32 products are scaled, exact and summed as Dot3, as in the
+// phase kernels), and then from every block to all in a fixed order.
 //
 // Measured against one cooperative launch per step with the matrix streamed
 // from L2 and three blocks for the small operator: 2,562 nodes, n = 31, heat
 // equation in float64, 3.8 iterations per step: 314 -> 52 us per step; 40k
-// torus, n = 50, two species in float32: 320 -> 90 us per step.
+// torus, n = 50, two species in float32: 320 -> 92 us per step (90 with sums of
+// float32 pairs, which lost accuracy and the range of small and large fields; 97
+// with float64 ones).
 //
 // Included by step.cu inside its anonymous namespace.
 
@@ -65,16 +67,61 @@ __device__ __forceinline__ void cluster_sync_all() {
     asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
 }
 
-// a row's product as it goes to the summing warp: float64, or an exact pair of
-// float32 values
+// A row's product as it goes to the summing warp.  Float64: the product itself.
+// Float32: two factors scaled by the caller, as their exact product p + e; or, in
+// the right-hand side's sums, whose scale is not known yet, the factors themselves,
+// which the summing warp scales to the block's largest.
 template <typename T>
 struct Term {
-    using type = typename PhaseAcc<T>::type;
-    __device__ static type of(T a, T b) {
-        type t;
-        acc_zero(t);
-        acc_add(t, a, b);
-        return t;
+    using type = double;
+    __device__ static double of(double a, double b) { return a * b; }
+    __device__ static double raw(double a, double b) { return a * b; }
+    // the sum of the block's rows (times 2^e; RAW: of factors) by one warp, valid in lane 0
+    template <bool RAW, int UN>
+    __device__ static double sum(const double* t, int rows, int ln, int) {
+        double s = t[ln];
+#pragma unroll 4
+        for (int r = ln + 32; r < rows; r += 32) s += t[r];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+        return s;
+    }
+};
+template <>
+struct Term<float> {
+    using type = float2;
+    __device__ static float2 of(float a, float b) {
+        const float p = __fmul_rn(a, b);
+        return make_float2(p, __fmaf_rn(a, b, -p));
+    }
+    __device__ static float2 raw(float a, float b) { return make_float2(a, b); }
+    template <bool RAW, int UN>
+    __device__ static double sum(const float2* t, int rows, int ln, int e) {
+        float fa = 1.f, fb = 1.f;
+        if (RAW) {
+            unsigned ma = 0, mb = 0;   // largest magnitudes (their bits order like integers)
+#pragma unroll 4
+            for (int r = ln; r < rows; r += 32) {
+                ma = max(ma, __float_as_uint(t[r].x) & 0x7fffffffu);
+                mb = max(mb, __float_as_uint(t[r].y) & 0x7fffffffu);
+            }
+            const int ea = unit_exp((int)(__reduce_max_sync(0xffffffffu, ma) >> 23) - 127);
+            const int eb = unit_exp((int)(__reduce_max_sync(0xffffffffu, mb) >> 23) - 127);
+            fa = unit_scale(ea);
+            fb = unit_scale(eb);
+            e = ea + eb;
+        }
+        // (UN: blocks of few rows run faster with less code, two species on the
+        // 60k sphere 95 -> 93 us a step, 150k rows with more, 166 -> 156)
+        Dot3 s;
+        acc_zero(s);
+#pragma unroll UN
+        for (int r = ln; r < rows; r += 32) {
+            const float2 x = t[r];
+            if (RAW) acc_add(s, x.x * fa, x.y * fb);
+            else acc_pair(s, x.x, x.y);
+        }
+        return fixed_value(warp_sum(s, e));
     }
 };
 
@@ -85,6 +132,7 @@ template <typename T>
 struct ResidentScalars {
     T beta[2], alpha[2], omega[2];
     int act[2], early[2], zero[2];
+    int e0[2], e[2];   // exponents of r-hat and of the iteration's vectors in the sums
 };
 
 // shared memory of a block, in this order (all offsets multiples of 16 bytes)
@@ -104,7 +152,7 @@ struct ResidentSmem {
 };
 
 // one block's view of the synchronisations
-template <typename T, bool CL>
+template <typename T, int TPR, bool CL>
 struct ResidentBlock {
     unsigned char* sm;
     ResidentSmem<T> L;
@@ -116,7 +164,6 @@ struct ResidentBlock {
 
     // x (node i of species sp) to wherever blocks gather from: the TPR lanes
     // of the row share the peers
-    template <int TPR>
     __device__ void publish(int sp, int64_t i, int lane, T x) {
         if (CL) {
             const uint32_t at = smem_u32(sm + L.gather) + (uint32_t)((sp * a.N + i) * sizeof(T));
@@ -137,9 +184,10 @@ struct ResidentBlock {
     }
     // KS sums per species over all rows (terms v of each row, written by its
     // lane 0), and the barrier that makes them, and what was published,
-    // visible; lane 0 of warp k then decides with the totals of species k
-    template <int KS, int NS, typename F>
-    __device__ bool reduce(const typename Term<T>::type (&v)[NS][KS], int row, bool writes, F decide) {
+    // visible; lane 0 of warp k then decides with the totals of species k.  exp_of:
+    // exponent of sum j of species k (or RAW terms)
+    template <int KS, int NS, bool RAW = false, typename E, typename F>
+    __device__ bool reduce(const typename Term<T>::type (&v)[NS][KS], int row, bool writes, E exp_of, F decide) {
         using V = typename Term<T>::type;
         V* terms = (V*)(sm + L.terms);
         if (writes) {
@@ -153,16 +201,12 @@ struct ResidentBlock {
         double* pp = CL ? (double*)(sm + L.part) + parity * RES_CLUSTER * RES_SUMS
                         : ri.part + (int64_t)parity * gridDim.x * RES_SUMS;
         for (int k = wid; k < NS * KS; k += nw) {
-            V s = terms[k * rows + ln];
-#pragma unroll 4
-            for (int r = ln + 32; r < rows; r += 32) s = acc_merge(s, terms[k * rows + r]);
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) s = acc_merge(s, acc_shfl_down(s, o));
+            const double s = Term<T>::template sum<RAW, TPR == 1 ? 4 : 2>(terms + k * rows, rows, ln, exp_of(k / KS, k % KS));
             if (CL) {
-                const double t = __shfl_sync(0xffffffffu, acc_value(s), 0);
+                const double t = __shfl_sync(0xffffffffu, s, 0);
                 if (ln < (int)gridDim.x) st_peer(peer_addr(smem_u32(pp + blockIdx.x * RES_SUMS + k), ln), t);
             } else if (ln == 0) {
-                __stcg(pp + (int64_t)blockIdx.x * RES_SUMS + k, acc_value(s));
+                __stcg(pp + (int64_t)blockIdx.x * RES_SUMS + k, s);
             }
         }
         if (!sync()) return false;
@@ -204,8 +248,9 @@ template <typename T, int TPR, int NS, bool CL>
 __global__ void __launch_bounds__(res_threads<T>(), 1) resident_kernel(Args<T> a, ResidentInfo ri) {
     extern __shared__ __align__(16) unsigned char res_smem[];
     using TM = Term<T>;
+    using PA = PhaseAcc<T>;
     const int rows = ri.spb * 32, RPW = 32 / TPR;
-    ResidentBlock<T, CL> B{res_smem, ResidentSmem<T>(ri.max_elems, rows, a.N, NS, CL), a, ri, rows};
+    ResidentBlock<T, TPR, CL> B{res_smem, ResidentSmem<T>(ri.max_elems, rows, a.N, NS, CL), a, ri, rows};
     T* sw = (T*)(res_smem + B.L.w);
     int32_t* si = (int32_t*)(res_smem + B.L.idx);
 
@@ -295,7 +340,7 @@ __global__ void __launch_bounds__(res_threads<T>(), 1) resident_kernel(Args<T> a
         const T kk[2] = {kc.k0, kc.k1};
 #pragma unroll
         for (int k = 0; k < NS; ++k)
-            if (own) B.template publish<TPR>(k, node, lane, x[k]);
+            if (own) B.publish(k, node, lane, x[k]);
         if (!B.sync()) return;
         // ---- right-hand side, r0 = b - A x
         T y[NS], b[2] = {T(0), T(0)};
@@ -308,11 +353,11 @@ __global__ void __launch_bounds__(res_threads<T>(), 1) resident_kernel(Args<T> a
             r[k] = b[k] - (kc.c0 * x[k] - kk[k] * y[k]);
             rh[k] = r[k];
             p[k] = q[k] = T(0);
-            d2[k][0] = TM::of(b[k], b[k]);
-            d2[k][1] = TM::of(r[k], r[k]);
+            d2[k][0] = TM::raw(b[k], b[k]);
+            d2[k][1] = TM::raw(r[k], r[k]);
         }
         it = 0;
-        if (!B.template reduce<2, NS>(d2, lrow, sums, [&](int k, const double (&tot)[2]) {
+        if (!B.template reduce<2, NS, true>(d2, lrow, sums, [](int, int) { return 0; }, [&](int k, const double (&tot)[2]) {
                 bnorm = sqrt(tot[0]);
                 limit2 = (a.tol * bnorm) * (a.tol * bnorm);
                 rho = tot[1];   // (r-hat, r0) = |r0|^2
@@ -326,11 +371,13 @@ __global__ void __launch_bounds__(res_threads<T>(), 1) resident_kernel(Args<T> a
                 sc.omega[k] = T(1);
                 sc.act[k] = active;
                 sc.zero[k] = bnorm == 0.0;
+                sc.e0[k] = sc.e[k] = PhaseAcc<T>::exp_of(rho);
             }))
             return;
 #pragma unroll
         for (int k = 0; k < NS; ++k)
             if (sc.zero[k]) x[k] = T(0);   // b = 0: x = 0
+        const auto both = [&](int k, int) { return 2 * sc.e[k]; };
         while ((sc.act[0] || (NS == 2 && sc.act[NS - 1])) && it < a.maxit) {
             ++it;
             // ---- A: p = r + beta (p - omega q)
@@ -338,7 +385,7 @@ __global__ void __launch_bounds__(res_threads<T>(), 1) resident_kernel(Args<T> a
             for (int k = 0; k < NS; ++k)
                 if (sc.act[k] && own) {
                     p[k] = r[k] + sc.beta[k] * (p[k] - sc.omega[k] * q[k]);
-                    B.template publish<TPR>(k, node, lane, p[k]);
+                    B.publish(k, node, lane, p[k]);
                 }
             if (!B.sync()) return;
             // ---- B: q = A p ; (r-hat, q)
@@ -346,9 +393,9 @@ __global__ void __launch_bounds__(res_threads<T>(), 1) resident_kernel(Args<T> a
 #pragma unroll
             for (int k = 0; k < NS; ++k) {
                 if (sc.act[k]) q[k] = kc.c0 * p[k] - kk[k] * y[k];
-                d1[k][0] = TM::of(rh[k], q[k]);
+                d1[k][0] = TM::of(PA::scaled(rh[k], unit_scale(sc.e0[k])), PA::scaled(q[k], unit_scale(sc.e[k])));
             }
-            if (!B.template reduce<1, NS>(d1, lrow, sums, [&](int k, const double (&tot)[1]) {
+            if (!B.template reduce<1, NS>(d1, lrow, sums, [&](int k, int) { return sc.e0[k] + sc.e[k]; }, [&](int k, const double (&tot)[1]) {
                     if (active) {
                         alpha = rho / tot[0];
                         if (tot[0] == 0.0 || !isfinite(alpha)) {
@@ -365,11 +412,11 @@ __global__ void __launch_bounds__(res_threads<T>(), 1) resident_kernel(Args<T> a
             for (int k = 0; k < NS; ++k) {
                 if (sc.act[k] && own) {
                     s[k] = r[k] - sc.alpha[k] * q[k];
-                    B.template publish<TPR>(k, node, lane, s[k]);
+                    B.publish(k, node, lane, s[k]);
                 }
-                d1[k][0] = TM::of(s[k], s[k]);
+                d1[k][0] = TM::of(PA::scaled(s[k], unit_scale(sc.e[k])), PA::scaled(s[k], unit_scale(sc.e[k])));
             }
-            if (!B.template reduce<1, NS>(d1, lrow, sums, [&](int k, const double (&tot)[1]) {
+            if (!B.template reduce<1, NS>(d1, lrow, sums, both, [&](int k, const double (&tot)[1]) {
                     const bool early = active && tot[0] <= limit2;
                     if (early) {
                         res2 = tot[0];
@@ -389,10 +436,11 @@ __global__ void __launch_bounds__(res_threads<T>(), 1) resident_kernel(Args<T> a
 #pragma unroll
             for (int k = 0; k < NS; ++k) {
                 if (sc.act[k]) t[k] = kc.c0 * s[k] - kk[k] * y[k];
-                d2[k][0] = TM::of(t[k], s[k]);
-                d2[k][1] = TM::of(t[k], t[k]);
+                const T ts = PA::scaled(t[k], unit_scale(sc.e[k]));
+                d2[k][0] = TM::of(ts, PA::scaled(s[k], unit_scale(sc.e[k])));
+                d2[k][1] = TM::of(ts, ts);
             }
-            if (!B.template reduce<2, NS>(d2, lrow, sums, [&](int k, const double (&tot)[2]) {
+            if (!B.template reduce<2, NS>(d2, lrow, sums, both, [&](int k, const double (&tot)[2]) {
                     if (active) {
                         omega = tot[0] / tot[1];
                         if (tot[1] == 0.0 || !isfinite(omega)) {
@@ -411,10 +459,11 @@ __global__ void __launch_bounds__(res_threads<T>(), 1) resident_kernel(Args<T> a
                     x[k] += sc.alpha[k] * p[k] + sc.omega[k] * s[k];
                     r[k] = s[k] - sc.omega[k] * t[k];
                 }
-                d2[k][0] = TM::of(rh[k], r[k]);
-                d2[k][1] = TM::of(r[k], r[k]);
+                const T rs = PA::scaled(r[k], unit_scale(sc.e[k]));
+                d2[k][0] = TM::of(PA::scaled(rh[k], unit_scale(sc.e0[k])), rs);
+                d2[k][1] = TM::of(rs, rs);
             }
-            if (!B.template reduce<2, NS>(d2, lrow, sums, [&](int k, const double (&tot)[2]) {
+            if (!B.template reduce<2, NS>(d2, lrow, sums, [&](int k, int j) { return (j ? sc.e[k] : sc.e0[k]) + sc.e[k]; }, [&](int k, const double (&tot)[2]) {
                     if (active) {
                         rho_prev = rho;
                         rho = tot[0];
@@ -431,6 +480,7 @@ __global__ void __launch_bounds__(res_threads<T>(), 1) resident_kernel(Args<T> a
                             sc.beta[k] = (T)beta;
                         }
                         res2 = tot[1];
+                        sc.e[k] = PhaseAcc<T>::exp_of(res2);
                     }
                     sc.act[k] = active;
                 }))
