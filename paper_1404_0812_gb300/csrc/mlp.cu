@@ -345,7 +345,7 @@ __device__ __forceinline__ void cp16(float* dst, const float* src) {
 
 // rows and features of the tile's samples, by asynchronous copies (loads in the
 // products' loops cost 15 us of L2 latency); they need no weights, so a step's
-// are on their way while the step before it still updates those
+// are on their way while the step before it (and nothing else) updates those
 template <int C>
 __device__ __forceinline__ void load_samples(float* smc, const ClusterTile& L, int64_t* row, int D,
                                              const float* feats, const int32_t* sel, int64_t s0, int ns, int rank) {
@@ -662,7 +662,7 @@ size_t tile_smem(int D) { return (size_t)(TS * D + 4 * TS * H + 2 * TS) * sizeof
 
 template <int C>
 rbffd_status launch_cluster_tiles(const rbffd_mlp* m, const float* feats, const float* target, const int32_t* sel,
-                                  int64_t count, int tiles, float* loss_part, cudaStream_t st) {
+                                  int64_t count, int tiles, float* loss_part, bool after_reduce, cudaStream_t st) {
     const size_t smem = (size_t)ClusterTile(m->D, C).total * sizeof(float);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(tiles * C));
@@ -676,7 +676,7 @@ rbffd_status launch_cluster_tiles(const rbffd_mlp* m, const float* feats, const 
     at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // see launch_reduce
     at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 2;
+    cfg.numAttrs = after_reduce ? 2 : 1;
     RBFFD_CUDA_TRY(cudaLaunchKernelEx(&cfg, mlp_tile_cluster<C>, (const float*)m->params, m->D, feats, target, sel,
                                       count, 1.f / (float)count, m->partial, loss_part));
     note_launch();
@@ -687,18 +687,22 @@ rbffd_status launch_cluster_tiles(const rbffd_mlp* m, const float* feats, const 
 // eight or four CTAs per tile while those stay within one wave of the chip, a
 // CTA per tile beyond (its register tiles move fewer shared-memory bytes per
 // FMA, and there are tiles enough), or where the weights of a large network
-// leave no room for a cluster's arrays.
+// leave no room for a cluster's arrays.  after_reduce: the kernel ahead on the
+// stream is this network's reduce_grad, which writes no samples; only then may the
+// tiles start while it drains, because they fetch their samples before they wait
+// for it.  Behind any other kernel, which may be the one that makes the samples and
+// may let its dependents start early, they are launched in plain stream order.
 constexpr size_t CLUSTER_SMEM_MAX = 227 * 1024;
 template <int C>
 bool cluster_fits(int D) { return ClusterTile(D, C).total * sizeof(float) + 1024 <= CLUSTER_SMEM_MAX; }
 
 rbffd_status gradient_tiles(const rbffd_mlp* m, const float* feats, const float* target, const int32_t* sel,
-                            int64_t count, float* loss_part, cudaStream_t st) {
+                            int64_t count, float* loss_part, bool after_reduce, cudaStream_t st) {
     const int64_t tiles = (count + TS - 1) / TS;
     if (tiles * 8 <= sm_count() && cluster_fits<8>(m->D))
-        return launch_cluster_tiles<8>(m, feats, target, sel, count, (int)tiles, loss_part, st);
+        return launch_cluster_tiles<8>(m, feats, target, sel, count, (int)tiles, loss_part, after_reduce, st);
     if (tiles * 4 <= sm_count() && cluster_fits<4>(m->D))
-        return launch_cluster_tiles<4>(m, feats, target, sel, count, (int)tiles, loss_part, st);
+        return launch_cluster_tiles<4>(m, feats, target, sel, count, (int)tiles, loss_part, after_reduce, st);
     mlp_tile<<<(unsigned)tiles, NT, tile_smem(m->D), st>>>(m->params, m->D, feats, target, sel, count,
                                                            1.f / (float)count, 1, nullptr, m->partial, loss_part);
     note_launch();
@@ -962,7 +966,7 @@ rbffd_status rbffd_mlp_loss_grad(const rbffd_mlp* mc, const float* feats, const 
     if (s != RBFFD_OK) return s;
     s = ensure_smem(m->D);
     if (s != RBFFD_OK) return s;
-    s = gradient_tiles(m, feats, target, nullptr, count, m->loss + 4096, st);
+    s = gradient_tiles(m, feats, target, nullptr, count, m->loss + 4096, false, st);
     if (s != RBFFD_OK) return s;
     s = launch_reduce(m, (int)tiles, grad, nullptr, nullptr, nullptr, 0, 0.f, 0, st);
     if (s != RBFFD_OK) return s;
@@ -1015,7 +1019,7 @@ rbffd_status rbffd_mlp_train(rbffd_mlp* m, const float* feats, const float* targ
             int64_t nb = std::min<int64_t>(batch, count - b0);
             unsigned tiles = (unsigned)((nb + TS - 1) / TS);
             ++m->adam_t;   // the step counter lives with the network's moments
-            s = gradient_tiles(m, feats, target, perm_d + b0, nb, m->loss + 4096, st);
+            s = gradient_tiles(m, feats, target, perm_d + b0, nb, m->loss + 4096, b > 0, st);
             if (s != RBFFD_OK) return s;
             s = launch_reduce(m, (int)tiles, nullptr, m->params, m->adam_m, m->adam_v, m->adam_t, lr, (int)b, st);
             if (s != RBFFD_OK) return s;
