@@ -497,10 +497,13 @@ __global__ void __launch_bounds__(SOLVE_THREADS) solve_kernel(SolveArgs<T, TV> a
 // owner of the next block updates and solves it first and copies its 32 values
 // to all CTAs while they update the rest, so a block costs one triangle, one
 // 32-column update of 32 rows and a cluster barrier.  The back substitution is
-// the same on mirrored rows, its rows scaled by 1 / U_ii so that the triangle's
-// chain has no division.  2,400 rows, bands of about 300: 4.2 -> 0.6 ms per
-// solve of two species (0.88 with the next block's coefficients loaded in the
-// step that uses them).
+// the same on mirrored rows, for z = D x with the triangle's columns divided by
+// their U_ii, so that its chain has no division and every product of a coefficient
+// and an unknown still carries one rounding beside its own (the coefficient's
+// instead of the unknown's); x = z / U_ii follows.  2,400 rows, bands of about 300: 4.2 -> 0.53 ms per solve of two
+// species (0.88 with the next block's coefficients loaded in the step that uses
+// them; 0.69 with a quotient in every step of the triangle's chain; 0.52 with rows
+// scaled by a rounded 1 / U_ii, which rounds twice more).
 // ---------------------------------------------------------------------------
 constexpr int NB = 32;                 // rows of a block
 constexpr int BLK_CTAS = 8;            // CTAs of the cluster
@@ -519,11 +522,59 @@ __device__ __forceinline__ void st_cluster(uint32_t a, float v) {
     asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
 }
 
+// Division of several numbers by the same d.  Float64: with the reciprocal to twice
+// the precision, h = fl(1 / d) and l = fl(fl(1 - d h) h), of which the residual is
+// exact in an FMA, fma(t, h, t l) errs by half an ulp and 2^-105 of the quotient, a
+// division's rounding, in two instructions (a division is ten).  A product with h
+// alone rounds twice, and h overflows for a subnormal d.  Divisors near the ends of
+// the range, where h or l leaves it, and float32 ones are divided by.
+template <typename T>
+struct Divisor {
+    static constexpr int ROWS = 1;   // rows of shared memory that hold a block's
+    T d;
+    __device__ static Divisor of(T d) { return Divisor{d}; }
+    __device__ static Divisor get(const T (*at)[NB], int lane) { return Divisor{at[0][lane]}; }
+    __device__ void put(T (*at)[NB], int lane) const { at[0][lane] = d; }
+    __device__ Divisor lane(int k) const { return Divisor{__shfl_sync(0xffffffffu, d, k)}; }
+    __device__ T quotient(T t) const { return t / d; }
+    // (by integers: a float64 comparison takes the float64 unit)
+    __device__ static bool normal(float q) { return (__float_as_uint(q) >> 23 & 0xffu) - 1u < 0xfeu; }
+    __device__ static bool zero(float q) { return __float_as_uint(q) << 1 == 0u; }
+};
+template <>
+struct Divisor<double> {
+    static constexpr int ROWS = 3;
+    double d, h, l;
+    __device__ static Divisor of(double d) {
+        const double h = 1.0 / d;
+        return Divisor{d, h, fma(-d, h, 1.0) * h};
+    }
+    __device__ static Divisor get(const double (*at)[NB], int lane) {
+        return Divisor{at[0][lane], at[1][lane], at[2][lane]};
+    }
+    __device__ void put(double (*at)[NB], int lane) const {
+        at[0][lane] = d;
+        at[1][lane] = h;
+        at[2][lane] = l;
+    }
+    __device__ Divisor lane(int k) const {
+        return Divisor{__shfl_sync(0xffffffffu, d, k), __shfl_sync(0xffffffffu, h, k),
+                       __shfl_sync(0xffffffffu, l, k)};
+    }
+    __device__ double quotient(double t) const {
+        const int e = (__double2hiint(d) >> 20) & 0x7ff;
+        return e < 1023 - 900 || e > 1023 + 900 ? t / d : fma(t, h, t * l);
+    }
+    __device__ static bool normal(double q) { return ((unsigned)__double2hiint(q) >> 20 & 0x7ffu) - 1u < 0x7feu; }
+    __device__ static bool zero(double q) { return ((__double2hiint(q) << 1) | __double2loint(q)) == 0; }
+};
+
 // One triangular sweep: forward with L, or (BACK) with U on mirrored rows
 // r' = N - 1 - r.  in / out: the right-hand side and the result by row.
 template <typename T, bool BACK, typename TI, typename TO>
 __device__ void block_sweep(const SolveSys<T>& f, int64_t N, int64_t kl, int64_t ku, const TI* in, TO* out, T* ring,
-                            int slots, T (*ybuf)[NB], T (*part)[NB], T (*tri)[NB], int rank) {
+                            int slots, T (*ybuf)[NB], T (*part)[NB], T (*tri)[NB], unsigned char* undivided,
+                            int rank) {
     const int64_t bw = BACK ? kl + ku : kl, ldab = 2 * kl + ku + 1;
     const int64_t nblk = (N + NB - 1) / NB, reach = (bw + NB - 1) / NB;   // blocks a block reaches below itself
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -542,9 +593,10 @@ __device__ void block_sweep(const SolveSys<T>& f, int64_t N, int64_t kl, int64_t
     // A block's coefficients are fetched in the step before their use, at its
     // start (the barrier at its end waits for loads still in flight), by the
     // UPD warps that update the next block: eight columns of the update each,
-    // kept in registers, and eight of the triangle, put in shared memory
-    // scaled by U's diagonal (back sweep).
+    // kept in registers, and eight of the triangle, put in shared memory divided
+    // by their columns' diagonal (back sweep).
     constexpr int CW = NB / UPD;
+    static_assert(CW == 8 && UPD == 4, "a byte of flags per warp");
     T tcol[CW], upd[CW], diag = T(1);
     auto fetch = [&](int64_t b) {
         const int64_t r0 = b * NB, r = r0 + lane;
@@ -557,18 +609,41 @@ __device__ void block_sweep(const SolveSys<T>& f, int64_t N, int64_t kl, int64_t
         if (BACK) diag = r < N ? f.udiag[N - 1 - r] : T(1);
     };
     auto store_triangle = [&]() {
-        const T d = BACK ? T(1) / diag : T(1);
+        if (BACK) {
+            // a column whose coefficients leave the range when divided is not divided
+            const Divisor<T> d = Divisor<T>::of(diag);
+            unsigned whole = 0;
 #pragma unroll
-        for (int c = 0; c < CW; ++c) tri[warp * CW + c][lane] = BACK ? tcol[c] * d : tcol[c];
-        if (warp == 0) tri[NB][lane] = d;
+            for (int c = 0; c < CW; ++c) {
+                const T q = d.lane(warp * CW + c).quotient(tcol[c]);
+                const bool out = !Divisor<T>::normal(q) && !Divisor<T>::zero(tcol[c]);
+                const bool keep = __any_sync(0xffffffffu, out);
+                tri[warp * CW + c][lane] = keep ? tcol[c] : q;
+                whole |= (unsigned)keep << c;
+            }
+            if (lane == 0) undivided[warp] = (unsigned char)whole;
+            if (warp == 0) d.put(tri + NB, lane);
+        } else {
+#pragma unroll
+            for (int c = 0; c < CW; ++c) tri[warp * CW + c][lane] = tcol[c];
+        }
     };
     // solve the triangle of block b (its rows updated) by one warp, copy the
     // result to all CTAs and to `out`
     auto solve = [&](int64_t b, T y) {
         const int64_t r = b * NB + lane;
-        if (BACK) y *= tri[NB][lane];
+        const unsigned whole = BACK ? *reinterpret_cast<const unsigned*>(undivided) : 0u;
+        if (whole == 0u) {
 #pragma unroll
-        for (int c = 0; c < NB; ++c) y = fma(-tri[c][lane], __shfl_sync(0xffffffffu, y, c), y);
+            for (int c = 0; c < NB; ++c) y = fma(-tri[c][lane], __shfl_sync(0xffffffffu, y, c), y);
+        } else {
+#pragma unroll 1
+            for (int c = 0; c < NB; ++c) {
+                const T z = __shfl_sync(0xffffffffu, y, c);
+                y = fma(-tri[c][lane], whole >> c & 1u ? z / tri[NB][c] : z, y);
+            }
+        }
+        if (BACK) y = Divisor<T>::get(tri + NB, lane).quotient(y);
 #pragma unroll
         for (int p = 0; p < BLK_CTAS; ++p) st_cluster(peer_smem(&ybuf[b & 1][lane], p), y);
         if (r < N) out[BACK ? N - 1 - r : r] = (TO)y;
@@ -636,7 +711,8 @@ __host__ __device__ inline int block_slots(int64_t bw) { return (int)(((bw + NB 
 template <typename T, typename TV>
 __global__ void __cluster_dims__(BLK_CTAS, 1, 1) __launch_bounds__(BLK_THREADS) solve_blocks_kernel(SolveArgs<T, TV> a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ T ybuf[2][NB], part[UPD][NB], tri[NB + 1][NB];
+    __shared__ T ybuf[2][NB], part[UPD][NB], tri[NB + Divisor<T>::ROWS][NB];
+    __shared__ __align__(4) unsigned char undivided[UPD];   // back sweep: columns of the triangle, a bit each
     T* ring = reinterpret_cast<T*>(smem_raw);
     const int sp = blockIdx.x / BLK_CTAS, rank = blockIdx.x % BLK_CTAS;
     const int ord = a.ord_flag ? *((volatile const int*)a.ord_flag) : 1;
@@ -644,11 +720,11 @@ __global__ void __cluster_dims__(BLK_CTAS, 1, 1) __launch_bounds__(BLK_THREADS) 
     T* wy = a.work + sp * (2 * a.N + 16);
     const int slots = block_slots(a.kl + a.ku);
     cluster_barrier();   // all CTAs run before their shared memory is written
-    block_sweep<T, false>(f, a.N, a.kl, a.ku, a.b[sp], wy, ring, slots, ybuf, part, tri, rank);
+    block_sweep<T, false>(f, a.N, a.kl, a.ku, a.b[sp], wy, ring, slots, ybuf, part, tri, undivided, rank);
     // the forward results, written by every CTA, are read by all
     __threadfence();
     cluster_barrier();
-    block_sweep<T, true>(f, a.N, a.kl, a.ku, wy, a.x[sp], ring, slots, ybuf, part, tri, rank);
+    block_sweep<T, true>(f, a.N, a.kl, a.ku, wy, a.x[sp], ring, slots, ybuf, part, tri, undivided, rank);
 }
 
 template <typename T>
