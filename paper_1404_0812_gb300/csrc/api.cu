@@ -68,6 +68,17 @@ cudaError_t pool_alloc_bytes(void** p, size_t bytes, cudaStream_t st) {
     return cudaMallocFromPoolAsync(p, bytes, pool, st);
 }
 
+rbffd_status allow_shared(const void* kernel) {
+    int dev = 0, most = 0;
+    cudaFuncAttributes fa;
+    RBFFD_CUDA_TRY(cudaGetDevice(&dev));
+    RBFFD_CUDA_TRY(cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+    RBFFD_CUDA_TRY(cudaFuncGetAttributes(&fa, kernel));
+    RBFFD_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        most - (int)fa.sharedSizeBytes));
+    return RBFFD_OK;
+}
+
 int sm_count() {
     int dev = 0, n = 0;
     cudaGetDevice(&dev);

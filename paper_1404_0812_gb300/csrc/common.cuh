@@ -27,6 +27,12 @@ void set_error(const char* fmt, ...);
         }                                                                         \
     } while (0)
 
+#define RBFFD_TRY(expr)                                                           \
+    do {                                                                          \
+        const rbffd_status _s = (expr);                                           \
+        if (_s != RBFFD_OK) return _s;                                            \
+    } while (0)
+
 #define RBFFD_CHECK_ARG(cond, msg)                                                \
     do {                                                                          \
         if (!(cond)) {                                                            \
@@ -203,4 +209,9 @@ rbffd_status lu_solve_step(rbffd_lu* const (&fac)[4][2], int nspecies, const voi
                            int vec_dtype, const int* ord_flag, void* work, int* err, cudaStream_t st);
 void lu_free(rbffd_lu* lu);
 int sm_count();
+
+// Lets launches of a kernel ask for any dynamic shared memory a block can have on
+// this device (api.cu).  The limit belongs to the function, not to a launch: set to
+// each launch's own size, it made another thread's larger launch fail.
+rbffd_status allow_shared(const void* kernel);
 }  // namespace rbffd

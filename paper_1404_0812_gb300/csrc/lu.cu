@@ -746,8 +746,7 @@ int solve_depth(int64_t kl, int64_t ku) {
 template <typename T, typename TV, int D>
 rbffd_status launch_solve_d(const SolveArgs<T, TV>& a, int nspecies, cudaStream_t st) {
     const size_t smem = solve_smem<T>(a.kl, a.ku, D);
-    RBFFD_CUDA_TRY(cudaFuncSetAttribute(solve_kernel<T, TV, D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)smem));
+    RBFFD_TRY(allow_shared((const void*)solve_kernel<T, TV, D>));
     solve_kernel<T, TV, D><<<nspecies, SOLVE_THREADS, smem, st>>>(a);
     note_launch();
     RBFFD_CUDA_TRY(cudaGetLastError());
@@ -759,8 +758,7 @@ rbffd_status launch_solve(const SolveArgs<T, TV>& a, int nspecies, bool intercha
     const int D = solve_depth<T>(a.kl, a.ku);
     if (D > 0 && !interchanges) {
         const size_t smem = (size_t)block_slots(a.kl + a.ku) * NB * sizeof(T);
-        RBFFD_CUDA_TRY(cudaFuncSetAttribute(solve_blocks_kernel<T, TV>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                            (int)smem));
+        RBFFD_TRY(allow_shared((const void*)solve_blocks_kernel<T, TV>));
         solve_blocks_kernel<T, TV><<<nspecies * BLK_CTAS, BLK_THREADS, smem, st>>>(a);
         note_launch();
         RBFFD_CUDA_TRY(cudaGetLastError());
@@ -812,7 +810,7 @@ rbffd_status factor_t(const rbffd_op* op, rbffd_lu* lu, cudaStream_t st) {
     RBFFD_CUDA_TRY(cudaMemsetAsync(flags, 0, 3 * sizeof(int), st));
     a.bar = bar;
     a.flags = flags;
-    RBFFD_CUDA_TRY(cudaFuncSetAttribute(factor_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    RBFFD_TRY(allow_shared((const void*)factor_kernel<T>));
     int per_sm = 0;
     RBFFD_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, factor_kernel<T>, FACTOR_THREADS, smem));
     RBFFD_CHECK_ARG(per_sm >= 1, "banded LU: the factorisation kernel does not fit on an SM");

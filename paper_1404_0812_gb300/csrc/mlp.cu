@@ -751,8 +751,7 @@ rbffd_status launch_epoch(const rbffd_mlp* m, EpochArgs a, int tiles, cudaStream
     at[1].val.cooperative = 1;
     cfg.attrs = at;
     cfg.numAttrs = 2;
-    RBFFD_CUDA_TRY(cudaFuncSetAttribute(mlp_epoch_cluster<C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)cfg.dynamicSmemBytes));
+    RBFFD_TRY(allow_shared((const void*)mlp_epoch_cluster<C>));
     int resident = 0;
     RBFFD_CUDA_TRY(cudaOccupancyMaxActiveClusters(&resident, mlp_epoch_cluster<C>, &cfg));
     if (resident < tiles) return RBFFD_OK;
@@ -795,15 +794,10 @@ rbffd_status epoch_launch(const rbffd_mlp* m, const float* feats, const float* t
     return s;
 }
 
-rbffd_status ensure_smem(int D) {
-    RBFFD_CUDA_TRY(cudaFuncSetAttribute(mlp_tile, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)tile_smem(D)));
-    if (cluster_fits<8>(D))
-        RBFFD_CUDA_TRY(cudaFuncSetAttribute(mlp_tile_cluster<8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)(ClusterTile(D, 8).total * sizeof(float))));
-    if (cluster_fits<4>(D))
-        RBFFD_CUDA_TRY(cudaFuncSetAttribute(mlp_tile_cluster<4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)(ClusterTile(D, 4).total * sizeof(float))));
+rbffd_status ensure_smem() {
+    RBFFD_TRY(allow_shared((const void*)mlp_tile));
+    RBFFD_TRY(allow_shared((const void*)mlp_tile_cluster<8>));
+    RBFFD_TRY(allow_shared((const void*)mlp_tile_cluster<4>));
     return RBFFD_OK;
 }
 
@@ -828,7 +822,7 @@ rbffd_status ensure_train_ws(rbffd_mlp* m, int64_t tiles) {
 rbffd_status predict_launch(const rbffd_mlp* m, const float* feats, int64_t count, float* out,
                             cudaStream_t st) {
     if (count <= 0) return RBFFD_OK;
-    rbffd_status s = ensure_smem(m->D);
+    rbffd_status s = ensure_smem();
     if (s != RBFFD_OK) return s;
     unsigned tiles = (unsigned)((count + TS - 1) / TS);
     mlp_tile<<<tiles, NT, tile_smem(m->D), st>>>(m->params, m->D, feats, nullptr, nullptr, count, 0.f,
@@ -964,7 +958,7 @@ rbffd_status rbffd_mlp_loss_grad(const rbffd_mlp* mc, const float* feats, const 
     int64_t tiles = (count + TS - 1) / TS;
     rbffd_status s = ensure_train_ws(m, tiles);
     if (s != RBFFD_OK) return s;
-    s = ensure_smem(m->D);
+    s = ensure_smem();
     if (s != RBFFD_OK) return s;
     s = gradient_tiles(m, feats, target, nullptr, count, m->loss + 4096, false, st);
     if (s != RBFFD_OK) return s;
@@ -991,7 +985,7 @@ rbffd_status rbffd_mlp_train(rbffd_mlp* m, const float* feats, const float* targ
     int64_t tiles_per_batch = (batch + TS - 1) / TS;
     rbffd_status s = ensure_train_ws(m, tiles_per_batch);
     if (s != RBFFD_OK) return s;
-    s = ensure_smem(m->D);
+    s = ensure_smem();
     if (s != RBFFD_OK) return s;
     int32_t* perm_d = nullptr;
     RBFFD_CUDA_TRY(pool_alloc(&perm_d, count * sizeof(int32_t), st));

@@ -250,13 +250,13 @@ __global__ void __launch_bounds__(SORT_THREADS) sort_one_tile(const uint64_t* __
 rbffd_status sort_keys_device(uint64_t* key, int64_t N, int32_t* perm, cudaStream_t st) {
     const size_t smem = sizeof(TileShared);
     if (N <= TILE) {
-        RBFFD_CUDA_TRY(cudaFuncSetAttribute(sort_one_tile, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        RBFFD_TRY(allow_shared((const void*)sort_one_tile));
         sort_one_tile<<<1, SORT_THREADS, smem, st>>>(key, (int)N, perm);
         note_launch();
         RBFFD_CUDA_TRY(cudaGetLastError());
         return RBFFD_OK;
     }
-    RBFFD_CUDA_TRY(cudaFuncSetAttribute(sort_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    RBFFD_TRY(allow_shared((const void*)sort_scatter));
     const int ntiles = (int)((N + TILE - 1) / TILE);
     uint64_t* key2 = nullptr;
     int32_t *val = nullptr, *val2 = nullptr, *counts = nullptr;

@@ -568,7 +568,7 @@ rbffd_status resident_launch_as(Args<T>& a, const ResidentPlan& p, const Residen
     const int threads = std::max(64, p.spb * 32 * TPR);   // at least a warp per species
     if (p.cluster) {
         auto* fn = resident_kernel<T, TPR, NS, true>;
-        RBFFD_CUDA_TRY(cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem));
+        RBFFD_TRY(allow_shared((const void*)fn));
         RBFFD_CUDA_TRY(cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(p.blocks);
@@ -584,7 +584,7 @@ rbffd_status resident_launch_as(Args<T>& a, const ResidentPlan& p, const Residen
         RBFFD_CUDA_TRY(cudaLaunchKernelEx(&cfg, fn, a, ri));
     } else {
         auto* fn = resident_kernel<T, TPR, NS, false>;
-        RBFFD_CUDA_TRY(cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem));
+        RBFFD_TRY(allow_shared((const void*)fn));
         RBFFD_CUDA_TRY(cudaMemsetAsync(a.bar, 0, sizeof(unsigned long long), st));
         ResidentInfo r = ri;
         void* args[] = {&a, &r};

@@ -1112,7 +1112,7 @@ __global__ void __launch_bounds__(32) team_weights_kernel(TeamWeightArgs B) {
 
 // one-warp blocks resident on the chip with the given shared memory each
 rbffd_status resident_warps(const void* kernel, size_t smem, int* warps) {
-    RBFFD_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    RBFFD_TRY(allow_shared(kernel));
     int per_sm = 0;
     RBFFD_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, 32, smem));
     *warps = std::max(1, per_sm) * sm_count();
