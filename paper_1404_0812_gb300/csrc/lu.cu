@@ -227,8 +227,6 @@ __global__ void __launch_bounds__(FACTOR_THREADS) factor_kernel(FactorArgs<T> a)
 // ---------------------------------------------------------------------------
 // substitutions
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
 __device__ __forceinline__ void mbar_init(uint64_t* bar) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_addr(bar)) : "memory");
 }
@@ -510,18 +508,6 @@ constexpr int BLK_CTAS = 8;            // CTAs of the cluster
 constexpr int BLK_THREADS = 512, BLK_WARPS = BLK_THREADS / 32;
 constexpr int UPD = 4;                 // warps that update the next block, 8 columns each
 
-__device__ __forceinline__ uint32_t peer_smem(const void* p, uint32_t rank) {
-    uint32_t r;
-    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_addr(p)), "r"(rank));
-    return r;
-}
-__device__ __forceinline__ void st_cluster(uint32_t a, double v) {
-    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
-}
-__device__ __forceinline__ void st_cluster(uint32_t a, float v) {
-    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
-}
-
 // Division of several numbers by the same d.  Float64: with the reciprocal to twice
 // the precision, h = fl(1 / d) and l = fl(fl(1 - d h) h), of which the residual is
 // exact in an FMA, fma(t, h, t l) errs by half an ulp and 2^-105 of the quotient, a
@@ -645,7 +631,7 @@ __device__ void block_sweep(const SolveSys<T>& f, int64_t N, int64_t kl, int64_t
         }
         if (BACK) y = Divisor<T>::get(tri + NB, lane).quotient(y);
 #pragma unroll
-        for (int p = 0; p < BLK_CTAS; ++p) st_cluster(peer_smem(&ybuf[b & 1][lane], p), y);
+        for (int p = 0; p < BLK_CTAS; ++p) st_cluster(peer_addr(smem_addr(&ybuf[b & 1][lane]), p), y);
         if (r < N) out[BACK ? N - 1 - r : r] = (TO)y;
     };
     // the window's first blocks, and the first triangle

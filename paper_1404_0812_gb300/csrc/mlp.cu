@@ -466,8 +466,7 @@ __device__ __forceinline__ void cluster_gradient(float* smc, const ClusterTile& 
     for (int e = t; e < C * OWN * (H / 4); e += NT) {
         const int p = e / (OWN * (H / 4)), q = e - p * (OWN * (H / 4));
         if (p == rank) continue;
-        uint32_t pb;
-        asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(pb) : "r"(base), "r"(p));
+        const uint32_t pb = peer_addr(base, p);
         const int off = first * H + 4 * q;
         const int col = (4 * q) % H;
         if (col >= p * (H / C) && col < (p + 1) * (H / C))
@@ -480,7 +479,7 @@ __device__ __forceinline__ void cluster_gradient(float* smc, const ClusterTile& 
             st_peer4(pb + 4 * o1, *reinterpret_cast<const float4*>(smc + o1));
         }
     }
-    asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
+    cluster_barrier();
     // ---- this CTA's rows of the tile's gradient
     float* gW1 = G;
     float* gb1 = gW1 + (int64_t)D * H;

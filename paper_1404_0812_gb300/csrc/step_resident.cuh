@@ -46,27 +46,6 @@ struct ResidentInfo {
     double* part;        // grid form: 2 x blocks x RES_SUMS
 };
 
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ uint32_t peer_addr(uint32_t a, uint32_t rank) {
-    uint32_t r;
-    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
-    return r;
-}
-__device__ __forceinline__ void st_peer(uint32_t a, float v) {
-    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
-}
-__device__ __forceinline__ void st_peer(uint32_t a, double v) {
-    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
-}
-__device__ __forceinline__ uint32_t cluster_rank() {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-__device__ __forceinline__ void cluster_sync_all() {
-    asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
-}
-
 // A row's product as it goes to the summing warp.  Float64: the product itself.
 // Float32: two factors scaled by the caller, as their exact product p + e; or, in
 // the right-hand side's sums, whose scale is not known yet, the factors themselves,
@@ -166,8 +145,8 @@ struct ResidentBlock {
     // of the row share the peers
     __device__ void publish(int sp, int64_t i, int lane, T x) {
         if (CL) {
-            const uint32_t at = smem_u32(sm + L.gather) + (uint32_t)((sp * a.N + i) * sizeof(T));
-            for (int p = lane; p < (int)gridDim.x; p += TPR) st_peer(peer_addr(at, p), x);
+            const uint32_t at = smem_addr(sm + L.gather) + (uint32_t)((sp * a.N + i) * sizeof(T));
+            for (int p = lane; p < (int)gridDim.x; p += TPR) st_cluster(peer_addr(at, p), x);
         } else if (lane == 0) {
             ((T*)ri.gather)[sp * a.N + i] = x;
         }
@@ -177,7 +156,7 @@ struct ResidentBlock {
     }
     __device__ bool sync() {
         if (CL) {
-            cluster_sync_all();
+            cluster_barrier();
             return true;
         }
         return grid_sync(a.bar, target += gridDim.x, a.flags);
@@ -204,7 +183,7 @@ struct ResidentBlock {
             const double s = Term<T>::template sum<RAW, TPR == 1 ? 4 : 2>(terms + k * rows, rows, ln, exp_of(k / KS, k % KS));
             if (CL) {
                 const double t = __shfl_sync(0xffffffffu, s, 0);
-                if (ln < (int)gridDim.x) st_peer(peer_addr(smem_u32(pp + blockIdx.x * RES_SUMS + k), ln), t);
+                if (ln < (int)gridDim.x) st_cluster(peer_addr(smem_addr(pp + blockIdx.x * RES_SUMS + k), ln), t);
             } else if (ln == 0) {
                 __stcg(pp + (int64_t)blockIdx.x * RES_SUMS + k, s);
             }
@@ -333,7 +312,7 @@ __global__ void __launch_bounds__(res_threads<T>(), 1) resident_kernel(Args<T> a
     double bnorm = 0.0, limit2 = 0.0, rho = 0.0, rho_prev = 1.0, alpha = 1.0, omega = 1.0, res2 = 0.0;
     bool active = false, fail = false;
     int iters = 0, it = 0, nhist = ri.nhist;
-    if (CL) cluster_sync_all();   // every block of the cluster runs before its shared memory is written
+    if (CL) cluster_barrier();   // every block of the cluster runs before its shared memory is written
 
     for (int64_t step = 0; step < ri.nsteps; ++step) {
         const StepCoef<T> kc = step_coef_at(a, nhist, (int)step);
@@ -563,35 +542,19 @@ ResidentPlan resident_plan(const GroupInfo& gi, int64_t N, int ns, int sms) {
     return best;
 }
 
-template <typename T, int TPR, int NS>
-rbffd_status resident_launch_as(Args<T>& a, const ResidentPlan& p, const ResidentInfo& ri, cudaStream_t st) {
-    const int threads = std::max(64, p.spb * 32 * TPR);   // at least a warp per species
-    if (p.cluster) {
-        auto* fn = resident_kernel<T, TPR, NS, true>;
-        RBFFD_TRY(allow_shared((const void*)fn));
-        RBFFD_CUDA_TRY(cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(p.blocks);
-        cfg.blockDim = dim3(threads);
-        cfg.dynamicSmemBytes = p.smem;
-        cfg.stream = st;
-        cudaLaunchAttribute at;
-        at.id = cudaLaunchAttributeClusterDimension;
-        at.val.clusterDim.x = p.blocks;
-        at.val.clusterDim.y = at.val.clusterDim.z = 1;
-        cfg.attrs = &at;
-        cfg.numAttrs = 1;
-        RBFFD_CUDA_TRY(cudaLaunchKernelEx(&cfg, fn, a, ri));
-    } else {
-        auto* fn = resident_kernel<T, TPR, NS, false>;
-        RBFFD_TRY(allow_shared((const void*)fn));
-        RBFFD_CUDA_TRY(cudaMemsetAsync(a.bar, 0, sizeof(unsigned long long), st));
-        ResidentInfo r = ri;
-        void* args[] = {&a, &r};
-        RBFFD_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)fn, dim3(p.blocks), dim3(threads), args, p.smem, st));
+// the kernel of a form; float64 rows have one lane each
+template <typename T, int NS, bool CL>
+const void* resident_fn(int tpr) {
+    if constexpr (sizeof(T) == 4) {
+        if (tpr == 4) return (const void*)resident_kernel<T, 4, NS, CL>;
+        if (tpr == 2) return (const void*)resident_kernel<T, 2, NS, CL>;
     }
-    note_launch();
-    return RBFFD_OK;
+    return (const void*)resident_kernel<T, 1, NS, CL>;
+}
+template <typename T>
+const void* resident_fn(const ResidentPlan& p, int ns) {
+    if (p.cluster) return ns == 1 ? resident_fn<T, 1, true>(p.tpr) : resident_fn<T, 2, true>(p.tpr);
+    return ns == 1 ? resident_fn<T, 1, false>(p.tpr) : resident_fn<T, 2, false>(p.tpr);
 }
 
 template <typename T>
@@ -605,12 +568,28 @@ rbffd_status resident_launch(Args<T>& a, const ResidentPlan& p, int nhist, int64
     ri.nhist = nhist;
     ri.gather = gather;
     ri.part = part;
-    if (a.ns == 1) {
-        if (p.tpr == 1) return resident_launch_as<T, 1, 1>(a, p, ri, st);
-        if (sizeof(T) == 4 && p.tpr == 2) return resident_launch_as<T, 2, 1>(a, p, ri, st);
-        return resident_launch_as<T, 4, 1>(a, p, ri, st);
+    const void* fn = resident_fn<T>(p, a.ns);
+    RBFFD_TRY(allow_shared(fn));
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(p.blocks);
+    cfg.blockDim = dim3(std::max(64, p.spb * 32 * p.tpr));   // at least a warp per species
+    cfg.dynamicSmemBytes = p.smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at;
+    if (p.cluster) {
+        RBFFD_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+        at.id = cudaLaunchAttributeClusterDimension;
+        at.val.clusterDim.x = p.blocks;
+        at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    } else {
+        RBFFD_CUDA_TRY(cudaMemsetAsync(a.bar, 0, sizeof(unsigned long long), st));
+        at.id = cudaLaunchAttributeCooperative;
+        at.val.cooperative = 1;
     }
-    if (p.tpr == 1) return resident_launch_as<T, 1, 2>(a, p, ri, st);
-    if (sizeof(T) == 4 && p.tpr == 2) return resident_launch_as<T, 2, 2>(a, p, ri, st);
-    return resident_launch_as<T, 4, 2>(a, p, ri, st);
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    void* args[] = {&a, &ri};
+    RBFFD_CUDA_TRY(cudaLaunchKernelExC(&cfg, fn, args));
+    note_launch();
+    return RBFFD_OK;
 }
