@@ -14,6 +14,7 @@
 // phase-kernel section below says why and how).  A direct step is three
 // launches: right-hand side, substitutions (lu.cu), report.
 #include "common.cuh"
+#include "step_plan.cuh"
 
 #include <algorithm>
 #include <climits>
@@ -64,6 +65,8 @@ struct rbffd_step_ws {
     PhaseCtl* ctl;                    // phase-kernel path: loop state
     double* pp;                       //   per-block partial sums
     double* rpart;                    // resident kernel: per-block sums of two reductions
+    rbffd::ResidentPlan plan[2];      //   and its shape by number of species
+    bool planned[2];
 };
 
 namespace rbffd {
@@ -1185,7 +1188,12 @@ rbffd_status run_steps(Args<T>& a, rbffd_step_ws* ws, int64_t nsteps, bool use_g
     static_assert(sizeof(Args<T>) <= sizeof(ws->graph_args), "graph key too small");
     if (!lu && nsteps > 0) {
         // operators that fit the chip's shared memory: one launch for all steps
-        const ResidentPlan plan = resident_plan<T>(a.gi, a.N, a.ns, sm_count());
+        ResidentPlan& plan = ws->plan[a.ns - 1];
+        if (!ws->planned[a.ns - 1]) {
+            plan = resident_plan<T>(a.gi, a.N, a.ns, sm_count(),
+                                    [&](const ResidentPlan& p) { return cluster_resides<T>(p, a.ns); });
+            ws->planned[a.ns - 1] = true;
+        }
         if (plan.blocks > 0)
             return resident_launch(a, plan, nhist, nsteps, ws->vec, ws->rpart, st);
     }
@@ -1289,8 +1297,7 @@ extern "C" rbffd_status rbffd_step_imex(rbffd_op* op, rbffd_state* s, const rbff
         ws = op->step = nullptr;
     }
     if (!ws) {
-        ws = new rbffd_step_ws();
-        memset(ws, 0, sizeof(*ws));
+        ws = new rbffd_step_ws();   // value-initialised: all zero
         op->step = ws;
         ws->elem = elem;
         ws->N = op->N;

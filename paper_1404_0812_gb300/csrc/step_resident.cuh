@@ -30,13 +30,6 @@
 //
 // Included by step.cu inside its anonymous namespace.
 
-constexpr int RES_SUMS = 6;        // sums of one reduction, at most
-constexpr int RES_CLUSTER = 16;    // blocks of a cluster
-
-// threads per block, at most (float64 rows hold twice the registers)
-template <typename T>
-constexpr int res_threads() { return sizeof(T) == 8 ? 512 : 1024; }
-
 struct ResidentInfo {
     int spb;             // slices of 32 rows per block
     int max_elems;       // matrix elements of a block, at most
@@ -104,31 +97,7 @@ struct Term<float> {
     }
 };
 
-// what one lane per species decides and every thread of the block reads (the
-// scalar arithmetic is float64: on all warps it would cost more than the
-// products)
-template <typename T>
-struct ResidentScalars {
-    T beta[2], alpha[2], omega[2];
-    int act[2], early[2], zero[2];
-    int e0[2], e[2];   // exponents of r-hat and of the iteration's vectors in the sums
-};
-
-// shared memory of a block, in this order (all offsets multiples of 16 bytes)
-template <typename T>
-struct ResidentSmem {
-    size_t w, idx, gather, terms, part, scal, total;
-    __host__ __device__ ResidentSmem(int max_elems, int rows, int64_t N, int ns, bool cluster) {
-        auto up = [](size_t x) { return (x + 15) & ~(size_t)15; };
-        w = 0;
-        idx = up(w + (size_t)max_elems * sizeof(T));
-        gather = up(idx + (size_t)max_elems * sizeof(int32_t));
-        terms = up(gather + (cluster ? (size_t)ns * N * sizeof(T) : 0));
-        part = up(terms + (size_t)RES_SUMS * rows * sizeof(typename Term<T>::type));
-        scal = up(part + (cluster ? 2 * RES_CLUSTER * RES_SUMS * sizeof(double) : 0));
-        total = up(scal + sizeof(ResidentScalars<T>));
-    }
-};
+static_assert(sizeof(Term<float>::type) == RES_TERM && sizeof(Term<double>::type) == RES_TERM, "size of a term");
 
 // one block's view of the synchronisations
 template <typename T, int TPR, bool CL>
@@ -487,61 +456,6 @@ __global__ void __launch_bounds__(res_threads<T>(), 1) resident_kernel(Args<T> a
         if (lead) (k == 0 ? a.u : a.v)[node] = x[k];
 }
 
-// A plan of the resident kernel for an operator: TPR lanes per row, slices per
-// block, blocks and form; blocks = 0 when the operator does not fit.
-struct ResidentPlan {
-    int blocks = 0, tpr = 1, spb = 0, max_elems = 0;
-    bool cluster = false;
-    size_t smem = 0;
-};
-
-// elements of the largest run of spb consecutive slices
-inline int64_t largest_block(const GroupInfo& gi, int spb, int64_t* slices) {
-    std::vector<int64_t> start(1, 0);   // element offset of each slice
-    for (int g = 0; g < gi.ngroups; ++g) {
-        const int64_t ns = (gi.row_begin[g + 1] - gi.row_begin[g] + 31) / 32;
-        for (int64_t k = 0; k < ns; ++k) start.push_back(start.back() + (int64_t)32 * gi.npad[g]);
-    }
-    const int64_t n = (int64_t)start.size() - 1;
-    int64_t most = 0;
-    for (int64_t b = 0; b < n; b += spb) most = std::max(most, start[std::min(n, b + spb)] - start[b]);
-    *slices = n;
-    return most;
-}
-
-constexpr size_t RES_SMEM_MAX = 227 * 1024;
-
-template <typename T>
-ResidentPlan resident_plan(const GroupInfo& gi, int64_t N, int ns, int sms) {
-    ResidentPlan best;
-    for (int form = 0; form < 2 && !best.blocks; ++form) {
-        ResidentPlan p;
-        p.cluster = form == 0;
-        int64_t slices = 0;
-        largest_block(gi, 1, &slices);
-        const int64_t blocks = std::min<int64_t>(slices, p.cluster ? RES_CLUSTER : sms);
-        p.spb = (int)((slices + blocks - 1) / blocks);
-        if (p.spb * 32 > res_threads<T>()) continue;
-        p.blocks = (int)((slices + p.spb - 1) / p.spb);
-        if (p.cluster)   // a power of two; the last blocks may have no rows
-            for (int c = 1;; c *= 2)
-                if (c >= p.blocks) {
-                    p.blocks = c;
-                    break;
-                }
-        const int64_t elems = largest_block(gi, p.spb, &slices);
-        if (elems * (int64_t)(sizeof(T) + 4) > (int64_t)RES_SMEM_MAX) continue;
-        p.max_elems = (int)elems;
-        p.smem = ResidentSmem<T>(p.max_elems, p.spb * 32, N, ns, p.cluster).total;
-        if (p.smem > RES_SMEM_MAX) continue;
-        // float64 rows gain nothing from more lanes (the float64 unit is the
-        // bound); float32 ones take up to four
-        while (sizeof(T) == 4 && p.tpr < 4 && p.spb * 32 * p.tpr * 2 <= res_threads<T>()) p.tpr *= 2;
-        best = p;
-    }
-    return best;
-}
-
 // the kernel of a form; float64 rows have one lane each
 template <typename T, int NS, bool CL>
 const void* resident_fn(int tpr) {
@@ -557,6 +471,43 @@ const void* resident_fn(const ResidentPlan& p, int ns) {
     return ns == 1 ? resident_fn<T, 1, false>(p.tpr) : resident_fn<T, 2, false>(p.tpr);
 }
 
+// a launch of the plan's kernel, and whether the device can hold its cluster (the
+// launch of a cluster that no partition of the device has room for fails)
+template <typename T>
+rbffd_status resident_config(const ResidentPlan& p, const void* fn, cudaLaunchConfig_t* cfg,
+                             cudaLaunchAttribute* at) {
+    RBFFD_TRY(allow_shared(fn));
+    memset(cfg, 0, sizeof(*cfg));
+    cfg->gridDim = dim3(p.blocks);
+    cfg->blockDim = dim3(std::max(64, p.spb * 32 * p.tpr));   // at least a warp per species
+    cfg->dynamicSmemBytes = p.smem;
+    if (p.cluster) {
+        RBFFD_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+        at->id = cudaLaunchAttributeClusterDimension;
+        at->val.clusterDim.x = p.blocks;
+        at->val.clusterDim.y = at->val.clusterDim.z = 1;
+    } else {
+        at->id = cudaLaunchAttributeCooperative;
+        at->val.cooperative = 1;
+    }
+    cfg->attrs = at;
+    cfg->numAttrs = 1;
+    return RBFFD_OK;
+}
+template <typename T>
+bool cluster_resides(const ResidentPlan& p, int ns) {
+    const void* fn = resident_fn<T>(p, ns);
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute at;
+    int n = 0;
+    if (resident_config<T>(p, fn, &cfg, &at) != RBFFD_OK) return false;
+    if (cudaOccupancyMaxActiveClusters(&n, fn, &cfg) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    return n >= 1;
+}
+
 template <typename T>
 rbffd_status resident_launch(Args<T>& a, const ResidentPlan& p, int nhist, int64_t nsteps, void* gather, double* part,
                              cudaStream_t st) {
@@ -569,25 +520,11 @@ rbffd_status resident_launch(Args<T>& a, const ResidentPlan& p, int nhist, int64
     ri.gather = gather;
     ri.part = part;
     const void* fn = resident_fn<T>(p, a.ns);
-    RBFFD_TRY(allow_shared(fn));
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(p.blocks);
-    cfg.blockDim = dim3(std::max(64, p.spb * 32 * p.tpr));   // at least a warp per species
-    cfg.dynamicSmemBytes = p.smem;
-    cfg.stream = st;
+    cudaLaunchConfig_t cfg;
     cudaLaunchAttribute at;
-    if (p.cluster) {
-        RBFFD_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-        at.id = cudaLaunchAttributeClusterDimension;
-        at.val.clusterDim.x = p.blocks;
-        at.val.clusterDim.y = at.val.clusterDim.z = 1;
-    } else {
-        RBFFD_CUDA_TRY(cudaMemsetAsync(a.bar, 0, sizeof(unsigned long long), st));
-        at.id = cudaLaunchAttributeCooperative;
-        at.val.cooperative = 1;
-    }
-    cfg.attrs = &at;
-    cfg.numAttrs = 1;
+    RBFFD_TRY(resident_config<T>(p, fn, &cfg, &at));
+    cfg.stream = st;
+    if (!p.cluster) RBFFD_CUDA_TRY(cudaMemsetAsync(a.bar, 0, sizeof(unsigned long long), st));
     void* args[] = {&a, &ri};
     RBFFD_CUDA_TRY(cudaLaunchKernelExC(&cfg, fn, args));
     note_launch();
