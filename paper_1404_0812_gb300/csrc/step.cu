@@ -64,6 +64,8 @@ struct rbffd_step_ws {
     double* ywork;                    // the LU substitutions' work: per species 2 N + 16 float64
     PhaseCtl* ctl;                    // phase-kernel path: loop state
     double* pp;                       //   per-block partial sums
+    int* more_host;                   //   host loop: pinned word in which a phase says whether the loop goes on
+    int more_seq;                     //   and the number of the last phase that was launched to do so
     double* rpart;                    // resident kernel: per-block sums of two reductions
     rbffd::ResidentPlan plan[2];      //   and its shape by number of species
     bool planned[2];
@@ -86,6 +88,7 @@ void step_ws_free(rbffd_step_ws* ws) {
     cudaFree(ws->ywork);
     cudaFree(ws->ctl);
     cudaFree(ws->pp);
+    if (ws->more_host) cudaFreeHost(ws->more_host);
     cudaFree(ws->rpart);
     delete ws;
 }
@@ -123,6 +126,8 @@ struct Args {
     PhaseCtl* ctl;                         // phase-kernel path: loop state and totals
     double* pp;                            //   per-block partial sums (blocks x 8)
     cudaGraphConditionalHandle cond;       //   WHILE handle of the step graph (0: host loop)
+    int* more_host;                        //   host loop: where R and E say 2 more_seq + (the loop goes on)
+    int more_seq;
 };
 
 enum { VB = 0, VR = 1, VRH = 2, VP = 3, VQ = 4, VS = 5, VT = 6 };
@@ -624,11 +629,13 @@ __device__ const double* phase_reduce(const A (&v)[K], double* pp, unsigned int*
     return tot;
 }
 
-// the loop continues while a species runs (m: ballot of the deciding lanes)
-__device__ __forceinline__ void set_more(PhaseCtl* c, cudaGraphConditionalHandle h, int more) {
+// the loop continues while a species runs
+template <typename T>
+__device__ __forceinline__ void set_more(const Args<T>& a, int more) {
     if (threadIdx.x == 0) {
-        c->more = more;
-        if (h) cudaGraphSetConditional(h, (unsigned)more);
+        a.ctl->more = more;
+        if (a.cond) cudaGraphSetConditional(a.cond, (unsigned)more);
+        if (a.more_host) *(volatile int*)a.more_host = 2 * a.more_seq + more;
     }
 }
 
@@ -674,7 +681,7 @@ __global__ void __launch_bounds__(PT, PT_MINB) phase_R(Args<T> a) {
         c->s[k] = z;
         c->it = 0;
         const unsigned m = __ballot_sync(3u, z.active);
-        set_more(c, a.cond, m != 0 && a.maxit > 0);
+        set_more(a, m != 0 && a.maxit > 0);
     }
 }
 
@@ -708,6 +715,7 @@ __device__ __forceinline__ void st4v(double* p, const double (&w)[4]) {
 template <typename T>
 __global__ void __launch_bounds__(PV, PV_BPS) phase_A(Args<T> a) {
     const PhaseCtl* c = a.ctl;
+    if (!c->more) return;   // (an iteration the host loop launched ahead)
     const int64_t S = (int64_t)gridDim.x * PV, t0 = blockIdx.x * (int64_t)PV + threadIdx.x;
     for (int k = 0; k < a.ns; ++k) {
         if (!c->s[k].actA) continue;
@@ -753,6 +761,7 @@ __device__ __forceinline__ int64_t back_row(int64_t k, int64_t Np) { return Np -
 template <typename T>
 __global__ void __launch_bounds__(PT, PT_MINB) phase_B(Args<T> a) {
     PhaseCtl* c = a.ctl;
+    if (!c->more) return;   // (an iteration the host loop launched ahead)
     const bool a0 = c->s[0].actA, a1 = a.ns == 2 && c->s[1].actA;
     const StepCoef<T> kc = step_coef(a);
     using PA = PhaseAcc<T>;
@@ -794,6 +803,7 @@ __global__ void __launch_bounds__(PT, PT_MINB) phase_B(Args<T> a) {
 template <typename T>
 __global__ void __launch_bounds__(PV, PV_BPS) phase_C(Args<T> a) {
     PhaseCtl* c = a.ctl;
+    if (!c->more) return;   // (an iteration the host loop launched ahead)
     using PA = PhaseAcc<T>;
     typename PA::type d[2];
     for (auto& x : d) acc_zero(x);
@@ -852,6 +862,7 @@ __global__ void __launch_bounds__(PV, PV_BPS) phase_C(Args<T> a) {
 template <typename T>
 __global__ void __launch_bounds__(PT, PT_MINB) phase_D(Args<T> a) {
     PhaseCtl* c = a.ctl;
+    if (!c->more) return;   // (an iteration the host loop launched ahead)
     const StepCoef<T> kc = step_coef(a);
     const bool two = a.ns == 2;
     const bool e0 = c->s[0].early, e1 = two && c->s[1].early;
@@ -905,6 +916,7 @@ __device__ __forceinline__ void e_update(T alpha, T omega, T& x, T p, T s, T t, 
 template <typename T>
 __global__ void __launch_bounds__(PV, PV_BPS) phase_E(Args<T> a) {
     PhaseCtl* c = a.ctl;
+    if (!c->more) return;   // (an iteration the host loop launched ahead)
     using PA = PhaseAcc<T>;
     typename PA::type d[4];
     for (auto& x : d) acc_zero(x);
@@ -986,7 +998,7 @@ __global__ void __launch_bounds__(PV, PV_BPS) phase_E(Args<T> a) {
         const unsigned m = __ballot_sync(3u, z.active);   // both lanes have read c->it
         c->s[k] = z;
         c->it = it;
-        set_more(c, a.cond, m != 0 && it < a.maxit);
+        set_more(a, m != 0 && it < a.maxit);
     }
 }
 
@@ -1101,21 +1113,49 @@ void phase_grids(const Args<T>& a, unsigned* g_rows, unsigned* g_vec) {
 }
 
 // One step of the phase-kernel path from the host (no graph): R, then the
-// iterations while the loop state says so (the condition is read back after
-// each iteration), then F -- the same kernels and arithmetic as the graph.
+// iterations while the loop state says so, then F -- the same kernels and
+// arithmetic as the graph.  R and E write into pinned host memory whether the loop
+// goes on, and an iteration is launched before its predecessor has done so (it does
+// nothing if the loop is over): with a copy and a wait between iterations the GPU
+// idled for longer than the phases of thin rows take (one species in float64,
+// n = 7, 120k rows: 331 us a step, so 283; the cooperative
+// kernel that these rows had before 313, replayed 226).
 template <typename T>
-rbffd_status phased_step_host(Args<T>& a, rbffd_step_ws* ws, cudaStream_t st) {
+rbffd_status phased_step_host(Args<T> a, rbffd_step_ws* ws, cudaStream_t st) {
     unsigned gr, gv;
     phase_grids(a, &gr, &gv);
     a.cond = 0;
+    if (!ws->more_host) {
+        RBFFD_CUDA_TRY(cudaMallocHost(&ws->more_host, sizeof(int)));
+        *ws->more_host = 0;
+    }
+    a.more_host = ws->more_host;
+    auto next = [&] { a.more_seq = ws->more_seq = (ws->more_seq + 1) & 0x3fffffff; };
+    // what phase `seq` said; a later word means that it said yes
+    auto goes_on = [&](int seq, bool* more) -> rbffd_status {
+        for (int64_t polls = 1;; ++polls) {
+            const int word = *(volatile int*)ws->more_host;
+            if (((word >> 1) - seq & 0x3fffffff) < 0x20000000) {
+                *more = (word >> 1) != seq || (word & 1);
+                return RBFFD_OK;
+            }
+            if (polls % 4096 == 0) {   // the stream drained or failed without a word
+                const cudaError_t e = cudaStreamQuery(st);
+                if (e == cudaErrorNotReady) continue;
+                RBFFD_CUDA_TRY(e);
+                if (((*(volatile int*)ws->more_host >> 1) - seq & 0x3fffffff) < 0x20000000) continue;
+                set_error("the steps' loop state did not arrive");
+                return RBFFD_ECUDA;
+            }
+        }
+    };
+    next();
     phase_R<T><<<gr, PT, 0, st>>>(a);
     note_launch();
     RBFFD_CUDA_TRY(cudaGetLastError());
-    for (;;) {
-        int more = 0;
-        RBFFD_CUDA_TRY(cudaMemcpyAsync(&more, &ws->ctl->more, sizeof(int), cudaMemcpyDeviceToHost, st));
-        RBFFD_CUDA_TRY(cudaStreamSynchronize(st));
-        if (!more) break;
+    for (bool more = true; more;) {
+        const int seq = a.more_seq;
+        next();
         phase_A<T><<<gv, PV, 0, st>>>(a);
         phase_B<T><<<gr, PT, 0, st>>>(a);
         phase_C<T><<<gv, PV, 0, st>>>(a);
@@ -1123,6 +1163,7 @@ rbffd_status phased_step_host(Args<T>& a, rbffd_step_ws* ws, cudaStream_t st) {
         phase_E<T><<<gv, PV, 0, st>>>(a);
         note_launch(5);
         RBFFD_CUDA_TRY(cudaGetLastError());
+        RBFFD_TRY(goes_on(seq, &more));
     }
     phase_F<T><<<gr, PT, 0, st>>>(a);
     note_launch();
