@@ -20,15 +20,21 @@ namespace {
 constexpr int BOX_THREADS = 256;
 
 // bounding box of n boxes (in: 6 doubles each, lo then hi) or, with X, of
-// nodes: one box per block into out (min and max are exact: any order)
+// nodes: one box per block into out (min and max are exact: any order); a node that
+// is not finite makes the box infinite
 __global__ void __launch_bounds__(BOX_THREADS) bbox_blocks(const double* __restrict__ X, const double* __restrict__ in,
                                                           int64_t n, double* __restrict__ out) {
     __shared__ double w[6][BOX_THREADS / 32];
     double v[6] = {INFINITY, INFINITY, INFINITY, -INFINITY, -INFINITY, -INFINITY};
     for (int64_t i = blockIdx.x * (int64_t)BOX_THREADS + threadIdx.x; i < n; i += (int64_t)gridDim.x * BOX_THREADS)
         for (int a = 0; a < 3; ++a) {
-            v[a] = fmin(v[a], X ? X[3 * i + a] : in[6 * i + a]);
-            v[3 + a] = fmax(v[3 + a], X ? X[3 * i + a] : in[6 * i + 3 + a]);
+            double lo = X ? X[3 * i + a] : in[6 * i + a], hi = X ? lo : in[6 * i + 3 + a];
+            if (X && (__double2hiint(lo) & 0x7ff00000) == 0x7ff00000) {   // (fmin and fmax would drop a NaN)
+                lo = -INFINITY;
+                hi = INFINITY;
+            }
+            v[a] = fmin(v[a], lo);
+            v[3 + a] = fmax(v[3 + a], hi);
         }
     for (int o = 16; o > 0; o >>= 1)
         for (int a = 0; a < 3; ++a) {
