@@ -988,6 +988,11 @@ rbffd_status rbffd_mlp_train(rbffd_mlp* m, const float* feats, const float* targ
     if (s != RBFFD_OK) return s;
     int32_t* perm_d = nullptr;
     RBFFD_CUDA_TRY(pool_alloc(&perm_d, count * sizeof(int32_t), st));
+    struct Freed {   // whichever way the call ends
+        int32_t* p;
+        cudaStream_t st;
+        ~Freed() { cudaFreeAsync(p, st); }
+    } freed{perm_d, st};
     std::vector<int32_t> perm(count), next;
     for (int64_t i = 0; i < count; ++i) perm[i] = (int32_t)i;
     std::mt19937_64 rng(seed);
@@ -1029,9 +1034,8 @@ rbffd_status rbffd_mlp_train(rbffd_mlp* m, const float* feats, const float* targ
             RBFFD_CUDA_TRY(cudaMemcpyAsync(&gave_up, barrier_words(m) + 1, sizeof(int), cudaMemcpyDeviceToHost, st));
         RBFFD_CUDA_TRY(cudaStreamSynchronize(st));
         if (gave_up) {
-            cudaFreeAsync(perm_d, st);
             set_error("rbffd_mlp_train: a grid barrier of the training kernel gave up");
-            return RBFFD_ECUDA;
+            return RBFFD_TIMEOUT;
         }
         perm.swap(next);
         if (loss_host) {
@@ -1040,7 +1044,6 @@ rbffd_status rbffd_mlp_train(rbffd_mlp* m, const float* feats, const float* targ
             loss_host[ep] = (float)(tot / (double)count);
         }
     }
-    cudaFreeAsync(perm_d, st);
     RBFFD_CUDA_TRY(cudaStreamSynchronize(st));
     return RBFFD_OK;
 }

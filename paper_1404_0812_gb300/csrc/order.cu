@@ -264,12 +264,11 @@ rbffd_status sort_keys_device(uint64_t* key, int64_t N, int32_t* perm, cudaStrea
     }
     RBFFD_TRY(allow_shared((const void*)sort_scatter));
     const int ntiles = (int)((N + TILE - 1) / TILE);
+    // one allocation: nothing is left behind where it fails
     uint64_t* key2 = nullptr;
-    int32_t *val = nullptr, *val2 = nullptr, *counts = nullptr;
-    RBFFD_CUDA_TRY(pool_alloc(&key2, (size_t)N * sizeof(uint64_t), st));
-    RBFFD_CUDA_TRY(pool_alloc(&val, (size_t)N * sizeof(int32_t), st));
-    RBFFD_CUDA_TRY(pool_alloc(&val2, (size_t)N * sizeof(int32_t), st));
-    RBFFD_CUDA_TRY(pool_alloc(&counts, ((size_t)BINS * ntiles + BINS) * sizeof(int32_t), st));
+    RBFFD_CUDA_TRY(pool_alloc(&key2, (size_t)N * (sizeof(uint64_t) + 2 * sizeof(int32_t)) +
+                                         (size_t)BINS * (ntiles + 1) * sizeof(int32_t), st));
+    int32_t *val = reinterpret_cast<int32_t*>(key2 + N), *val2 = val + N, *counts = val2 + N;
     int32_t* totals = counts + (size_t)BINS * ntiles;
     const uint64_t* k_in = key;
     uint64_t* k_out = key2;
@@ -282,16 +281,14 @@ rbffd_status sort_keys_device(uint64_t* key, int64_t N, int32_t* perm, cudaStrea
         sort_scatter<<<ntiles, SORT_THREADS, smem, st>>>(k_in, v_in, N, 8 * p, ntiles, counts, totals,
                                                         final_pass ? nullptr : k_out, final_pass ? perm : v_out);
         note_launch(3);
-        RBFFD_CUDA_TRY(cudaGetLastError());
         k_in = k_out;
         k_out = k_out == key ? key2 : key;
         v_in = v_out;
         v_out = v_out == val ? val2 : val;
     }
+    const cudaError_t e = cudaGetLastError();
     cudaFreeAsync(key2, st);
-    cudaFreeAsync(val, st);
-    cudaFreeAsync(val2, st);
-    cudaFreeAsync(counts, st);
+    RBFFD_CUDA_TRY(e);
     return RBFFD_OK;
 }
 
