@@ -68,14 +68,8 @@ cudaError_t pool_alloc_bytes(void** p, size_t bytes, cudaStream_t st) {
     return cudaMallocFromPoolAsync(p, bytes, pool, st);
 }
 
-rbffd_status allow_shared(const void* kernel) {
-    int dev = 0, most = 0;
-    cudaFuncAttributes fa;
-    RBFFD_CUDA_TRY(cudaGetDevice(&dev));
-    RBFFD_CUDA_TRY(cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-    RBFFD_CUDA_TRY(cudaFuncGetAttributes(&fa, kernel));
-    RBFFD_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        most - (int)fa.sharedSizeBytes));
+rbffd_status allow_shared(const void* kernel, int kept) {
+    RBFFD_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - kept));
     return RBFFD_OK;
 }
 

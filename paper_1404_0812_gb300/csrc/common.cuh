@@ -223,8 +223,9 @@ rbffd_status lu_solve_step(rbffd_lu* const (&fac)[4][2], int nspecies, const voi
 void lu_free(rbffd_lu* lu);
 int sm_count();
 
-// Lets launches of a kernel ask for any dynamic shared memory a block can have on
-// this device (api.cu).  The limit belongs to the function, not to a launch: set to
-// each launch's own size, it made another thread's larger launch fail.
-rbffd_status allow_shared(const void* kernel);
+// Lets launches of a kernel ask for all of a block's 227 KB but `kept` bytes (at least
+// the kernel's static arrays) as dynamic shared memory (api.cu).  The limit belongs to
+// the function, not to a launch: set to each launch's own size, it made another
+// thread's larger launch fail.
+rbffd_status allow_shared(const void* kernel, int kept = 1024);
 }  // namespace rbffd

@@ -744,7 +744,7 @@ rbffd_status launch_solve(const SolveArgs<T, TV>& a, int nspecies, bool intercha
     const int D = solve_depth<T>(a.kl, a.ku);
     if (D > 0 && !interchanges) {
         const size_t smem = (size_t)block_slots(a.kl + a.ku) * NB * sizeof(T);
-        RBFFD_TRY(allow_shared((const void*)solve_blocks_kernel<T, TV>));
+        RBFFD_TRY(allow_shared((const void*)solve_blocks_kernel<T, TV>, 12 * 1024));
         solve_blocks_kernel<T, TV><<<nspecies * BLK_CTAS, BLK_THREADS, smem, st>>>(a);
         note_launch();
         RBFFD_CUDA_TRY(cudaGetLastError());
@@ -796,7 +796,7 @@ rbffd_status factor_t(const rbffd_op* op, rbffd_lu* lu, cudaStream_t st) {
     RBFFD_CUDA_TRY(cudaMemsetAsync(flags, 0, 3 * sizeof(int), st));
     a.bar = bar;
     a.flags = flags;
-    RBFFD_TRY(allow_shared((const void*)factor_kernel<T>));
+    RBFFD_TRY(allow_shared((const void*)factor_kernel<T>, 12 * 1024));
     int per_sm = 0;
     RBFFD_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, factor_kernel<T>, FACTOR_THREADS, smem));
     RBFFD_CHECK_ARG(per_sm >= 1, "banded LU: the factorisation kernel does not fit on an SM");

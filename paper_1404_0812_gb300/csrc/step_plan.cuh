@@ -67,8 +67,8 @@ inline int64_t largest_block(const GroupInfo& gi, int64_t slices, int spb) {
     return most;
 }
 
-// (a block's share less the grid barrier's own 16 bytes)
-constexpr size_t RES_SMEM_MAX = 227 * 1024 - 16;
+constexpr int RES_STATIC = 16;     // the grid barrier's own bytes
+constexpr size_t RES_SMEM_MAX = 227 * 1024 - RES_STATIC;
 
 // resides(plan): the device has room for the cluster of a plan.  Where it has not (a
 // partition of a GPU may have fewer SMs side by side), the cooperative grid takes the

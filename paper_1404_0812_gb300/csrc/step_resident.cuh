@@ -325,7 +325,9 @@ __global__ void __launch_bounds__(res_threads<T>(), 1) resident_kernel(Args<T> a
 #pragma unroll
         for (int k = 0; k < NS; ++k)
             if (sc.zero[k]) x[k] = T(0);   // b = 0: x = 0
-        const auto both = [&](int k, int) { return 2 * sc.e[k]; };
+        // exponents of the sums' factors and their scales (float32 only)
+        const auto e0 = [&](int k) { return sizeof(T) == 4 ? (int)sc.e0[k] : 0; };
+        const auto e = [&](int k) { return sizeof(T) == 4 ? (int)sc.e[k] : 0; };
         while ((sc.act[0] || (NS == 2 && sc.act[NS - 1])) && it < a.maxit) {
             ++it;
             // ---- A: p = r + beta (p - omega q)
@@ -341,9 +343,9 @@ __global__ void __launch_bounds__(res_threads<T>(), 1) resident_kernel(Args<T> a
 #pragma unroll
             for (int k = 0; k < NS; ++k) {
                 if (sc.act[k]) q[k] = kc.c0 * p[k] - kk[k] * y[k];
-                d1[k][0] = TM::of(PA::scaled(rh[k], unit_scale(sc.e0[k])), PA::scaled(q[k], unit_scale(sc.e[k])));
+                d1[k][0] = TM::of(PA::scaled(rh[k], unit_scale(e0(k))), PA::scaled(q[k], unit_scale(e(k))));
             }
-            if (!B.template reduce<1, NS>(d1, lrow, sums, [&](int k, int) { return sc.e0[k] + sc.e[k]; }, [&](int k, const double (&tot)[1]) {
+            if (!B.template reduce<1, NS>(d1, lrow, sums, [&](int k, int) { return e0(k) + e(k); }, [&](int k, const double (&tot)[1]) {
                     if (active) {
                         alpha = rho / tot[0];
                         if (tot[0] == 0.0 || !isfinite(alpha)) {
@@ -362,9 +364,9 @@ __global__ void __launch_bounds__(res_threads<T>(), 1) resident_kernel(Args<T> a
                     s[k] = r[k] - sc.alpha[k] * q[k];
                     B.publish(k, node, lane, s[k]);
                 }
-                d1[k][0] = TM::of(PA::scaled(s[k], unit_scale(sc.e[k])), PA::scaled(s[k], unit_scale(sc.e[k])));
+                d1[k][0] = TM::of(PA::scaled(s[k], unit_scale(e(k))), PA::scaled(s[k], unit_scale(e(k))));
             }
-            if (!B.template reduce<1, NS>(d1, lrow, sums, both, [&](int k, const double (&tot)[1]) {
+            if (!B.template reduce<1, NS>(d1, lrow, sums, [&](int k, int) { return 2 * e(k); }, [&](int k, const double (&tot)[1]) {
                     const bool early = active && tot[0] <= limit2;
                     if (early) {
                         res2 = tot[0];
@@ -384,11 +386,11 @@ __global__ void __launch_bounds__(res_threads<T>(), 1) resident_kernel(Args<T> a
 #pragma unroll
             for (int k = 0; k < NS; ++k) {
                 if (sc.act[k]) t[k] = kc.c0 * s[k] - kk[k] * y[k];
-                const T ts = PA::scaled(t[k], unit_scale(sc.e[k]));
-                d2[k][0] = TM::of(ts, PA::scaled(s[k], unit_scale(sc.e[k])));
+                const T ts = PA::scaled(t[k], unit_scale(e(k)));
+                d2[k][0] = TM::of(ts, PA::scaled(s[k], unit_scale(e(k))));
                 d2[k][1] = TM::of(ts, ts);
             }
-            if (!B.template reduce<2, NS>(d2, lrow, sums, both, [&](int k, const double (&tot)[2]) {
+            if (!B.template reduce<2, NS>(d2, lrow, sums, [&](int k, int) { return 2 * e(k); }, [&](int k, const double (&tot)[2]) {
                     if (active) {
                         omega = tot[0] / tot[1];
                         if (tot[1] == 0.0 || !isfinite(omega)) {
@@ -407,11 +409,11 @@ __global__ void __launch_bounds__(res_threads<T>(), 1) resident_kernel(Args<T> a
                     x[k] += sc.alpha[k] * p[k] + sc.omega[k] * s[k];
                     r[k] = s[k] - sc.omega[k] * t[k];
                 }
-                const T rs = PA::scaled(r[k], unit_scale(sc.e[k]));
-                d2[k][0] = TM::of(PA::scaled(rh[k], unit_scale(sc.e0[k])), rs);
+                const T rs = PA::scaled(r[k], unit_scale(e(k)));
+                d2[k][0] = TM::of(PA::scaled(rh[k], unit_scale(e0(k))), rs);
                 d2[k][1] = TM::of(rs, rs);
             }
-            if (!B.template reduce<2, NS>(d2, lrow, sums, [&](int k, int j) { return (j ? sc.e[k] : sc.e0[k]) + sc.e[k]; }, [&](int k, const double (&tot)[2]) {
+            if (!B.template reduce<2, NS>(d2, lrow, sums, [&](int k, int j) { return (j ? e(k) : e0(k)) + e(k); }, [&](int k, const double (&tot)[2]) {
                     if (active) {
                         rho_prev = rho;
                         rho = tot[0];
@@ -476,7 +478,7 @@ const void* resident_fn(const ResidentPlan& p, int ns) {
 template <typename T>
 rbffd_status resident_config(const ResidentPlan& p, const void* fn, cudaLaunchConfig_t* cfg,
                              cudaLaunchAttribute* at) {
-    RBFFD_TRY(allow_shared(fn));
+    RBFFD_TRY(allow_shared(fn, RES_STATIC));
     memset(cfg, 0, sizeof(*cfg));
     cfg->gridDim = dim3(p.blocks);
     cfg->blockDim = dim3(std::max(64, p.spb * 32 * p.tpr));   // at least a warp per species
