@@ -1031,9 +1031,7 @@ def run_ours(args):
     step_info = {"ms": round(step_ms, 3), "loop_iterations_per_step": step_its,
                  "ell_passes_per_step": round(step_passes / 10.0, 2),
                  "ell_GB_s": round(ell_gbs, 1),
-                 "path": ("phase kernels under a WHILE graph node"
-                          if N_NODES >= 1024 * torch.cuda.get_device_properties(dev).multi_processor_count
-                          else "cooperative")}
+                 "path": "phase kernels under a WHILE graph node"}   # (1M rows: past the resident kernel)
     hbm = None
     try:
         hbm = json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json")))["hbm_gbs"]
@@ -1100,7 +1098,26 @@ def run_ours(args):
                                    f"Brent eps search, full G^d weights",
                          "one_core": round(cpu1["count"] / cpu1["seconds"], 3)},
     }
-    print(json.dumps(line))
+    print(json.dumps({"details": line}), file=sys.stderr)
+    print(json.dumps(short_line(line)))
+
+
+# what the one line on stdout holds; everything measured beside it (other
+# configurations, phases, steps, training) goes to stderr as one JSON object
+SHORT = {"roofline": ("bound", "kernel", "achieved", "peak", "unit", "frac", "peak_source", "search_ms"),
+         "e2e": ("value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step", "warmup"),
+         "imex_step": ("ms", "ell_GB_s", "ell_frac_of_measured_hbm")}
+DETAILS = ("phases_ms", "learned_speedup", "apply", "mlp_train", "other_configs", "rates")
+
+
+def short_line(line):
+    """The result line without its details: a few hundred bytes per key, so
+    that whoever keeps only the end of the output has all of it."""
+    out = {k: v for k, v in line.items() if k not in DETAILS}
+    for k, keys in SHORT.items():
+        if isinstance(out.get(k), dict):
+            out[k] = {q: out[k][q] for q in keys if q in out[k]}
+    return out
 
 
 def run_reference(args):
