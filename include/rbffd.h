@@ -73,8 +73,10 @@ typedef struct {
     const double* eps_override; /* device, N, or NULL: fixed eps per node (no
                                    search; kappa/evals reported as NaN/0) */
     const rbffd_mlp* mlp[RBFFD_MAX_GROUPS]; /* learned networks (may be NULL) */
-    int block_threads;        /* 0 = autotuned / default launch shape */
-    int blocks_per_sm;        /* 0 = autotuned / default launch shape */
+    int block_threads;        /* launch shape of the lane-per-stencil kernels: */
+    int blocks_per_sm;        /*   non-zero chooses them; both 0: the library's
+                                 choice by stencil size and rows (several lanes
+                                 per stencil where one each leaves the chip idle) */
     double eps_lo;            /* search range of the dimensionless eps * r_s */
     double eps_hi;            /*   (r_s = the stencil's largest centre distance);
                                  0 = unbounded on that side.  A stencil whose
@@ -104,7 +106,11 @@ void rbffd_build_opts_default(rbffd_build_opts* opts);
  * (and its time in *best_ms, -1 when it came from the cache).  Arguments as
  * in rbffd_build_operator; cache_path (may be NULL) is a text file of
  * previous results keyed by device, stencil sizes, kernel and kappa_T; a hit
- * skips the timing.  Synchronises the stream.
+ * skips the timing.  Synchronises the stream.  It times the lane-per-stencil
+ * kernels only, and a shape passed to rbffd_build_operator chooses them: for sets
+ * below about 80,000 nodes (40,000 from n = 57 on, 250,000 or 100,000 with
+ * networks) the default, a shape of zeros, is the faster build (2,562 nodes of n =
+ * 31: 6 against 31 ms).
  */
 rbffd_status rbffd_autotune_build(const double* nodes, const double* normals, int64_t N,
                                   const int32_t* n_per_node, int n_uniform,

@@ -72,7 +72,11 @@ constexpr size_t RES_SMEM_MAX = 227 * 1024 - RES_STATIC;
 
 // resides(plan): the device has room for the cluster of a plan.  Where it has not (a
 // partition of a GPU may have fewer SMs side by side), the cooperative grid takes the
-// operator.
+// operator.  The cluster comes first wherever its shared memory holds the operator (us
+// a step, n = 31, cluster / grid: heat equation in float64, 642 rows 45/69, 2,562
+// 54/71, 3,500 58/75, 5,000 70/72, 6,300 84/74; two species in float32, 642 rows 15/25,
+// 2,562 26/29, 5,000 28/30, 6,300 34/32: its last fifth, above 5k rows, would be as
+// fast or up to a fifth faster on the grid).
 template <typename T, typename F>
 ResidentPlan resident_plan(const GroupInfo& gi, int64_t N, int ns, int sms, F resides) {
     int64_t slices = 0;
@@ -96,8 +100,10 @@ ResidentPlan resident_plan(const GroupInfo& gi, int64_t N, int ns, int sms, F re
         p.max_elems = (int)elems;
         p.smem = ResidentSmem<T>(p.max_elems, p.spb * 32, N, ns, p.cluster).total;
         if (p.smem > RES_SMEM_MAX) continue;
-        // float64 rows gain nothing from more lanes (the float64 unit is the
-        // bound); float32 ones take up to four
+        // float32 rows take up to four lanes, float64 ones have one (us a step, n = 31,
+        // one / two lanes: one species, 642 rows 45/39, 1,280 48/44, 2,562 54/57, 3,500
+        // 58/63, 20k 78/76; two species, 2,562 63/71, 6,300 95/80, 20k 137/140: the
+        // float64 unit is the bound unless a block has few rows)
         while (sizeof(T) == 4 && p.tpr < 4 && p.spb * 32 * p.tpr * 2 <= res_threads<T>()) p.tpr *= 2;
         if (p.cluster && !resides(p)) continue;
         return p;
