@@ -206,9 +206,8 @@ __device__ __forceinline__ StepCoef<T> step_coef(const Args<T>& a) {
     return step_coef_at(a, *((volatile int*)(a.flags + 2)), *((volatile int*)(a.flags + 3)));
 }
 
-// Dot-product accumulators.  Float64 sums and those of a right-hand side are
-// float64.  The float32 sums of an iteration are carried in three float32 values
-// by the dot product DotK with K = 3 (Ogita, Rump & Oishi, "Accurate sum and dot
+// Dot-product accumulators.  Float64 sums are float64.  Float32 sums are carried in
+// three float32 values by the dot product DotK with K = 3 (Ogita, Rump & Oishi, "Accurate sum and dot
 // product", SIAM J. Sci. Comput. 26 (2005), Algorithm 5.10, the last level a plain
 // sum): each product a b split exactly into p + e by an FMA (TwoProduct), sums by
 // Knuth's error-free TwoSum, the errors of the second level added at the end.  The
@@ -251,7 +250,7 @@ __device__ __forceinline__ float unit_scale(int e) { return __int_as_float((127 
 // of 20 bits (by adding and subtracting 1.5 2^23), relative to the largest of them
 // all, and integers are summed exactly by warp reductions.  What is cut off is below
 // 2^-55 of the largest value, a float64 rounding's share.  (With a shuffle tree of
-// Dot3 values, 40k torus, two species: 84.5 us a step, with this 80.)
+// Dot3 values 40k rows of n = 50, two species, took 84.5 us a step, with this 81.)
 struct Fixed {
     long long n;   // value n 2^e
     int e;
@@ -1117,9 +1116,8 @@ void phase_grids(const Args<T>& a, unsigned* g_rows, unsigned* g_vec) {
 // arithmetic as the graph.  R and E write into pinned host memory whether the loop
 // goes on, and an iteration is launched before its predecessor has done so (it does
 // nothing if the loop is over): with a copy and a wait between iterations the GPU
-// idled for longer than the phases of thin rows take (one species in float64,
-// n = 7, 120k rows: 331 us a step, so 283; the cooperative
-// kernel that these rows had before 313, replayed 226).
+// idled for longer than the phases of thin rows take (one species in float64, n = 7,
+// 120k rows: 331 us a step, so 283; replayed 226; one cooperative launch a step 313).
 template <typename T>
 rbffd_status phased_step_host(Args<T> a, rbffd_step_ws* ws, cudaStream_t st) {
     unsigned gr, gv;

@@ -24,9 +24,9 @@
 // Measured against one cooperative launch per step with the matrix streamed
 // from L2 and three blocks for the small operator: 2,562 nodes, n = 31, heat
 // equation in float64, 3.8 iterations per step: 314 -> 52 us per step; 40k
-// torus, n = 50, two species in float32: 320 -> 92 us per step (90 with sums of
-// float32 pairs, which lost accuracy and the range of small and large fields; 97
-// with float64 ones).
+// torus, n = 50, two species in float32: 320 -> 92 us per step (its sums: a sphere of
+// the same size 82 us with these, 78 with pairs of float32 values, which lost accuracy
+// and the range of small and large fields, 85 with float64 ones).
 //
 // Included by step.cu inside its anonymous namespace.
 
